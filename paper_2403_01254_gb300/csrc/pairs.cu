@@ -696,6 +696,10 @@ __device__ __forceinline__ void ldsm_x4_t(unsigned (&r)[4], const void* p) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
 }
+__device__ __forceinline__ void ldsm_x2_t(unsigned (&r)[2], const void* p) {
+    const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(a));
+}
 __device__ __forceinline__ void ldsm_x2(unsigned& r0, unsigned& r1, const void* p) {
     const unsigned a = (unsigned)__cvta_generic_to_shared(p);
     asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(a));
@@ -723,6 +727,14 @@ __device__ __forceinline__ void mma_f16_16816(float (&d)[4], const unsigned (&a)
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
+// The first MMA of a sum: d = A B with the addend a zero operand of its own,
+// so no accumulator registers are cleared beforehand.
+__device__ __forceinline__ void mma_f16_16816_first(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+        "{%10,%10,%10,%10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+}
 
 // (lo, hi) rounded to FP16 (nearest even), lo in the low half
 __device__ __forceinline__ unsigned f16x2_rn(float lo, float hi) {
@@ -730,24 +742,22 @@ __device__ __forceinline__ unsigned f16x2_rn(float lo, float hi) {
     asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
-__device__ __forceinline__ float2 f16x2_to_f32(unsigned v) {
-    float2 r;
-    asm("{\n\t.reg .f16 l, h;\n\tmov.b32 {l, h}, %2;\n\tcvt.f32.f16 %0, l;\n\tcvt.f32.f16 %1, h;\n\t}"
-        : "=f"(r.x), "=f"(r.y) : "r"(v));
-    return r;
-}
-// v0 ~ hi.lo + lo.lo, v1 ~ hi.hi + lo.hi: two FP16 pieces per value (22 bits)
+// v0 ~ hi.lo + lo.lo, v1 ~ hi.hi + lo.hi: two FP16 pieces per value (22 bits).
+// The remainders v - hi are one mixed FP16 x FP16 + FP32 FMA each (exact: hi
+// holds the leading bits of v), without widening hi first.
 __device__ __forceinline__ void split_f16x2(float v0, float v1, unsigned& hi, unsigned& lo) {
     hi = f16x2_rn(v0, v1);
-    const float2 h = f16x2_to_f32(hi);
-    lo = f16x2_rn(v0 - h.x, v1 - h.y);
+    float r0, r1;
+    asm("{\n\t.reg .f16 l, h, m;\n\tmov.b32 {l, h}, %2;\n\tmov.b16 m, 0xBC00;\n\t"
+        "fma.rn.f32.f16 %0, l, m, %3;\n\tfma.rn.f32.f16 %1, h, m, %4;\n\t}"
+        : "=f"(r0), "=f"(r1) : "r"(hi), "f"(v0), "f"(v1));
+    lo = f16x2_rn(r0, r1);
 }
 
-// w when t < thr (the pair is inside r_c), counted in cnt; else 0
-__device__ __forceinline__ float inside_count(float t, float thr, float w, int& cnt) {
+// 1 when t < thr (the pair is inside r_c), else 0
+__device__ __forceinline__ float inside_mask(float t, float thr) {
     float r;
-    asm("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %2, %3;\n\tselp.f32 %0, %4, 0f00000000, p;\n\t@p add.s32 %1, %1, 1;\n\t}"
-        : "=f"(r), "+r"(cnt) : "f"(t), "f"(thr), "f"(w));
+    asm("set.lt.f32.f32 %0, %1, %2;" : "=f"(r) : "f"(t), "f"(thr));
     return r;
 }
 
@@ -768,15 +778,18 @@ struct DenseSmem {
     static constexpr int CL = QL + MAXQ * LW;                     // [32][LW] the batch's candidate label rows
     static constexpr int CG = CL + 32 * LW;                       // [16][12] candidate pairs (2p, 2p+1):
                                                                   //   x0 x0' x1 x1' | x2 x2' thr thr' | xk xk' - -
-    static constexpr int CF = CG + 16 * 12;                       // [32][16] features: FP16 hi (8 words), lo (8);
-                                                                  //   16-byte chunks XOR-swizzled by (c >> 1) & 3;
-                                                                  //   at the unit's end [32 queries][16] FP32 sums
+    static constexpr int CF = CG + 16 * 12;                       // [32][12] features in FP16: hi of features 0..7,
+                                                                  //   tile 1 (hi 8, hi 9, lo 8, lo 9, zeros), lo of
+                                                                  //   features 0..7 (a 48-byte row: conflict-free
+                                                                  //   ldmatrix); at the unit's end [32 queries][12]
+                                                                  //   FP32 sums
     // running per-query sums of the moment MMAs, in the accumulator layout:
     // feature tile 0 as [m tile][lane] float4; feature tile 1 holds only
-    // features 8 and 9 (lanes with t4 = 0), as [m tile][g] float4
-    static constexpr int RUN = CF + 32 * 16;
+    // features 8 and 9, their hi parts in the lanes with t4 = 0 and their lo
+    // parts in those with t4 = 1, as [m tile][g][t4] float4
+    static constexpr int RUN = CF + 32 * 12;
     static constexpr int RUN1 = RUN + (MAXQ / 16) * 32 * 4;
-    static constexpr int RING = RUN1 + (MAXQ / 16) * 8 * 4;      // [CQ_N] float4 candidate ring
+    static constexpr int RING = RUN1 + (MAXQ / 16) * 16 * 4;     // [CQ_N] float4 candidate ring
     static constexpr int ROWS = RING + 4 * CQ_N;                  // [40] stencil rows
     static constexpr int WORDS = ROWS + 40;
 };
@@ -866,12 +879,25 @@ __device__ __forceinline__ void mma_f16_16816_r(float (&d)[4], unsigned a0, unsi
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// s += A B over NKC chunks: BF16 (F16 false) or FP16 operands.
-template <int NKC, bool F16>
+__device__ __forceinline__ void mma_bf16_16816_first(float (&d)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3,
+                                                     unsigned b0, unsigned b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+        "{%10,%10,%10,%10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
+}
+
+// s += A B over NKC chunks: BF16 (F16 false) or FP16 operands; FIRST: s = A B.
+template <int NKC, bool F16, bool FIRST>
 __device__ __forceinline__ void gram_chunks(float (&s)[4], const unsigned (&qa)[2 * NKC], const unsigned (&cb)[NKC]) {
+    if constexpr (FIRST && NKC == 1) s[0] = s[1] = s[2] = s[3] = 0.f;
 #pragma unroll
     for (int kc = 0; kc + 1 < NKC; kc += 2) {
-        if constexpr (F16) mma_f16_16816_r(s, qa[2 * kc], qa[2 * kc + 1], qa[2 * kc + 2], qa[2 * kc + 3], cb[kc], cb[kc + 1]);
+        if (FIRST && kc == 0) {
+            const unsigned a[4] = {qa[0], qa[1], qa[2], qa[3]};
+            if constexpr (F16) mma_f16_16816_first(s, a, cb[0], cb[1]);
+            else mma_bf16_16816_first(s, a[0], a[1], a[2], a[3], cb[0], cb[1]);
+        } else if constexpr (F16) mma_f16_16816_r(s, qa[2 * kc], qa[2 * kc + 1], qa[2 * kc + 2], qa[2 * kc + 3], cb[kc], cb[kc + 1]);
         else mma_bf16_16816_r(s, qa[2 * kc], qa[2 * kc + 1], qa[2 * kc + 2], qa[2 * kc + 3], cb[kc], cb[kc + 1]);
     }
     if constexpr (NKC & 1) {
@@ -972,13 +998,13 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int k0, float
     const int n_mt = (qcount + 15) >> 4;        // m tiles of 16 queries that hold queries
     const u64 KG2 = f2(gp.kg, gp.kg);
     // this lane's running sums (feature tile 0 for every lane, tile 1 for
-    // the lanes holding features 8 and 9), in shared memory
+    // the lanes holding features 8 and 9, hi and lo parts), in shared memory
     float4* run0 = reinterpret_cast<float4*>(wb + L::RUN) + lane;       // [mt * 32]
-    float4* run1 = reinterpret_cast<float4*>(wb + L::RUN1) + g;         // [mt * 8], t4 == 0
+    float4* run1 = reinterpret_cast<float4*>(wb + L::RUN1) + 2 * g + (t4 & 1);   // [mt * 16], t4 < 2
 #pragma unroll
     for (int mt = 0; mt < L::MAXQ / 16; ++mt) {
         run0[32 * mt] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (t4 == 0) run1[8 * mt] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (t4 < 2) run1[16 * mt] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     int cnt = 0;
     int c_s = 0, qhead = 0, qlen = 0;
@@ -1030,16 +1056,15 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int k0, float
             split_f16x2(u0 * u0, u0 * u1, h2, l2);
             split_f16x2(u0 * u2, u1 * u1, h3, l3);
             split_f16x2(u1 * u2, u2 * u2, h4, l4);
-            const int sw = (lane >> 1) & 3;
-            uint4* frow = reinterpret_cast<uint4*>(cf + 16 * lane);
-            frow[0 ^ sw] = make_uint4(h0, h1, h2, h3);
-            frow[1 ^ sw] = make_uint4(h4, 0u, 0u, 0u);
-            frow[2 ^ sw] = make_uint4(l0, l1, l2, l3);
-            frow[3 ^ sw] = make_uint4(l4, 0u, 0u, 0u);
+            uint4* frow = reinterpret_cast<uint4*>(cf + 12 * lane);
+            frow[0] = make_uint4(h0, h1, h2, h3);
+            frow[1] = make_uint4(h4, l4, 0u, 0u);
+            frow[2] = make_uint4(l0, l1, l2, l3);
         }
         qhead = (qhead + nb) & (CQ_N - 1);
         qlen -= nb;
         __syncwarp();
+        u64 n_in = 0ull;     // pairs inside r_c of this lane's elements of the batch, as FP32 counts
         // m tiles one after another, not unrolled: the smaller loop body ran
         // faster (LiDAR 0.344 -> 0.284 ms, window 2.00 -> 1.85 ms, mapping
         // within 1%)
@@ -1064,16 +1089,16 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int k0, float
                 const unsigned* crowp = cl + (8 * nt + (lane & 7)) * LW;
                 unsigned cb[NKC];
                 load_b_chunks<NKC>(cb, crowp);
-                float s[4] = {0.f, 0.f, 0.f, 0.f};
+                float s[4];
                 if constexpr (SPLIT) {
                     // FP32 labels: hi*hi + hi*lo + lo*hi of the FP16 parts
                     unsigned cbl[NKC];
                     load_b_chunks<NKC>(cbl, crowp + PW);
-                    gram_chunks<NKC, true>(s, qa, cb);
-                    gram_chunks<NKC, true>(s, qa, cbl);
-                    gram_chunks<NKC, true>(s, qal, cb);
+                    gram_chunks<NKC, true, true>(s, qa, cb);
+                    gram_chunks<NKC, true, false>(s, qa, cbl);
+                    gram_chunks<NKC, true, false>(s, qal, cb);
                 } else {
-                    gram_chunks<NKC, false>(s, qa, cb);
+                    gram_chunks<NKC, false, true>(s, qa, cb);
                 }
                 const int p = 4 * nt + t4;
                 const ulonglong2 c01 = *reinterpret_cast<const ulonglong2*>(cg + 12 * p);
@@ -1095,28 +1120,32 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int k0, float
                     const u64 T = ffma2(c01.x, QA.x, ffma2(c01.y, QA.y, ffma2(c2t.x, QB.x, QB.y)));
                     const float2 t = f2_split(T);
                     const float2 a = f2_split(ffma2(T, KG2, XK));
-                    const float w0 = s[2 * i] * ex2_approx(a.x), w1 = s[2 * i + 1] * ex2_approx(a.y);
-                    split_f16x2(inside_count(t.x, thr.x, w0, cnt), inside_count(t.y, thr.y, w1, cnt),
-                                ah[nt >> 1][2 * (nt & 1) + i], al[nt >> 1][2 * (nt & 1) + i]);
+                    const u64 in = f2(inside_mask(t.x, thr.x), inside_mask(t.y, thr.y));
+                    n_in = fadd2(n_in, in);
+                    const float2 w = f2_split(fmul2(fmul2(f2(s[2 * i], s[2 * i + 1]), in),
+                                                    f2(ex2_approx(a.x), ex2_approx(a.y))));
+                    split_f16x2(w.x, w.y, ah[nt >> 1][2 * (nt & 1) + i], al[nt >> 1][2 * (nt & 1) + i]);
                 }
             }
             // per query: sum over the batch's candidates of w (1, x, x x^T);
             // feature B fragments (FP16 hi and lo) of each 16-candidate k step
-            float t[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+            float t[2][4];
 #pragma unroll
             for (int ks = 0; ks < 2; ++ks) {
-                unsigned fh[4], fl[4];
-                const int c = 16 * ks + (lane & 7) + 8 * ((lane >> 3) & 1);
-                const int sw = (c >> 1) & 3;
-                const unsigned* rowp = cf + 16 * c;
-                ldsm_x4_t(fh, rowp + 4 * ((lane >> 4) ^ sw));
-                ldsm_x4_t(fl, rowp + 4 * ((2 + (lane >> 4)) ^ sw));
-#pragma unroll
-                for (int n2 = 0; n2 < 2; ++n2) {
-                    mma_f16_16816(t[n2], ah[ks], fh[2 * n2], fh[2 * n2 + 1]);
-                    mma_f16_16816(t[n2], ah[ks], fl[2 * n2], fl[2 * n2 + 1]);
-                    mma_f16_16816(t[n2], al[ks], fh[2 * n2], fh[2 * n2 + 1]);
+                unsigned fh[4], fl[2];
+                const unsigned* rowp = cf + 12 * (16 * ks + (lane & 7) + 8 * ((lane >> 3) & 1));
+                ldsm_x4_t(fh, rowp + 4 * (lane >> 4));
+                ldsm_x2_t(fl, rowp + 8);
+                if (ks == 0) {
+                    mma_f16_16816_first(t[0], ah[ks], fh[0], fh[1]);
+                    mma_f16_16816_first(t[1], ah[ks], fh[2], fh[3]);
+                } else {
+                    mma_f16_16816(t[0], ah[ks], fh[0], fh[1]);
+                    mma_f16_16816(t[1], ah[ks], fh[2], fh[3]);
                 }
+                mma_f16_16816(t[1], al[ks], fh[2], fh[3]);
+                mma_f16_16816(t[0], ah[ks], fl[0], fl[1]);
+                mma_f16_16816(t[0], al[ks], fh[0], fh[1]);
             }
             {
                 float4 r = run0[32 * mt];
@@ -1125,16 +1154,18 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int k0, float
                 r.z += t[0][2];
                 r.w += t[0][3];
                 run0[32 * mt] = r;
-                if (t4 == 0) {     // features 8, 9 (the other columns of tile 1 are zero)
-                    float4 r1 = run1[8 * mt];
+                if (t4 < 2) {      // features 8, 9: hi (t4 = 0) and lo parts (the other columns of tile 1 are zero)
+                    float4 r1 = run1[16 * mt];
                     r1.x += t[1][0];
                     r1.y += t[1][1];
                     r1.z += t[1][2];
                     r1.w += t[1][3];
-                    run1[8 * mt] = r1;
+                    run1[16 * mt] = r1;
                 }
             }
         }
+        const float2 n2 = f2_split(n_in);
+        cnt += (int)n2.x + (int)n2.y;
     }
     // unit end: per-query sums through shared memory to one lane per query
     // (32 queries at a time), formed into this lane's moments
@@ -1144,7 +1175,7 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int k0, float
 #pragma unroll
     for (int k = 0; k < 9; ++k) Mdy[k] = 0.f;
     const float s0 = ldexpf(1.f, -KW), s1 = ldexpf(1.f, ex - KW), s2 = ldexpf(1.f, 2 * ex - KW);
-    float* sq = reinterpret_cast<float*>(cf);    // [32][16] (features 0..9 used)
+    float* sq = reinterpret_cast<float*>(cf);    // [32][12] (features 0..9 used)
 #pragma unroll
     for (int h = 0; h < L::MAXQ / 32; ++h) {
         __syncwarp();
@@ -1153,19 +1184,20 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int k0, float
             const int mt = 2 * h + m2;
             const int q0 = 16 * m2 + g;
             const float4 r = run0[32 * mt];
-            *reinterpret_cast<float2*>(sq + 16 * q0 + 2 * t4) = make_float2(r.x, r.y);
-            *reinterpret_cast<float2*>(sq + 16 * (q0 + 8) + 2 * t4) = make_float2(r.z, r.w);
+            *reinterpret_cast<float2*>(sq + 12 * q0 + 2 * t4) = make_float2(r.x, r.y);
+            *reinterpret_cast<float2*>(sq + 12 * (q0 + 8) + 2 * t4) = make_float2(r.z, r.w);
             if (t4 == 0) {
-                const float4 r1 = run1[8 * mt];
-                *reinterpret_cast<float2*>(sq + 16 * q0 + 8) = make_float2(r1.x, r1.y);
-                *reinterpret_cast<float2*>(sq + 16 * (q0 + 8) + 8) = make_float2(r1.z, r1.w);
+                const float4 rh = run1[16 * mt], rl = run1[16 * mt + 1];
+                const float4 r1 = make_float4(rh.x + rl.x, rh.y + rl.y, rh.z + rl.z, rh.w + rl.w);
+                *reinterpret_cast<float2*>(sq + 12 * q0 + 8) = make_float2(r1.x, r1.y);
+                *reinterpret_cast<float2*>(sq + 12 * (q0 + 8) + 8) = make_float2(r1.z, r1.w);
             }
         }
         __syncwarp();
         const int q = lane + 32 * h;
-        const float4* rq = reinterpret_cast<const float4*>(sq + 16 * lane);
+        const float4* rq = reinterpret_cast<const float4*>(sq + 12 * lane);
         const float4 r0 = rq[0], r1 = rq[1];
-        const float2 r2 = *reinterpret_cast<const float2*>(sq + 16 * lane + 8);
+        const float2 r2 = *reinterpret_cast<const float2*>(sq + 12 * lane + 8);
         float y[3];
         if constexpr (SPLIT) {
             const float4 qm = reinterpret_cast<const float4*>(qg)[q];
