@@ -276,13 +276,19 @@ rkhsba_status build(rkhsba_ctx* c, const double* xyz, const float* sem, const fl
     RK_TRY(alloc(c, &c->d_xf, E));
     RK_TRY(alloc(c, &c->d_qkey, Q));
     RK_TRY(alloc(c, &c->d_qkey_alt, Q));
-    RK_TRY(alloc(c, &c->d_qval, Q));
-    RK_TRY(alloc(c, &c->d_qval_alt, Q));
+    // the query order and the unsorted records are done with when the units
+    // are cut, so the dense pair kernel's per-query sums take their place
+    const bool per_query = pairs_per_query(c->gp);
+    RK_TRY(alloc(c, &c->d_qval, 2 * Q));
+    c->d_qval_alt = c->d_qval + Q;
     RK_TRY(alloc(c, &c->d_qhist, (long long)radix_hist_elems(Q)));
-    RK_TRY(alloc(c, &c->d_qrec, Q));
+    RK_TRY(alloc(c, &c->d_qrec, per_query ? 2 * Q : Q));
+    if (per_query) {
+        c->d_qs8 = reinterpret_cast<float*>(c->d_qrec);
+        c->d_qs2 = reinterpret_cast<float*>(c->d_qval);
+    }
     RK_TRY(alloc(c, &c->d_slots, Q));
-    RK_TRY(alloc(c, &c->d_bin_first, c->total_bins));
-    RK_TRY(alloc(c, &c->d_unit_start, Q));
+    RK_TRY(alloc(c, &c->d_units, Q));
     RK_TRY(alloc(c, &c->d_ucount, 4));
     RK_TRY(alloc(c, &c->d_acc, (long long)E * ACC_N));
     RK_TRY(alloc(c, &c->d_eout, E));
@@ -317,10 +323,8 @@ void run_binning(rkhsba_ctx* c, const double* poses, const int* done) {
                    c->d_scan_ws, c->d_err + 1, st, &alt);
     c->q_sorted_key = alt ? c->d_qkey_alt : c->d_qkey;
     const int* qv = alt ? c->d_qval_alt : c->d_qval;
-    launch_query_gather(c->q_sorted_key, qv, c->d_qrec, c->Q_total, c->gp.key_sub, c->d_slots, c->d_bin_first, done,
-                        st);
-    launch_units(c->q_sorted_key, c->d_bin_first, c->Q_total, c->tune_uq, c->gp.key_sub, c->d_unit_start,
-                 c->d_ucount, done, st);
+    launch_units(c->q_sorted_key, qv, c->d_qrec, c->Q_total, c->tune_uq, c->gp.key_sub, c->d_edges, c->E, c->d_slots,
+                 c->d_units, c->d_ucount, done, st);
 }
 
 // One evaluation at the device poses `poses`, results into the cand
@@ -335,7 +339,7 @@ void eval_pre(rkhsba_ctx* c, const double* poses, const int* done) {
 
 void eval_pairs(rkhsba_ctx* c, const int* done) {
     c->phase_begin(2);
-    launch_pairs(PairLaunch{c->d_unit_start, c->d_ucount, c->d_ucount + 1, done, c->num_sms, c->tune_ctas,
+    launch_pairs(PairLaunch{c->d_units, c->d_ucount, c->d_ucount + 1, done, c->num_sms, c->tune_ctas,
                             c->stream},
                  c->pair_args());
     c->phase_end();
@@ -344,6 +348,7 @@ void eval_pairs(rkhsba_ctx* c, const int* done) {
 void eval_post(rkhsba_ctx* c, const int* done) {
     cudaStream_t st = c->stream;
     c->phase_begin(3);
+    if (pairs_per_query(c->gp)) launch_query_moments(c->pair_args(), c->num_sms, done, st);
     launch_edge_assemble(c->d_edges, c->E, c->d_xf, c->d_acc, c->p.sigma * c->p.sigma, c->d_eout, done, st);
     cudaMemsetAsync(c->d_H_cand, 0, sizeof(double) * 36LL * c->K * c->K, st);
     launch_frame_assemble(c->d_edges, c->E, c->K, c->d_inc_off, c->d_inc_list, c->d_eout, c->d_H_cand,
@@ -547,7 +552,7 @@ void ctx_iter_post(rkhsba_ctx* c) {
 }
 PairJob ctx_pair_job(const rkhsba_ctx* c) {
     PairJob j{};
-    j.unit_start = c->d_unit_start;
+    j.units = c->d_units;
     j.n_units = c->d_ucount;
     j.done = &c->d_state->done;
     j.a = c->pair_args();
@@ -720,9 +725,9 @@ rkhsba_status rkhsba_edge_pairs(rkhsba_ctx* c, const double* poses, int32_t edge
     }
     cudaMemsetAsync(dn, 0, sizeof(unsigned long long), st);
     cudaMemsetAsync(c->d_ucount + 1, 0, sizeof(int), st);
-    launch_emit_pairs(c->d_unit_start, c->d_ucount, c->d_ucount + 1, c->q_sorted_key, c->d_slots, c->Q_total,
-                      c->d_edges, c->E, c->d_frames, c->d_cell_start, c->d_pts4, c->gp, edge, c->d_perm_local,
-                      capacity, c->tune_uq, di, dj, dn, c->num_sms, st);
+    launch_emit_pairs(c->d_units, c->d_ucount, c->d_ucount + 1, c->q_sorted_key, c->d_slots, c->Q_total,
+                      c->d_edges, c->d_frames, c->d_cell_start, c->d_pts4, c->gp, edge, c->d_perm_local,
+                      capacity, di, dj, dn, c->num_sms, st);
     unsigned long long n = 0;
     cudaMemcpyAsync(&n, dn, sizeof(n), cudaMemcpyDeviceToHost, st);
     cudaError_t es = cudaStreamSynchronize(st);

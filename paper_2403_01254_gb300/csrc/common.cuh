@@ -116,15 +116,16 @@ struct PairArgs {
     const void* sem_sorted;   // label rows in the same order (FP32 or BF16), or NULL
     const float4* col4;       // colours in the same order, or NULL
     long long* acc;           // [E][ACC_N] fixed-point moments
+    float* qs8;               // [Q][8], [Q][2]: per sorted query sum_c w (1, x, x x^T) of the
+    float* qs2;               //   dense pair kernel (scaled), read by k_query_moments
     int E;
-    int uq;                   // queries per unit (1..32; up to 64 for the dense kernel with BF16 labels)
     GridParams gp;
 };
 
 // One problem of a batched pair launch: its unit list and LM state flag
 // (a job whose solve is done contributes no units).
 struct PairJob {
-    const int* unit_start;
+    const int2* units;
     const int* n_units;
     const int* done;
     PairArgs a;
@@ -133,7 +134,7 @@ constexpr int MAX_PAIR_JOBS = 64;   // problems in one batched pair launch
 
 // Launch state of a single-problem pair launch.
 struct PairLaunch {
-    const int* unit_start;
+    const int2* units;        // (first sorted query, edge << 7 | queries)
     const int* n_units;
     int* unit_counter;        // zeroed by the caller
     const int* done;          // LM state flag or NULL
@@ -182,25 +183,28 @@ void launch_edge_setup(const double* poses, const EdgeDev* edges, int E, const F
 void launch_query_keys(const EdgeDev* edges, int E, const FrameDev* frames, const EdgeXf* xf,
                        const uint32_t* pt_cell, const float4* pts4, GridParams gp, long long Q,
                        uint32_t* qkey, int* qval, float4* qrec, const int* done, cudaStream_t st);
-void launch_query_gather(const uint32_t* qkey_sorted, const int* qval_sorted, const float4* qrec,
-                         long long Q, int sub, float4* slots, int* bin_first, const int* done,
-                         cudaStream_t st);
-void launch_units(const uint32_t* qkey_sorted, const int* bin_first, long long Q, int uq, int sub, int* unit_start,
-                  int* n_units, const int* done, cudaStream_t st);
+void launch_units(const uint32_t* qkey_sorted, const int* qval_sorted, const float4* qrec, long long Q, int uq,
+                  int sub, const EdgeDev* edges, int E, float4* slots, int2* units, int* n_units, const int* done,
+                  cudaStream_t st);
 void launch_pairs(const PairLaunch& L, const PairArgs& A);
-// Largest unit (queries of one home cell per warp) the pair kernel of this
-// layout takes: 64 for the dense tile kernel with BF16 labels, else 32.
+// The dense pair kernel leaves per-query sums (PairArgs::qs8, qs2), which
+// launch_query_moments turns into the edges' moments; the others add to the
+// moments themselves.
+bool pairs_per_query(const GridParams& gp);
+void launch_query_moments(const PairArgs& A, int num_sms, const int* done, cudaStream_t st);
+// Largest unit_queries setting of this layout: 64 for the dense tile kernel
+// with BF16 labels, else 32 (64 is taken as two units of 32).
 int pair_unit_max(const GridParams& gp);
 // One persistent launch over the units of n_jobs problems (device array
-// `jobs`) that share the label layout, colour use and variant of `layout`,
-// with units of at most max_uq queries; false when the layout has no batched
-// kernel (top_k variant) or n_jobs is out of range.  *counter must be zero.
-bool launch_pairs_multi(const PairJob* jobs, int n_jobs, const GridParams& layout, int max_uq, int* counter,
-                        int num_sms, int ctas_per_sm, cudaStream_t st);
-void launch_emit_pairs(const int* unit_start, const int* n_units, int* unit_counter,
+// `jobs`) that share the label layout, colour use and variant of `layout`;
+// false when the layout has no batched kernel (top_k variant) or n_jobs is
+// out of range.  *counter must be zero.
+bool launch_pairs_multi(const PairJob* jobs, int n_jobs, const GridParams& layout, int* counter, int num_sms,
+                        int ctas_per_sm, cudaStream_t st);
+void launch_emit_pairs(const int2* units, const int* n_units, int* unit_counter,
                        const uint32_t* qkey, const float4* slots, long long Q, const EdgeDev* edges,
-                       int E, const FrameDev* frames, const int* cell_start, const float4* pts4,
-                       GridParams gp, int edge_sel, const int* perm_local, long long capacity, int uq,
+                       const FrameDev* frames, const int* cell_start, const float4* pts4,
+                       GridParams gp, int edge_sel, const int* perm_local, long long capacity,
                        int* i_out, int* j_out, unsigned long long* n_out, int num_sms,
                        cudaStream_t st);
 

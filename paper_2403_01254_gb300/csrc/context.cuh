@@ -75,8 +75,9 @@ struct rkhsba_ctx {
     long long* d_qhist = nullptr;
     float4* d_qrec = nullptr;          // per query: offset from home centre, point index
     float4* d_slots = nullptr;         // the same in sorted order
-    int* d_bin_first = nullptr;        // first sorted query of each home cell
-    int* d_unit_start = nullptr;       // units of <= tune_uq queries of one home cell
+    int2* d_units = nullptr;           // units of <= tune_uq queries of one home cell
+    float* d_qs8 = nullptr;            // per-query sums of the dense pair kernel (d_qs8 on d_qrec,
+    float* d_qs2 = nullptr;            //   d_qs2 on d_qval / d_qval_alt: both free once the units are cut)
     int* d_ucount = nullptr;           // [2]: number of units, unit counter
     const uint32_t* q_sorted_key = nullptr;
     long long* d_acc = nullptr;
@@ -126,8 +127,9 @@ struct rkhsba_ctx {
         a.sem_sorted = d_sem;
         a.col4 = d_col4;
         a.acc = d_acc;
+        a.qs8 = d_qs8;
+        a.qs2 = d_qs2;
         a.E = E;
-        a.uq = tune_uq;
         a.gp = gp;
         return a;
     }

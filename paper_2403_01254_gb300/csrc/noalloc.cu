@@ -239,12 +239,12 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
     long long* d_run = cv.take<long long>(N);
     uint32_t* d_qkey = cv.take<uint32_t>(Q);
     uint32_t* d_qkey_alt = cv.take<uint32_t>(Q);
-    int* d_qval = cv.take<int>(Q);
-    int* d_qval_alt = cv.take<int>(Q);
-    float4* d_qrec = cv.take<float4>(Q);
+    int* d_qval = cv.take<int>(2 * Q);      // qval, then its alternate; at last the dense kernel's sums
+    int* d_qval_alt = d_qval + Q;
+    const bool per_query = pairs_per_query(gp);
+    float4* d_qrec = cv.take<float4>(per_query ? 2 * Q : Q);
     float4* d_slots = cv.take<float4>(Q);
-    int* d_bin_first = cv.take<int>(bins);
-    int* d_units = cv.take<int>(Q);
+    int2* d_units = cv.take<int2>(Q);
     int* d_ucount = cv.take<int>(4);
     long long* d_acc = cv.take<long long>((long long)E * ACC_N);
     EdgeOut* d_eout = cv.take<EdgeOut>(E);
@@ -277,8 +277,8 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
     bool qalt = false;
     radix_sort_u32(d_qkey, d_qval, d_qkey_alt, d_qval_alt, Q, qbits, d_hist, d_ws, d_err + 1, st, &qalt);
     const uint32_t* qk = qalt ? d_qkey_alt : d_qkey;
-    launch_query_gather(qk, qalt ? d_qval_alt : d_qval, d_qrec, Q, gp.key_sub, d_slots, d_bin_first, nullptr, st);
-    launch_units(qk, d_bin_first, Q, UNIT_Q, gp.key_sub, d_units, d_ucount, nullptr, st);
+    launch_units(qk, qalt ? d_qval_alt : d_qval, d_qrec, Q, UNIT_Q, gp.key_sub, d_edges, E, d_slots, d_units,
+                 d_ucount, nullptr, st);
     {
         PairArgs a{};
         a.qkey = qk;
@@ -291,10 +291,12 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
         a.sem_sorted = d_sem_sorted;
         a.col4 = d_col4;
         a.acc = d_acc;
+        a.qs8 = per_query ? reinterpret_cast<float*>(d_qrec) : nullptr;
+        a.qs2 = per_query ? reinterpret_cast<float*>(d_qval) : nullptr;
         a.E = E;
-        a.uq = UNIT_Q;
         a.gp = gp;
         launch_pairs(PairLaunch{d_units, d_ucount, d_ucount + 1, nullptr, num_sms, 0, st}, a);
+        if (per_query) launch_query_moments(a, num_sms, nullptr, st);
     }
     launch_edge_assemble(d_edges, E, d_xf, d_acc, p.sigma * p.sigma, d_eout, nullptr, st);
     SCK(cudaMemsetAsync(d_H, 0, sizeof(double) * 36LL * K * K, st));

@@ -178,37 +178,57 @@ __global__ void k_query_keys(const EdgeDev* __restrict__ edges, int E, const Fra
     }
 }
 
-// sorted query records, and the first sorted query of every home cell (keys
-// >> sub are home-cell keys)
-__global__ void k_query_gather(const uint32_t* __restrict__ key, const int* __restrict__ val,
-                               const float4* __restrict__ qrec, long long Q, int sub, float4* __restrict__ slots,
-                               int* __restrict__ bin_first, const int* done) {
-    if (done && *done) return;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < Q;
-         k += (long long)gridDim.x * blockDim.x) {
-        slots[k] = qrec[val[k]];
-        const uint32_t kk = key[k];
-        if (kk != NO_KEY && (k == 0 || (key[k - 1] >> sub) != (kk >> sub))) bin_first[kk >> sub] = (int)k;
-    }
-}
-
-// a unit starts at the first query of a home cell and every uq queries
-// after (uq <= 32); one atomic per block reserves the block's slots in the
-// unit list
-__global__ void __launch_bounds__(256) k_units(const uint32_t* __restrict__ key, const int* __restrict__ bin_first,
-                                               long long Q, int uq, int sub, int* __restrict__ unit_start,
+// Sorted query records and the unit list, in one pass over the sorted keys: a
+// unit starts at the first query of a home cell and every uq queries after.
+// A block takes 256 sorted queries; where its first one continues a cell of
+// an earlier block, the block looks back over the keys, 256 at a time, for
+// that cell's first query.  One atomic per block reserves its slots in the
+// unit list; a record is (first sorted query, edge << 7 | queries), so that
+// no warp of the pair kernels searches for either.
+__global__ void __launch_bounds__(256) k_units(const uint32_t* __restrict__ key, const int* __restrict__ val,
+                                               const float4* __restrict__ qrec, long long Q, int uq, int sub,
+                                               const EdgeDev* __restrict__ edges, int E,
+                                               float4* __restrict__ slots, int2* __restrict__ units,
                                                int* __restrict__ n_units, const int* done) {
     if (done && *done) return;
-    __shared__ int s_cnt[8];
-    __shared__ int s_base;
+    __shared__ int s_cnt[8], s_first[8];
+    __shared__ int s_base, s_start;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (long long base = (long long)blockIdx.x * blockDim.x; base < Q; base += (long long)gridDim.x * blockDim.x) {
         const long long k = base + threadIdx.x;
-        bool st = false;
+        uint32_t kk = NO_KEY, prev = NO_KEY;
         if (k < Q) {
-            const uint32_t kk = key[k];
-            st = kk != NO_KEY && ((k - bin_first[kk >> sub]) % uq) == 0;
+            slots[k] = qrec[val[k]];
+            kk = key[k];
+            if (k > 0) prev = key[k - 1];
         }
+        const bool valid = kk != NO_KEY;
+        const bool head = valid && (k == 0 || (prev >> sub) != (kk >> sub));   // first query of its cell
+        // last cell head at or before this query inside the block
+        const unsigned hm = __ballot_sync(FULL, head) & (0xffffffffu >> (31 - lane));
+        int start = hm ? warp * 32 + 31 - __clz(hm) : -1;
+        if (lane == 31) s_first[warp] = start;
+        if (threadIdx.x == 0) s_start = -1;
+        __syncthreads();
+        if (start < 0)
+            for (int w = warp - 1; w >= 0 && start < 0; --w) start = s_first[w];
+        // the cell that the block's first query continues
+        const uint32_t c0 = key[base];
+        long long from = base;
+        if (c0 != NO_KEY && base > 0 && (key[base - 1] >> sub) == (c0 >> sub)) {
+            for (long long hi = base - 1; hi >= 0; hi -= 256) {
+                const long long p = hi - threadIdx.x;
+                const bool other = p < 0 || (key[p] >> sub) != (c0 >> sub);
+                if (other) atomicMax(&s_start, (int)(p < 0 ? 0 : p + 1));
+                __syncthreads();
+                const bool found = s_start >= 0;
+                __syncthreads();
+                if (found) break;
+            }
+            from = s_start;
+        }
+        const long long run = start >= 0 ? base + start : from;
+        const bool st = valid && ((k - run) % uq) == 0;
         const unsigned m = __ballot_sync(FULL, st);
         if (lane == 0) s_cnt[warp] = __popc(m);
         __syncthreads();
@@ -218,7 +238,18 @@ __global__ void __launch_bounds__(256) k_units(const uint32_t* __restrict__ key,
             s_base = tot ? atomicAdd(n_units, tot) : 0;
         }
         __syncthreads();
-        if (st) unit_start[s_base + s_cnt[warp] + __popc(m & ((1u << lane) - 1u))] = (int)k;
+        if (st) {
+            // queries of the cell from here on, uq at most (gallop, then bisect)
+            int n = 1;
+            while (n < uq && k + n < Q && (key[k + n] >> sub) == (kk >> sub)) n *= 2;
+            int lo = n / 2 + 1, hi = n < uq ? n : uq;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (k + mid < Q && (key[k + mid] >> sub) == (kk >> sub)) lo = mid + 1; else hi = mid;
+            }
+            units[s_base + s_cnt[warp] + __popc(m & ((1u << lane) - 1u))] =
+                make_int2((int)k, (find_edge_bin(edges, E, kk >> sub) << 7) | lo);
+        }
         __syncthreads();
     }
 }
@@ -369,18 +400,6 @@ struct SemRow<0, false> {
 
 
 constexpr int PAIR_T = 256;
-#ifndef RK_PAIR_MINB
-#define RK_PAIR_MINB 2              // resident CTAs per SM the register budget targets
-#endif
-// Resident CTAs per SM the register budget of a dense tile kernel targets:
-// three for BF16 rows of <= 24 values and units of <= 32 queries (75 KB of
-// shared memory per CTA, so three fit; 80 registers with a few bytes of
-// spills: window workload 1.85 -> 1.73 ms per evaluation), else two (the
-// larger layouts fit only two CTAs' shared memory).
-template <int DP, bool BF16, int DENSE>
-__host__ __device__ constexpr int dense_min_blocks() {
-    return (BF16 && DENSE == 1 && DP <= 24) ? 3 : 2;
-}
 constexpr int UQ = UNIT_Q;          // queries per unit: one 32-bit mask word
 static_assert(UQ == 32, "units hold 32 queries");
 
@@ -404,6 +423,7 @@ __device__ __forceinline__ float ex2_approx(float x) {
 // sum w0 x x^T (6), sum x dc^T (9), with w0 = sum w, dc = sum w d of one
 // candidate over its queries.
 constexpr int N_ACC = 28;
+constexpr int ROWS_WORDS = 9 * 4 + 9 * 2 + 2;   // segment list of the candidate stream (Rows)
 constexpr int CQ_N = 64;            // ring of candidates that survived the unit's box test
 constexpr int GRAM_LD = 32;         // row stride (floats) of the BF16 label Gram tile, stored
                                     // [query][candidate]: the walk's lane c reads column c,
@@ -412,104 +432,92 @@ constexpr int A_W = 0, A_D = 1, A_Q = 4, A_SWX = 10, A_SWXX = 13, A_SXD = 19;
 
 template <int DP, bool BF16, bool COLOR>
 __host__ __device__ constexpr int warp_smem_words() {
-    return UQ * 4 + UQ * 4 + (COLOR ? UQ * 4 : 0) + UQ * SemRow<DP, BF16>::WORDS + 4 * 10 + 32 * N_ACC +
+    return UQ * 4 + UQ * 4 + (COLOR ? UQ * 4 : 0) + UQ * SemRow<DP, BF16>::WORDS + ROWS_WORDS + 32 * N_ACC +
            4 * CQ_N + ((BF16 && DP > 0) ? 32 * GRAM_LD : 0);
 }
 
+// The candidate stream of a unit: the points of the 3x3x3 cells around its
+// home cell are nine contiguous ranges (rows of three x-adjacent cells).  Cells
+// farther than the cutoff from the bounding box of the unit's queries are left
+// out, and rows without points skipped; what is left is a list of segments.
 struct Rows {
-    int* rb;    // [9] first point of the row (three x-adjacent cells)
-    int* b1;    // [9] first point of the home-x cell
-    int* b2;    // [9] first point of the x+1 cell
-    int* pre;   // [10] prefix of row lengths
+    int4* seg;     // [<= 9] first and end point, first point of the home-x cell, of the x+1 cell
+    float2* off;   // [<= 9] y and z offset of the row's cells from the home cell
 };
 
-// Rows of the 3x3x3 stencil around home cell (hx, hy, hz): lanes 0..8 fill one
-// row each; returns the total candidate count.
-__device__ __forceinline__ int build_rows(const Rows& R, const int* __restrict__ cell_start, long long coff,
-                                          int dx0, int dy0, int dz0, int hx, int hy, int hz, int lane) {
-    int len = 0, rb = 0, b1 = 0, b2 = 0;
+// Fills the segment list (lanes 0..8 take a row each); returns the number of
+// points on it and, in n_seg, of segments.  thr: squared cutoff with a margin,
+// so that no cell holding a candidate that passes the box test is left out.
+__device__ __forceinline__ int build_rows(const Rows& R, const int* __restrict__ cell_start, const FrameDev& F,
+                                          int hx, int hy, int hz, float blo0, float blo1, float blo2, float bhi0,
+                                          float bhi1, float bhi2, float hf, float thr, int lane, int& n_seg) {
+    int len = 0;
+    int4 sg = make_int4(0, 0, 0, 0);
+    const int dy = (lane % 3) - 1, dz = (lane / 3) - 1;
+    const float oy = (float)dy * hf, oz = (float)dz * hf;
     if (lane < 9) {
-        const int ny = hy + (lane % 3) - 1, nz = hz + (lane / 3) - 1;
-        if (ny >= 0 && ny < dy0 && nz >= 0 && nz < dz0) {
-            const long long g0 = coff + ((long long)nz * dy0 + ny) * dx0;
-            const int xlo = max(hx - 1, 0), xhi = min(hx + 1, dx0 - 1);
-            rb = cell_start[g0 + xlo];
-            len = cell_start[g0 + xhi + 1] - rb;
-            b1 = cell_start[g0 + hx];
-            b2 = cell_start[g0 + hx + 1];
+        const int ny = hy + dy, nz = hz + dz;
+        const float hw = 0.50001f * hf;      // half a cell, with a margin for the rounding of the offsets
+        const float ey = fmaxf(fmaxf(blo1 - (oy + hw), (oy - hw) - bhi1), 0.f);
+        const float ez = fmaxf(fmaxf(blo2 - (oz + hw), (oz - hw) - bhi2), 0.f);
+        const float left = 1.0001f * thr - fmaf(ey, ey, ez * ez);     // what the x distance may use
+        if (ny >= 0 && ny < F.dim[1] && nz >= 0 && nz < F.dim[2] && left > 0.f) {
+            const float el = fmaxf(blo0 + hf - hw, 0.f), er = fmaxf(hf - hw - bhi0, 0.f);
+            const int xlo = max(hx - (el * el < left ? 1 : 0), 0), xhi = min(hx + (er * er < left ? 1 : 0), F.dim[0] - 1);
+            const int* c = cell_start + F.cell_off + ((long long)nz * F.dim[1] + ny) * F.dim[0];
+            sg.x = c[xlo];
+            sg.y = c[xhi + 1];
+            sg.z = c[hx];
+            sg.w = c[hx + 1];
+            len = sg.y - sg.x;
         }
     }
-    int inc = len;
-#pragma unroll
-    for (int o = 1; o < 16; o <<= 1) {
-        const int u = __shfl_up_sync(FULL, inc, o);
-        if (lane >= o) inc += u;
+    const unsigned m = __ballot_sync(FULL, len > 0);
+    if (len > 0) {
+        const int at = __popc(m & ((1u << lane) - 1u));
+        R.seg[at] = sg;
+        R.off[at] = make_float2(oy, oz);
     }
-    if (lane < 9) {
-        R.rb[lane] = rb;
-        R.b1[lane] = b1;
-        R.b2[lane] = b2;
-        R.pre[lane] = inc - len;
-    }
-    const int total = __shfl_sync(FULL, inc, 8);
-    if (lane == 9) R.pre[9] = total;
+    n_seg = __popc(m);
+    const int total = __reduce_add_sync(FULL, len);
     __syncwarp();
     return total;
 }
 
-// Candidate v of the unit's stream: point index and offset (dx, dy, dz) of
-// its cell from the home cell.
-__device__ __forceinline__ int stream_point(const Rows& R, int v, int& dx, int& dy, int& dz) {
-    int r = 0;
-#pragma unroll
-    for (int k = 1; k < 9; ++k) r += (R.pre[k] <= v) ? 1 : 0;
-    const int i = R.rb[r] + (v - R.pre[r]);
-    dx = (i >= R.b1[r]) + (i >= R.b2[r]) - 1;
-    dy = (r % 3) - 1;
-    dz = (r / 3) - 1;
-    return i;
-}
-
-// The same with the row prefix held in registers (pre[0] = 0).
-__device__ __forceinline__ int stream_point_r(const Rows& R, const int (&pre)[9], int v, int& dx, int& dy, int& dz) {
-    int r = 0;
-#pragma unroll
-    for (int k = 1; k < 9; ++k) r += (pre[k] <= v) ? 1 : 0;
-    int base = pre[0];
-#pragma unroll
-    for (int k = 1; k < 9; ++k) base = (r == k) ? pre[k] : base;
-    const int i = R.rb[r] + (v - base);
-    dx = (i >= R.b1[r]) + (i >= R.b2[r]) - 1;
-    dy = (r % 3) - 1;
-    dz = (r / 3) - 1;
-    return i;
-}
-
-// Unit header shared by the pair and the pair-list kernels: home cell of the
-// unit starting at sorted query k0, and the number of its queries (<= UQ).
-__device__ __forceinline__ int unit_queries(const uint32_t* __restrict__ qkey, long long Q, int k0,
-                                            uint32_t key0, int lane, int uq, int sub) {
-    // units start every uq queries of a home cell, so a unit holds at most uq
-    // of them even when the cell continues past k0 + uq
-    const long long k1 = (long long)k0 + lane;
-    const bool m1 = k1 < Q && (qkey[k1] >> sub) == (key0 >> sub);
-    const int n = __popc(__ballot_sync(FULL, m1));
-    return n < uq ? n : uq;
-}
-
-// The same for units of up to 64 queries (the dense tile unit and the
-// pair-list kernel).
-__device__ __forceinline__ int unit_queries64(const uint32_t* __restrict__ qkey, long long Q, int k0,
-                                              uint32_t key0, int lane, int uq, int sub) {
-    int n = unit_queries(qkey, Q, k0, key0, lane, uq, sub);
-    if (n == 32 && uq > 32) {
-        const long long k1 = (long long)k0 + 32 + lane;
-        const bool m1 = k1 < Q && (qkey[k1] >> sub) == (key0 >> sub);
-        n = 32 + __popc(__ballot_sync(FULL, m1));
-        n = n < uq ? n : uq;
+// A lane's place in the stream: it starts at point `lane` of the list and
+// steps 32 points at a time, crossing into the next segment when it must.
+struct Cursor {
+    int i, end, r, b1, b2;
+    float oy, oz;
+    __device__ __forceinline__ void enter(const Rows& R, int seg, int skip) {
+        const int4 sg = R.seg[seg];
+        const float2 o = R.off[seg];
+        r = seg;
+        i = sg.x + skip;
+        end = sg.y;
+        b1 = sg.z;
+        b2 = sg.w;
+        oy = o.x;
+        oz = o.y;
     }
-    return n;
-}
+    __device__ __forceinline__ void settle(const Rows& R, int n_seg) {
+        while (i >= end && r + 1 < n_seg) enter(R, r + 1, i - end);
+    }
+    __device__ __forceinline__ void start(const Rows& R, int n_seg, int lane) {
+        enter(R, 0, lane);
+        settle(R, n_seg);
+    }
+    __device__ __forceinline__ void next(const Rows& R, int n_seg) {
+        i += 32;
+        settle(R, n_seg);
+    }
+    __device__ __forceinline__ bool valid() const { return i < end; }
+    // point i relative to the home cell's centre, with its index
+    __device__ __forceinline__ float4 point(const float4* __restrict__ pts4, float hf) const {
+        const float4 p = __ldg(pts4 + i);
+        return make_float4(p.x + (i >= b2 ? hf : (i >= b1 ? 0.f : -hf)), p.y + oy, p.z + oz, __int_as_float(i));
+    }
+};
 
 // One step of the moment reduce-scatter: lanes whose bit `o` is clear keep
 // the lower half of their values, the others the upper half, and each adds
@@ -525,32 +533,12 @@ __device__ __forceinline__ void reduce_half(long long (&v)[32], int lane) {
     }
 }
 
-// Unit end, shared by the pair kernels: the lane's moments about the home
-// cell centre move to frame-a coordinates (y' += o), are rounded to 64-bit
-// fixed point and reduce-scattered over the warp (lane k ends with the warp
-// total of moment k), and added to the edge's accumulators with one integer
-// atomic per moment.
-__device__ __forceinline__ void store_moments(float W, const float (&Dv)[3], float (&Sy)[3], float (&Myy)[6],
-                                              float (&Mdy)[9], const float* Qm, int cnt, const FrameDev& Fa,
-                                              int hx, int hy, int hz, const GridParams& gp,
-                                              const float* __restrict__ scl, long long* __restrict__ acc_e,
-                                              int lane) {
-    const float o[3] = {((float)(hx + Fa.lo[0]) + 0.5f) * gp.hf, ((float)(hy + Fa.lo[1]) + 0.5f) * gp.hf,
-                        ((float)(hz + Fa.lo[2]) + 0.5f) * gp.hf};
-    {
-        int t6 = 0;
-#pragma unroll
-        for (int mm = 0; mm < 3; ++mm)
-#pragma unroll
-            for (int l = mm; l < 3; ++l, ++t6)
-                Myy[t6] += Sy[mm] * o[l] + o[mm] * Sy[l] + W * o[mm] * o[l];
-#pragma unroll
-        for (int mm = 0; mm < 3; ++mm)
-#pragma unroll
-            for (int l = 0; l < 3; ++l) Mdy[3 * mm + l] = fmaf(Dv[mm], o[l], Mdy[3 * mm + l]);
-#pragma unroll
-        for (int mm = 0; mm < 3; ++mm) Sy[mm] = fmaf(W, o[mm], Sy[mm]);
-    }
+// A lane's moments (frame-a coordinates) rounded to 64-bit fixed point,
+// reduce-scattered over the warp (lane k ends with the warp total of moment k)
+// and added to the edge's accumulators with one integer atomic per moment.
+__device__ __forceinline__ void add_moments(float W, const float (&Dv)[3], const float (&Sy)[3], const float (&Myy)[6],
+                                            const float (&Mdy)[9], const float* Qm, int cnt,
+                                            const float* __restrict__ scl, long long* __restrict__ acc_e, int lane) {
     long long vals[32];
 #pragma unroll
     for (int k = 0; k < 32; ++k) {
@@ -571,6 +559,31 @@ __device__ __forceinline__ void store_moments(float W, const float (&Dv)[3], flo
     reduce_half<1>(vals, lane);
     if (lane < N_MOM && vals[0] != 0)
         atomicAdd(reinterpret_cast<unsigned long long*>(acc_e + lane), (unsigned long long)vals[0]);
+}
+
+// Unit end of the pair kernels that sum moments themselves: the lane's moments
+// about the home cell centre move to frame-a coordinates (y' += o) and are
+// added to the edge's.
+__device__ __forceinline__ void store_moments(float W, const float (&Dv)[3], float (&Sy)[3], float (&Myy)[6],
+                                              float (&Mdy)[9], const float* Qm, int cnt, const FrameDev& Fa,
+                                              int hx, int hy, int hz, const GridParams& gp,
+                                              const float* __restrict__ scl, long long* __restrict__ acc_e,
+                                              int lane) {
+    const float o[3] = {((float)(hx + Fa.lo[0]) + 0.5f) * gp.hf, ((float)(hy + Fa.lo[1]) + 0.5f) * gp.hf,
+                        ((float)(hz + Fa.lo[2]) + 0.5f) * gp.hf};
+    int t6 = 0;
+#pragma unroll
+    for (int mm = 0; mm < 3; ++mm)
+#pragma unroll
+        for (int l = mm; l < 3; ++l, ++t6)
+            Myy[t6] += Sy[mm] * o[l] + o[mm] * Sy[l] + W * o[mm] * o[l];
+#pragma unroll
+    for (int mm = 0; mm < 3; ++mm)
+#pragma unroll
+        for (int l = 0; l < 3; ++l) Mdy[3 * mm + l] = fmaf(Dv[mm], o[l], Mdy[3 * mm + l]);
+#pragma unroll
+    for (int mm = 0; mm < 3; ++mm) Sy[mm] = fmaf(W, o[mm], Sy[mm]);
+    add_moments(W, Dv, Sy, Myy, Mdy, Qm, cnt, scl, acc_e, lane);
 }
 
 // BF16 labels: the candidate x query label products of a batch come from the
@@ -761,38 +774,48 @@ __device__ __forceinline__ float inside_mask(float t, float thr) {
     return r;
 }
 
-// Per-warp shared memory of the dense path, in 32-bit words.  Label rows:
-// BF16 rows as stored (DP values); FP32 rows (SPLIT) as an FP16 hi part and an
-// FP16 lo part of DPH values each (DP rounded up to 8), scaled by a power of two.
-template <int DP, bool SPLIT, int MQ = 32>
+// Per-warp shared memory of the dense path, in 32-bit words: the batch's
+// candidates only (the unit's queries live in registers).  Label rows: BF16
+// rows as stored (DP values); FP32 rows (SPLIT) as an FP16 hi part and an FP16
+// lo part of DPH values each (DP rounded up to 8), scaled by a power of two.
+template <int DP, bool SPLIT>
 struct DenseSmem {
     static constexpr int DPH = SPLIT ? ((DP + 7) / 8) * 8 : DP;    // values per part
     static constexpr int PW = DPH / 2;                            // words per part
     static constexpr int RW = SPLIT ? 2 * PW : PW;                // words per staged row
     static constexpr int LW = (RW % 8 == 0) ? RW + 4 : RW;        // row stride: 4 x odd, conflict-free ldmatrix
-    static constexpr int MAXQ = SPLIT ? 32 : MQ;                  // queries per unit (m tiles of 16: MAXQ / 16)
-    static constexpr int QGW = SPLIT ? 4 : 8;                     // query geometry words:
-                                                                  //   (mx mx my my mz mz yy yy) or (mx my mz yy), m = -2y
-    static constexpr int QG = 0;                                  // [MAXQ][QGW]
-    static constexpr int QL = QG + MAXQ * QGW;                    // [MAXQ][LW] query label rows
-    static constexpr int CL = QL + MAXQ * LW;                     // [32][LW] the batch's candidate label rows
+    static constexpr int CL = 0;                                  // [32][LW] candidate label rows (first the
+                                                                  //   unit's query rows, on their way to registers)
     static constexpr int CG = CL + 32 * LW;                       // [16][12] candidate pairs (2p, 2p+1):
                                                                   //   x0 x0' x1 x1' | x2 x2' thr thr' | xk xk' - -
     static constexpr int CF = CG + 16 * 12;                       // [32][12] features in FP16: hi of features 0..7,
                                                                   //   tile 1 (hi 8, hi 9, lo 8, lo 9, zeros), lo of
                                                                   //   features 0..7 (a 48-byte row: conflict-free
-                                                                  //   ldmatrix); at the unit's end [32 queries][12]
-                                                                  //   FP32 sums
-    // running per-query sums of the moment MMAs, in the accumulator layout:
-    // feature tile 0 as [m tile][lane] float4; feature tile 1 holds only
-    // features 8 and 9, their hi parts in the lanes with t4 = 0 and their lo
-    // parts in those with t4 = 1, as [m tile][g][t4] float4
-    static constexpr int RUN = CF + 32 * 12;
-    static constexpr int RUN1 = RUN + (MAXQ / 16) * 32 * 4;
-    static constexpr int RING = RUN1 + (MAXQ / 16) * 16 * 4;     // [CQ_N] float4 candidate ring
-    static constexpr int ROWS = RING + 4 * CQ_N;                  // [40] stencil rows
-    static constexpr int WORDS = ROWS + 40;
+                                                                  //   ldmatrix)
+    static constexpr int RING = CF + 32 * 12;                     // [CQ_N] float4 candidate ring
+    static constexpr int ROWS = RING + 4 * CQ_N;                  // the stream's segments
+    static constexpr int WORDS = ROWS + ROWS_WORDS;
 };
+
+// Power-of-two scales of the dense path's FP16 operands, from the frames'
+// label-norm bounds and the cell size (see "Scaling" above): the weights carry
+// 2^kw, the features 2^-ex, FP32 labels 2^-el.
+struct DenseScales {
+    int kw, ex, el;
+};
+__device__ __forceinline__ DenseScales dense_scales(float norm_a, float norm_b, float hf, bool split) {
+    DenseScales d;
+    int ew;
+    frexpf(norm_a * norm_b, &ew);
+    frexpf(hf, &d.ex);
+    d.kw = min(max(14 - ew, -100), 100);
+    d.el = 0;
+    if (split) {
+        frexpf(fmaxf(norm_a, norm_b), &d.el);
+        d.el = min(max(d.el, -60), 60);
+    }
+    return d;
+}
 
 // Stage one label row into shared memory: BF16 rows copied; FP32 rows scaled
 // by ls and split into FP16 hi and lo parts (zeros beyond DP); a zero row when
@@ -906,86 +929,66 @@ __device__ __forceinline__ void gram_chunks(float (&s)[4], const unsigned (&qa)[
     }
 }
 
-template <int DP, bool SPLIT, int MQ>
-__device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int k0, float* wb, int lane) {
-    using L = DenseSmem<DP, SPLIT, MQ>;
+// One unit of the dense path: <= 32 queries of one frame-a home cell, MT m
+// tiles of 16.  The queries live in registers for the whole unit (geometry as
+// FP32 pairs, label rows as A fragments, running sums as accumulators), so
+// that a batch reads each candidate's geometry, label row and features from
+// shared memory once for all its queries: at one 16-query tile per read the
+// shared-memory pipe was the kernel's bound (82% busy on the mapping workload,
+// 98 wavefronts per 16 x 32 tile; 32 here).
+template <int DP, bool SPLIT>
+__device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int2 unit, float* wb, int lane) {
+    using L = DenseSmem<DP, SPLIT>;
     constexpr int LW = L::LW, PW = L::PW;
     constexpr int NKC = L::DPH / 8;             // 8-wide chunks of a label row part (1..4)
     const GridParams& gp = A.gp;
-    float* qg = wb + L::QG;
-    unsigned* ql = reinterpret_cast<unsigned*>(wb + L::QL);
     unsigned* cl = reinterpret_cast<unsigned*>(wb + L::CL);
     float* cg = wb + L::CG;
     unsigned* cf = reinterpret_cast<unsigned*>(wb + L::CF);
     float4* cq = reinterpret_cast<float4*>(wb + L::RING);
-    int* ri = reinterpret_cast<int*>(wb + L::ROWS);
-    const Rows R{ri, ri + 9, ri + 18, ri + 27};
+    const Rows R{reinterpret_cast<int4*>(wb + L::ROWS), reinterpret_cast<float2*>(wb + L::ROWS + 36)};
     const int g = lane >> 2, t4 = lane & 3;
     const float INF = __int_as_float(0x7f800000);
 
-    const uint32_t kq0 = A.qkey[k0];
-    const int qcount = unit_queries64(A.qkey, A.Q, k0, kq0, lane, L::MAXQ < A.uq ? L::MAXQ : A.uq, gp.key_sub);
-    const uint32_t key0 = kq0 >> gp.key_sub;
-    const int e = find_edge_bin(A.edges, A.E, key0);
+    const int k0 = unit.x, qcount = unit.y & 127, e = unit.y >> 7;
+    const uint32_t key0 = A.qkey[k0] >> gp.key_sub;
     const FrameDev& Fa = A.frames[A.edges[e].a];
     const FrameDev& Fb = A.frames[A.edges[e].b];
-    const int dx0 = Fa.dim[0], dy0 = Fa.dim[1], dz0 = Fa.dim[2];
     const int cell = (int)(key0 - A.edges[e].bin_off);
-    const int hx = cell % dx0, hy = (cell / dx0) % dy0, hz = cell / (dx0 * dy0);
-    // power-of-two scales of the FP16 operands
-    int ew, ex;
-    frexpf(Fa.sem_norm_max * Fb.sem_norm_max, &ew);
-    frexpf(gp.hf, &ex);
-    const int KW = min(max(14 - ew, -100), 100);
+    const int hx = cell % Fa.dim[0], hy = (cell / Fa.dim[0]) % Fa.dim[1], hz = cell / (Fa.dim[0] * Fa.dim[1]);
+    const DenseScales sc = dense_scales(Fa.sem_norm_max, Fb.sem_norm_max, gp.hf, SPLIT);
     // FP32 labels enter the FP16 parts scaled by ls = 2^-el (|l| ls < 1), so
     // the products carry 2^-2el, which the exponent offset undoes
-    int el = 0;
-    if constexpr (SPLIT) {
-        frexpf(fmaxf(Fa.sem_norm_max, Fb.sem_norm_max), &el);
-        el = min(max(el, -60), 60);
-    }
-    const float ls = ldexpf(1.f, -el);
-    const float kwf = (float)(KW + 2 * el);
-    const float xs = ldexpf(1.f, -ex);
-    __syncwarp();
-    // stage the unit's queries: geometry, label rows (zero rows for absent
-    // queries, whose |y|^2 = inf fails every test), bounding box
+    const float ls = ldexpf(1.f, -sc.el);
+    const float kwf = (float)(sc.kw + 2 * sc.el);
+    const float xs = ldexpf(1.f, -sc.ex);
+    // this lane's queries, rows g + 8 i: -2 y and |y|^2 doubled into pairs
+    // (absent ones: |y|^2 = inf fails every test), and the unit's bounding box
+    u64 qm[4][4];
     float blo0 = INF, blo1 = INF, blo2 = INF, bhi0 = -INF, bhi1 = -INF, bhi2 = -INF;
 #pragma unroll
-    for (int h = 0; h < L::MAXQ / 32; ++h) {
-        const int q = lane + 32 * h;
-        float4* q4 = reinterpret_cast<float4*>(qg) + (L::QGW / 4) * q;
-        const bool qv = q < qcount;
-        int s = 0;
-        if (qv) {
-            const float4 r = A.slots[(long long)k0 + q];
+    for (int i = 0; i < 4; ++i) {
+        float mx = 0.f, my = 0.f, mz = 0.f, yy = INF;
+        if (g + 8 * i < qcount) {
+            const float4 r = A.slots[(long long)k0 + g + 8 * i];
             blo0 = fminf(blo0, r.x);
             bhi0 = fmaxf(bhi0, r.x);
             blo1 = fminf(blo1, r.y);
             bhi1 = fmaxf(bhi1, r.y);
             blo2 = fminf(blo2, r.z);
             bhi2 = fmaxf(bhi2, r.z);
-            s = __float_as_int(r.w);
-            const float mx = -2.f * r.x, my = -2.f * r.y, mz = -2.f * r.z;
-            const float yy = fmaf(r.x, r.x, fmaf(r.y, r.y, r.z * r.z));
-            if constexpr (SPLIT) {
-                q4[0] = make_float4(mx, my, mz, yy);
-            } else {
-                q4[0] = make_float4(mx, mx, my, my);
-                q4[1] = make_float4(mz, mz, yy, yy);
-            }
-        } else {
-            if constexpr (SPLIT) {
-                q4[0] = make_float4(0.f, 0.f, 0.f, INF);
-            } else {
-                q4[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-                q4[1] = make_float4(0.f, 0.f, INF, INF);
-            }
+            mx = -2.f * r.x;
+            my = -2.f * r.y;
+            mz = -2.f * r.z;
+            yy = fmaf(r.x, r.x, fmaf(r.y, r.y, r.z * r.z));
         }
-        stage_label_row<DP, SPLIT>(ql + q * LW, A.sem_sorted, s, ls, qv);
+        qm[i][0] = f2(mx, mx);
+        qm[i][1] = f2(my, my);
+        qm[i][2] = f2(mz, mz);
+        qm[i][3] = f2(yy, yy);
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int o = 16; o >= 4; o >>= 1) {
         blo0 = fminf(blo0, __shfl_xor_sync(FULL, blo0, o));
         blo1 = fminf(blo1, __shfl_xor_sync(FULL, blo1, o));
         blo2 = fminf(blo2, __shfl_xor_sync(FULL, blo2, o));
@@ -993,267 +996,312 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int k0, float
         bhi1 = fmaxf(bhi1, __shfl_xor_sync(FULL, bhi1, o));
         bhi2 = fmaxf(bhi2, __shfl_xor_sync(FULL, bhi2, o));
     }
-    const int C = build_rows(R, A.cell_start, Fa.cell_off, dx0, dy0, dz0, hx, hy, hz, lane);
+    __syncwarp();
     const float box_thr = gp.rc2 * 1.0001f;
-    const int n_mt = (qcount + 15) >> 4;        // m tiles of 16 queries that hold queries
-    const u64 KG2 = f2(gp.kg, gp.kg);
-    // this lane's running sums (feature tile 0 for every lane, tile 1 for
-    // the lanes holding features 8 and 9, hi and lo parts), in shared memory
-    float4* run0 = reinterpret_cast<float4*>(wb + L::RUN) + lane;       // [mt * 32]
-    float4* run1 = reinterpret_cast<float4*>(wb + L::RUN1) + 2 * g + (t4 & 1);   // [mt * 16], t4 < 2
-#pragma unroll
-    for (int mt = 0; mt < L::MAXQ / 16; ++mt) {
-        run0[32 * mt] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (t4 < 2) run1[16 * mt] = make_float4(0.f, 0.f, 0.f, 0.f);
+    int n_seg;
+    const int C = build_rows(R, A.cell_start, Fa, hx, hy, hz, blo0, blo1, blo2, bhi0, bhi1, bhi2, gp.hf, box_thr, lane,
+                             n_seg);
+    // query label rows (zero rows for absent queries) as A fragments, through
+    // the candidates' rows
+    {
+        const bool qv = lane < qcount;
+        const int s = qv ? __float_as_int(A.slots[(long long)k0 + lane].w) : 0;
+        stage_label_row<DP, SPLIT>(cl + lane * LW, A.sem_sorted, s, ls, qv);
     }
+    __syncwarp();
+    unsigned qa[2][2 * NKC], qal[SPLIT ? 2 : 1][SPLIT ? 2 * NKC : 1];
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) {
+        const unsigned* qrowp = cl + (16 * mt + (lane & 7) + 8 * ((lane >> 3) & 1)) * LW;
+        load_a_chunks<NKC>(qa[mt], qrowp);
+        if constexpr (SPLIT) load_a_chunks<NKC>(qal[mt], qrowp + PW);
+    }
+    __syncwarp();
+    const u64 KG2 = f2(gp.kg, gp.kg);
+    // running sums of the moment MMAs, in the accumulator layout: feature tile
+    // 0, and tile 1 (features 8 and 9: hi parts in the lanes with t4 = 0, lo
+    // parts in those with t4 = 1, zeros elsewhere)
+    float run[2][2][4];
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int n2 = 0; n2 < 2; ++n2)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) run[mt][n2][k] = 0.f;
     int cnt = 0;
-    int c_s = 0, qhead = 0, qlen = 0;
-    while (c_s < C || qlen > 0) {
-        while (qlen < 32 && c_s < C) {
-            const int v = c_s + lane;
-            bool keep = false;
-            float4 ent = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (v < C) {
-                int dx, dy, dz;
-                const int i = stream_point(R, v, dx, dy, dz);
-                const float4 p = __ldg(A.pts4 + i);
-                ent.x = fmaf((float)dx, gp.hf, p.x);
-                ent.y = fmaf((float)dy, gp.hf, p.y);
-                ent.z = fmaf((float)dz, gp.hf, p.z);
-                ent.w = __int_as_float(i);
-                const float e0 = fmaxf(fmaxf(blo0 - ent.x, ent.x - bhi0), 0.f);
-                const float e1 = fmaxf(fmaxf(blo1 - ent.y, ent.y - bhi1), 0.f);
-                const float e2 = fmaxf(fmaxf(blo2 - ent.z, ent.z - bhi2), 0.f);
-                keep = fmaf(e0, e0, fmaf(e1, e1, e2 * e2)) < box_thr;
+    // the batches, compiled for one and for two m tiles
+    auto batches = [&](auto mtc) {
+        constexpr int MT = decltype(mtc)::value;
+        int c_s = 0, qhead = 0, qlen = 0;
+        Cursor cur;
+        cur.start(R, n_seg, lane);
+        while (c_s < C || qlen > 0) {
+            while (qlen < 32 && c_s < C) {
+                bool keep = false;
+                float4 ent = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (cur.valid()) {
+                    ent = cur.point(A.pts4, gp.hf);
+                    const float e0 = fmaxf(fmaxf(blo0 - ent.x, ent.x - bhi0), 0.f);
+                    const float e1 = fmaxf(fmaxf(blo1 - ent.y, ent.y - bhi1), 0.f);
+                    const float e2 = fmaxf(fmaxf(blo2 - ent.z, ent.z - bhi2), 0.f);
+                    keep = fmaf(e0, e0, fmaf(e1, e1, e2 * e2)) < box_thr;
+                }
+                const unsigned bal = __ballot_sync(FULL, keep);
+                if (keep) cq[(qhead + qlen + __popc(bal & ((1u << lane) - 1u))) & (CQ_N - 1)] = ent;
+                qlen += __popc(bal);
+                c_s += 32;
+                cur.next(R, n_seg);
             }
-            const unsigned bal = __ballot_sync(FULL, keep);
-            if (keep) cq[(qhead + qlen + __popc(bal & ((1u << lane) - 1u))) & (CQ_N - 1)] = ent;
-            qlen += __popc(bal);
-            c_s += 32;
-        }
-        __syncwarp();
-        const int nb = qlen < 32 ? qlen : 32;
-        if (nb == 0) break;
-        // lane c stages candidate c of the batch (absent ones: zero rows,
-        // zero features, thr = -inf)
-        {
-            const bool has = lane < nb;
-            const float4 ent = has ? cq[(qhead + lane) & (CQ_N - 1)] : make_float4(0.f, 0.f, 0.f, 0.f);
-            const int i = __float_as_int(ent.w);
-            stage_label_row<DP, SPLIT>(cl + lane * LW, A.sem_sorted, i, ls, has);
-            const float x0 = ent.x, x1 = ent.y, x2 = ent.z;
-            const float xx = fmaf(x0, x0, fmaf(x1, x1, x2 * x2));
-            float* cgp = cg + 12 * (lane >> 1) + (lane & 1);
-            cgp[0] = x0;
-            cgp[2] = x1;
-            cgp[4] = x2;
-            cgp[6] = has ? gp.rc2 - xx : -INF;
-            cgp[8] = fmaf(xx, gp.kg, kwf);
-            const float u0 = x0 * xs, u1 = x1 * xs, u2 = x2 * xs;
-            unsigned h0, h1, h2, h3, h4, l0, l1, l2, l3, l4;
-            split_f16x2(has ? 1.f : 0.f, u0, h0, l0);
-            split_f16x2(u1, u2, h1, l1);
-            split_f16x2(u0 * u0, u0 * u1, h2, l2);
-            split_f16x2(u0 * u2, u1 * u1, h3, l3);
-            split_f16x2(u1 * u2, u2 * u2, h4, l4);
-            uint4* frow = reinterpret_cast<uint4*>(cf + 12 * lane);
-            frow[0] = make_uint4(h0, h1, h2, h3);
-            frow[1] = make_uint4(h4, l4, 0u, 0u);
-            frow[2] = make_uint4(l0, l1, l2, l3);
-        }
-        qhead = (qhead + nb) & (CQ_N - 1);
-        qlen -= nb;
-        __syncwarp();
-        u64 n_in = 0ull;     // pairs inside r_c of this lane's elements of the batch, as FP32 counts
-        // m tiles one after another, not unrolled: the smaller loop body ran
-        // faster (LiDAR 0.344 -> 0.284 ms, window 2.00 -> 1.85 ms, mapping
-        // within 1%)
+            __syncwarp();
+            const int nb = qlen < 32 ? qlen : 32;
+            if (nb == 0) break;
+            // lane c stages candidate c of the batch (absent ones: zero rows,
+            // zero features, thr = -inf)
+            {
+                const bool has = lane < nb;
+                const float4 ent = has ? cq[(qhead + lane) & (CQ_N - 1)] : make_float4(0.f, 0.f, 0.f, 0.f);
+                const int i = __float_as_int(ent.w);
+                stage_label_row<DP, SPLIT>(cl + lane * LW, A.sem_sorted, i, ls, has);
+                const float x0 = ent.x, x1 = ent.y, x2 = ent.z;
+                const float xx = fmaf(x0, x0, fmaf(x1, x1, x2 * x2));
+                float* cgp = cg + 12 * (lane >> 1) + (lane & 1);
+                cgp[0] = x0;
+                cgp[2] = x1;
+                cgp[4] = x2;
+                cgp[6] = has ? gp.rc2 - xx : -INF;
+                cgp[8] = fmaf(xx, gp.kg, kwf);
+                const float u0 = x0 * xs, u1 = x1 * xs, u2 = x2 * xs;
+                unsigned h0, h1, h2, h3, h4, l0, l1, l2, l3, l4;
+                split_f16x2(has ? 1.f : 0.f, u0, h0, l0);
+                split_f16x2(u1, u2, h1, l1);
+                split_f16x2(u0 * u0, u0 * u1, h2, l2);
+                split_f16x2(u0 * u2, u1 * u1, h3, l3);
+                split_f16x2(u1 * u2, u2 * u2, h4, l4);
+                uint4* frow = reinterpret_cast<uint4*>(cf + 12 * lane);
+                frow[0] = make_uint4(h0, h1, h2, h3);
+                frow[1] = make_uint4(h4, l4, 0u, 0u);
+                frow[2] = make_uint4(l0, l1, l2, l3);
+            }
+            qhead = (qhead + nb) & (CQ_N - 1);
+            qlen -= nb;
+            __syncwarp();
+            u64 n_in = 0ull;     // pairs inside r_c of this lane's elements of the batch, as FP32 counts
+            // 16 candidates at a time (one k step of the moment MMAs), not
+            // unrolled: the smaller loop body fetches faster
 #pragma unroll 1
-        for (int mt = 0; mt < L::MAXQ / 16; ++mt) {
-            if (mt >= n_mt) break;
-            // query-side A fragments of the label products: rows 16 mt ..
-            // 16 mt + 15 (FP32 labels: hi and lo parts)
-            const unsigned* qrowp = ql + (16 * mt + (lane & 7) + 8 * ((lane >> 3) & 1)) * LW;
-            unsigned qa[2 * NKC];
-            load_a_chunks<NKC>(qa, qrowp);
-            unsigned qal[SPLIT ? 2 * NKC : 1];
-            if constexpr (SPLIT) load_a_chunks<NKC>(qal, qrowp + PW);
-            // per candidate tile nt (8 candidates): label products, then the
-            // weights of rows q0 = 16 mt + g, q0 + 8 and columns 8 nt + 2 t4,
-            // + 1, split into the FP16 A operands of the moment MMAs
-            unsigned ah[2][4], al[2][4];
-            const ulonglong2* q2 = reinterpret_cast<const ulonglong2*>(qg);
-            const float4* qg4 = reinterpret_cast<const float4*>(qg);
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                const unsigned* crowp = cl + (8 * nt + (lane & 7)) * LW;
-                unsigned cb[NKC];
-                load_b_chunks<NKC>(cb, crowp);
-                float s[4];
-                if constexpr (SPLIT) {
-                    // FP32 labels: hi*hi + hi*lo + lo*hi of the FP16 parts
-                    unsigned cbl[NKC];
-                    load_b_chunks<NKC>(cbl, crowp + PW);
-                    gram_chunks<NKC, true, true>(s, qa, cb);
-                    gram_chunks<NKC, true, false>(s, qa, cbl);
-                    gram_chunks<NKC, true, false>(s, qal, cb);
-                } else {
-                    gram_chunks<NKC, false, true>(s, qa, cb);
-                }
-                const int p = 4 * nt + t4;
-                const ulonglong2 c01 = *reinterpret_cast<const ulonglong2*>(cg + 12 * p);
-                const ulonglong2 c2t = *reinterpret_cast<const ulonglong2*>(cg + 12 * p + 4);
-                const u64 XK = *reinterpret_cast<const u64*>(cg + 12 * p + 8);
-                const float2 thr = f2_split(c2t.y);
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const int q = 16 * mt + g + 8 * i;
-                    ulonglong2 QA, QB;
-                    if constexpr (SPLIT) {
-                        const float4 qv = qg4[q];
-                        QA = make_ulonglong2(f2(qv.x, qv.x), f2(qv.y, qv.y));
-                        QB = make_ulonglong2(f2(qv.z, qv.z), f2(qv.w, qv.w));
-                    } else {
-                        QA = q2[2 * q];
-                        QB = q2[2 * q + 1];
-                    }
-                    const u64 T = ffma2(c01.x, QA.x, ffma2(c01.y, QA.y, ffma2(c2t.x, QB.x, QB.y)));
-                    const float2 t = f2_split(T);
-                    const float2 a = f2_split(ffma2(T, KG2, XK));
-                    const u64 in = f2(inside_mask(t.x, thr.x), inside_mask(t.y, thr.y));
-                    n_in = fadd2(n_in, in);
-                    const float2 w = f2_split(fmul2(fmul2(f2(s[2 * i], s[2 * i + 1]), in),
-                                                    f2(ex2_approx(a.x), ex2_approx(a.y))));
-                    split_f16x2(w.x, w.y, ah[nt >> 1][2 * (nt & 1) + i], al[nt >> 1][2 * (nt & 1) + i]);
-                }
-            }
-            // per query: sum over the batch's candidates of w (1, x, x x^T);
-            // feature B fragments (FP16 hi and lo) of each 16-candidate k step
-            float t[2][4];
-#pragma unroll
             for (int ks = 0; ks < 2; ++ks) {
+                if (16 * ks >= nb) break;
+                // label products, then the weights of this lane's rows and of
+                // columns 8 nt + 2 t4, + 1, split into the FP16 A operands of
+                // the moment MMAs
+                unsigned ah[MT][4], al[MT][4];
+#pragma unroll
+                for (int n1 = 0; n1 < 2; ++n1) {
+                    const int nt = 2 * ks + n1;
+                    const unsigned* crowp = cl + (8 * nt + (lane & 7)) * LW;
+                    unsigned cb[NKC];
+                    [[maybe_unused]] unsigned cbl[NKC];
+                    load_b_chunks<NKC>(cb, crowp);
+                    if constexpr (SPLIT) load_b_chunks<NKC>(cbl, crowp + PW);
+                    const int p = 4 * nt + t4;
+                    const ulonglong2 c01 = *reinterpret_cast<const ulonglong2*>(cg + 12 * p);
+                    const ulonglong2 c2t = *reinterpret_cast<const ulonglong2*>(cg + 12 * p + 4);
+                    const u64 XK = *reinterpret_cast<const u64*>(cg + 12 * p + 8);
+                    const float2 thr = f2_split(c2t.y);
+#pragma unroll
+                    for (int mt = 0; mt < MT; ++mt) {
+                        float s[4];
+                        if constexpr (SPLIT) {
+                            // FP32 labels: hi*hi + hi*lo + lo*hi of the FP16 parts
+                            gram_chunks<NKC, true, true>(s, qa[mt], cb);
+                            gram_chunks<NKC, true, false>(s, qa[mt], cbl);
+                            gram_chunks<NKC, true, false>(s, qal[mt], cb);
+                        } else {
+                            gram_chunks<NKC, false, true>(s, qa[mt], cb);
+                        }
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            const u64(&m)[4] = qm[2 * mt + i];
+                            const u64 T = ffma2(c01.x, m[0], ffma2(c01.y, m[1], ffma2(c2t.x, m[2], m[3])));
+                            const float2 t = f2_split(T);
+                            const float2 a = f2_split(ffma2(T, KG2, XK));
+                            const u64 in = f2(inside_mask(t.x, thr.x), inside_mask(t.y, thr.y));
+                            n_in = fadd2(n_in, in);
+                            const float2 w = f2_split(fmul2(fmul2(f2(s[2 * i], s[2 * i + 1]), in),
+                                                            f2(ex2_approx(a.x), ex2_approx(a.y))));
+                            split_f16x2(w.x, w.y, ah[mt][2 * n1 + i], al[mt][2 * n1 + i]);
+                        }
+                    }
+                }
+                // per query: sum over the 16 candidates of w (1, x, x x^T);
+                // feature B fragments, FP16 hi and lo
                 unsigned fh[4], fl[2];
                 const unsigned* rowp = cf + 12 * (16 * ks + (lane & 7) + 8 * ((lane >> 3) & 1));
                 ldsm_x4_t(fh, rowp + 4 * (lane >> 4));
                 ldsm_x2_t(fl, rowp + 8);
-                if (ks == 0) {
-                    mma_f16_16816_first(t[0], ah[ks], fh[0], fh[1]);
-                    mma_f16_16816_first(t[1], ah[ks], fh[2], fh[3]);
-                } else {
-                    mma_f16_16816(t[0], ah[ks], fh[0], fh[1]);
-                    mma_f16_16816(t[1], ah[ks], fh[2], fh[3]);
-                }
-                mma_f16_16816(t[1], al[ks], fh[2], fh[3]);
-                mma_f16_16816(t[0], ah[ks], fl[0], fl[1]);
-                mma_f16_16816(t[0], al[ks], fh[0], fh[1]);
-            }
-            {
-                float4 r = run0[32 * mt];
-                r.x += t[0][0];
-                r.y += t[0][1];
-                r.z += t[0][2];
-                r.w += t[0][3];
-                run0[32 * mt] = r;
-                if (t4 < 2) {      // features 8, 9: hi (t4 = 0) and lo parts (the other columns of tile 1 are zero)
-                    float4 r1 = run1[16 * mt];
-                    r1.x += t[1][0];
-                    r1.y += t[1][1];
-                    r1.z += t[1][2];
-                    r1.w += t[1][3];
-                    run1[16 * mt] = r1;
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt) {
+                    float t[2][4];
+                    mma_f16_16816_first(t[0], ah[mt], fh[0], fh[1]);
+                    mma_f16_16816_first(t[1], ah[mt], fh[2], fh[3]);
+                    mma_f16_16816(t[1], al[mt], fh[2], fh[3]);
+                    mma_f16_16816(t[0], ah[mt], fl[0], fl[1]);
+                    mma_f16_16816(t[0], al[mt], fh[0], fh[1]);
+#pragma unroll
+                    for (int n2 = 0; n2 < 2; ++n2)
+#pragma unroll
+                        for (int k = 0; k < 4; k += 2) {
+                            const float2 r = f2_split(fadd2(f2(run[mt][n2][k], run[mt][n2][k + 1]),
+                                                            f2(t[n2][k], t[n2][k + 1])));
+                            run[mt][n2][k] = r.x;
+                            run[mt][n2][k + 1] = r.y;
+                        }
                 }
             }
+            const float2 n2 = f2_split(n_in);
+            cnt += (int)n2.x + (int)n2.y;
         }
-        const float2 n2 = f2_split(n_in);
-        cnt += (int)n2.x + (int)n2.y;
+    };
+    if (C > 0) {
+        if (qcount > 16) batches(std::integral_constant<int, 2>{});
+        else batches(std::integral_constant<int, 1>{});
     }
-    // unit end: per-query sums through shared memory to one lane per query
-    // (32 queries at a time), formed into this lane's moments
-    float W = 0.f, Dv[3] = {0.f, 0.f, 0.f}, Sy[3] = {0.f, 0.f, 0.f}, Myy[6], Mdy[9], Qm[6];
+    // unit end: the per-query sums as they are; k_query_moments forms the moments
+    float* qs8 = A.qs8 + 8LL * k0;
+    float* qs2 = A.qs2 + 2LL * k0;
 #pragma unroll
-    for (int k = 0; k < 6; ++k) Myy[k] = Qm[k] = 0.f;
+    for (int mt = 0; mt < 2; ++mt) {
+        float (&r1)[4] = run[mt][1];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) Mdy[k] = 0.f;
-    const float s0 = ldexpf(1.f, -KW), s1 = ldexpf(1.f, ex - KW), s2 = ldexpf(1.f, 2 * ex - KW);
-    float* sq = reinterpret_cast<float*>(cf);    // [32][12] (features 0..9 used)
+        for (int k = 0; k < 4; ++k) r1[k] += __shfl_xor_sync(FULL, r1[k], 1);    // hi and lo parts of features 8, 9
 #pragma unroll
-    for (int h = 0; h < L::MAXQ / 32; ++h) {
-        __syncwarp();
-#pragma unroll
-        for (int m2 = 0; m2 < 2; ++m2) {
-            const int mt = 2 * h + m2;
-            const int q0 = 16 * m2 + g;
-            const float4 r = run0[32 * mt];
-            *reinterpret_cast<float2*>(sq + 12 * q0 + 2 * t4) = make_float2(r.x, r.y);
-            *reinterpret_cast<float2*>(sq + 12 * (q0 + 8) + 2 * t4) = make_float2(r.z, r.w);
-            if (t4 == 0) {
-                const float4 rh = run1[16 * mt], rl = run1[16 * mt + 1];
-                const float4 r1 = make_float4(rh.x + rl.x, rh.y + rl.y, rh.z + rl.z, rh.w + rl.w);
-                *reinterpret_cast<float2*>(sq + 12 * q0 + 8) = make_float2(r1.x, r1.y);
-                *reinterpret_cast<float2*>(sq + 12 * (q0 + 8) + 8) = make_float2(r1.z, r1.w);
+        for (int i = 0; i < 2; ++i) {
+            const int q = 16 * mt + 8 * i + g;
+            if (q < qcount) {
+                *reinterpret_cast<float2*>(qs8 + 8 * q + 2 * t4) = make_float2(run[mt][0][2 * i], run[mt][0][2 * i + 1]);
+                if (t4 == 0) *reinterpret_cast<float2*>(qs2 + 2 * q) = make_float2(r1[2 * i], r1[2 * i + 1]);
             }
         }
-        __syncwarp();
-        const int q = lane + 32 * h;
-        const float4* rq = reinterpret_cast<const float4*>(sq + 12 * lane);
-        const float4 r0 = rq[0], r1 = rq[1];
-        const float2 r2 = *reinterpret_cast<const float2*>(sq + 12 * lane + 8);
-        float y[3];
-        if constexpr (SPLIT) {
-            const float4 qm = reinterpret_cast<const float4*>(qg)[q];
-            y[0] = -0.5f * qm.x;
-            y[1] = -0.5f * qm.y;
-            y[2] = -0.5f * qm.z;
-        } else {
-            const float4 qm = reinterpret_cast<const float4*>(qg)[2 * q];
-            y[0] = -0.5f * qm.x;
-            y[1] = -0.5f * qm.z;
-            y[2] = -0.5f * qg[8 * q + 4];
-        }
-        const float k = r0.x * s0;
-        const float X1[3] = {r0.y * s1, r0.z * s1, r0.w * s1};
-        const float X2[6] = {r1.x * s2, r1.y * s2, r1.z * s2, r1.w * s2, r2.x * s2, r2.y * s2};
-        float ky[3], D[3];
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            ky[m] = k * y[m];
-            D[m] = X1[m] - ky[m];
-        }
-        W += k;
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            Sy[m] += ky[m];
-            Dv[m] += D[m];
-        }
-        int t6 = 0;
-#pragma unroll
-        for (int m = 0; m < 3; ++m)
-#pragma unroll
-            for (int l = m; l < 3; ++l, ++t6) {
-                const float kyy = ky[m] * y[l];
-                Myy[t6] += kyy;
-                Qm[t6] += X2[t6] - X1[m] * y[l] - y[m] * X1[l] + kyy;
-            }
-#pragma unroll
-        for (int m = 0; m < 3; ++m)
-#pragma unroll
-            for (int l = 0; l < 3; ++l) Mdy[3 * m + l] = fmaf(D[m], y[l], Mdy[3 * m + l]);
     }
-    store_moments(W, Dv, Sy, Myy, Mdy, Qm, cnt, Fa, hx, hy, hz, gp, A.edges[e].scale,
-                  A.acc + (long long)e * ACC_N, lane);
+    cnt = __reduce_add_sync(FULL, cnt);
+    if (lane == 0 && cnt > 0)
+        atomicAdd(reinterpret_cast<unsigned long long*>(A.acc + (long long)e * ACC_N + N_MOM - 1),
+                  (unsigned long long)cnt);
 }
 
-// One unit (<= A.uq queries of one frame-a home cell, starting at sorted
-// query k0) of the pair sum: stage the queries, stream the candidates of the
+// Moments of the dense path, one query per lane: from the query's k, X1 and X2
+// (sum_c w (1, x, x x^T), powers of two undone exactly) and its place y it
+// forms, with o the home cell's centre,
+//   W = k, D = X1 - k y, sum w y', sum w y'y'^T, sum w d y'^T (y' = y + o)
+//   and Q = X2 - X1 y^T - y X1^T + k y y^T.
+// A lane adds its queries of the `per` (<= MOM_PER) groups of 32 sorted queries
+// that its warp takes, the sums are rounded to the edge's fixed point and
+// added in 64-bit integers.  As a pass of its own every lane has a query, and
+// the rounding and the reduction over the lanes are paid once per 128 queries;
+// at the end of each unit of the pair kernel they cost ~1000 instructions for
+// (LiDAR scenes) 8 queries in the median.
+constexpr int MOM_PER = 4;
+__global__ void __launch_bounds__(128, 5) k_query_moments(const PairArgs A, int per, const int* done) {
+    if (done && *done) return;
+    const int lane = threadIdx.x & 31;
+    const GridParams& gp = A.gp;
+    const long long w0 = ((long long)blockIdx.x * 4 + (threadIdx.x >> 5)) * per * 32;
+    float W = 0.f, D[3], Sy[3], Myy[6], Mdy[9], Q[6];
+    auto clear = [&]() {
+        W = 0.f;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) D[k] = Sy[k] = 0.f;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) Myy[k] = Q[k] = 0.f;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) Mdy[k] = 0.f;
+    };
+    clear();
+    // edge of the sums so far: its home-cell keys, scales and frame-a grid
+    int e_cur = -1, lo0 = 0, lo1 = 0, lo2 = 0, dim0 = 1, dim1 = 1;
+    long long bin_lo = 0, bin_hi = 0;
+    float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+    auto flush = [&]() {
+        if (e_cur >= 0)
+            add_moments(W, D, Sy, Myy, Mdy, Q, 0, A.edges[e_cur].scale, A.acc + (long long)e_cur * ACC_N, lane);
+    };
+    for (int r = 0; r < per; ++r) {
+        const long long k = w0 + 32LL * r + lane;
+        const uint32_t kq = k < A.Q ? A.qkey[k] : NO_KEY;
+        const bool valid = kq != NO_KEY;
+        unsigned todo = __ballot_sync(FULL, valid);
+        if (!todo) break;                    // keys of no home cell sort last
+        const long long key = (long long)(kq >> gp.key_sub);
+        float4 q = make_float4(0.f, 0.f, 0.f, 0.f), f0 = q, f1 = q;
+        float2 f2v = make_float2(0.f, 0.f);
+        if (valid) {
+            q = A.slots[k];
+            const float4* p8 = reinterpret_cast<const float4*>(A.qs8) + 2 * k;
+            f0 = p8[0];
+            f1 = p8[1];
+            f2v = reinterpret_cast<const float2*>(A.qs2)[k];
+        }
+        while (todo) {
+            const long long kl = __shfl_sync(FULL, key, __ffs(todo) - 1);
+            if (kl < bin_lo || kl >= bin_hi) {
+                flush();
+                clear();
+                e_cur = find_edge_bin(A.edges, A.E, kl);
+                const EdgeDev& Ed = A.edges[e_cur];
+                const FrameDev& Fa = A.frames[Ed.a];
+                lo0 = Fa.lo[0];
+                lo1 = Fa.lo[1];
+                lo2 = Fa.lo[2];
+                dim0 = Fa.dim[0];
+                dim1 = Fa.dim[1];
+                bin_lo = Ed.bin_off;
+                bin_hi = bin_lo + (long long)dim0 * dim1 * Fa.dim[2];
+                const DenseScales sc = dense_scales(Fa.sem_norm_max, A.frames[Ed.b].sem_norm_max, gp.hf, false);
+                s0 = ldexpf(1.f, -sc.kw);
+                s1 = ldexpf(1.f, sc.ex - sc.kw);
+                s2 = ldexpf(1.f, 2 * sc.ex - sc.kw);
+            }
+            const bool mine = valid && key >= bin_lo && key < bin_hi;
+            todo &= ~__ballot_sync(FULL, mine);
+            if (mine) {
+                const int cell = (int)(key - bin_lo);
+                const int row = cell / dim0, hx = cell - row * dim0, hz = row / dim1, hy = row - hz * dim1;
+                const float o[3] = {((float)(hx + lo0) + 0.5f) * gp.hf, ((float)(hy + lo1) + 0.5f) * gp.hf,
+                                    ((float)(hz + lo2) + 0.5f) * gp.hf};
+                const float y[3] = {q.x, q.y, q.z};
+                const float w = f0.x * s0;
+                const float X1[3] = {f0.y * s1, f0.z * s1, f0.w * s1};
+                const float X2[6] = {f1.x * s2, f1.y * s2, f1.z * s2, f1.w * s2, f2v.x * s2, f2v.y * s2};
+                W += w;
+                int t6 = 0;
+#pragma unroll
+                for (int m = 0; m < 3; ++m) {
+                    const float ky = w * y[m], d = X1[m] - ky;
+                    D[m] += d;
+                    Sy[m] += fmaf(w, o[m], ky);
+#pragma unroll
+                    for (int l = m; l < 3; ++l, ++t6) {
+                        const float kyy = ky * y[l], kyl = w * y[l];
+                        Myy[t6] += kyy + (ky * o[l] + o[m] * kyl + w * o[m] * o[l]);
+                        Q[t6] += X2[t6] - X1[m] * y[l] - y[m] * X1[l] + kyy;
+                    }
+#pragma unroll
+                    for (int l = 0; l < 3; ++l) Mdy[3 * m + l] += fmaf(d, o[l], d * y[l]);
+                }
+            }
+        }
+    }
+    flush();
+}
+
+// One unit (queries of one frame-a home cell) of the pair sum: stage the queries, stream the candidates of the
 // 27-cell stencil, test, walk and fold, and add the unit's moments to its
 // edge.  wb is the warp's shared-memory block.
 template <int DP, bool BF16, bool COLOR>
-__device__ __forceinline__ void pair_unit(const PairArgs& A, int k0, float* wb, int lane) {
+__device__ __forceinline__ void pair_unit(const PairArgs& A, int2 unit, float* wb, int lane) {
     const uint32_t* __restrict__ qkey = A.qkey;
     const float4* __restrict__ slots = A.slots;
-    const long long Q = A.Q;
     const EdgeDev* __restrict__ edges = A.edges;
-    const int E = A.E;
     const FrameDev* __restrict__ frames = A.frames;
     const int* __restrict__ cell_start = A.cell_start;
     const float4* __restrict__ pts4 = A.pts4;
@@ -1266,22 +1314,19 @@ __device__ __forceinline__ void pair_unit(const PairArgs& A, int k0, float* wb, 
     float* smt = wb + 4 * UQ;                                         // [UQ/2][8] test records
     float4* scq = reinterpret_cast<float4*>(wb + 8 * UQ);             // [UQ] query colours
     float* ssq = wb + (COLOR ? 12 : 8) * UQ;                          // [UQ][SW] query labels
-    int* ri = reinterpret_cast<int*>(ssq + UQ * SW);
-    const Rows R{ri, ri + 9, ri + 18, ri + 27};
-    float4* sacc = reinterpret_cast<float4*>(ri + 40) + lane * (N_ACC / 4);   // this lane's unit sums
-    float4* cq = reinterpret_cast<float4*>(ri + 40) + 32 * (N_ACC / 4);       // candidate ring
+    float* ri = ssq + UQ * SW;
+    const Rows R{reinterpret_cast<int4*>(ri), reinterpret_cast<float2*>(ri + 36)};
+    float4* sacc = reinterpret_cast<float4*>(ri + ROWS_WORDS) + lane * (N_ACC / 4);   // this lane's unit sums
+    float4* cq = reinterpret_cast<float4*>(ri + ROWS_WORDS) + 32 * (N_ACC / 4);       // candidate ring
     float* gram = reinterpret_cast<float*>(cq + CQ_N);                        // [query][candidate] (BF16)
     const ulonglong2* walk2 = reinterpret_cast<const ulonglong2*>(smw);
     const ulonglong2* test2 = reinterpret_cast<const ulonglong2*>(smt);
     const u64 H2 = f2(0.5f, 0.5f);
-    const uint32_t kq0 = qkey[k0];
-    const int qcount = unit_queries(qkey, Q, k0, kq0, lane, A.uq, gp.key_sub);
-    const uint32_t key0 = kq0 >> gp.key_sub;                 // home-cell key
-    const int e = find_edge_bin(edges, E, key0);
+    const int k0 = unit.x, qcount = unit.y & 127, e = unit.y >> 7;
+    const uint32_t key0 = qkey[k0] >> gp.key_sub;            // home-cell key
     const FrameDev& Fa = frames[edges[e].a];
-    const int dx0 = Fa.dim[0], dy0 = Fa.dim[1], dz0 = Fa.dim[2];
     const int cell = (int)(key0 - edges[e].bin_off);
-    const int hx = cell % dx0, hy = (cell / dx0) % dy0, hz = cell / (dx0 * dy0);
+    const int hx = cell % Fa.dim[0], hy = (cell / Fa.dim[0]) % Fa.dim[1], hz = cell / (Fa.dim[0] * Fa.dim[1]);
     __syncwarp();
     // bounding box of the unit's queries (home-centre coordinates)
     float blo0 = __int_as_float(0x7f800000), blo1 = blo0, blo2 = blo0;
@@ -1320,20 +1365,17 @@ __device__ __forceinline__ void pair_unit(const PairArgs& A, int k0, float* wb, 
         bhi1 = fmaxf(bhi1, __shfl_xor_sync(FULL, bhi1, o));
         bhi2 = fmaxf(bhi2, __shfl_xor_sync(FULL, bhi2, o));
     }
-    const int C = build_rows(R, cell_start, Fa.cell_off, dx0, dy0, dz0, hx, hy, hz, lane);
-    const int np = (qcount + 1) >> 1;
     // a candidate farther than r_c from the query box pairs with none of
     // the queries; the margin keeps every candidate the exact test passes
     const float box_thr = gp.rc2 * 1.0001f;
-    // BF16 labels: the Gram path leaves registers free, so the stencil row
-    // prefix, the query-side MMA fragments and the per-lane unit sums live
-    // in registers instead of shared memory
+    int n_seg;
+    const int C = build_rows(R, cell_start, Fa, hx, hy, hz, blo0, blo1, blo2, bhi0, bhi1, bhi2, gp.hf, box_thr, lane, n_seg);
+    if (C == 0) return;
+    const int np = (qcount + 1) >> 1;
+    // BF16 labels: the Gram path leaves registers free, so the query-side MMA
+    // fragments and the per-lane unit sums live in registers instead of
+    // shared memory
     constexpr bool REG = BF16 && DP > 0;
-    int pre[9];
-    if constexpr (REG) {
-#pragma unroll
-        for (int k = 0; k < 9; ++k) pre[k] = R.pre[k];
-    }
     GramB<(BF16 && DP > 0) ? DP : 16> gb;
     if constexpr (REG) gb.load(ssq, lane);
 
@@ -1349,23 +1391,16 @@ __device__ __forceinline__ void pair_unit(const PairArgs& A, int k0, float* wb, 
     }
     int cnt = 0;
     int c_s = 0, qhead = 0, qlen = 0;            // stream position, ring head and fill
+    Cursor cur;
+    cur.start(R, n_seg, lane);
     while (c_s < C || qlen > 0) {
         // stream the 27-cell candidates through the box test into the
         // ring until it holds a full batch (or the stream ends)
         while (qlen < 32 && c_s < C) {
-            const int v = c_s + lane;
             bool keep = false;
             float4 ent = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (v < C) {
-                int dx, dy, dz;
-                int i;
-                if constexpr (REG) i = stream_point_r(R, pre, v, dx, dy, dz);
-                else i = stream_point(R, v, dx, dy, dz);
-                const float4 p = __ldg(pts4 + i);
-                ent.x = fmaf((float)dx, gp.hf, p.x);
-                ent.y = fmaf((float)dy, gp.hf, p.y);
-                ent.z = fmaf((float)dz, gp.hf, p.z);
-                ent.w = __int_as_float(i);
+            if (cur.valid()) {
+                ent = cur.point(pts4, gp.hf);
                 const float e0 = fmaxf(fmaxf(blo0 - ent.x, ent.x - bhi0), 0.f);
                 const float e1 = fmaxf(fmaxf(blo1 - ent.y, ent.y - bhi1), 0.f);
                 const float e2 = fmaxf(fmaxf(blo2 - ent.z, ent.z - bhi2), 0.f);
@@ -1375,6 +1410,7 @@ __device__ __forceinline__ void pair_unit(const PairArgs& A, int k0, float* wb, 
             if (keep) cq[(qhead + qlen + __popc(bal & ((1u << lane) - 1u))) & (CQ_N - 1)] = ent;
             qlen += __popc(bal);
             c_s += 32;
+            cur.next(R, n_seg);
         }
         __syncwarp();
         const int nb = qlen < 32 ? qlen : 32;
@@ -1514,6 +1550,7 @@ __device__ __forceinline__ void pair_unit(const PairArgs& A, int k0, float* wb, 
                 sacc[k] = make_float4(a[4 * k], a[4 * k + 1], a[4 * k + 2], a[4 * k + 3]);
         }
     }
+    if (!__any_sync(FULL, cnt != 0)) return;     // no pair: every sum is zero
     float a_s[REG ? 1 : N_ACC];
     float* a = REG ? racc : a_s;
     if constexpr (!REG) {
@@ -1554,26 +1591,22 @@ __device__ __forceinline__ void pair_unit(const PairArgs& A, int k0, float* wb, 
 
 }
 
-// Shared-memory words per warp of the bit-walk (DENSE false) or the dense
-// tile unit (BF16 labels, no colour).
-// DENSE: 0 bit walk, 1 dense tile with units of <= 32 queries, 2 dense tile
-// with units of <= 64 queries (BF16 labels).
-template <int DP, bool BF16, bool COLOR, int DENSE>
+// Shared-memory words per warp of the bit-walk or the dense tile unit.
+template <int DP, bool BF16, bool COLOR, bool DENSE>
 __host__ __device__ constexpr int unit_smem_words() {
-    if constexpr (DENSE > 0) return DenseSmem<(DP > 0 ? DP : 8), !BF16, DENSE == 2 ? 64 : 32>::WORDS;
+    if constexpr (DENSE) return DenseSmem<(DP > 0 ? DP : 8), !BF16>::WORDS;
     else return warp_smem_words<DP, BF16, COLOR>();
 }
 
-template <int DP, bool BF16, bool COLOR, int DENSE>
-__device__ __forceinline__ void run_unit(const PairArgs& A, int k0, float* wb, int lane) {
-    if constexpr (DENSE > 0 && DP > 0 && !COLOR) pair_unit_dense<DP, !BF16, DENSE == 2 ? 64 : 32>(A, k0, wb, lane);
-    else pair_unit<DP, BF16, COLOR>(A, k0, wb, lane);
+template <int DP, bool BF16, bool COLOR, bool DENSE>
+__device__ __forceinline__ void run_unit(const PairArgs& A, int2 unit, float* wb, int lane) {
+    if constexpr (DENSE && DP > 0 && !COLOR) pair_unit_dense<DP, !BF16>(A, unit, wb, lane);
+    else pair_unit<DP, BF16, COLOR>(A, unit, wb, lane);
 }
 
-template <int DP, bool BF16, bool COLOR, int DENSE>
-__global__ void __launch_bounds__(PAIR_T, DENSE ? dense_min_blocks<DP, BF16, DENSE>()
-                                                  : ((BF16 && DP > 0) ? 2 : RK_PAIR_MINB))
-k_pairs(const int* __restrict__ unit_start, const int* __restrict__ n_units, int* unit_counter,
+template <int DP, bool BF16, bool COLOR, bool DENSE>
+__global__ void __launch_bounds__(PAIR_T, 2)
+k_pairs(const int2* __restrict__ units, const int* __restrict__ n_units, int* unit_counter,
         const PairArgs A, const int* done) {
     if (done && *done) return;
     extern __shared__ float4 smem4[];
@@ -1586,7 +1619,7 @@ k_pairs(const int* __restrict__ unit_start, const int* __restrict__ n_units, int
         if (lane == 0) u = atomicAdd(unit_counter, 1);
         u = __shfl_sync(FULL, u, 0);
         if (u >= nu) break;
-        run_unit<DP, BF16, COLOR, DENSE>(A, unit_start[u], wb, lane);
+        run_unit<DP, BF16, COLOR, DENSE>(A, units[u], wb, lane);
     }
 }
 
@@ -1596,9 +1629,8 @@ k_pairs(const int* __restrict__ unit_start, const int* __restrict__ n_units, int
 // the job by binary search over the prefix, and run the unit with that
 // job's arrays.  Every job adds into its own fixed-point accumulators, so a
 // problem's results do not depend on which other problems share the launch.
-template <int DP, bool BF16, bool COLOR, int DENSE>
-__global__ void __launch_bounds__(PAIR_T, DENSE ? dense_min_blocks<DP, BF16, DENSE>()
-                                                  : ((BF16 && DP > 0) ? 2 : RK_PAIR_MINB))
+template <int DP, bool BF16, bool COLOR, bool DENSE>
+__global__ void __launch_bounds__(PAIR_T, 2)
 k_pairs_multi(const PairJob* __restrict__ jobs, int n_jobs, int* unit_counter) {
     __shared__ int s_pref[MAX_PAIR_JOBS + 1];
     extern __shared__ float4 smem4[];
@@ -1638,7 +1670,7 @@ k_pairs_multi(const PairJob* __restrict__ jobs, int n_jobs, int* unit_counter) {
             if (s_pref[mid] <= u) lo = mid; else hi = mid - 1;
         }
         const PairJob* J = jobs + lo;
-        run_unit<DP, BF16, COLOR, DENSE>(J->a, J->unit_start[u - s_pref[lo]], wb, lane);
+        run_unit<DP, BF16, COLOR, DENSE>(J->a, J->units[u - s_pref[lo]], wb, lane);
     }
 }
 
@@ -1651,17 +1683,17 @@ k_pairs_multi(const PairJob* __restrict__ jobs, int n_jobs, int* unit_counter) {
 // sum w d y'^T = D y^T.
 template <int DP, bool BF16, bool COLOR>
 __host__ __device__ constexpr int warp_smem_words_topk() {
-    return 32 * 4 + 32 * SemRow<DP, BF16>::WORDS + (COLOR ? 32 * 4 : 0) + 4 * CQ_N + 4 * 10;
+    return 32 * 4 + 32 * SemRow<DP, BF16>::WORDS + (COLOR ? 32 * 4 : 0) + 4 * CQ_N + ROWS_WORDS;
 }
 
 template <int DP, bool BF16, bool COLOR>
 __global__ void __launch_bounds__(PAIR_T, 2)
-k_pairs_topk(const int* __restrict__ unit_start, const int* __restrict__ n_units, int* unit_counter,
-             const uint32_t* __restrict__ qkey, const float4* __restrict__ slots, long long Q,
-             const EdgeDev* __restrict__ edges, int E, const FrameDev* __restrict__ frames,
+k_pairs_topk(const int2* __restrict__ units, const int* __restrict__ n_units, int* unit_counter,
+             const uint32_t* __restrict__ qkey, const float4* __restrict__ slots,
+             const EdgeDev* __restrict__ edges, const FrameDev* __restrict__ frames,
              const int* __restrict__ cell_start, const float4* __restrict__ pts4,
              const void* __restrict__ sem_sorted, const float4* __restrict__ col4, GridParams gp,
-             long long* __restrict__ acc, int uq, const int* done) {
+             long long* __restrict__ acc, const int* done) {
     if (done && *done) return;
     extern __shared__ float4 smem4[];
     constexpr int SW = SemRow<DP, BF16>::WORDS;
@@ -1672,8 +1704,7 @@ k_pairs_topk(const int* __restrict__ unit_start, const int* __restrict__ n_units
     float* srow = wb + 4 * 32;                                        // [32][SW] their label rows
     float4* scc = reinterpret_cast<float4*>(srow + 32 * SW);          // [32] their colours
     float4* cq = reinterpret_cast<float4*>(wb + 4 * 32 + 32 * SW + (COLOR ? 4 * 32 : 0));   // ring
-    int* ri = reinterpret_cast<int*>(cq + CQ_N);
-    const Rows R{ri, ri + 9, ri + 18, ri + 27};
+    const Rows R{reinterpret_cast<int4*>(cq + CQ_N), reinterpret_cast<float2*>(cq + CQ_N + 9)};
     const float NEG_INF = -__int_as_float(0x7f800000);
     const int nu = *n_units;
     for (;;) {
@@ -1681,15 +1712,12 @@ k_pairs_topk(const int* __restrict__ unit_start, const int* __restrict__ n_units
         if (lane == 0) u = atomicAdd(unit_counter, 1);
         u = __shfl_sync(FULL, u, 0);
         if (u >= nu) break;
-        const int k0 = unit_start[u];
-        const uint32_t kq0 = qkey[k0];
-        const int qcount = unit_queries(qkey, Q, k0, kq0, lane, uq, gp.key_sub);
-        const uint32_t key0 = kq0 >> gp.key_sub;
-        const int e = find_edge_bin(edges, E, key0);
+        const int2 unit = units[u];
+        const int k0 = unit.x, qcount = unit.y & 127, e = unit.y >> 7;
+        const uint32_t key0 = qkey[k0] >> gp.key_sub;
         const FrameDev& Fa = frames[edges[e].a];
-        const int dx0 = Fa.dim[0], dy0 = Fa.dim[1], dz0 = Fa.dim[2];
         const int cell = (int)(key0 - edges[e].bin_off);
-        const int hx = cell % dx0, hy = (cell / dx0) % dy0, hz = cell / (dx0 * dy0);
+        const int hx = cell % Fa.dim[0], hy = (cell / Fa.dim[0]) % Fa.dim[1], hz = cell / (Fa.dim[0] * Fa.dim[1]);
         // this lane's query
         const bool qv = lane < qcount;
         const float4 r = qv ? slots[(long long)k0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1712,8 +1740,11 @@ k_pairs_topk(const int* __restrict__ unit_start, const int* __restrict__ n_units
             bhi2 = fmaxf(bhi2, __shfl_xor_sync(FULL, bhi2, o));
         }
         __syncwarp();
-        const int C = build_rows(R, cell_start, Fa.cell_off, dx0, dy0, dz0, hx, hy, hz, lane);
         const float box_thr = gp.rc2 * 1.0001f;
+        int n_seg;
+        const int C = build_rows(R, cell_start, Fa, hx, hy, hz, blo0, blo1, blo2, bhi0, bhi1, bhi2, gp.hf, box_thr, lane,
+                                 n_seg);
+        if (C == 0) continue;
         float tw[TOPK_MAX], t0[TOPK_MAX], t1[TOPK_MAX], t2[TOPK_MAX];   // w descending, d = x - y
 #pragma unroll
         for (int k = 0; k < TOPK_MAX; ++k) {
@@ -1721,19 +1752,14 @@ k_pairs_topk(const int* __restrict__ unit_start, const int* __restrict__ n_units
             t0[k] = t1[k] = t2[k] = 0.f;
         }
         int c_s = 0, qhead = 0, qlen = 0;
+        Cursor cur;
+        cur.start(R, n_seg, lane);
         while (c_s < C || qlen > 0) {
             while (qlen < 32 && c_s < C) {
-                const int v = c_s + lane;
                 bool keep = false;
                 float4 ent = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (v < C) {
-                    int dx, dy, dz;
-                    const int i = stream_point(R, v, dx, dy, dz);
-                    const float4 p = __ldg(pts4 + i);
-                    ent.x = fmaf((float)dx, gp.hf, p.x);
-                    ent.y = fmaf((float)dy, gp.hf, p.y);
-                    ent.z = fmaf((float)dz, gp.hf, p.z);
-                    ent.w = __int_as_float(i);
+                if (cur.valid()) {
+                    ent = cur.point(pts4, gp.hf);
                     const float e0 = fmaxf(fmaxf(blo0 - ent.x, ent.x - bhi0), 0.f);
                     const float e1 = fmaxf(fmaxf(blo1 - ent.y, ent.y - bhi1), 0.f);
                     const float e2 = fmaxf(fmaxf(blo2 - ent.z, ent.z - bhi2), 0.f);
@@ -1743,6 +1769,7 @@ k_pairs_topk(const int* __restrict__ unit_start, const int* __restrict__ n_units
                 if (keep) cq[(qhead + qlen + __popc(bal & ((1u << lane) - 1u))) & (CQ_N - 1)] = ent;
                 qlen += __popc(bal);
                 c_s += 32;
+                cur.next(R, n_seg);
             }
             __syncwarp();
             const int nb = qlen < 32 ? qlen : 32;
@@ -1808,6 +1835,7 @@ k_pairs_topk(const int* __restrict__ unit_start, const int* __restrict__ n_units
                 ++cnt;
             }
         }
+        if (!__any_sync(FULL, cnt != 0)) continue;   // no pair: every sum is zero
         const float y[3] = {r.x, r.y, r.z};
         float Sy[3], Myy[6], Mdy[9];
         int t6 = 0;
@@ -1827,53 +1855,50 @@ k_pairs_topk(const int* __restrict__ unit_start, const int* __restrict__ n_units
 // Same search and the same cutoff test, geometry only: writes the pair list
 // of one edge (verification).
 __global__ void __launch_bounds__(PAIR_T)
-k_emit_pairs(const int* __restrict__ unit_start, const int* __restrict__ n_units, int* unit_counter,
-             const uint32_t* __restrict__ qkey, const float4* __restrict__ slots, long long Q,
-             const EdgeDev* __restrict__ edges, int E, const FrameDev* __restrict__ frames,
+k_emit_pairs(const int2* __restrict__ units, const int* __restrict__ n_units, int* unit_counter,
+             const uint32_t* __restrict__ qkey, const float4* __restrict__ slots,
+             const EdgeDev* __restrict__ edges, const FrameDev* __restrict__ frames,
              const int* __restrict__ cell_start, const float4* __restrict__ pts4, GridParams gp,
-             int edge_sel, const int* __restrict__ perm_local, long long capacity, int uq,
+             int edge_sel, const int* __restrict__ perm_local, long long capacity,
              int* __restrict__ i_out, int* __restrict__ j_out, unsigned long long* n_out) {
-    __shared__ float4 s_m[PAIR_T / 32][64];
-    __shared__ int s_j[PAIR_T / 32][64];
-    __shared__ int s_rows[PAIR_T / 32][40];
+    __shared__ float4 s_m[PAIR_T / 32][UQ];
+    __shared__ int s_j[PAIR_T / 32][UQ];
+    __shared__ int4 s_rows[PAIR_T / 32][ROWS_WORDS / 4];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     float4* sm = s_m[warp];
-    const Rows R{s_rows[warp], s_rows[warp] + 9, s_rows[warp] + 18, s_rows[warp] + 27};
+    const Rows R{s_rows[warp], reinterpret_cast<float2*>(s_rows[warp] + 9)};
     const int nu = *n_units;
     for (;;) {
         int u = 0;
         if (lane == 0) u = atomicAdd(unit_counter, 1);
         u = __shfl_sync(FULL, u, 0);
         if (u >= nu) break;
-        const int k0 = unit_start[u];
-        const uint32_t kq0 = qkey[k0];
-        const uint32_t key0 = kq0 >> gp.key_sub;
-        const int e = find_edge_bin(edges, E, key0);
+        const int2 unit = units[u];
+        const int k0 = unit.x, qcount = unit.y & 127, e = unit.y >> 7;
         if (e != edge_sel) continue;
-        const int qcount = unit_queries64(qkey, Q, k0, kq0, lane, uq, gp.key_sub);
+        const uint32_t key0 = qkey[k0] >> gp.key_sub;
         const FrameDev& Fa = frames[edges[e].a];
-        const int dx0 = Fa.dim[0], dy0 = Fa.dim[1], dz0 = Fa.dim[2];
         const int cell = (int)(key0 - edges[e].bin_off);
-        const int hx = cell % dx0, hy = (cell / dx0) % dy0, hz = cell / (dx0 * dy0);
+        const int hx = cell % Fa.dim[0], hy = (cell / Fa.dim[0]) % Fa.dim[1], hz = cell / (Fa.dim[0] * Fa.dim[1]);
         __syncwarp();
-        for (int h = 0; h < 2; ++h) {
-            const int q = lane + 32 * h;
-            if (q < qcount) {
-                const float4 r = slots[(long long)k0 + q];
-                sm[q] = make_float4(-2.f * r.x, -2.f * r.y, -2.f * r.z, fmaf(r.x, r.x, fmaf(r.y, r.y, r.z * r.z)));
-                s_j[warp][q] = perm_local[__float_as_int(r.w)];
-            }
+        if (lane < qcount) {
+            const float4 r = slots[(long long)k0 + lane];
+            sm[lane] = make_float4(-2.f * r.x, -2.f * r.y, -2.f * r.z, fmaf(r.x, r.x, fmaf(r.y, r.y, r.z * r.z)));
+            s_j[warp][lane] = perm_local[__float_as_int(r.w)];
         }
-        const int C = build_rows(R, cell_start, Fa.cell_off, dx0, dy0, dz0, hx, hy, hz, lane);
-        for (int c0 = 0; c0 < C; c0 += 32) {
-            const int v = c0 + lane;
-            if (v >= C) continue;
-            int dx, dy, dz;
-            const int i = stream_point(R, v, dx, dy, dz);
-            const float4 p = __ldg(pts4 + i);
-            const float x0 = fmaf((float)dx, gp.hf, p.x), x1 = fmaf((float)dy, gp.hf, p.y),
-                        x2 = fmaf((float)dz, gp.hf, p.z);
+        const float INF = __int_as_float(0x7f800000);
+        int n_seg;
+        const int C = build_rows(R, cell_start, Fa, hx, hy, hz, -INF, -INF, -INF, INF, INF, INF, gp.hf, gp.rc2, lane,
+                                 n_seg);      // every cell: no query box
+        if (C == 0) continue;
+        Cursor cur;
+        cur.start(R, n_seg, lane);
+        for (int c0 = 0; c0 < C; c0 += 32, cur.next(R, n_seg)) {
+            if (!cur.valid()) continue;
+            const float4 x = cur.point(pts4, gp.hf);
+            const int i = __float_as_int(x.w);
+            const float x0 = x.x, x1 = x.y, x2 = x.z;
             const float thr = gp.rc2 - fmaf(x0, x0, fmaf(x1, x1, x2 * x2));
             for (int j = 0; j < qcount; ++j) {
                 const float4 m = sm[j];
@@ -1927,13 +1952,13 @@ inline bool dense_path(const GridParams& gp) {
 #endif
 }
 
-template <int DP, bool BF16, bool COLOR, int DENSE>
+template <int DP, bool BF16, bool COLOR, bool DENSE>
 void launch_k_pairs(const PairLaunch& L, const PairArgs& A) {
     const size_t smem = sizeof(float) * (PAIR_T / 32) * unit_smem_words<DP, BF16, COLOR, DENSE>();
     static int resident = 0;   // opt in to > 48 KB and size the persistent grid, once per instantiation
     const int r = pair_blocks_per_sm(k_pairs<DP, BF16, COLOR, DENSE>, smem, &resident);
     k_pairs<DP, BF16, COLOR, DENSE><<<pair_grid(L.num_sms, r, L.ctas_per_sm), PAIR_T, smem, L.stream>>>(
-        L.unit_start, L.n_units, L.unit_counter, A, L.done);
+        L.units, L.n_units, L.unit_counter, A, L.done);
 }
 
 template <int DP, bool BF16, bool COLOR>
@@ -1943,26 +1968,20 @@ void run_pairs(const PairLaunch& L, const PairArgs& A) {
         static int resident = 0;
         const int r = pair_blocks_per_sm(k_pairs_topk<DP, BF16, COLOR>, smem, &resident);
         k_pairs_topk<DP, BF16, COLOR><<<pair_grid(L.num_sms, r, L.ctas_per_sm), PAIR_T, smem, L.stream>>>(
-            L.unit_start, L.n_units, L.unit_counter, A.qkey, A.slots, A.Q, A.edges, A.E, A.frames, A.cell_start,
-            A.pts4, A.sem_sorted, A.col4, A.gp, A.acc, A.uq, L.done);
+            L.units, L.n_units, L.unit_counter, A.qkey, A.slots, A.edges, A.frames, A.cell_start, A.pts4,
+            A.sem_sorted, A.col4, A.gp, A.acc, L.done);
         return;
     }
     if constexpr (DP > 0 && !COLOR) {
         if (dense_path(A.gp)) {
-            if constexpr (BF16) {
-                if (A.uq > 32) {
-                    launch_k_pairs<DP, BF16, COLOR, 2>(L, A);
-                    return;
-                }
-            }
-            launch_k_pairs<DP, BF16, COLOR, 1>(L, A);
+            launch_k_pairs<DP, BF16, COLOR, true>(L, A);
             return;
         }
     }
-    launch_k_pairs<DP, BF16, COLOR, 0>(L, A);
+    launch_k_pairs<DP, BF16, COLOR, false>(L, A);
 }
 
-template <int DP, bool BF16, bool COLOR, int DENSE>
+template <int DP, bool BF16, bool COLOR, bool DENSE>
 void launch_k_pairs_multi(const PairJob* jobs, int n_jobs, int* counter, int num_sms, int ctas_per_sm,
                           cudaStream_t st) {
     const size_t smem = sizeof(float) * (PAIR_T / 32) * unit_smem_words<DP, BF16, COLOR, DENSE>();
@@ -1972,23 +1991,16 @@ void launch_k_pairs_multi(const PairJob* jobs, int n_jobs, int* counter, int num
         jobs, n_jobs, counter);
 }
 
-// max_uq: the largest unit size among the jobs
 template <int DP, bool BF16, bool COLOR>
 void run_pairs_multi(const PairJob* jobs, int n_jobs, int* counter, int num_sms, int ctas_per_sm, bool dense,
-                     int max_uq, cudaStream_t st) {
+                     cudaStream_t st) {
     if constexpr (DP > 0 && !COLOR) {
         if (dense) {
-            if constexpr (BF16) {
-                if (max_uq > 32) {
-                    launch_k_pairs_multi<DP, BF16, COLOR, 2>(jobs, n_jobs, counter, num_sms, ctas_per_sm, st);
-                    return;
-                }
-            }
-            launch_k_pairs_multi<DP, BF16, COLOR, 1>(jobs, n_jobs, counter, num_sms, ctas_per_sm, st);
+            launch_k_pairs_multi<DP, BF16, COLOR, true>(jobs, n_jobs, counter, num_sms, ctas_per_sm, st);
             return;
         }
     }
-    launch_k_pairs_multi<DP, BF16, COLOR, 0>(jobs, n_jobs, counter, num_sms, ctas_per_sm, st);
+    launch_k_pairs_multi<DP, BF16, COLOR, false>(jobs, n_jobs, counter, num_sms, ctas_per_sm, st);
 }
 
 // Calls F.template operator()<DP, BF16>() for the label layout of gp
@@ -2033,20 +2045,13 @@ void launch_query_keys(const EdgeDev* edges, int E, const FrameDev* frames, cons
     count_launch();
 }
 
-void launch_query_gather(const uint32_t* qkey_sorted, const int* qval_sorted, const float4* qrec,
-                         long long Q, int sub, float4* slots, int* bin_first, const int* done,
-                         cudaStream_t st) {
+void launch_units(const uint32_t* qkey_sorted, const int* qval_sorted, const float4* qrec, long long Q, int uq,
+                  int sub, const EdgeDev* edges, int E, float4* slots, int2* units, int* n_units, const int* done,
+                  cudaStream_t st) {
     if (Q <= 0) return;
-    k_query_gather<<<blocks_for(Q, 256), 256, 0, st>>>(qkey_sorted, qval_sorted, qrec, Q, sub, slots, bin_first,
-                                                      done);
-    count_launch();
-}
-
-void launch_units(const uint32_t* qkey_sorted, const int* bin_first, long long Q, int uq, int sub, int* unit_start,
-                  int* n_units, const int* done, cudaStream_t st) {
-    if (Q <= 0) return;
-    if (uq < 1 || uq > 64) uq = UQ;
-    k_units<<<blocks_for(Q, 256), 256, 0, st>>>(qkey_sorted, bin_first, Q, uq, sub, unit_start, n_units, done);
+    if (uq < 1 || uq > UQ) uq = UQ;      // larger units are taken as units of 32
+    k_units<<<blocks_for(Q, 256), 256, 0, st>>>(qkey_sorted, qval_sorted, qrec, Q, uq, sub, edges, E, slots, units,
+                                                n_units, done);
     count_launch();
 }
 
@@ -2065,44 +2070,55 @@ struct MultiLaunch {
     int n_jobs;
     bool color;
     bool dense;
-    int max_uq;
     int* counter;
     int num_sms, ctas_per_sm;
     cudaStream_t st;
     template <int DP, bool BF16>
     void operator()() const {
-        if (color) run_pairs_multi<DP, BF16, true>(jobs, n_jobs, counter, num_sms, ctas_per_sm, dense, max_uq, st);
-        else run_pairs_multi<DP, BF16, false>(jobs, n_jobs, counter, num_sms, ctas_per_sm, dense, max_uq, st);
+        if (color) run_pairs_multi<DP, BF16, true>(jobs, n_jobs, counter, num_sms, ctas_per_sm, dense, st);
+        else run_pairs_multi<DP, BF16, false>(jobs, n_jobs, counter, num_sms, ctas_per_sm, dense, st);
     }
 };
 }  // namespace
 
 int pair_unit_max(const GridParams& gp) { return (dense_path(gp) && gp.sem_bf16) ? 64 : UQ; }
 
+bool pairs_per_query(const GridParams& gp) { return dense_path(gp); }
+
+void launch_query_moments(const PairArgs& A, int num_sms, const int* done, cudaStream_t st) {
+    if (A.Q <= 0) return;
+    // groups of 32 queries per warp: as many as leave a few warps for every
+    // scheduler
+    const long long groups = (A.Q + 31) / 32;
+    int per = (int)(groups / (16LL * num_sms));
+    per = per < 1 ? 1 : (per > MOM_PER ? MOM_PER : per);
+    k_query_moments<<<blocks_for((groups + per - 1) / per, 4), 128, 0, st>>>(A, per, done);
+    count_launch();
+}
+
 void launch_pairs(const PairLaunch& L, const PairArgs& A) {
     if (A.Q <= 0) return;
     if (with_label_layout(A.gp, SingleLaunch{L, A})) count_launch();
 }
 
-bool launch_pairs_multi(const PairJob* jobs, int n_jobs, const GridParams& layout, int max_uq, int* counter,
-                        int num_sms, int ctas_per_sm, cudaStream_t st) {
+bool launch_pairs_multi(const PairJob* jobs, int n_jobs, const GridParams& layout, int* counter, int num_sms,
+                        int ctas_per_sm, cudaStream_t st) {
     if (n_jobs <= 0 || n_jobs > MAX_PAIR_JOBS || layout.top_k > 0) return false;
     const bool ok = with_label_layout(layout, MultiLaunch{jobs, n_jobs, layout.color != 0, dense_path(layout),
-                                                          max_uq, counter, num_sms, ctas_per_sm, st});
+                                                          counter, num_sms, ctas_per_sm, st});
     if (ok) count_launch();
     return ok;
 }
 
-void launch_emit_pairs(const int* unit_start, const int* n_units, int* unit_counter,
+void launch_emit_pairs(const int2* units, const int* n_units, int* unit_counter,
                        const uint32_t* qkey, const float4* slots, long long Q, const EdgeDev* edges,
-                       int E, const FrameDev* frames, const int* cell_start, const float4* pts4,
-                       GridParams gp, int edge_sel, const int* perm_local, long long capacity, int uq,
+                       const FrameDev* frames, const int* cell_start, const float4* pts4,
+                       GridParams gp, int edge_sel, const int* perm_local, long long capacity,
                        int* i_out, int* j_out, unsigned long long* n_out, int num_sms,
                        cudaStream_t st) {
     if (Q <= 0) return;
-    if (uq < 1 || uq > 64) uq = UQ;
-    k_emit_pairs<<<num_sms * 2, PAIR_T, 0, st>>>(unit_start, n_units, unit_counter, qkey, slots, Q, edges, E,
-                                                 frames, cell_start, pts4, gp, edge_sel, perm_local, capacity, uq,
+    k_emit_pairs<<<num_sms * 2, PAIR_T, 0, st>>>(units, n_units, unit_counter, qkey, slots, edges, frames,
+                                                 cell_start, pts4, gp, edge_sel, perm_local, capacity,
                                                  i_out, j_out, n_out);
     count_launch();
 }

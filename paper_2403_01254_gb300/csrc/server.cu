@@ -79,7 +79,7 @@ double ms_between(Clock::time_point a, Clock::time_point b) {
 
 // Device bytes a problem will hold, from its sizes (mirrors the buffers of
 // rkhsba_create): points, labels, sort buffers, grids over the frames'
-// bounding boxes, per-edge queries and home cells, and the 6K system.
+// bounding boxes, per-edge queries, and the 6K system.
 size_t estimate_bytes(const Req& r) {
     const double rc = (r.p.cutoff_mult > 0 ? r.p.cutoff_mult : 3.0) * r.p.ell;
     const double h = rc * (1.0 + 1.0 / 1024.0);
@@ -99,15 +99,11 @@ size_t estimate_bytes(const Req& r) {
         }
         off += r.n[m];
     }
-    double N = (double)off, Q = 0, bins = 0, C = 0;
+    double N = (double)off, Q = 0, C = 0;
     for (int m = 0; m < r.K; ++m) C += cells[m];
-    for (int e = 0; e < r.E; ++e) {
-        int a = std::min(r.edges[2 * e], r.edges[2 * e + 1]), b = std::max(r.edges[2 * e], r.edges[2 * e + 1]);
-        Q += (double)r.n[b];
-        bins += cells[a];
-    }
+    for (int e = 0; e < r.E; ++e) Q += (double)r.n[std::max(r.edges[2 * e], r.edges[2 * e + 1])];
     const double D = r.p.sem_dim;
-    const double bytes = N * (24 + 8 * D + 16 + 16 + 40 + 12) + Q * 68 + bins * 4 + C * 4 +
+    const double bytes = N * (24 + 8 * D + 16 + 16 + 40 + 12) + Q * 80 + C * 4 +
                          (double)r.K * r.K * 36 * 8 * 2 + (double)r.E * 1600 + (4 << 20);
     return (size_t)(bytes * 1.25);
 }
@@ -403,7 +399,7 @@ bool rkhsba_server::tuning_for(Req* r, rkhsba_tuning* t) {
 // neighbour-limited variant (its own kernel) run whole iterations on their
 // streams.
 void rkhsba_server::issue_round(const std::vector<Req*>& batch, int n_iter) {
-    struct Group { int key; GridParams layout; int ctas; int max_uq; std::vector<Req*> reqs; };
+    struct Group { int key; GridParams layout; int ctas; std::vector<Req*> reqs; };
     std::vector<Group> groups;
     for (Req* r : batch) {
         const GridParams g = ctx_layout(r->ctx);
@@ -421,11 +417,10 @@ void rkhsba_server::issue_round(const std::vector<Req*>& batch, int n_iter) {
         for (Group& x : groups)
             if (x.key == key && (int)x.reqs.size() < MAX_PAIR_JOBS) grp = &x;
         if (!grp) {
-            groups.push_back({key, g, ctx_tune_ctas(r->ctx), 0, {}});
+            groups.push_back({key, g, ctx_tune_ctas(r->ctx), {}});
             grp = &groups.back();
         }
         grp->reqs.push_back(r);
-        grp->max_uq = std::max(grp->max_uq, ctx_tune_uq(r->ctx));
     }
     if (groups.empty()) return;
     RoundSlot* rs_free = nullptr;
@@ -456,7 +451,7 @@ void rkhsba_server::issue_round(const std::vector<Req*>& batch, int n_iter) {
             const int n = (int)grp.reqs.size();
             for (Req* r : grp.reqs) cudaStreamWaitEvent(rst, r->ev, 0);
             cudaMemsetAsync(counters + gi, 0, sizeof(int), rst);
-            launch_pairs_multi(jobs + off, n, grp.layout, grp.max_uq, counters + gi, num_sms, grp.ctas, rst);
+            launch_pairs_multi(jobs + off, n, grp.layout, counters + gi, num_sms, grp.ctas, rst);
             off += n;
             ++gi;
         }
