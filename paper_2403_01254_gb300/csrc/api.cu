@@ -279,10 +279,11 @@ rkhsba_status build(rkhsba_ctx* c, const double* xyz, const float* sem, const fl
     // the query order and the unsorted records are done with when the units
     // are cut, so the dense pair kernel's per-query sums take their place
     const bool per_query = pairs_per_query(c->gp);
-    RK_TRY(alloc(c, &c->d_qval, 2 * Q));
+    const int parts = per_query ? 1 << part_max_for(c->gp, Q, c->num_sms) : 1;
+    RK_TRY(alloc(c, &c->d_qval, 2 * Q * parts));
     c->d_qval_alt = c->d_qval + Q;
     RK_TRY(alloc(c, &c->d_qhist, (long long)radix_hist_elems(Q)));
-    RK_TRY(alloc(c, &c->d_qrec, per_query ? 2 * Q : Q));
+    RK_TRY(alloc(c, &c->d_qrec, per_query ? 2 * Q * parts : Q));
     if (per_query) {
         c->d_qs8 = reinterpret_cast<float*>(c->d_qrec);
         c->d_qs2 = reinterpret_cast<float*>(c->d_qval);
@@ -339,7 +340,7 @@ void eval_pre(rkhsba_ctx* c, const double* poses, const int* done) {
 
 void eval_pairs(rkhsba_ctx* c, const int* done) {
     c->phase_begin(2);
-    launch_pairs(PairLaunch{c->d_units, c->d_ucount, c->d_ucount + 1, done, c->num_sms, c->tune_ctas,
+    launch_pairs(PairLaunch{c->d_ucount + 1, done, c->num_sms, c->tune_ctas,
                             c->stream},
                  c->pair_args());
     c->phase_end();
@@ -552,8 +553,6 @@ void ctx_iter_post(rkhsba_ctx* c) {
 }
 PairJob ctx_pair_job(const rkhsba_ctx* c) {
     PairJob j{};
-    j.units = c->d_units;
-    j.n_units = c->d_ucount;
     j.done = &c->d_state->done;
     j.a = c->pair_args();
     return j;

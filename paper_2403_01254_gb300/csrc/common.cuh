@@ -109,6 +109,10 @@ struct PairArgs {
     const uint32_t* qkey;     // sorted home-cell keys of the queries
     const float4* slots;      // sorted query records (offset from the home centre, point index)
     long long Q;              // queries over all edges
+    const int2* units;        // (first sorted query, edge << 7 | queries)
+    const int* n_units;
+    int part_max, part_target;   // a unit's stream is cut into up to 2^part_max parts until there are
+                                 //   part_target items (part_max = 0: never)
     const EdgeDev* edges;
     const FrameDev* frames;
     const int* cell_start;
@@ -116,8 +120,8 @@ struct PairArgs {
     const void* sem_sorted;   // label rows in the same order (FP32 or BF16), or NULL
     const float4* col4;       // colours in the same order, or NULL
     long long* acc;           // [E][ACC_N] fixed-point moments
-    float* qs8;               // [Q][8], [Q][2]: per sorted query sum_c w (1, x, x x^T) of the
-    float* qs2;               //   dense pair kernel (scaled), read by k_query_moments
+    float* qs8;               // [parts][Q][8], [parts][Q][2]: per sorted query sum_c w (1, x, x x^T) of
+    float* qs2;               //   the dense pair kernel (scaled), read by k_query_moments
     int E;
     GridParams gp;
 };
@@ -125,17 +129,26 @@ struct PairArgs {
 // One problem of a batched pair launch: its unit list and LM state flag
 // (a job whose solve is done contributes no units).
 struct PairJob {
-    const int2* units;
-    const int* n_units;
     const int* done;
     PairArgs a;
 };
 constexpr int MAX_PAIR_JOBS = 64;   // problems in one batched pair launch
 
+// Cutting of units into parts: items for two per resident warp (16
+// warps per SM) are wanted, in 2^3 parts per unit at most.  A problem of more
+// queries than 32 per wanted item has the items as units; the top_k variant's
+// selection needs a unit's whole stream.  Measured with 1, 2 and 4 items per
+// warp: four scans of 8000 points of one object, without labels, 492 us per
+// pair launch uncut, 289 / 272 / 266 us; an RGB-D pair of 2000 points 16 us uncut,
+// 18 / 24 / 24 us (short streams gain nothing).
+constexpr int PART_MAX = 3;
+inline int part_target_for(int num_sms) { return 32 * num_sms; }
+inline int part_max_for(const GridParams& gp, long long Q, int num_sms) {
+    return (gp.top_k > 0 || Q > 32LL * part_target_for(num_sms)) ? 0 : PART_MAX;
+}
+
 // Launch state of a single-problem pair launch.
 struct PairLaunch {
-    const int2* units;        // (first sorted query, edge << 7 | queries)
-    const int* n_units;
     int* unit_counter;        // zeroed by the caller
     const int* done;          // LM state flag or NULL
     int num_sms;

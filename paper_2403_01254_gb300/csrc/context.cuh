@@ -127,6 +127,10 @@ struct rkhsba_ctx {
         a.sem_sorted = d_sem;
         a.col4 = d_col4;
         a.acc = d_acc;
+        a.units = d_units;
+        a.n_units = d_ucount;
+        a.part_max = rk::part_max_for(gp, Q_total, num_sms);
+        a.part_target = rk::part_target_for(num_sms);
         a.qs8 = d_qs8;
         a.qs2 = d_qs2;
         a.E = E;

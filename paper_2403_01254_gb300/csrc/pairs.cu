@@ -484,8 +484,7 @@ __device__ __forceinline__ int build_rows(const Rows& R, const int* __restrict__
     return total;
 }
 
-// A lane's place in the stream: it starts at point `lane` of the list and
-// steps 32 points at a time, crossing into the next segment when it must.
+// A lane's place in the stream: it starts at a point of the list and steps 32 points at a time, crossing into the next segment when it must.
 struct Cursor {
     int i, end, r, b1, b2;
     float oy, oz;
@@ -503,8 +502,8 @@ struct Cursor {
     __device__ __forceinline__ void settle(const Rows& R, int n_seg) {
         while (i >= end && r + 1 < n_seg) enter(R, r + 1, i - end);
     }
-    __device__ __forceinline__ void start(const Rows& R, int n_seg, int lane) {
-        enter(R, 0, lane);
+    __device__ __forceinline__ void start(const Rows& R, int n_seg, int at) {
+        enter(R, 0, at);
         settle(R, n_seg);
     }
     __device__ __forceinline__ void next(const Rows& R, int n_seg) {
@@ -518,6 +517,26 @@ struct Cursor {
         return make_float4(p.x + (i >= b2 ? hf : (i >= b1 ? 0.f : -hf)), p.y + oy, p.z + oz, __int_as_float(i));
     }
 };
+
+// Parts that the candidate stream of a unit is cut into, as a power of two
+// (log2): problems with few units (dense small clouds) would leave most warps
+// idle behind a few long streams, so their units are shared by up to
+// 2^part_max warps until part_target items are there.  Set by the problem's own
+// units alone, so that its results do not depend on what shares a launch.
+__device__ __forceinline__ int part_shift(const PairArgs& A, int n_units) {
+    int s = 0;
+    while (s < A.part_max && ((long long)n_units << s) < A.part_target) ++s;
+    return s;
+}
+// Chunks [c0, c1) of 32 stream points that part `part` of 2^shift takes: an
+// even share, but four at least (short streams stay whole, and their other
+// parts are empty).
+__device__ __forceinline__ void part_range(int C, int part, int shift, int& c0, int& c1) {
+    const int n = (int)(((long long)C + 31) >> 5);
+    const int per = max((n + (1 << shift) - 1) >> shift, 4);
+    c0 = min(part * per, n);
+    c1 = min(c0 + per, n);
+}
 
 // One step of the moment reduce-scatter: lanes whose bit `o` is clear keep
 // the lower half of their values, the others the upper half, and each adds
@@ -936,8 +955,8 @@ __device__ __forceinline__ void gram_chunks(float (&s)[4], const unsigned (&qa)[
 // shared memory once for all its queries: at one 16-query tile per read the
 // shared-memory pipe was the kernel's bound (82% busy on the mapping workload,
 // 98 wavefronts per 16 x 32 tile; 32 here).
-template <int DP, bool SPLIT>
-__device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int2 unit, float* wb, int lane) {
+template <int DP, bool SPLIT, bool PARTS>
+__device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int2 unit, int part, int shift, float* wb, int lane) {
     using L = DenseSmem<DP, SPLIT>;
     constexpr int LW = L::LW, PW = L::PW;
     constexpr int NKC = L::DPH / 8;             // 8-wide chunks of a label row part (1..4)
@@ -1001,6 +1020,8 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int2 unit, fl
     int n_seg;
     const int C = build_rows(R, A.cell_start, Fa, hx, hy, hz, blo0, blo1, blo2, bhi0, bhi1, bhi2, gp.hf, box_thr, lane,
                              n_seg);
+    int c_lo = 0, c_hi = (int)(((long long)C + 31) >> 5);    // chunks of the stream
+    if constexpr (PARTS) part_range(C, part, shift, c_lo, c_hi);
     // query label rows (zero rows for absent queries) as A fragments, through
     // the candidates' rows
     {
@@ -1032,11 +1053,11 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int2 unit, fl
     // the batches, compiled for one and for two m tiles
     auto batches = [&](auto mtc) {
         constexpr int MT = decltype(mtc)::value;
-        int c_s = 0, qhead = 0, qlen = 0;
+        int c_s = c_lo, qhead = 0, qlen = 0;
         Cursor cur;
-        cur.start(R, n_seg, lane);
-        while (c_s < C || qlen > 0) {
-            while (qlen < 32 && c_s < C) {
+        cur.start(R, n_seg, 32 * c_lo + lane);
+        while (c_s < c_hi || qlen > 0) {
+            while (qlen < 32 && c_s < c_hi) {
                 bool keep = false;
                 float4 ent = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (cur.valid()) {
@@ -1049,7 +1070,7 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int2 unit, fl
                 const unsigned bal = __ballot_sync(FULL, keep);
                 if (keep) cq[(qhead + qlen + __popc(bal & ((1u << lane) - 1u))) & (CQ_N - 1)] = ent;
                 qlen += __popc(bal);
-                c_s += 32;
+                ++c_s;
                 cur.next(R, n_seg);
             }
             __syncwarp();
@@ -1162,13 +1183,14 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int2 unit, fl
             cnt += (int)n2.x + (int)n2.y;
         }
     };
-    if (C > 0) {
+    if (c_lo < c_hi) {
         if (qcount > 16) batches(std::integral_constant<int, 2>{});
         else batches(std::integral_constant<int, 1>{});
     }
     // unit end: the per-query sums as they are; k_query_moments forms the moments
-    float* qs8 = A.qs8 + 8LL * k0;
-    float* qs2 = A.qs2 + 2LL * k0;
+    const long long at = (PARTS ? A.Q * part : 0LL) + k0;
+    float* qs8 = A.qs8 + 8 * at;
+    float* qs2 = A.qs2 + 2 * at;
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt) {
         float (&r1)[4] = run[mt][1];
@@ -1221,6 +1243,7 @@ __global__ void __launch_bounds__(128, 5) k_query_moments(const PairArgs A, int 
     int e_cur = -1, lo0 = 0, lo1 = 0, lo2 = 0, dim0 = 1, dim1 = 1;
     long long bin_lo = 0, bin_hi = 0;
     float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+    const int parts = 1 << part_shift(A, *A.n_units);
     auto flush = [&]() {
         if (e_cur >= 0)
             add_moments(W, D, Sy, Myy, Mdy, Q, 0, A.edges[e_cur].scale, A.acc + (long long)e_cur * ACC_N, lane);
@@ -1240,6 +1263,13 @@ __global__ void __launch_bounds__(128, 5) k_query_moments(const PairArgs A, int 
             f0 = p8[0];
             f1 = p8[1];
             f2v = reinterpret_cast<const float2*>(A.qs2)[k];
+            for (int p = 1; p < parts; ++p) {
+                const float4 g0 = p8[2 * A.Q * p], g1 = p8[2 * A.Q * p + 1];
+                const float2 g2 = reinterpret_cast<const float2*>(A.qs2)[A.Q * p + k];
+                f0 = make_float4(f0.x + g0.x, f0.y + g0.y, f0.z + g0.z, f0.w + g0.w);
+                f1 = make_float4(f1.x + g1.x, f1.y + g1.y, f1.z + g1.z, f1.w + g1.w);
+                f2v = make_float2(f2v.x + g2.x, f2v.y + g2.y);
+            }
         }
         while (todo) {
             const long long kl = __shfl_sync(FULL, key, __ffs(todo) - 1);
@@ -1298,7 +1328,7 @@ __global__ void __launch_bounds__(128, 5) k_query_moments(const PairArgs A, int 
 // 27-cell stencil, test, walk and fold, and add the unit's moments to its
 // edge.  wb is the warp's shared-memory block.
 template <int DP, bool BF16, bool COLOR>
-__device__ __forceinline__ void pair_unit(const PairArgs& A, int2 unit, float* wb, int lane) {
+__device__ __forceinline__ void pair_unit(const PairArgs& A, int2 unit, int part, int shift, float* wb, int lane) {
     const uint32_t* __restrict__ qkey = A.qkey;
     const float4* __restrict__ slots = A.slots;
     const EdgeDev* __restrict__ edges = A.edges;
@@ -1370,7 +1400,9 @@ __device__ __forceinline__ void pair_unit(const PairArgs& A, int2 unit, float* w
     const float box_thr = gp.rc2 * 1.0001f;
     int n_seg;
     const int C = build_rows(R, cell_start, Fa, hx, hy, hz, blo0, blo1, blo2, bhi0, bhi1, bhi2, gp.hf, box_thr, lane, n_seg);
-    if (C == 0) return;
+    int c_s, c_hi;                               // chunks of the stream
+    part_range(C, part, shift, c_s, c_hi);
+    if (c_s >= c_hi) return;
     const int np = (qcount + 1) >> 1;
     // BF16 labels: the Gram path leaves registers free, so the query-side MMA
     // fragments and the per-lane unit sums live in registers instead of
@@ -1390,13 +1422,13 @@ __device__ __forceinline__ void pair_unit(const PairArgs& A, int2 unit, float* w
         for (int k = 0; k < N_ACC / 4; ++k) sacc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     int cnt = 0;
-    int c_s = 0, qhead = 0, qlen = 0;            // stream position, ring head and fill
+    int qhead = 0, qlen = 0;                     // ring head and fill
     Cursor cur;
-    cur.start(R, n_seg, lane);
-    while (c_s < C || qlen > 0) {
+    cur.start(R, n_seg, 32 * c_s + lane);
+    while (c_s < c_hi || qlen > 0) {
         // stream the 27-cell candidates through the box test into the
         // ring until it holds a full batch (or the stream ends)
-        while (qlen < 32 && c_s < C) {
+        while (qlen < 32 && c_s < c_hi) {
             bool keep = false;
             float4 ent = make_float4(0.f, 0.f, 0.f, 0.f);
             if (cur.valid()) {
@@ -1409,7 +1441,7 @@ __device__ __forceinline__ void pair_unit(const PairArgs& A, int2 unit, float* w
             const unsigned bal = __ballot_sync(FULL, keep);
             if (keep) cq[(qhead + qlen + __popc(bal & ((1u << lane) - 1u))) & (CQ_N - 1)] = ent;
             qlen += __popc(bal);
-            c_s += 32;
+            ++c_s;
             cur.next(R, n_seg);
         }
         __syncwarp();
@@ -1598,28 +1630,32 @@ __host__ __device__ constexpr int unit_smem_words() {
     else return warp_smem_words<DP, BF16, COLOR>();
 }
 
-template <int DP, bool BF16, bool COLOR, bool DENSE>
-__device__ __forceinline__ void run_unit(const PairArgs& A, int2 unit, float* wb, int lane) {
-    if constexpr (DENSE && DP > 0 && !COLOR) pair_unit_dense<DP, !BF16>(A, unit, wb, lane);
-    else pair_unit<DP, BF16, COLOR>(A, unit, wb, lane);
+// PARTS false (the dense path of problems that never cut units): the kernel
+// without part numbers, 2% faster on the mapping and window workloads.
+template <int DP, bool BF16, bool COLOR, bool DENSE, bool PARTS>
+__device__ __forceinline__ void run_unit(const PairArgs& A, int item, int shift, float* wb, int lane) {
+    const int2 unit = A.units[PARTS ? item >> shift : item];
+    const int part = PARTS ? item & ((1 << shift) - 1) : 0;
+    if constexpr (DENSE && DP > 0 && !COLOR) pair_unit_dense<DP, !BF16, PARTS>(A, unit, part, shift, wb, lane);
+    else pair_unit<DP, BF16, COLOR>(A, unit, part, shift, wb, lane);
 }
 
-template <int DP, bool BF16, bool COLOR, bool DENSE>
+template <int DP, bool BF16, bool COLOR, bool DENSE, bool PARTS>
 __global__ void __launch_bounds__(PAIR_T, 2)
-k_pairs(const int2* __restrict__ units, const int* __restrict__ n_units, int* unit_counter,
-        const PairArgs A, const int* done) {
+k_pairs(int* unit_counter, const PairArgs A, const int* done) {
     if (done && *done) return;
     extern __shared__ float4 smem4[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     float* wb = reinterpret_cast<float*>(smem4) + warp * unit_smem_words<DP, BF16, COLOR, DENSE>();
-    const int nu = *n_units;
+    const int shift = PARTS ? part_shift(A, *A.n_units) : 0;
+    const int items = *A.n_units << shift;
     for (;;) {
         int u = 0;
         if (lane == 0) u = atomicAdd(unit_counter, 1);
         u = __shfl_sync(FULL, u, 0);
-        if (u >= nu) break;
-        run_unit<DP, BF16, COLOR, DENSE>(A, units[u], wb, lane);
+        if (u >= items) break;
+        run_unit<DP, BF16, COLOR, DENSE, PARTS>(A, u, shift, wb, lane);
     }
 }
 
@@ -1632,7 +1668,7 @@ k_pairs(const int2* __restrict__ units, const int* __restrict__ n_units, int* un
 template <int DP, bool BF16, bool COLOR, bool DENSE>
 __global__ void __launch_bounds__(PAIR_T, 2)
 k_pairs_multi(const PairJob* __restrict__ jobs, int n_jobs, int* unit_counter) {
-    __shared__ int s_pref[MAX_PAIR_JOBS + 1];
+    __shared__ int s_pref[MAX_PAIR_JOBS + 1], s_shift[MAX_PAIR_JOBS];
     extern __shared__ float4 smem4[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -1643,7 +1679,9 @@ k_pairs_multi(const PairJob* __restrict__ jobs, int n_jobs, int* unit_counter) {
             int n = 0;
             if (j < n_jobs) {
                 const int* dn = jobs[j].done;
-                n = (dn && *dn) ? 0 : *jobs[j].n_units;
+                n = (dn && *dn) ? 0 : *jobs[j].a.n_units;
+                s_shift[j] = part_shift(jobs[j].a, n);
+                n <<= s_shift[j];
             }
             int inc = n;
 #pragma unroll
@@ -1669,8 +1707,7 @@ k_pairs_multi(const PairJob* __restrict__ jobs, int n_jobs, int* unit_counter) {
             const int mid = (lo + hi + 1) >> 1;
             if (s_pref[mid] <= u) lo = mid; else hi = mid - 1;
         }
-        const PairJob* J = jobs + lo;
-        run_unit<DP, BF16, COLOR, DENSE>(J->a, J->units[u - s_pref[lo]], wb, lane);
+        run_unit<DP, BF16, COLOR, DENSE, true>(jobs[lo].a, u - s_pref[lo], s_shift[lo], wb, lane);
     }
 }
 
@@ -1952,13 +1989,13 @@ inline bool dense_path(const GridParams& gp) {
 #endif
 }
 
-template <int DP, bool BF16, bool COLOR, bool DENSE>
+template <int DP, bool BF16, bool COLOR, bool DENSE, bool PARTS>
 void launch_k_pairs(const PairLaunch& L, const PairArgs& A) {
     const size_t smem = sizeof(float) * (PAIR_T / 32) * unit_smem_words<DP, BF16, COLOR, DENSE>();
     static int resident = 0;   // opt in to > 48 KB and size the persistent grid, once per instantiation
-    const int r = pair_blocks_per_sm(k_pairs<DP, BF16, COLOR, DENSE>, smem, &resident);
-    k_pairs<DP, BF16, COLOR, DENSE><<<pair_grid(L.num_sms, r, L.ctas_per_sm), PAIR_T, smem, L.stream>>>(
-        L.units, L.n_units, L.unit_counter, A, L.done);
+    const int r = pair_blocks_per_sm(k_pairs<DP, BF16, COLOR, DENSE, PARTS>, smem, &resident);
+    k_pairs<DP, BF16, COLOR, DENSE, PARTS><<<pair_grid(L.num_sms, r, L.ctas_per_sm), PAIR_T, smem, L.stream>>>(
+        L.unit_counter, A, L.done);
 }
 
 template <int DP, bool BF16, bool COLOR>
@@ -1968,17 +2005,18 @@ void run_pairs(const PairLaunch& L, const PairArgs& A) {
         static int resident = 0;
         const int r = pair_blocks_per_sm(k_pairs_topk<DP, BF16, COLOR>, smem, &resident);
         k_pairs_topk<DP, BF16, COLOR><<<pair_grid(L.num_sms, r, L.ctas_per_sm), PAIR_T, smem, L.stream>>>(
-            L.units, L.n_units, L.unit_counter, A.qkey, A.slots, A.edges, A.frames, A.cell_start, A.pts4,
+            A.units, A.n_units, L.unit_counter, A.qkey, A.slots, A.edges, A.frames, A.cell_start, A.pts4,
             A.sem_sorted, A.col4, A.gp, A.acc, L.done);
         return;
     }
     if constexpr (DP > 0 && !COLOR) {
         if (dense_path(A.gp)) {
-            launch_k_pairs<DP, BF16, COLOR, true>(L, A);
+            if (A.part_max > 0) launch_k_pairs<DP, BF16, COLOR, true, true>(L, A);
+            else launch_k_pairs<DP, BF16, COLOR, true, false>(L, A);
             return;
         }
     }
-    launch_k_pairs<DP, BF16, COLOR, false>(L, A);
+    launch_k_pairs<DP, BF16, COLOR, false, true>(L, A);
 }
 
 template <int DP, bool BF16, bool COLOR, bool DENSE>
