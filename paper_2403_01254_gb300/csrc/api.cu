@@ -119,17 +119,19 @@ rkhsba_status check_shape(rkhsba_ctx* ctx, int32_t n_frames, const int64_t* n_po
 
 void grid_fill(rkhsba_ctx* c, bool* keys_in_alt) {
     cudaStream_t st = c->stream;
-    launch_keys(c->d_xyz, c->N, c->K, c->d_pt_off, c->d_frames, c->gp.h_inv, c->d_keys, c->d_vals, st);
     int nbits = 0;
     while ((1LL << nbits) < c->C_total) ++nbits;
-    bool alt = false;
-    radix_sort_u32(c->d_keys, c->d_vals, c->d_keys_alt, c->d_vals_alt, c->N, nbits, c->d_hist,
-                   c->d_scan_ws, c->d_err + 1, st, &alt);
+    const RadixWs ws = radix_ws(c->N, nbits, c->d_hist, c->d_scan_ws);
+    cudaMemsetAsync(c->d_scan_ws, 0, sizeof(long long) * scan_ws_elems(c->N), st);
+    launch_keys(c->d_xyz, c->N, c->K, c->d_pt_off, c->d_frames, c->gp.h_inv, c->d_keys, ws, c->num_sms, st);
+    if (ws.npass == 0)      // one cell: the input order is the order
+        launch_iota(c->d_vals, c->N, st);
+    const bool alt = radix_sort_u32(c->d_keys, c->d_vals, c->d_keys_alt, c->d_vals_alt, c->N, ws, c->d_err + 1, nullptr,
+                                    st);
     const uint32_t* keys = alt ? c->d_keys_alt : c->d_keys;
     const int* perm = alt ? c->d_vals_alt : c->d_vals;
     launch_gather(c->d_xyz, c->d_sem_in, c->d_rgb_in, c->N, c->K, c->d_pt_off, keys, perm, c->gp,
-                  c->C_total, c->d_pts4, c->d_sem, c->d_col4, c->d_perm_local, c->d_cell_start,
-                  c->d_run, st);
+                  c->C_total, c->d_pts4, c->d_sem, c->d_col4, c->d_perm_local, c->d_cell_start, st);
     c->d_pt_cell = keys;
     *keys_in_alt = alt;
 }
@@ -237,8 +239,6 @@ rkhsba_status build(rkhsba_ctx* c, const double* xyz, const float* sem, const fl
     }
     if (c->gp.color) RK_TRY(alloc(c, &c->d_col4, N));
     RK_TRY(alloc(c, &c->d_perm_local, N));
-    RK_TRY(alloc(c, &c->d_run, N));
-    RK_TRY(alloc(c, &c->d_total, 4));
 
     // per-edge sizes (bins = cells of frame a's grid, queries = points of
     // frame b) and fixed-point scales
@@ -254,7 +254,7 @@ rkhsba_status build(rkhsba_ctx* c, const double* xyz, const float* sem, const fl
     long long scan_n = std::max<long long>((long long)radix_hist_elems(N),
                                            (long long)radix_hist_elems(c->Q_total));
     RK_TRY(alloc(c, &c->d_scan_ws, (long long)scan_ws_elems(scan_n) + 64));
-    RK_CUDA(c, cudaMemsetAsync(c->d_cell_start, 0, sizeof(int) * (c->C_total + 1), st));
+    if (N == 0) RK_CUDA(c, cudaMemsetAsync(c->d_cell_start, 0, sizeof(int) * (c->C_total + 1), st));
     bool alt = false;
     grid_fill(c, &alt);
     RK_CUDA(c, cudaGetLastError());
@@ -305,6 +305,8 @@ rkhsba_status build(rkhsba_ctx* c, const double* xyz, const float* sem, const fl
     RK_TRY(alloc(c, &c->d_state, 1));
     const long long nf = 6LL * (K - 1);
     RK_TRY(alloc(c, &c->d_lm_ws, nf * nf + 2 * nf + 16));
+    // blocks of frame pairs without an edge stay zero: no evaluation writes them
+    RK_CUDA(c, cudaMemsetAsync(c->d_H_cand, 0, sizeof(double) * n6 * n6, st));
     RK_CUDA(c, cudaMemsetAsync(c->d_state, 0, sizeof(LMState), st));
     RK_CUDA(c, cudaStreamSynchronize(st));
     RK_CUDA(c, cudaGetLastError());
@@ -315,13 +317,13 @@ rkhsba_status build(rkhsba_ctx* c, const double* xyz, const float* sem, const fl
 // sorted home-cell keys, sorted query records and the unit list.
 void run_binning(rkhsba_ctx* c, const double* poses, const int* done) {
     cudaStream_t st = c->stream;
-    launch_edge_setup(poses, c->d_edges, c->E, c->d_frames, c->gp.h, c->d_xf, done, st);
-    cudaMemsetAsync(c->d_ucount, 0, sizeof(int) * 4, st);
+    const RadixWs ws = radix_ws(c->Q_total, c->qbits, c->d_qhist, c->d_scan_ws);
+    launch_eval_setup(poses, c->d_edges, c->E, c->d_frames, c->gp.h, c->d_xf, c->d_scan_ws,
+                      (int)scan_ws_elems(c->Q_total), c->d_ucount, c->d_acc, done, st);
     launch_query_keys(c->d_edges, c->E, c->d_frames, c->d_xf, c->d_pt_cell, c->d_pts4, c->gp, c->Q_total,
-                      c->d_qkey, c->d_qval, c->d_qrec, done, st);
-    bool alt = false;
-    radix_sort_u32(c->d_qkey, c->d_qval, c->d_qkey_alt, c->d_qval_alt, c->Q_total, c->qbits, c->d_qhist,
-                   c->d_scan_ws, c->d_err + 1, st, &alt);
+                      c->d_qkey, c->d_qrec, ws, c->num_sms, done, st);
+    const bool alt = radix_sort_u32(c->d_qkey, c->d_qval, c->d_qkey_alt, c->d_qval_alt, c->Q_total, ws, c->d_err + 1,
+                                    done, st);
     c->q_sorted_key = alt ? c->d_qkey_alt : c->d_qkey;
     const int* qv = alt ? c->d_qval_alt : c->d_qval;
     launch_units(c->q_sorted_key, qv, c->d_qrec, c->Q_total, c->tune_uq, c->gp.key_sub, c->d_edges, c->E, c->d_slots,
@@ -334,7 +336,6 @@ void run_binning(rkhsba_ctx* c, const double* poses, const int* done) {
 void eval_pre(rkhsba_ctx* c, const double* poses, const int* done) {
     c->phase_begin(1);
     run_binning(c, poses, done);
-    cudaMemsetAsync(c->d_acc, 0, sizeof(long long) * c->E * ACC_N, c->stream);
     c->phase_end();
 }
 
@@ -346,21 +347,22 @@ void eval_pairs(rkhsba_ctx* c, const int* done) {
     c->phase_end();
 }
 
-void eval_post(rkhsba_ctx* c, const int* done) {
+// lm: the assembly ends with the LM loop's accept / reject step.
+void eval_post(rkhsba_ctx* c, const int* done, bool lm = false) {
     cudaStream_t st = c->stream;
     c->phase_begin(3);
     if (pairs_per_query(c->gp)) launch_query_moments(c->pair_args(), c->num_sms, done, st);
     launch_edge_assemble(c->d_edges, c->E, c->d_xf, c->d_acc, c->p.sigma * c->p.sigma, c->d_eout, done, st);
-    cudaMemsetAsync(c->d_H_cand, 0, sizeof(double) * 36LL * c->K * c->K, st);
+    const LMStep step{c->d_state, c->d_poses_cur, c->d_poses_cand, c->d_H_cur, c->d_b_cur};
     launch_frame_assemble(c->d_edges, c->E, c->K, c->d_inc_off, c->d_inc_list, c->d_eout, c->d_H_cand,
-                          c->d_b_cand, c->d_F_cand, c->d_n_cand, done, st);
+                          c->d_b_cand, c->d_F_cand, c->d_n_cand, done, lm ? &step : nullptr, st);
     c->phase_end();
 }
 
-void run_eval(rkhsba_ctx* c, const double* poses, const int* done) {
+void run_eval(rkhsba_ctx* c, const double* poses, const int* done, bool lm = false) {
     eval_pre(c, poses, done);
     eval_pairs(c, done);
-    eval_post(c, done);
+    eval_post(c, done, lm);
 }
 
 rkhsba_status check_poses(rkhsba_ctx* c, const double* poses) {
@@ -396,12 +398,7 @@ void reset_state(rkhsba_ctx* c) {
 
 void lm_initial(rkhsba_ctx* c) {
     const int* done = &c->d_state->done;
-    run_eval(c, c->d_poses_cand, done);
-    c->phase_begin(4);
-    launch_lm_accept(c->K, c->d_state, c->d_F_cand, c->d_n_cand, c->d_poses_cur, c->d_poses_cand,
-                     c->d_b_cur, c->d_b_cand, c->stream);
-    launch_copy_if_accepted(c->d_state, c->d_H_cur, c->d_H_cand, 36LL * c->K * c->K, c->stream);
-    c->phase_end();
+    run_eval(c, c->d_poses_cand, done, true);
     c->need_initial = false;
 }
 
@@ -419,12 +416,7 @@ void lm_iter_pre(rkhsba_ctx* c) {
 
 void lm_iter_post(rkhsba_ctx* c) {
     const int* done = &c->d_state->done;
-    eval_post(c, done);
-    c->phase_begin(4);
-    launch_lm_accept(c->K, c->d_state, c->d_F_cand, c->d_n_cand, c->d_poses_cur, c->d_poses_cand,
-                     c->d_b_cur, c->d_b_cand, c->stream);
-    launch_copy_if_accepted(c->d_state, c->d_H_cur, c->d_H_cand, 36LL * c->K * c->K, c->stream);
-    c->phase_end();
+    eval_post(c, done, true);
 }
 
 void lm_iteration(rkhsba_ctx* c) {
@@ -638,7 +630,6 @@ rkhsba_status rkhsba_rebuild(rkhsba_ctx* c) {
     if (!c) return fail(nullptr, RKHSBA_EINVAL, "ctx is NULL");
     bool alt = false;
     c->phase_begin(0);
-    cudaMemsetAsync(c->d_cell_start, 0, sizeof(int) * (c->C_total + 1), c->stream);
     grid_fill(c, &alt);
     c->phase_end();
     RK_CUDA(c, cudaGetLastError());

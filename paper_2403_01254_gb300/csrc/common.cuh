@@ -167,35 +167,45 @@ struct LMState {
     int done, status;         // status: 0 converged, 4 not converged
     int first, chol_fail, accepted;
     int n_accepted;           // accepted steps after the first evaluation
+    int ticket;               // blocks of the assembly that have finished
 };
 
 // ------------------------------------------------------------ launchers ----
 // scan.cu
 size_t scan_ws_elems(long long n);   // long longs of the radix sort's small workspace
-// Stable LSD sort of the low nbits of keys (payload vals); ends in the *_alt
-// buffers when *in_alt.  hist: radix_hist_elems(n) long longs; ws:
-// scan_ws_elems(n); *err |= 1 if a bounded wait of the look-back gave up.
-void radix_sort_u32(uint32_t* keys, int* vals, uint32_t* keys_alt, int* vals_alt, long long n,
-                    int nbits, long long* hist, long long* ws, int* err, cudaStream_t st, bool* in_alt);
 size_t radix_hist_elems(long long n);
+// Views of the scratch arrays of one sort of n keys of nbits: hist:
+// radix_hist_elems(n) long longs, ws: scan_ws_elems(n), which must be zero
+// before the kernel that makes the keys.
+struct RadixWs;
+RadixWs radix_ws(long long n, int nbits, long long* hist, long long* ws);
+// Stable LSD sort; vals receives the keys' first positions.  The kernel that
+// made the keys has counted their digits and cleared the tile records
+// (radix.cuh).  Returns whether the result is in the *_alt buffers; *err |= 1
+// if a bounded wait of the look-back gave up.  With *done set nothing is done
+// (the kernel that makes the keys and the one that clears ws heed it too).
+bool radix_sort_u32(uint32_t* keys, int* vals, uint32_t* keys_alt, int* vals_alt, long long n, const RadixWs& ws,
+                    int* err, const int* done, cudaStream_t st);
 
 // grid.cu
+void launch_iota(int* vals, long long n, cudaStream_t st);
 void launch_bbox(const double* xyz, const float* sem, const float* rgb, long long N, int K,
                  const long long* pt_off, int sem_dim, double h_inv, int* cmin, int* cmax,
                  unsigned* sem_norm_bits, int* err, cudaStream_t st);
 void launch_keys(const double* xyz, long long N, int K, const long long* pt_off,
-                 const FrameDev* frames, double h_inv, uint32_t* keys, int* vals, cudaStream_t st);
+                 const FrameDev* frames, double h_inv, uint32_t* keys, const RadixWs& ws, int num_sms,
+                 cudaStream_t st);
 void launch_gather(const double* xyz, const float* sem, const float* rgb, long long N, int K,
                    const long long* pt_off, const uint32_t* keys, const int* perm, GridParams gp,
                    long long C_total, float4* pts4, void* sem_sorted, float4* col4,
-                   int* perm_local, int* cell_start, long long* run_flag, cudaStream_t st);
+                   int* perm_local, int* cell_start, cudaStream_t st);
 
 // pairs.cu
-void launch_edge_setup(const double* poses, const EdgeDev* edges, int E, const FrameDev* frames,
-                       double h, EdgeXf* xf, const int* done, cudaStream_t st);
+void launch_eval_setup(const double* poses, const EdgeDev* edges, int E, const FrameDev* frames, double h, EdgeXf* xf,
+                       long long* ws, int n_ws, int* ucount, long long* acc, const int* done, cudaStream_t st);
 void launch_query_keys(const EdgeDev* edges, int E, const FrameDev* frames, const EdgeXf* xf,
                        const uint32_t* pt_cell, const float4* pts4, GridParams gp, long long Q,
-                       uint32_t* qkey, int* qval, float4* qrec, const int* done, cudaStream_t st);
+                       uint32_t* qkey, float4* qrec, const RadixWs& ws, int num_sms, const int* done, cudaStream_t st);
 void launch_units(const uint32_t* qkey_sorted, const int* qval_sorted, const float4* qrec, long long Q, int uq,
                   int sub, const EdgeDev* edges, int E, float4* slots, int2* units, int* n_units, const int* done,
                   cudaStream_t st);
@@ -224,17 +234,21 @@ void launch_emit_pairs(const int2* units, const int* n_units, int* unit_counter,
 // solve.cu
 void launch_edge_assemble(const EdgeDev* edges, int E, const EdgeXf* xf, const long long* acc,
                           double sigma2, EdgeOut* out, const int* done, cudaStream_t st);
+// The 6K system of one evaluation from the edges' results.  lm: also the
+// accept / reject step of the LM loop (and the copies of an accepted
+// candidate), done by the last block to finish.
+struct LMStep {
+    LMState* st;
+    double* poses_cur;
+    const double* poses_cand;
+    double* H_cur;
+    double* b_cur;
+};
 void launch_frame_assemble(const EdgeDev* edges, int E, int K, const int* inc_off,
                            const int* inc_list, const EdgeOut* eout, double* H, double* b,
-                           double* F, long long* npairs, const int* done, cudaStream_t st);
+                           double* F, long long* npairs, const int* done, const LMStep* lm, cudaStream_t st);
 void launch_lm_solve(int K, const double* H_cur, const double* b_cur, const double* poses_cur,
                      double* poses_cand, LMState* st_dev, double* ws, cudaStream_t st);
-void launch_lm_accept(int K, LMState* st_dev, const double* F_cand, const long long* n_cand,
-                      double* poses_cur, const double* poses_cand, double* b_cur,
-                      const double* b_cand, cudaStream_t st);
-void launch_copy_if_accepted(const LMState* st_dev, double* dst, const double* src,
-                             long long n, cudaStream_t st);
-
 }  // namespace rk
 
 #include "rkhsba.h"

@@ -1,7 +1,7 @@
 // Internal: the context of one problem and the host helpers shared by the
 // translation units that drive it (api.cu, init.cu).  Not part of the C ABI.
 #pragma once
-#include "common.cuh"
+#include "radix.cuh"
 
 #include <algorithm>
 #include <string>
@@ -60,9 +60,7 @@ struct rkhsba_ctx {
     void* d_sem = nullptr;
     float4* d_col4 = nullptr;
     int* d_perm_local = nullptr;
-    long long* d_run = nullptr;       // cell run starts of the sorted points
     const uint32_t* d_pt_cell = nullptr;  // grid cell key of every sorted point
-    long long* d_total = nullptr;      // scratch totals [4]
     long long* d_scan_ws = nullptr;
 
     long long total_bins = 0, Q_total = 0;

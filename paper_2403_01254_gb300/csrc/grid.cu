@@ -8,7 +8,7 @@
 // stable in the input order, and stored as FP32 offsets from their cell
 // centre.  Because points stay in frame-local coordinates the grid never
 // moves with the poses: only the queries of the other frame do.
-#include "common.cuh"
+#include "radix.cuh"
 
 #include <cuda_bf16.h>
 
@@ -114,19 +114,31 @@ __global__ void k_bbox(const double* __restrict__ xyz, const float* __restrict__
     }
 }
 
-__global__ void k_keys(const double* __restrict__ xyz, long long N, int K,
-                       const long long* __restrict__ pt_off, const FrameDev* __restrict__ frames,
-                       double h_inv, uint32_t* __restrict__ keys, int* __restrict__ vals) {
-    for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < N;
-         g += (long long)gridDim.x * blockDim.x) {
-        const FrameDev& F = frames[frame_of(pt_off, K, g)];
-        int l[3];
+// Grid cell key of every point; the block also counts its keys' digits and
+// clears its share of the sort's tile records (radix.cuh).
+__global__ void __launch_bounds__(RAD_T) k_keys(const double* __restrict__ xyz, long long N, int K,
+                                                const long long* __restrict__ pt_off,
+                                                const FrameDev* __restrict__ frames, double h_inv,
+                                                uint32_t* __restrict__ keys, RadixWs ws, int rounds) {
+    __shared__ int hist[RAD_PASSES][256];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) l[k] = (int)cell_q(xyz[3 * g + k], h_inv) - F.lo[k];
-        long long key = F.cell_off + ((long long)l[2] * F.dim[1] + l[1]) * F.dim[0] + l[0];
-        keys[g] = (uint32_t)key;
-        vals[g] = (int)g;
+    for (int p = 0; p < RAD_PASSES; ++p) hist[p][threadIdx.x] = 0;
+    __syncthreads();
+    for (int round = 0; round < rounds; ++round) {
+        const long long g = ((long long)blockIdx.x * rounds + round) * RAD_T + threadIdx.x;
+        uint32_t key = 0;
+        if (g < N) {
+            const FrameDev& F = frames[frame_of(pt_off, K, g)];
+            int l[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) l[k] = (int)cell_q(xyz[3 * g + k], h_inv) - F.lo[k];
+            key = (uint32_t)(F.cell_off + ((long long)l[2] * F.dim[1] + l[1]) * F.dim[0] + l[0]);
+            keys[g] = key;
+        }
+        radix_count(key, g < N, ws.npass, hist);
     }
+    __syncthreads();
+    radix_finish(ws, hist);
 }
 
 __global__ void k_gather(const double* __restrict__ xyz, const float* __restrict__ sem,
@@ -135,7 +147,7 @@ __global__ void k_gather(const double* __restrict__ xyz, const float* __restrict
                          const int* __restrict__ perm, GridParams gp, long long C_total,
                          float4* __restrict__ pts4, void* __restrict__ sem_sorted,
                          float4* __restrict__ col4, int* __restrict__ perm_local,
-                         int* __restrict__ cell_start, long long* __restrict__ run_flag) {
+                         int* __restrict__ cell_start) {
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < N;
          s += (long long)gridDim.x * blockDim.x) {
         const long long g = perm[s];
@@ -160,8 +172,6 @@ __global__ void k_gather(const double* __restrict__ xyz, const float* __restrict
             }
         }
         if (gp.color) col4[s] = make_float4(rgb[3 * g], rgb[3 * g + 1], rgb[3 * g + 2], 0.f);
-        const long long key = keys[s];
-        run_flag[s] = ((s == 0) || ((long long)keys[s - 1] != key)) ? 1 : 0;
     }
 }
 
@@ -182,6 +192,11 @@ __global__ void k_cell_start(const uint32_t* __restrict__ keys, long long N, lon
     }
 }
 
+__global__ void k_iota(int* __restrict__ vals, long long n) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        vals[i] = (int)i;
+}
+
 inline unsigned grid_for(long long n) {
     long long b = (n + GT - 1) / GT;
     if (b < 1) b = 1;
@@ -189,6 +204,12 @@ inline unsigned grid_for(long long n) {
     return (unsigned)b;
 }
 }  // namespace
+
+void launch_iota(int* vals, long long n, cudaStream_t st) {
+    if (n <= 0) return;
+    k_iota<<<grid_for(n), GT, 0, st>>>(vals, n);
+    count_launch();
+}
 
 void launch_bbox(const double* xyz, const float* sem, const float* rgb, long long N, int K,
                  const long long* pt_off, int sem_dim, double h_inv, int* cmin, int* cmax,
@@ -200,19 +221,22 @@ void launch_bbox(const double* xyz, const float* sem, const float* rgb, long lon
 }
 
 void launch_keys(const double* xyz, long long N, int K, const long long* pt_off,
-                 const FrameDev* frames, double h_inv, uint32_t* keys, int* vals, cudaStream_t st) {
+                 const FrameDev* frames, double h_inv, uint32_t* keys, const RadixWs& ws, int num_sms,
+                 cudaStream_t st) {
     if (N <= 0) return;
-    k_keys<<<grid_for(N), GT, 0, st>>>(xyz, N, K, pt_off, frames, h_inv, keys, vals);
+    const int rounds = radix_rounds(N, num_sms);
+    k_keys<<<(unsigned)((N + (long long)RAD_T * rounds - 1) / ((long long)RAD_T * rounds)), RAD_T, 0, st>>>(
+        xyz, N, K, pt_off, frames, h_inv, keys, ws, rounds);
     count_launch();
 }
 
 void launch_gather(const double* xyz, const float* sem, const float* rgb, long long N, int K,
                    const long long* pt_off, const uint32_t* keys, const int* perm, GridParams gp,
                    long long C_total, float4* pts4, void* sem_sorted, float4* col4,
-                   int* perm_local, int* cell_start, long long* run_flag, cudaStream_t st) {
+                   int* perm_local, int* cell_start, cudaStream_t st) {
     if (N <= 0) return;
     k_gather<<<grid_for(N), GT, 0, st>>>(xyz, sem, rgb, N, K, pt_off, keys, perm, gp, C_total,
-                                         pts4, sem_sorted, col4, perm_local, cell_start, run_flag);
+                                         pts4, sem_sorted, col4, perm_local, cell_start);
     k_cell_start<<<grid_for(C_total + 1), GT, 0, st>>>(keys, N, C_total, cell_start);
     count_launch(2);
 }

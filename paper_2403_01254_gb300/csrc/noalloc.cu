@@ -21,8 +21,8 @@
 // overlaps on the GPU (different streams, or different host threads)
 // overwrite each other's temporaries, so calls must be serialised by the
 // caller.
-#include "common.cuh"
 #include "layout.cuh"
+#include "radix.cuh"
 #include "rkhsba.h"
 
 #include <cmath>
@@ -183,7 +183,6 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
     int* d_inc_off = cv.take<int>(K + 1);
     int* d_inc_list = cv.take<int>(2 * E);
     double* d_poses = cv.take<double>(16 * K);
-    long long* d_total = cv.take<long long>(4);
     if (!cv.ok) return fail(RKHSBA_EINVAL, "static scratch too small");
     int cmin[3 * MAX_K], cmax[3 * MAX_K], errbits = 0;
     unsigned semn[MAX_K];
@@ -236,7 +235,6 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
     void* d_sem_sorted = sp > 0 ? (void*)cv.take<unsigned char>(N * sp * (gp.sem_bf16 ? 2 : 4)) : nullptr;
     float4* d_col4 = gp.color ? cv.take<float4>(N) : nullptr;
     int* d_perm_local = cv.take<int>(N);
-    long long* d_run = cv.take<long long>(N);
     uint32_t* d_qkey = cv.take<uint32_t>(Q);
     uint32_t* d_qkey_alt = cv.take<uint32_t>(Q);
     const bool per_query = pairs_per_query(gp);
@@ -267,21 +265,21 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
     SCK(cudaMemcpyAsync(d_poses, poses, sizeof(double) * 16 * K, cudaMemcpyHostToDevice, st));
 
     // ---- grid step (all temporaries that must start at zero are cleared) ----
-    SCK(cudaMemsetAsync(d_cell_start, 0, sizeof(int) * (C + 1), st));
-    launch_keys(d_xyz, N, K, d_pt_off, d_frames, gp.h_inv, d_keys, d_vals, st);
-    bool alt = false;
-    radix_sort_u32(d_keys, d_vals, d_keys_alt, d_vals_alt, N, cbits, d_hist, d_ws, d_err + 1, st, &alt);
+    if (N == 0) SCK(cudaMemsetAsync(d_cell_start, 0, sizeof(int) * (C + 1), st));
+    const RadixWs gws = radix_ws(N, cbits, d_hist, d_ws);
+    SCK(cudaMemsetAsync(d_ws, 0, sizeof(long long) * scan_ws_elems(N), st));
+    launch_keys(d_xyz, N, K, d_pt_off, d_frames, gp.h_inv, d_keys, gws, num_sms, st);
+    if (gws.npass == 0) launch_iota(d_vals, N, st);
+    const bool alt = radix_sort_u32(d_keys, d_vals, d_keys_alt, d_vals_alt, N, gws, d_err + 1, nullptr, st);
     const uint32_t* pt_cell = alt ? d_keys_alt : d_keys;
     launch_gather(d_xyz, d_sem, gp.color ? d_rgb : nullptr, N, K, d_pt_off, pt_cell, alt ? d_vals_alt : d_vals,
-                  gp, C, d_pts4, d_sem_sorted, d_col4, d_perm_local, d_cell_start, d_run, st);
+                  gp, C, d_pts4, d_sem_sorted, d_col4, d_perm_local, d_cell_start, st);
 
     // ---- evaluation ----
-    launch_edge_setup(d_poses, d_edges, E, d_frames, gp.h, d_xf, nullptr, st);
-    SCK(cudaMemsetAsync(d_ucount, 0, sizeof(int) * 4, st));
-    SCK(cudaMemsetAsync(d_acc, 0, sizeof(long long) * E * ACC_N, st));
-    launch_query_keys(d_edges, E, d_frames, d_xf, pt_cell, d_pts4, gp, Q, d_qkey, d_qval, d_qrec, nullptr, st);
-    bool qalt = false;
-    radix_sort_u32(d_qkey, d_qval, d_qkey_alt, d_qval_alt, Q, qbits, d_hist, d_ws, d_err + 1, st, &qalt);
+    const RadixWs qws = radix_ws(Q, qbits, d_hist, d_ws);
+    launch_eval_setup(d_poses, d_edges, E, d_frames, gp.h, d_xf, d_ws, (int)scan_ws_elems(Q), d_ucount, d_acc, nullptr, st);
+    launch_query_keys(d_edges, E, d_frames, d_xf, pt_cell, d_pts4, gp, Q, d_qkey, d_qrec, qws, num_sms, nullptr, st);
+    const bool qalt = radix_sort_u32(d_qkey, d_qval, d_qkey_alt, d_qval_alt, Q, qws, d_err + 1, nullptr, st);
     const uint32_t* qk = qalt ? d_qkey_alt : d_qkey;
     launch_units(qk, qalt ? d_qval_alt : d_qval, d_qrec, Q, UNIT_Q, gp.key_sub, d_edges, E, d_slots, d_units,
                  d_ucount, nullptr, st);
@@ -310,7 +308,7 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
     }
     launch_edge_assemble(d_edges, E, d_xf, d_acc, p.sigma * p.sigma, d_eout, nullptr, st);
     SCK(cudaMemsetAsync(d_H, 0, sizeof(double) * 36LL * K * K, st));
-    launch_frame_assemble(d_edges, E, K, d_inc_off, d_inc_list, d_eout, d_H, d_b, d_F, d_n, nullptr, st);
+    launch_frame_assemble(d_edges, E, K, d_inc_off, d_inc_list, d_eout, d_H, d_b, d_F, d_n, nullptr, nullptr, st);
 
     // ---- results to the caller's host buffers ----
     double F = 0.0;

@@ -28,7 +28,7 @@
 // No FP64 arithmetic runs per query: the frame-a position of a frame-b cell
 // centre comes from a per-edge affine map held as double-float pairs, evaluated
 // with error-free transformations (Dekker product, Knuth sum) on the FP32 pipe.
-#include "common.cuh"
+#include "radix.cuh"
 
 #include <type_traits>
 
@@ -62,39 +62,52 @@ __device__ __forceinline__ df df_mul_f(float hi, float lo, float c) {
     return fast_two_sum(p, fmaf(lo, c, e));
 }
 
-__global__ void k_edge_setup(const double* __restrict__ poses, const EdgeDev* __restrict__ edges,
-                             int E, const FrameDev* __restrict__ frames, double h,
-                             EdgeXf* __restrict__ xf, const int* done) {
+// Start of an evaluation: the edges' transforms, one warp per edge (nine lanes
+// an entry of R_ab each: FP64 chains of a few operations instead of the ~100 of
+// one thread per edge, 8.4 us at 28 edges), and everything cleared that the
+// evaluation counts or adds into: the sort's digit counts and tile counters,
+// the unit counters and the edges' accumulators.
+__global__ void __launch_bounds__(128) k_eval_setup(const double* __restrict__ poses, const EdgeDev* __restrict__ edges,
+                                                    int E, const FrameDev* __restrict__ frames, double h,
+                                                    EdgeXf* __restrict__ xf, long long* __restrict__ ws, int n_ws,
+                                                    int* __restrict__ ucount, long long* __restrict__ acc,
+                                                    const int* done) {
     if (done && *done) return;
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= E) return;
-    const double* Ta = poses + 16 * edges[e].a;
-    const double* Tb = poses + 16 * edges[e].b;
-    const FrameDev& Fb = frames[edges[e].b];
-    EdgeXf X;
-    // R_ab = R_a^T R_b,  t_ab = R_a^T (t_b - t_a)
-    for (int r = 0; r < 3; ++r)
-        for (int c = 0; c < 3; ++c) {
-            double s = 0.0;
-            for (int k = 0; k < 3; ++k) s += Ta[4 * k + r] * Tb[4 * k + c];
-            X.R[3 * r + c] = s;
-            X.Rf[3 * r + c] = (float)s;
+    const int gt = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+    for (int i = gt; i < n_ws; i += nt) ws[i] = 0;
+    for (long long i = gt; i < (long long)E * ACC_N; i += nt) acc[i] = 0;
+    if (gt < 4) ucount[gt] = 0;
+    const int lane = threadIdx.x & 31;
+    for (int e = gt >> 5; e < E; e += nt >> 5) {
+        const double* Ta = poses + 16 * edges[e].a;
+        const double* Tb = poses + 16 * edges[e].b;
+        const FrameDev& Fb = frames[edges[e].b];
+        EdgeXf& X = xf[e];
+        // R_ab = R_a^T R_b (lane 3 r + c: entry (r, c)),  t_ab = R_a^T (t_b - t_a) (lanes 9..11)
+        const int r = lane < 9 ? lane / 3 : lane - 9, c = lane % 3;
+        double v = 0.0, prod = 0.0;
+        if (lane < 9) {
+            for (int k = 0; k < 3; ++k) v += Ta[4 * k + r] * Tb[4 * k + c];
+            X.R[lane] = v;
+            X.Rf[lane] = (float)v;
+            // P(l) = h R l + [R (lo_b + 1/2) h + t]
+            const double A = h * v;
+            X.Ahi[lane] = (float)A;
+            X.Alo[lane] = (float)(A - (double)(float)A);
+            prod = v * ((double)Fb.lo[c] + 0.5) * h;
+        } else if (lane < 12) {
+            v = Ta[r] * (Tb[3] - Ta[3]) + Ta[4 + r] * (Tb[7] - Ta[7]) + Ta[8 + r] * (Tb[11] - Ta[11]);
+            X.t[r] = v;
         }
-    const double dt[3] = {Tb[3] - Ta[3], Tb[7] - Ta[7], Tb[11] - Ta[11]};
-    for (int r = 0; r < 3; ++r) X.t[r] = Ta[r] * dt[0] + Ta[4 + r] * dt[1] + Ta[8 + r] * dt[2];
-    // P(l) = h R l + [R (lo_b + 1/2) h + t]
-    for (int r = 0; r < 3; ++r) {
-        double B = X.t[r];
-        for (int c = 0; c < 3; ++c) {
-            const double A = h * X.R[3 * r + c];
-            X.Ahi[3 * r + c] = (float)A;
-            X.Alo[3 * r + c] = (float)(A - (double)(float)A);
-            B += X.R[3 * r + c] * ((double)Fb.lo[c] + 0.5) * h;
+        const int src = lane >= 9 && lane < 12 ? 3 * r : 0;
+        const double p0 = __shfl_sync(FULL, prod, src), p1 = __shfl_sync(FULL, prod, src + 1),
+                     p2 = __shfl_sync(FULL, prod, src + 2);
+        if (lane >= 9 && lane < 12) {
+            const double B = v + p0 + p1 + p2;
+            X.Bhi[r] = (float)B;
+            X.Blo[r] = (float)(B - (double)(float)B);
         }
-        X.Bhi[r] = (float)B;
-        X.Blo[r] = (float)(B - (double)(float)B);
     }
-    xf[e] = X;
 }
 
 __device__ __forceinline__ int find_edge_q(const EdgeDev* __restrict__ edges, int E, long long q) {
@@ -116,15 +129,23 @@ __device__ __forceinline__ int find_edge_bin(const EdgeDev* __restrict__ edges, 
 }
 
 // One thread per query: frame-a home cell key and the query's FP32 offset
-// from that cell's centre.
-__global__ void k_query_keys(const EdgeDev* __restrict__ edges, int E, const FrameDev* __restrict__ frames,
-                             const EdgeXf* __restrict__ xf, const uint32_t* __restrict__ pt_cell,
-                             const float4* __restrict__ pts4, GridParams gp, long long Q,
-                             uint32_t* __restrict__ qkey, int* __restrict__ qval,
-                             float4* __restrict__ qrec, const int* done) {
+// from that cell's centre.  The block also counts its keys' digits and clears
+// its share of the sort's tile records (radix.cuh).
+__global__ void __launch_bounds__(RAD_T) k_query_keys(const EdgeDev* __restrict__ edges, int E,
+                                                      const FrameDev* __restrict__ frames,
+                                                      const EdgeXf* __restrict__ xf, const uint32_t* __restrict__ pt_cell,
+                                                      const float4* __restrict__ pts4, GridParams gp, long long Q,
+                                                      uint32_t* __restrict__ qkey, float4* __restrict__ qrec,
+                                                      RadixWs ws, int rounds, const int* done) {
     if (done && *done) return;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < Q;
-         q += (long long)gridDim.x * blockDim.x) {
+    __shared__ int hist[RAD_PASSES][256];
+#pragma unroll
+    for (int p = 0; p < RAD_PASSES; ++p) hist[p][threadIdx.x] = 0;
+    __syncthreads();
+    for (int round = 0; round < rounds; ++round) {
+        const long long q = ((long long)blockIdx.x * rounds + round) * RAD_T + threadIdx.x;
+        uint32_t key = NO_KEY;
+        if (q < Q) {
         const int e = find_edge_q(edges, E, q);
         const EdgeDev& Ed = edges[e];
         const FrameDev& Fa = frames[Ed.a];
@@ -164,7 +185,6 @@ __global__ void k_query_keys(const EdgeDev* __restrict__ edges, int E, const Fra
         const int hy = (int)(K[1] + my) - Fa.lo[1];
         const int hz = (int)(K[2] + mz) - Fa.lo[2];
         const float ox = fmaf(-mx, gp.hf, vx), oy = fmaf(-my, gp.hf, vy), oz = fmaf(-mz, gp.hf, vz);
-        uint32_t key = NO_KEY;
         if (hx >= 0 && hy >= 0 && hz >= 0 && hx < Fa.dim[0] && hy < Fa.dim[1] && hz < Fa.dim[2]) {
             key = (uint32_t)(Ed.bin_off + ((long long)hz * Fa.dim[1] + hy) * Fa.dim[0] + hx);
             // with key_sub = 3 the low bits hold the query's octant of its home
@@ -173,9 +193,12 @@ __global__ void k_query_keys(const EdgeDev* __restrict__ edges, int E, const Fra
                 key = (key << 3) | (ox >= 0.f ? 1u : 0u) | (oy >= 0.f ? 2u : 0u) | (oz >= 0.f ? 4u : 0u);
         }
         qkey[q] = key;
-        qval[q] = (int)q;
         qrec[q] = make_float4(ox, oy, oz, __int_as_float(s));
+        }
+        radix_count(key, q < Q, ws.npass, hist);
     }
+    __syncthreads();
+    radix_finish(ws, hist);
 }
 
 // Sorted query records and the unit list, in one pass over the sorted keys: a
@@ -1216,37 +1239,41 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int2 unit, in
 // forms, with o the home cell's centre,
 //   W = k, D = X1 - k y, sum w y', sum w y'y'^T, sum w d y'^T (y' = y + o)
 //   and Q = X2 - X1 y^T - y X1^T + k y y^T.
-// A lane adds its queries of the `per` (<= MOM_PER) groups of 32 sorted queries
-// that its warp takes, the sums are rounded to the edge's fixed point and
-// added in 64-bit integers.  As a pass of its own every lane has a query, and
-// the rounding and the reduction over the lanes are paid once per 128 queries;
-// at the end of each unit of the pair kernel they cost ~1000 instructions for
-// (LiDAR scenes) 8 queries in the median.
-constexpr int MOM_PER = 4;
-__global__ void __launch_bounds__(128, 5) k_query_moments(const PairArgs A, int per, const int* done) {
+// Each query's moments are rounded to the edge's fixed point on their own, so
+// that the integer sums do not depend on which queries share a lane or a warp
+// (an edge's results are the same whatever other edges there are); a lane adds
+// its queries of the `per` (<= MOM_PER) groups of 32 sorted queries that its warp
+// takes, and the warp reduces once per edge it meets.  As a pass of its own every
+// lane has a query, and the reduction is paid once per 256 queries; at the end of each
+// unit of the pair kernel both cost ~1000 instructions for (LiDAR scenes) 8
+// queries in the median.
+constexpr int MOM_PER = 8;
+__global__ void __launch_bounds__(128, 4) k_query_moments(const PairArgs A, int per, const int* done) {
     if (done && *done) return;
     const int lane = threadIdx.x & 31;
     const GridParams& gp = A.gp;
     const long long w0 = ((long long)blockIdx.x * 4 + (threadIdx.x >> 5)) * per * 32;
-    float W = 0.f, D[3], Sy[3], Myy[6], Mdy[9], Q[6];
-    auto clear = [&]() {
-        W = 0.f;
+    long long v[32];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) D[k] = Sy[k] = 0.f;
-#pragma unroll
-        for (int k = 0; k < 6; ++k) Myy[k] = Q[k] = 0.f;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) Mdy[k] = 0.f;
-    };
-    clear();
+    for (int k = 0; k < 32; ++k) v[k] = 0;
     // edge of the sums so far: its home-cell keys, scales and frame-a grid
     int e_cur = -1, lo0 = 0, lo1 = 0, lo2 = 0, dim0 = 1, dim1 = 1;
     long long bin_lo = 0, bin_hi = 0;
     float s0 = 0.f, s1 = 0.f, s2 = 0.f;
     const int parts = 1 << part_shift(A, *A.n_units);
+    float c0 = 0.f, c1 = 0.f, c2 = 0.f, c3 = 0.f, c4 = 0.f, c5 = 0.f;
     auto flush = [&]() {
-        if (e_cur >= 0)
-            add_moments(W, D, Sy, Myy, Mdy, Q, 0, A.edges[e_cur].scale, A.acc + (long long)e_cur * ACC_N, lane);
+        if (e_cur < 0) return;
+        reduce_half<16>(v, lane);
+        reduce_half<8>(v, lane);
+        reduce_half<4>(v, lane);
+        reduce_half<2>(v, lane);
+        reduce_half<1>(v, lane);
+        if (lane < N_MOM - 1 && v[0] != 0)
+            atomicAdd(reinterpret_cast<unsigned long long*>(A.acc + (long long)e_cur * ACC_N + lane),
+                      (unsigned long long)v[0]);
+#pragma unroll
+        for (int k = 0; k < 32; ++k) v[k] = 0;
     };
     for (int r = 0; r < per; ++r) {
         const long long k = w0 + 32LL * r + lane;
@@ -1275,7 +1302,6 @@ __global__ void __launch_bounds__(128, 5) k_query_moments(const PairArgs A, int 
             const long long kl = __shfl_sync(FULL, key, __ffs(todo) - 1);
             if (kl < bin_lo || kl >= bin_hi) {
                 flush();
-                clear();
                 e_cur = find_edge_bin(A.edges, A.E, kl);
                 const EdgeDev& Ed = A.edges[e_cur];
                 const FrameDev& Fa = A.frames[Ed.a];
@@ -1290,6 +1316,12 @@ __global__ void __launch_bounds__(128, 5) k_query_moments(const PairArgs A, int 
                 s0 = ldexpf(1.f, -sc.kw);
                 s1 = ldexpf(1.f, sc.ex - sc.kw);
                 s2 = ldexpf(1.f, 2 * sc.ex - sc.kw);
+                c0 = Ed.scale[MC_W];
+                c1 = Ed.scale[MC_D];
+                c2 = Ed.scale[MC_SY];
+                c3 = Ed.scale[MC_MYY];
+                c4 = Ed.scale[MC_MDY];
+                c5 = Ed.scale[MC_Q];
             }
             const bool mine = valid && key >= bin_lo && key < bin_hi;
             todo &= ~__ballot_sync(FULL, mine);
@@ -1302,21 +1334,21 @@ __global__ void __launch_bounds__(128, 5) k_query_moments(const PairArgs A, int 
                 const float w = f0.x * s0;
                 const float X1[3] = {f0.y * s1, f0.z * s1, f0.w * s1};
                 const float X2[6] = {f1.x * s2, f1.y * s2, f1.z * s2, f1.w * s2, f2v.x * s2, f2v.y * s2};
-                W += w;
+                v[0] += to_fixed(w, c0);
                 int t6 = 0;
 #pragma unroll
                 for (int m = 0; m < 3; ++m) {
                     const float ky = w * y[m], d = X1[m] - ky;
-                    D[m] += d;
-                    Sy[m] += fmaf(w, o[m], ky);
+                    v[1 + m] += to_fixed(d, c1);
+                    v[4 + m] += to_fixed(fmaf(w, o[m], ky), c2);
 #pragma unroll
                     for (int l = m; l < 3; ++l, ++t6) {
                         const float kyy = ky * y[l], kyl = w * y[l];
-                        Myy[t6] += kyy + (ky * o[l] + o[m] * kyl + w * o[m] * o[l]);
-                        Q[t6] += X2[t6] - X1[m] * y[l] - y[m] * X1[l] + kyy;
+                        v[7 + t6] += to_fixed(kyy + (ky * o[l] + o[m] * kyl + w * o[m] * o[l]), c3);
+                        v[22 + t6] += to_fixed(X2[t6] - X1[m] * y[l] - y[m] * X1[l] + kyy, c5);
                     }
 #pragma unroll
-                    for (int l = 0; l < 3; ++l) Mdy[3 * m + l] += fmaf(d, o[l], d * y[l]);
+                    for (int l = 0; l < 3; ++l) v[13 + 3 * m + l] += to_fixed(fmaf(d, o[l], d * y[l]), c4);
                 }
             }
         }
@@ -2068,18 +2100,20 @@ bool with_label_layout(const GridParams& gp, const F& f) {
 }
 }  // namespace
 
-void launch_edge_setup(const double* poses, const EdgeDev* edges, int E, const FrameDev* frames,
-                       double h, EdgeXf* xf, const int* done, cudaStream_t st) {
-    k_edge_setup<<<(E + 127) / 128, 128, 0, st>>>(poses, edges, E, frames, h, xf, done);
+void launch_eval_setup(const double* poses, const EdgeDev* edges, int E, const FrameDev* frames, double h, EdgeXf* xf,
+                       long long* ws, int n_ws, int* ucount, long long* acc, const int* done, cudaStream_t st) {
+    k_eval_setup<<<(unsigned)(E < 4 * 592 ? (E + 3) / 4 : 592), 128, 0, st>>>(poses, edges, E, frames, h, xf, ws, n_ws,
+                                                                              ucount, acc, done);
     count_launch();
 }
 
 void launch_query_keys(const EdgeDev* edges, int E, const FrameDev* frames, const EdgeXf* xf,
                        const uint32_t* pt_cell, const float4* pts4, GridParams gp, long long Q,
-                       uint32_t* qkey, int* qval, float4* qrec, const int* done, cudaStream_t st) {
+                       uint32_t* qkey, float4* qrec, const RadixWs& ws, int num_sms, const int* done, cudaStream_t st) {
     if (Q <= 0) return;
-    k_query_keys<<<blocks_for(Q, 256), 256, 0, st>>>(edges, E, frames, xf, pt_cell, pts4, gp, Q, qkey, qval,
-                                                    qrec, done);
+    const int rounds = radix_rounds(Q, num_sms);
+    k_query_keys<<<(unsigned)((Q + (long long)RAD_T * rounds - 1) / ((long long)RAD_T * rounds)), RAD_T, 0, st>>>(
+        edges, E, frames, xf, pt_cell, pts4, gp, Q, qkey, qrec, ws, rounds, done);
     count_launch();
 }
 

@@ -1,203 +1,224 @@
-// Stable LSD radix sort of uint32 keys with an int32 payload: the plumbing of
-// the grid build (points by cell) and of the per-evaluation query binning
-// (queries by home cell).  The pair sum needs a spatial index (the paper
-// names GPU voxel hashing as future work); this one is rebuilt by sorting.
+// Stable LSD radix sort of uint32 keys with an int32 payload (the key's first
+// position): the plumbing of the grid build (points by cell) and of the
+// per-evaluation query binning (queries by home cell).  The pair sum needs a
+// spatial index (the paper names GPU voxel hashing as future work); this one is
+// rebuilt by sorting.
 //
-// One counting kernel reads the keys once and histograms every 8-bit digit;
-// each pass is then a single kernel ("one sweep"): a block takes the next
-// tile of 2048 keys (tiles are handed out in order by an atomic counter),
-// ranks its keys stably (match.any inside a warp, per-warp digit counts
-// across warps, rounds of 256 keys in input order), publishes its per-digit
-// counts, and obtains the counts of all earlier tiles by looking back over
-// their published records (decoupled look-back): a record holds a flag
-// (aggregate of the tile / inclusive prefix up to the tile) and a count in
-// one 64-bit word.  Every wait is bounded; a wait that gives up sets an error
-// word and the kernel finishes with what it has.
-#include "common.cuh"
+// The kernels that make the keys also histogram their 8-bit digits (radix.cuh);
+// each pass is then a single kernel ("one sweep"): a block takes the next tile
+// of keys (tiles are handed out in order by an atomic counter), ranks its keys
+// stably (each warp its own run of keys by match.any and a digit counter of its
+// own; one exclusive sum over the warps), publishes its per-digit counts, obtains
+// the counts of all earlier tiles by looking back over their published records
+// (decoupled look-back, eight records read at a time), and writes the tile in
+// digit order from shared memory.  A record holds a flag (aggregate of the tile
+// / inclusive prefix up to the tile) and a count in one 64-bit word.  Every wait
+// is bounded; a wait that gives up sets an error word and the kernel finishes
+// with what it has.
+//
+// Ranking by warps costs two block barriers per tile where rounds of 256 keys in
+// input order cost three each (24 per tile of 2048).
+#include "radix.cuh"
 
+#include <utility>
 #include <vector>
 
 namespace rk {
 
 namespace {
-constexpr int RAD_T = 256;
-constexpr int RAD_IPT = 8;
-constexpr int RAD_TILE = RAD_T * RAD_IPT;        // 2048 keys per tile
 constexpr int RAD_WARPS = RAD_T / 32;
-constexpr int MAX_PASS = 4;
 constexpr unsigned long long ST_AGG = 1ull << 62;      // count = this tile's
 constexpr unsigned long long ST_PRE = 2ull << 62;      // count = tiles 0..t inclusive
 constexpr unsigned long long ST_CNT = (1ull << 62) - 1ull;
 constexpr int SPIN_LIMIT = 1 << 22;         // polls of one look-back wait before it gives up
-
-__global__ void __launch_bounds__(RAD_T) k_radix_counts(const uint32_t* __restrict__ keys, long long n,
-                                                        int npass, unsigned long long* __restrict__ counts) {
-    __shared__ int c[MAX_PASS][256];
-#pragma unroll
-    for (int p = 0; p < MAX_PASS; ++p) c[p][threadIdx.x] = 0;
-    __syncthreads();
-    const long long base = (long long)blockIdx.x * RAD_TILE;
-#pragma unroll
-    for (int k = 0; k < RAD_IPT; ++k) {
-        const long long i = base + (long long)k * RAD_T + threadIdx.x;
-        if (i < n) {
-            const uint32_t key = keys[i];
-            for (int p = 0; p < npass; ++p) atomicAdd(&c[p][(key >> (8 * p)) & 255u], 1);
-        }
-    }
-    __syncthreads();
-    for (int p = 0; p < npass; ++p)
-        if (c[p][threadIdx.x]) atomicAdd(&counts[256 * p + threadIdx.x], (unsigned long long)c[p][threadIdx.x]);
-}
+constexpr int LOOK = 8;                     // records a look-back reads at a time
 
 // exclusive scan of one value per thread over a 256-thread block
-__device__ __forceinline__ long long block_excl_scan256(long long v, long long* s_warp) {
+template <typename T>
+__device__ __forceinline__ T block_excl_scan256(T v, T* s_warp) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    long long inc = v;
+    T inc = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const long long u = __shfl_up_sync(0xffffffffu, inc, o);
+        const T u = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += u;
     }
     if (lane == 31) s_warp[warp] = inc;
     __syncthreads();
-    long long before = 0;
-    for (int w = 0; w < warp; ++w) before += s_warp[w];
+    T before = 0;
+#pragma unroll
+    for (int w = 0; w < RAD_WARPS; ++w) before += w < warp ? s_warp[w] : T(0);
     __syncthreads();
     return before + inc - v;
 }
 
+// FIRST: the payload is the key's position, not read.
+template <int IPT, bool FIRST>
 __global__ void __launch_bounds__(RAD_T) k_onesweep(const uint32_t* __restrict__ kin,
                                                     const int* __restrict__ vin,
                                                     uint32_t* __restrict__ kout, int* __restrict__ vout,
                                                     long long n, int shift,
                                                     const unsigned long long* __restrict__ counts,
                                                     unsigned long long* status, int* tile_ctr, int* err,
-                                                    int spin_limit) {
+                                                    int spin_limit, const int* done) {
+    if (done && *done) return;
+    constexpr int TILE = RAD_T * IPT;
     __shared__ int s_tile;
-    __shared__ int run[256];
     __shared__ int wcnt[RAD_WARPS][256];
-    __shared__ long long s_base[256];
+    __shared__ int s_loc[256];            // first place of a digit inside the tile
+    __shared__ long long s_out[256];      // what to add to a place inside the tile for its place in the output
     __shared__ long long s_warp[RAD_WARPS];
+    __shared__ int s_warpi[RAD_WARPS];
+    __shared__ uint32_t s_key[TILE];
+    __shared__ int s_val[TILE];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) s_tile = atomicAdd(tile_ctr, 1);
-    run[tid] = 0;
 #pragma unroll
     for (int w = 0; w < RAD_WARPS; ++w) wcnt[w][tid] = 0;
     __syncthreads();
     const int t = s_tile;
-    const long long base = (long long)t * RAD_TILE;
+    const long long base = (long long)t * TILE;
     const unsigned lt = (1u << lane) - 1u;
-    uint32_t key[RAD_IPT];
-    int val[RAD_IPT], dig[RAD_IPT], rank[RAD_IPT];
-    // all loads of the tile first (independent), then the ranking rounds
+    const int off = warp * (32 * IPT) + lane;       // a warp's keys are one run of the input
+    uint32_t key[IPT];
+    int val[IPT], rank[IPT];
 #pragma unroll
-    for (int r = 0; r < RAD_IPT; ++r) {
-        const long long i = base + (long long)r * RAD_T + tid;
+    for (int r = 0; r < IPT; ++r) {
+        const long long i = base + off + 32 * r;
         key[r] = i < n ? kin[i] : 0u;
-        val[r] = i < n ? vin[i] : 0;
+        val[r] = FIRST ? (int)i : (i < n ? vin[i] : 0);
     }
-    // stable ranks inside the tile: round r holds keys base + 256 r + tid
 #pragma unroll
-    for (int r = 0; r < RAD_IPT; ++r) {
-        const long long i = base + (long long)r * RAD_T + tid;
-        const bool valid = i < n;
+    for (int r = 0; r < IPT; ++r) {
+        const bool valid = base + off + 32 * r < n;
         const int d = valid ? (int)((key[r] >> shift) & 255u) : 256;
-        dig[r] = d;
         const unsigned peers = __match_any_sync(0xffffffffu, d);
-        const int lr = __popc(peers & lt);
-        if (valid && lr == 0) wcnt[warp][d] = __popc(peers);
-        __syncthreads();
-        rank[r] = 0;
-        if (valid) {
-            int off = run[d] + lr;
-            for (int w = 0; w < warp; ++w) off += wcnt[w][d];
-            rank[r] = off;
+        const int leader = __ffs(peers) - 1;
+        int old = 0;
+        if (valid && lane == leader) {
+            old = wcnt[warp][d];
+            wcnt[warp][d] = old + __popc(peers);
         }
-        __syncthreads();
-        int add = 0;
-#pragma unroll
-        for (int w = 0; w < RAD_WARPS; ++w) {
-            add += wcnt[w][tid];
-            wcnt[w][tid] = 0;
-        }
-        run[tid] += add;
-        __syncthreads();
+        rank[r] = __shfl_sync(0xffffffffu, old, leader) + __popc(peers & lt);
+        __syncwarp();
     }
-    // publish this tile's count of digit tid, then look back for the prefix
+    __syncthreads();
+    // digit tid: exclusive sum over the warps, this tile's count
     const int d = tid;
-    const long long cnt = run[d];
+    int cnt = 0;
+#pragma unroll
+    for (int w = 0; w < RAD_WARPS; ++w) {
+        const int c = wcnt[w][d];
+        wcnt[w][d] = cnt;
+        cnt += c;
+    }
+    // publish it, then look back for the prefix
     volatile unsigned long long* st = status + (long long)t * 256 + d;
+    *st = (t == 0 ? ST_PRE : ST_AGG) | (unsigned long long)cnt;
+    const int loc = block_excl_scan256<int>(cnt, s_warpi);
+    const long long first = block_excl_scan256<long long>((long long)counts[d], s_warp);
+    s_loc[d] = loc;
+    __syncthreads();
+    // the tile in digit order (places below the tile's key count)
+#pragma unroll
+    for (int r = 0; r < IPT; ++r) {
+        if (base + off + 32 * r < n) {
+            const int dd = (int)((key[r] >> shift) & 255u);
+            const int at = s_loc[dd] + wcnt[warp][dd] + rank[r];
+            s_key[at] = key[r];
+            s_val[at] = val[r];
+        }
+    }
     long long excl = 0;
-    if (t == 0) {
-        *st = ST_PRE | (unsigned long long)cnt;
-    } else {
-        *st = ST_AGG | (unsigned long long)cnt;
-        bool gave_up = false;
-        for (int p = t - 1; p >= 0 && !gave_up; --p) {
-            volatile unsigned long long* sp = status + (long long)p * 256 + d;
-            unsigned long long v = *sp;
-            int spins = 0;
-            while ((v >> 62) == 0ull) {
-                if (++spins > spin_limit) {   // give up: the prefix stays short, writes stay in bounds
-                    atomicOr(err, 1);
-                    gave_up = true;
-                    break;
+    if (t > 0) {
+        bool open = true;                           // no inclusive prefix met yet
+        for (int p = t - 1; p >= 0 && open; p -= LOOK) {
+            unsigned long long v[LOOK];
+#pragma unroll
+            for (int j = 0; j < LOOK; ++j)
+                v[j] = p - j >= 0 ? *(volatile unsigned long long*)(status + (long long)(p - j) * 256 + d) : 0ull;
+#pragma unroll
+            for (int j = 0; j < LOOK; ++j) {
+                if (open && p - j >= 0) {
+                    volatile unsigned long long* sp = status + (long long)(p - j) * 256 + d;
+                    int spins = 0;
+                    while ((v[j] >> 62) == 0ull) {
+                        if (++spins > spin_limit) {   // give up: the prefix stays short, writes stay in bounds
+                            atomicOr(err, 1);
+                            open = false;
+                            break;
+                        }
+                        __nanosleep(20);
+                        v[j] = *sp;
+                    }
+                    excl += (long long)(v[j] & ST_CNT);
+                    if ((v[j] >> 62) == 2ull) open = false;
                 }
-                __nanosleep(32);
-                v = *sp;
             }
-            excl += (long long)(v & ST_CNT);
-            if ((v >> 62) == 2ull) break;
         }
         *st = ST_PRE | (unsigned long long)(excl + cnt);
     }
-    s_base[d] = block_excl_scan256((long long)counts[d], s_warp) + excl;
+    s_out[d] = first + excl - loc;
     __syncthreads();
+    const int m = n - base < TILE ? (int)(n - base) : TILE;
 #pragma unroll
-    for (int r = 0; r < RAD_IPT; ++r) {
-        const long long i = base + (long long)r * RAD_T + tid;
-        if (i < n) {
-            const long long o = s_base[dig[r]] + rank[r];
-            kout[o] = key[r];
-            vout[o] = val[r];
+    for (int r = 0; r < IPT; ++r) {
+        const int j = tid + RAD_T * r;
+        if (j < m) {
+            const uint32_t k = s_key[j];
+            const long long o = s_out[(k >> shift) & 255u] + j;
+            kout[o] = k;
+            vout[o] = s_val[j];
         }
     }
 }
-}  // namespace
 
-size_t scan_ws_elems(long long) { return (size_t)(MAX_PASS * 256 + 2 * MAX_PASS); }
-
-size_t radix_hist_elems(long long n) {
-    const long long nb = (n + RAD_TILE - 1) / RAD_TILE;
-    return (size_t)(MAX_PASS * 256 * (nb > 0 ? nb : 1));
-}
-
-void radix_sort_u32(uint32_t* keys, int* vals, uint32_t* keys_alt, int* vals_alt, long long n,
-                    int nbits, long long* hist, long long* ws, int* err, cudaStream_t st, bool* in_alt) {
-    *in_alt = false;
-    if (n <= 0 || nbits <= 0) return;
-    const int nb = (int)((n + RAD_TILE - 1) / RAD_TILE);
-    const int npass = (nbits + 7) / 8;
-    unsigned long long* status = reinterpret_cast<unsigned long long*>(hist);
-    unsigned long long* counts = reinterpret_cast<unsigned long long*>(ws);
-    int* ctr = reinterpret_cast<int*>(ws + MAX_PASS * 256);
-    cudaMemsetAsync(status, 0, sizeof(unsigned long long) * 256 * (size_t)nb * npass, st);
-    cudaMemsetAsync(ws, 0, sizeof(long long) * scan_ws_elems(n), st);
-    k_radix_counts<<<nb, RAD_T, 0, st>>>(keys, n, npass, counts);
-    count_launch();
+template <int IPT>
+void sort_passes(uint32_t* keys, int* vals, uint32_t* keys_alt, int* vals_alt, long long n, const RadixWs& ws,
+                 int* err, const int* done, cudaStream_t st) {
+    const long long nb = (n + RAD_T * IPT - 1) / (RAD_T * IPT);
     uint32_t* ki = keys;
     int* vi = vals;
     uint32_t* ko = keys_alt;
     int* vo = vals_alt;
-    for (int p = 0; p < npass; ++p) {
-        k_onesweep<<<nb, RAD_T, 0, st>>>(ki, vi, ko, vo, n, 8 * p, counts + 256 * p,
-                                         status + (size_t)256 * nb * p, ctr + p, err, SPIN_LIMIT);
+    for (int p = 0; p < ws.npass; ++p) {
+        auto kernel = p == 0 ? k_onesweep<IPT, true> : k_onesweep<IPT, false>;
+        kernel<<<(unsigned)nb, RAD_T, 0, st>>>(ki, vi, ko, vo, n, 8 * p, ws.counts + 256 * p,
+                                               ws.status + (size_t)256 * nb * p, ws.ctr + p, err, SPIN_LIMIT, done);
         count_launch();
-        uint32_t* tk = ki; ki = ko; ko = tk;
-        int* tv = vi; vi = vo; vo = tv;
-        *in_alt = !*in_alt;
+        std::swap(ki, ko);
+        std::swap(vi, vo);
     }
+}
+// Tiles of 4096 keys once there are enough of them for every SM several times
+// over (half the records per key: 51.6 M keys, see the launch), else of 2048.
+constexpr long long BIG_SORT = 4096LL * 152 * 8;
+}  // namespace
+
+size_t scan_ws_elems(long long) { return (size_t)(RAD_PASSES * 256 + 2 * RAD_PASSES); }
+
+size_t radix_hist_elems(long long n) {
+    const long long nb = (n + RAD_TILE_MIN - 1) / RAD_TILE_MIN;
+    return (size_t)(RAD_PASSES * 256 * (nb > 0 ? nb : 1));
+}
+
+RadixWs radix_ws(long long n, int nbits, long long* hist, long long* ws) {
+    RadixWs r{};
+    r.counts = reinterpret_cast<unsigned long long*>(ws);
+    r.ctr = reinterpret_cast<int*>(ws + RAD_PASSES * 256);
+    r.status = reinterpret_cast<unsigned long long*>(hist);
+    r.npass = (nbits + 7) / 8;
+    const long long tile = n >= BIG_SORT ? 4096 : 2048;
+    r.n_status = 256 * ((n + tile - 1) / tile) * r.npass;
+    return r;
+}
+
+bool radix_sort_u32(uint32_t* keys, int* vals, uint32_t* keys_alt, int* vals_alt, long long n, const RadixWs& ws,
+                    int* err, const int* done, cudaStream_t st) {
+    if (n <= 0 || ws.npass <= 0) return false;
+    if (n >= BIG_SORT) sort_passes<16>(keys, vals, keys_alt, vals_alt, n, ws, err, done, st);
+    else sort_passes<8>(keys, vals, keys_alt, vals_alt, n, ws, err, done, st);
+    return (ws.npass & 1) != 0;
 }
 
 }  // namespace rk
@@ -217,7 +238,7 @@ extern "C" rkhsba_status rkhsba_selftest_lookback_timeout(int32_t spin_limit, in
         set_thread_error("rkhsba_selftest_lookback_timeout: spin_limit must be in [1, 2^20]");
         return RKHSBA_EINVAL;
     }
-    const long long n = 2LL * RAD_TILE;
+    const long long n = 2LL * RAD_TILE_MIN;
     const long long G = 256;                        // guard words on each side of the outputs
     uint32_t* kin = nullptr;
     uint32_t* kout = nullptr;
@@ -256,11 +277,12 @@ extern "C" rkhsba_status rkhsba_selftest_lookback_timeout(int32_t spin_limit, in
     if ((e = cudaMemset(kout, 0xAB, sizeof(uint32_t) * (n + 2 * G))) != cudaSuccess) return cuda_fail(e);
     if ((e = cudaMemset(vout, 0xAB, sizeof(int) * (n + 2 * G))) != cudaSuccess) return cuda_fail(e);
     if ((e = cudaMemset(status, 0, sizeof(unsigned long long) * 2 * 256)) != cudaSuccess) return cuda_fail(e);
-    if ((e = cudaMemset(counts, 0, sizeof(unsigned long long) * 256)) != cudaSuccess) return cuda_fail(e);
+    std::vector<unsigned long long> hc(256, 0ull);
+    for (long long i = 0; i < n; ++i) ++hc[hk[i] & 255u];
+    if ((e = cudaMemcpy(counts, hc.data(), sizeof(unsigned long long) * 256, cudaMemcpyHostToDevice)) != cudaSuccess)
+        return cuda_fail(e);
     if ((e = cudaMemcpy(ctl, ctl0, sizeof(ctl0), cudaMemcpyHostToDevice)) != cudaSuccess) return cuda_fail(e);
-    k_radix_counts<<<2, RAD_T>>>(kin, n, 1, counts);
-    count_launch();
-    k_onesweep<<<1, RAD_T>>>(kin, vin, kout + G, vout + G, n, 0, counts, status, ctl, ctl + 1, spin_limit);
+    k_onesweep<RAD_TILE_MIN / RAD_T, false><<<1, RAD_T>>>(kin, vin, kout + G, vout + G, n, 0, counts, status, ctl, ctl + 1, spin_limit, nullptr);
     count_launch();
     if ((e = cudaDeviceSynchronize()) != cudaSuccess) return cuda_fail(e);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e);

@@ -25,149 +25,178 @@ __device__ __forceinline__ void skew(const double* v, double S[3][3]) {
     S[2][0] = -v[1]; S[2][1] = v[0];  S[2][2] = 0.0;
 }
 
-__global__ void k_edge_assemble(const EdgeDev* __restrict__ edges, int E, const EdgeXf* __restrict__ xf,
-                                const long long* __restrict__ acc, double sigma2,
-                                EdgeOut* __restrict__ out, const int* done) {
-    if (done && *done) return;
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= E) return;
-    const long long* a = acc + (long long)e * ACC_N;
-    const EdgeDev& Ed = edges[e];
-    double m[28];
-    for (int k = 0; k < 28; ++k) m[k] = (double)a[k] * Ed.inv_scale[moment_class(k)];
-    const double W = m[0];
-    const double D[3] = {m[1], m[2], m[3]};
-    const double Sy[3] = {m[4], m[5], m[6]};
-    const double Myy[3][3] = {{m[7], m[8], m[9]}, {m[8], m[10], m[11]}, {m[9], m[11], m[12]}};
-    const double Mdy[3][3] = {{m[13], m[14], m[15]}, {m[16], m[17], m[18]}, {m[19], m[20], m[21]}};
-    const double Q[3][3] = {{m[22], m[23], m[24]}, {m[23], m[25], m[26]}, {m[24], m[26], m[27]}};
-    const EdgeXf& X = xf[e];
-    const double* R = X.R;
-    const double* t = X.t;
-
-    double Sx[3], St[3], Gx[3], Gt[3];
-    double Mxx[3][3], Mxt[3][3], Mtt[3][3];
-    for (int i = 0; i < 3; ++i) {
-        Sx[i] = Sy[i] + D[i];
-        St[i] = Sy[i] - W * t[i];
-    }
-    for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) {
-            const double Mxy = Myy[i][j] + Mdy[i][j];                 // sum w x y'^T
-            Mxx[i][j] = Myy[i][j] + Mdy[i][j] + Mdy[j][i] + Q[i][j];   // sum w x x^T
-            Mxt[i][j] = Mxy - Sx[i] * t[j];                             // sum w x y~^T
-            Mtt[i][j] = Myy[i][j] - Sy[i] * t[j] - t[i] * Sy[j] + W * t[i] * t[j];
-        }
-    // sum w x (x) d = sum w y' (x) d
-    Gx[0] = Mdy[2][1] - Mdy[1][2];
-    Gx[1] = Mdy[0][2] - Mdy[2][0];
-    Gx[2] = Mdy[1][0] - Mdy[0][1];
-    // sum w y~ (x) d, y~ = y' - t_ab
-    Gt[0] = Gx[0] - (t[1] * D[2] - t[2] * D[1]);
-    Gt[1] = Gx[1] - (t[2] * D[0] - t[0] * D[2]);
-    Gt[2] = Gx[2] - (t[0] * D[1] - t[1] * D[0]);
-
-    EdgeOut o;
-    o.F = sigma2 * W;
-    o.E = Q[0][0] + Q[1][1] + Q[2][2];
-    o.n = a[28];
-    o.pad = 0;
-    // b_a = [D; Gx],  b_b = -[R^T D; R^T Gt]
-    for (int i = 0; i < 3; ++i) {
-        o.b[i] = D[i];
-        o.b[3 + i] = Gx[i];
-        o.b[6 + i] = -(R[i] * D[0] + R[3 + i] * D[1] + R[6 + i] * D[2]);
-        o.b[9 + i] = -(R[i] * Gt[0] + R[3 + i] * Gt[1] + R[6 + i] * Gt[2]);
-    }
-    double* H = o.H;
-    for (int k = 0; k < 144; ++k) H[k] = 0.0;
-    double Kx[3][3], Kt[3][3], Kb[3][3];
-    skew(Sx, Kx);
-    skew(St, Kt);
-    // frame-b quantities in b's own axes: Sb = R^T St, Mb = R^T Mtt R
-    double Sb[3], Mb[3][3], T1[3][3];
-    for (int i = 0; i < 3; ++i) Sb[i] = R[i] * St[0] + R[3 + i] * St[1] + R[6 + i] * St[2];
-    for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) T1[i][j] = Mtt[i][0] * R[j] + Mtt[i][1] * R[3 + j] + Mtt[i][2] * R[6 + j];
-    for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) Mb[i][j] = R[i] * T1[0][j] + R[3 + i] * T1[1][j] + R[6 + i] * T1[2][j];
-    skew(Sb, Kb);
-    const double trx = Mxx[0][0] + Mxx[1][1] + Mxx[2][2];
-    const double trb = Mb[0][0] + Mb[1][1] + Mb[2][2];
-    const double trxt = Mxt[0][0] + Mxt[1][1] + Mxt[2][2];
-    // right factors of the a-b block: [S~]x R, [Sx]x R, (Mxt^T - tr I) R
-    double KtR[3][3], KxR[3][3], NR[3][3];
-    for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) {
-            double s1 = 0.0, s2 = 0.0, s3 = 0.0;
-            for (int k = 0; k < 3; ++k) {
-                s1 += Kt[i][k] * R[3 * k + j];
-                s2 += Kx[i][k] * R[3 * k + j];
-                const double Nik = Mxt[k][i] - (i == k ? trxt : 0.0);
-                s3 += Nik * R[3 * k + j];
-            }
-            KtR[i][j] = s1; KxR[i][j] = s2; NR[i][j] = s3;
-        }
-    for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) {
-            const double id = (i == j) ? 1.0 : 0.0;
-            // H_aa
-            H[12 * i + j] = W * id;
-            H[12 * i + 3 + j] = -Kx[i][j];
-            H[12 * (3 + i) + j] = Kx[i][j];
-            H[12 * (3 + i) + 3 + j] = trx * id - Mxx[i][j];
-            // H_bb
-            H[12 * (6 + i) + 6 + j] = W * id;
-            H[12 * (6 + i) + 9 + j] = -Kb[i][j];
-            H[12 * (9 + i) + 6 + j] = Kb[i][j];
-            H[12 * (9 + i) + 9 + j] = trb * id - Mb[i][j];
-            // H_ab and its transpose
-            const double ab00 = -W * R[3 * i + j];
-            const double ab01 = KtR[i][j];
-            const double ab10 = -KxR[i][j];
-            const double ab11 = NR[i][j];
-            H[12 * i + 6 + j] = ab00;
-            H[12 * i + 9 + j] = ab01;
-            H[12 * (3 + i) + 6 + j] = ab10;
-            H[12 * (3 + i) + 9 + j] = ab11;
-            H[12 * (6 + j) + i] = ab00;
-            H[12 * (9 + j) + i] = ab01;
-            H[12 * (6 + j) + 3 + i] = ab10;
-            H[12 * (9 + j) + 3 + i] = ab11;
-        }
-    out[e] = o;
+// entry (i, j) of the cross-product matrix [v]x
+__device__ __forceinline__ double skew_at(const double* v, int i, int j) {
+    if (i == j) return 0.0;
+    const double x = v[3 - i - j];
+    return j == (i + 1) % 3 ? -x : x;
 }
+
+// One block per edge, the entries of each stage over its threads: as one thread
+// per edge the ~1000 dependent FP64 operations took 15.6 us at any edge count.
+__global__ void __launch_bounds__(64) k_edge_assemble(const EdgeDev* __restrict__ edges, const EdgeXf* __restrict__ xf,
+                                                      const long long* __restrict__ acc, double sigma2,
+                                                      EdgeOut* __restrict__ out, const int* done) {
+    if (done && *done) return;
+    __shared__ double m[28], R[9], t[3];
+    __shared__ double Mxx[9], Mxt[9], Mtt[9], Sx[3], St[3], T1[9], Mb[9], Sb[3], KtR[9], KxR[9], NR[9];
+    const int e = blockIdx.x, tid = threadIdx.x;
+    const long long* a = acc + (long long)e * ACC_N;
+    EdgeOut& o = out[e];
+    if (tid < 28) m[tid] = (double)a[tid] * edges[e].inv_scale[moment_class(tid)];
+    else if (tid < 37) R[tid - 28] = xf[e].R[tid - 28];
+    else if (tid < 40) t[tid - 37] = xf[e].t[tid - 37];
+    else if (tid == 40) o.n = a[28];
+    __syncthreads();
+    const double W = m[0];
+    const double* D = m + 1;
+    const double* Sy = m + 4;
+    // place of (i, j) among the six upper entries of a symmetric matrix
+    auto sym = [](int i, int j) { return i <= j ? (i == 0 ? j : (i == 1 ? 2 + j : 5)) : (j == 0 ? i : (j == 1 ? 2 + i : 5)); };
+    const int i = (tid % 9) / 3, j = tid % 3;
+    if (tid < 27) {
+        const double myy = m[7 + sym(i, j)], mij = m[13 + 3 * i + j], mji = m[13 + 3 * j + i];   // Mdy
+        if (tid < 9) Mxx[tid] = myy + mij + mji + m[22 + sym(i, j)];              // sum w x x^T
+        else if (tid < 18) Mxt[tid - 9] = (myy + mij) - (Sy[i] + D[i]) * t[j];    // sum w x y~^T
+        else Mtt[tid - 18] = myy - Sy[i] * t[j] - t[i] * Sy[j] + W * t[i] * t[j];
+    } else if (tid < 30) {
+        Sx[tid - 27] = Sy[tid - 27] + D[tid - 27];
+    } else if (tid < 33) {
+        St[tid - 30] = Sy[tid - 30] - W * t[tid - 30];
+    } else if (tid == 33) {
+        o.F = sigma2 * W;
+        o.E = m[22] + m[25] + m[27];
+        o.pad = 0;
+    } else if (tid < 46) {
+        // b_a = [D; Gx],  b_b = -[R^T D; R^T Gt], with Gx = sum w x (x) d =
+        // sum w y' (x) d and Gt = sum w y~ (x) d, y~ = y' - t_ab
+        const int k = tid - 34, c = k % 3;
+        const double G[3] = {m[20] - m[18], m[15] - m[19], m[16] - m[14]};
+        double v;
+        if (k < 3) v = D[c];
+        else if (k < 6) v = G[c];
+        else if (k < 9) v = -(R[c] * D[0] + R[3 + c] * D[1] + R[6 + c] * D[2]);
+        else {
+            const double Gt[3] = {G[0] - (t[1] * D[2] - t[2] * D[1]), G[1] - (t[2] * D[0] - t[0] * D[2]),
+                                  G[2] - (t[0] * D[1] - t[1] * D[0])};
+            v = -(R[c] * Gt[0] + R[3 + c] * Gt[1] + R[6 + c] * Gt[2]);
+        }
+        o.b[k] = v;
+    }
+    __syncthreads();
+    // right factors of the a-b block: [S~]x R, [Sx]x R, (Mxt^T - tr I) R; and
+    // frame-b quantities in b's own axes: Sb = R^T St, Mb = R^T Mtt R
+    if (tid < 9) {
+        T1[tid] = Mtt[3 * i] * R[j] + Mtt[3 * i + 1] * R[3 + j] + Mtt[3 * i + 2] * R[6 + j];
+    } else if (tid < 36) {
+        const double trxt = Mxt[0] + Mxt[4] + Mxt[8];
+        double v = 0.0;
+        for (int k = 0; k < 3; ++k) {
+            const double f = tid < 18 ? skew_at(St, i, k) : (tid < 27 ? skew_at(Sx, i, k)
+                                                                      : Mxt[3 * k + i] - (i == k ? trxt : 0.0));
+            v += f * R[3 * k + j];
+        }
+        (tid < 18 ? KtR : (tid < 27 ? KxR : NR))[tid % 9] = v;
+    } else if (tid < 39) {
+        const int c = tid - 36;
+        Sb[c] = R[c] * St[0] + R[3 + c] * St[1] + R[6 + c] * St[2];
+    }
+    __syncthreads();
+    if (tid < 9) Mb[tid] = R[i] * T1[j] + R[3 + i] * T1[3 + j] + R[6 + i] * T1[6 + j];
+    __syncthreads();
+    const double trx = Mxx[0] + Mxx[4] + Mxx[8], trb = Mb[0] + Mb[4] + Mb[8];
+    for (int k = tid; k < 144; k += 64) {
+        int r = k / 12, c = k % 12;
+        if (r >= 6 && c < 6) { const int x = r; r = c; c = x; }      // the a-b block's transpose
+        const int p = r % 3, q = c % 3;
+        const bool rot_r = (r / 3) & 1, rot_c = (c / 3) & 1;
+        const double id = p == q ? 1.0 : 0.0;
+        double v;
+        if (c < 6 || r >= 6) {                                        // H_aa, H_bb
+            const bool b = r >= 6;
+            const double* S = b ? Sb : Sx;
+            const double* M = b ? Mb : Mxx;
+            if (!rot_r && !rot_c) v = W * id;
+            else if (rot_r && rot_c) v = (b ? trb : trx) * id - M[3 * p + q];
+            else v = rot_r ? skew_at(S, p, q) : -skew_at(S, p, q);
+        } else if (!rot_r) {                                          // H_ab
+            v = rot_c ? KtR[3 * p + q] : -W * R[3 * p + q];
+        } else {
+            v = rot_c ? NR[3 * p + q] : -KxR[3 * p + q];
+        }
+        o.H[k] = v;
+    }
+}
+
+// The LM loop's decision on an evaluated candidate (one thread): returns
+// whether it is accepted.
+__device__ int lm_accept(LMState* S, double F, long long n) {
+    S->pair_terms += n;
+    S->n_cand = n;
+    int acc;
+    if (S->first) {
+        acc = 1;
+        S->first = 0;
+        S->F_cur = F;
+    } else {
+        S->iters += 1;
+        const double step = S->step_inf;
+        if (F > S->F_cur) {
+            const double rel = (F - S->F_cur) / fmax(fabs(S->F_cur), 1e-300);
+            acc = 1;
+            S->F_cur = F;
+            S->n_accepted += 1;
+            S->lambda = fmax(S->lambda * 0.1, 1e-12);
+            if (step < S->tol_step || rel < S->tol_rel_f) { S->done = 1; S->status = 0; }
+        } else {
+            acc = 0;
+            S->lambda *= 10.0;
+            if (step < S->tol_step || S->lambda > 1e10) { S->done = 1; S->status = 0; }
+        }
+        if (!S->done && S->iters >= S->max_iters) { S->done = 1; S->status = 4; }
+    }
+    S->F_cand = F;
+    S->accepted = acc;
+    S->chol_fail = 0;
+    return acc;
+}
+
+// Systems of up to this many entries are copied by the accepting block itself
+// (one block copies 64 KB in a few us; larger ones take k_copy_if).
+constexpr long long ACCEPT_COPY = 8192;
+constexpr int FA_T = 128;
 
 // blocks [0, K): diagonal 6x6 block and gradient of frame m (sum over its
 // edges in edge order); [K, K+E): the off-diagonal block of edge e;
-// K+E: totals.  Every entry has one writer and a fixed summation order.
-__global__ void k_frame_assemble(const EdgeDev* __restrict__ edges, int E, int K,
-                                 const int* __restrict__ inc_off, const int* __restrict__ inc_list,
-                                 const EdgeOut* __restrict__ eo, double* __restrict__ H,
-                                 double* __restrict__ b, double* __restrict__ F,
-                                 long long* __restrict__ npairs, const int* done) {
+// K+E: totals.  Every entry has one writer and a fixed summation order.  With an
+// LM step the last block to finish decides on the candidate (its inputs come
+// from the other blocks' stores, read past L1).
+__global__ void __launch_bounds__(FA_T) k_frame_assemble(const EdgeDev* __restrict__ edges, int E, int K,
+                                                         const int* __restrict__ inc_off,
+                                                         const int* __restrict__ inc_list,
+                                                         const EdgeOut* __restrict__ eo, double* __restrict__ H,
+                                                         double* __restrict__ b, double* __restrict__ F,
+                                                         long long* __restrict__ npairs, const int* done, LMStep lm) {
     if (done && *done) return;
+    __shared__ double s_F[FA_T];
+    __shared__ long long s_n[FA_T];
+    __shared__ int s_last;
     const int ld = 6 * K;
     const int tid = threadIdx.x;
     const int blk = blockIdx.x;
     if (blk < K) {
         const int m = blk;
-        if (tid < 36) {
-            const int r = tid / 6, c = tid % 6;
+        if (tid < 42) {
+            const bool diag = tid < 36;
+            const int r = diag ? tid / 6 : tid - 36, c = diag ? tid % 6 : 0;
             double s = 0.0;
+#pragma unroll 4
             for (int k = inc_off[m]; k < inc_off[m + 1]; ++k) {
                 const int e = inc_list[k] >> 1, off = 6 * (inc_list[k] & 1);
-                s += eo[e].H[12 * (off + r) + off + c];
+                s += diag ? eo[e].H[12 * (off + r) + off + c] : eo[e].b[off + r];
             }
-            H[(long long)(6 * m + r) * ld + 6 * m + c] = s;
-        } else if (tid < 42) {
-            const int r = tid - 36;
-            double s = 0.0;
-            for (int k = inc_off[m]; k < inc_off[m + 1]; ++k) {
-                const int e = inc_list[k] >> 1, off = 6 * (inc_list[k] & 1);
-                s += eo[e].b[off + r];
-            }
-            b[6 * m + r] = s;
+            if (diag) H[(long long)(6 * m + r) * ld + 6 * m + c] = s;
+            else b[6 * m + r] = s;
         }
     } else if (blk < K + E) {
         const int e = blk - K;
@@ -178,16 +207,46 @@ __global__ void k_frame_assemble(const EdgeDev* __restrict__ edges, int E, int K
             H[(long long)(6 * a + r) * ld + 6 * bb + c] = v;
             H[(long long)(6 * bb + c) * ld + 6 * a + r] = v;
         }
-    } else if (tid == 0) {
+    } else {
         double s = 0.0;
         long long n = 0;
-        for (int e = 0; e < E; ++e) {
+        for (int e = tid; e < E; e += FA_T) {
             s += eo[e].F;
             n += eo[e].n;
         }
-        *F = s;
-        *npairs = n;
+        s_F[tid] = s;
+        s_n[tid] = n;
+        for (int o = FA_T / 2; o > 0; o >>= 1) {
+            __syncthreads();
+            if (tid < o) {
+                s_F[tid] += s_F[tid + o];
+                s_n[tid] += s_n[tid + o];
+            }
+        }
+        if (tid == 0) {
+            *F = s_F[0];
+            *npairs = s_n[0];
+        }
     }
+    if (!lm.st) return;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(&lm.st->ticket, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    __shared__ int s_acc;
+    if (tid == 0) {
+        lm.st->ticket = 0;
+        s_acc = lm_accept(lm.st, __ldcg(F), __ldcg(npairs));
+    }
+    __syncthreads();
+    if (!s_acc) return;
+    for (int i = tid; i < 16 * K; i += FA_T) lm.poses_cur[i] = lm.poses_cand[i];
+    for (int i = tid; i < 6 * K; i += FA_T) lm.b_cur[i] = __ldcg(b + i);
+    const long long nH = (long long)ld * ld;
+    if (nH <= ACCEPT_COPY)
+        for (long long i = tid; i < nH; i += FA_T) lm.H_cur[i] = __ldcg(H + i);
 }
 
 __device__ void se3_exp_dev(const double* xi, double T[12]) {
@@ -537,51 +596,6 @@ __global__ void __launch_bounds__(LM_T) k_lm_subst(int K, const double* __restri
     lm_finish(K, n, A, y, rinv, S->chol_fail, Tcur, Tcand, S, red);
 }
 
-__global__ void k_lm_accept(int K, LMState* S, const double* __restrict__ Fc,
-                            const long long* __restrict__ nc, double* __restrict__ Tcur,
-                            const double* __restrict__ Tcand, double* __restrict__ bcur,
-                            const double* __restrict__ bcand) {
-    __shared__ int s_acc;
-    if (S->done) return;
-    if (threadIdx.x == 0) {
-        const double F = *Fc;
-        const long long n = *nc;
-        S->pair_terms += n;
-        S->n_cand = n;
-        int acc;
-        if (S->first) {
-            acc = 1;
-            S->first = 0;
-            S->F_cur = F;
-        } else {
-            S->iters += 1;
-            const double step = S->step_inf;
-            if (F > S->F_cur) {
-                const double rel = (F - S->F_cur) / fmax(fabs(S->F_cur), 1e-300);
-                acc = 1;
-                S->F_cur = F;
-                S->n_accepted += 1;
-                S->lambda = fmax(S->lambda * 0.1, 1e-12);
-                if (step < S->tol_step || rel < S->tol_rel_f) { S->done = 1; S->status = 0; }
-            } else {
-                acc = 0;
-                S->lambda *= 10.0;
-                if (step < S->tol_step || S->lambda > 1e10) { S->done = 1; S->status = 0; }
-            }
-            if (!S->done && S->iters >= S->max_iters) { S->done = 1; S->status = 4; }
-        }
-        S->F_cand = F;
-        S->accepted = acc;
-        S->chol_fail = 0;
-        s_acc = acc;
-    }
-    __syncthreads();
-    if (s_acc) {
-        for (int i = threadIdx.x; i < 16 * K; i += blockDim.x) Tcur[i] = Tcand[i];
-        for (int i = threadIdx.x; i < 6 * K; i += blockDim.x) bcur[i] = bcand[i];
-    }
-}
-
 __global__ void k_copy_if(const LMState* S, double* __restrict__ dst, const double* __restrict__ src,
                           long long n) {
     if (!S->accepted) return;
@@ -593,16 +607,21 @@ __global__ void k_copy_if(const LMState* S, double* __restrict__ dst, const doub
 
 void launch_edge_assemble(const EdgeDev* edges, int E, const EdgeXf* xf, const long long* acc,
                           double sigma2, EdgeOut* out, const int* done, cudaStream_t st) {
-    k_edge_assemble<<<(E + 63) / 64, 64, 0, st>>>(edges, E, xf, acc, sigma2, out, done);
+    k_edge_assemble<<<E, 64, 0, st>>>(edges, xf, acc, sigma2, out, done);
     count_launch();
 }
 
 void launch_frame_assemble(const EdgeDev* edges, int E, int K, const int* inc_off,
                            const int* inc_list, const EdgeOut* eout, double* H, double* b,
-                           double* F, long long* npairs, const int* done, cudaStream_t st) {
-    k_frame_assemble<<<K + E + 1, 64, 0, st>>>(edges, E, K, inc_off, inc_list, eout, H, b, F, npairs,
-                                              done);
+                           double* F, long long* npairs, const int* done, const LMStep* lm, cudaStream_t st) {
+    k_frame_assemble<<<K + E + 1, FA_T, 0, st>>>(edges, E, K, inc_off, inc_list, eout, H, b, F, npairs, done,
+                                                 lm ? *lm : LMStep{});
     count_launch();
+    const long long nH = 36LL * K * K;
+    if (lm && nH > ACCEPT_COPY) {
+        k_copy_if<<<(unsigned)std::min<long long>((nH + 255) / 256, 1024), 256, 0, st>>>(lm->st, lm->H_cur, H, nH);
+        count_launch();
+    }
 }
 
 void launch_lm_solve(int K, const double* H_cur, const double* b_cur, const double* poses_cur,
@@ -640,22 +659,6 @@ void launch_lm_solve(int K, const double* H_cur, const double* b_cur, const doub
         return;
     }
     k_lm_solve<<<1, LM_T, smem, st>>>(K, H_cur, b_cur, poses_cur, poses_cand, st_dev, ws);
-    count_launch();
-}
-
-void launch_lm_accept(int K, LMState* st_dev, const double* F_cand, const long long* n_cand,
-                      double* poses_cur, const double* poses_cand, double* b_cur,
-                      const double* b_cand, cudaStream_t st) {
-    k_lm_accept<<<1, 128, 0, st>>>(K, st_dev, F_cand, n_cand, poses_cur, poses_cand, b_cur, b_cand);
-    count_launch();
-}
-
-void launch_copy_if_accepted(const LMState* st_dev, double* dst, const double* src, long long n,
-                             cudaStream_t st) {
-    long long blocks = (n + 255) / 256;
-    if (blocks > 1024) blocks = 1024;
-    if (blocks < 1) blocks = 1;
-    k_copy_if<<<(unsigned)blocks, 256, 0, st>>>(st_dev, dst, src, n);
     count_launch();
 }
 
