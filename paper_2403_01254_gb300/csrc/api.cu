@@ -276,18 +276,10 @@ rkhsba_status build(rkhsba_ctx* c, const double* xyz, const float* sem, const fl
     RK_TRY(alloc(c, &c->d_xf, E));
     RK_TRY(alloc(c, &c->d_qkey, Q));
     RK_TRY(alloc(c, &c->d_qkey_alt, Q));
-    // the query order and the unsorted records are done with when the units
-    // are cut, so the dense pair kernel's per-query sums take their place
-    const bool per_query = pairs_per_query(c->gp);
-    const int parts = per_query ? 1 << part_max_for(c->gp, Q, c->num_sms) : 1;
-    RK_TRY(alloc(c, &c->d_qval, 2 * Q * parts));
-    c->d_qval_alt = c->d_qval + Q;
+    RK_TRY(alloc(c, &c->d_qval, Q));
+    RK_TRY(alloc(c, &c->d_qval_alt, Q));
     RK_TRY(alloc(c, &c->d_qhist, (long long)radix_hist_elems(Q)));
-    RK_TRY(alloc(c, &c->d_qrec, per_query ? 2 * Q * parts : Q));
-    if (per_query) {
-        c->d_qs8 = reinterpret_cast<float*>(c->d_qrec);
-        c->d_qs2 = reinterpret_cast<float*>(c->d_qval);
-    }
+    RK_TRY(alloc(c, &c->d_qrec, Q));
     RK_TRY(alloc(c, &c->d_slots, Q));
     RK_TRY(alloc(c, &c->d_units, Q));
     RK_TRY(alloc(c, &c->d_ucount, 4));
@@ -351,7 +343,6 @@ void eval_pairs(rkhsba_ctx* c, const int* done) {
 void eval_post(rkhsba_ctx* c, const int* done, bool lm = false) {
     cudaStream_t st = c->stream;
     c->phase_begin(3);
-    if (pairs_per_query(c->gp)) launch_query_moments(c->pair_args(), c->num_sms, done, st);
     launch_edge_assemble(c->d_edges, c->E, c->d_xf, c->d_acc, c->p.sigma * c->p.sigma, c->d_eout, done, st);
     const LMStep step{c->d_state, c->d_poses_cur, c->d_poses_cand, c->d_H_cur, c->d_b_cur};
     launch_frame_assemble(c->d_edges, c->E, c->K, c->d_inc_off, c->d_inc_list, c->d_eout, c->d_H_cand,

@@ -120,8 +120,6 @@ struct PairArgs {
     const void* sem_sorted;   // label rows in the same order (FP32 or BF16), or NULL
     const float4* col4;       // colours in the same order, or NULL
     long long* acc;           // [E][ACC_N] fixed-point moments
-    float* qs8;               // [parts][Q][8], [parts][Q][2]: per sorted query sum_c w (1, x, x x^T) of
-    float* qs2;               //   the dense pair kernel (scaled), read by k_query_moments
     int E;
     GridParams gp;
 };
@@ -210,11 +208,6 @@ void launch_units(const uint32_t* qkey_sorted, const int* qval_sorted, const flo
                   int sub, const EdgeDev* edges, int E, float4* slots, int2* units, int* n_units, const int* done,
                   cudaStream_t st);
 void launch_pairs(const PairLaunch& L, const PairArgs& A);
-// The dense pair kernel leaves per-query sums (PairArgs::qs8, qs2), which
-// launch_query_moments turns into the edges' moments; the others add to the
-// moments themselves.
-bool pairs_per_query(const GridParams& gp);
-void launch_query_moments(const PairArgs& A, int num_sms, const int* done, cudaStream_t st);
 // Largest unit_queries setting of this layout: 64 for the dense tile kernel
 // with BF16 labels, else 32 (64 is taken as two units of 32).
 int pair_unit_max(const GridParams& gp);

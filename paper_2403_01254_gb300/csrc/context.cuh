@@ -74,8 +74,6 @@ struct rkhsba_ctx {
     float4* d_qrec = nullptr;          // per query: offset from home centre, point index
     float4* d_slots = nullptr;         // the same in sorted order
     int2* d_units = nullptr;           // units of <= tune_uq queries of one home cell
-    float* d_qs8 = nullptr;            // per-query sums of the dense pair kernel (d_qs8 on d_qrec,
-    float* d_qs2 = nullptr;            //   d_qs2 on d_qval / d_qval_alt: both free once the units are cut)
     int* d_ucount = nullptr;           // [2]: number of units, unit counter
     const uint32_t* q_sorted_key = nullptr;
     long long* d_acc = nullptr;
@@ -129,8 +127,6 @@ struct rkhsba_ctx {
         a.n_units = d_ucount;
         a.part_max = rk::part_max_for(gp, Q_total, num_sms);
         a.part_target = rk::part_target_for(num_sms);
-        a.qs8 = d_qs8;
-        a.qs2 = d_qs2;
         a.E = E;
         a.gp = gp;
         return a;

@@ -237,7 +237,9 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
     int* d_perm_local = cv.take<int>(N);
     uint32_t* d_qkey = cv.take<uint32_t>(Q);
     uint32_t* d_qkey_alt = cv.take<uint32_t>(Q);
-    const bool per_query = pairs_per_query(gp);
+    int* d_qval = cv.take<int>(Q);
+    int* d_qval_alt = cv.take<int>(Q);
+    float4* d_qrec = cv.take<float4>(Q);
     float4* d_slots = cv.take<float4>(Q);
     int2* d_units = cv.take<int2>(Q);
     int* d_ucount = cv.take<int>(4);
@@ -247,15 +249,6 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
     double* d_b = cv.take<double>(6 * K);
     double* d_F = cv.take<double>(1);
     long long* d_n = cv.take<long long>(1);
-    // query order and unsorted records; at last the dense kernel's per-query
-    // sums, in as many parts as the rest of the scratch holds
-    int part_max = part_max_for(gp, Q, num_sms);
-    const long long room = (long long)(SCRATCH_BYTES - cv.off) - 1024;
-    while (per_query && part_max > 0 && (40LL << part_max) * Q > room) --part_max;
-    const long long parts = per_query ? 1LL << part_max : 1;
-    int* d_qval = cv.take<int>(2 * Q * parts);
-    int* d_qval_alt = d_qval + Q;
-    float4* d_qrec = cv.take<float4>(per_query ? 2 * Q * parts : Q);
     if (!cv.ok) return fail(RKHSBA_EINVAL, "rkhsba_eval_static: problem does not fit the 32 MiB static scratch");
 
     SCK(cudaMemcpyAsync(d_frames, fh, sizeof(FrameDev) * K, cudaMemcpyHostToDevice, st));
@@ -297,14 +290,11 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
         a.acc = d_acc;
         a.units = d_units;
         a.n_units = d_ucount;
-        a.part_max = part_max;
+        a.part_max = part_max_for(gp, Q, num_sms);
         a.part_target = part_target_for(num_sms);
-        a.qs8 = per_query ? reinterpret_cast<float*>(d_qrec) : nullptr;
-        a.qs2 = per_query ? reinterpret_cast<float*>(d_qval) : nullptr;
         a.E = E;
         a.gp = gp;
         launch_pairs(PairLaunch{d_ucount + 1, nullptr, num_sms, 0, st}, a);
-        if (per_query) launch_query_moments(a, num_sms, nullptr, st);
     }
     launch_edge_assemble(d_edges, E, d_xf, d_acc, p.sigma * p.sigma, d_eout, nullptr, st);
     SCK(cudaMemsetAsync(d_H, 0, sizeof(double) * 36LL * K * K, st));

@@ -561,71 +561,59 @@ __device__ __forceinline__ void part_range(int C, int part, int shift, int& c0, 
     c1 = min(c0 + per, n);
 }
 
-// One step of the moment reduce-scatter: lanes whose bit `o` is clear keep
+// One step of the moment reduce-scatter: lanes whose bit N is clear keep
 // the lower half of their values, the others the upper half, and each adds
 // the half its partner sends.
 template <int N>
-__device__ __forceinline__ void reduce_half(long long (&v)[32], int lane) {
+__device__ __forceinline__ void reduce_half(float (&v)[32], int lane) {
     const bool up = (lane & N) != 0;
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-        const long long send = up ? v[k] : v[k + N];
-        const long long keep = up ? v[k + N] : v[k];
+        const float send = up ? v[k] : v[k + N];
+        const float keep = up ? v[k + N] : v[k];
         v[k] = keep + __shfl_xor_sync(FULL, send, N);
     }
 }
 
-// A lane's moments (frame-a coordinates) rounded to 64-bit fixed point,
-// reduce-scattered over the warp (lane k ends with the warp total of moment k)
-// and added to the edge's accumulators with one integer atomic per moment.
-__device__ __forceinline__ void add_moments(float W, const float (&Dv)[3], const float (&Sy)[3], const float (&Myy)[6],
-                                            const float (&Mdy)[9], const float* Qm, int cnt,
-                                            const float* __restrict__ scl, long long* __restrict__ acc_e, int lane) {
-    long long vals[32];
-#pragma unroll
-    for (int k = 0; k < 32; ++k) {
-        float val = 0.f;
-        if (k == 0) val = W;
-        else if (k < 4) val = Dv[k - 1];
-        else if (k < 7) val = Sy[k - 4];
-        else if (k < 13) val = Myy[k - 7];
-        else if (k < 22) val = Mdy[k - 13];
-        else if (k < 28) val = Qm[k - 22];
-        vals[k] = (k == N_MOM - 1) ? (long long)cnt
-                : (k < N_MOM ? to_fixed(val, __ldg(scl + moment_class(k))) : 0ll);
-    }
-    reduce_half<16>(vals, lane);
-    reduce_half<8>(vals, lane);
-    reduce_half<4>(vals, lane);
-    reduce_half<2>(vals, lane);
-    reduce_half<1>(vals, lane);
-    if (lane < N_MOM && vals[0] != 0)
-        atomicAdd(reinterpret_cast<unsigned long long*>(acc_e + lane), (unsigned long long)vals[0]);
-}
-
-// Unit end of the pair kernels that sum moments themselves: the lane's moments
-// about the home cell centre move to frame-a coordinates (y' += o) and are
-// added to the edge's.
-__device__ __forceinline__ void store_moments(float W, const float (&Dv)[3], float (&Sy)[3], float (&Myy)[6],
-                                              float (&Mdy)[9], const float* Qm, int cnt, const FrameDev& Fa,
+// Unit end, shared by the pair kernels: the lanes' moments about the home cell
+// centre are reduce-scattered over the warp (lane k ends with moment k, summed
+// in a fixed order), move to frame-a coordinates (y' += o), are rounded to 64-bit
+// fixed point and added to the edge's accumulators with one integer atomic per
+// moment.  What enters the accumulators depends on the unit alone, and their sums are
+// exact.  (Rounding all 28 moments of every lane first and reducing 64-bit
+// integers took four times the instructions, ~1000 a unit.)
+__device__ __forceinline__ void store_moments(float W, const float (&Dv)[3], const float (&Sy)[3], const float (&Myy)[6],
+                                              const float (&Mdy)[9], const float* Qm, int cnt, const FrameDev& Fa,
                                               int hx, int hy, int hz, const GridParams& gp,
                                               const float* __restrict__ scl, long long* __restrict__ acc_e,
                                               int lane) {
-    const float o[3] = {((float)(hx + Fa.lo[0]) + 0.5f) * gp.hf, ((float)(hy + Fa.lo[1]) + 0.5f) * gp.hf,
-                        ((float)(hz + Fa.lo[2]) + 0.5f) * gp.hf};
-    int t6 = 0;
+    float v[32];
 #pragma unroll
-    for (int mm = 0; mm < 3; ++mm)
-#pragma unroll
-        for (int l = mm; l < 3; ++l, ++t6)
-            Myy[t6] += Sy[mm] * o[l] + o[mm] * Sy[l] + W * o[mm] * o[l];
-#pragma unroll
-    for (int mm = 0; mm < 3; ++mm)
-#pragma unroll
-        for (int l = 0; l < 3; ++l) Mdy[3 * mm + l] = fmaf(Dv[mm], o[l], Mdy[3 * mm + l]);
-#pragma unroll
-    for (int mm = 0; mm < 3; ++mm) Sy[mm] = fmaf(W, o[mm], Sy[mm]);
-    add_moments(W, Dv, Sy, Myy, Mdy, Qm, cnt, scl, acc_e, lane);
+    for (int k = 0; k < 32; ++k)
+        v[k] = k == 0 ? W : k < 4 ? Dv[k - 1] : k < 7 ? Sy[k - 4] : k < 13 ? Myy[k - 7] : k < 22 ? Mdy[k - 13]
+             : k < 28 ? Qm[k - 22] : 0.f;
+    reduce_half<16>(v, lane);
+    reduce_half<8>(v, lane);
+    reduce_half<4>(v, lane);
+    reduce_half<2>(v, lane);
+    reduce_half<1>(v, lane);
+    cnt = __reduce_add_sync(FULL, cnt);
+    // rows m and columns l of the lane's moment: Sy (m), Myy and Mdy (m, l)
+    const bool in_sy = lane >= 4 && lane < 7, in_yy = lane >= 7 && lane < 13, in_dy = lane >= 13 && lane < 22;
+    const int q = lane - 13;
+    const int m = in_sy ? lane - 4 : in_yy ? (lane < 10 ? 0 : (lane < 12 ? 1 : 2)) : in_dy ? q / 3 : 0;
+    const int l = in_yy ? (lane < 10 ? lane - 7 : (lane < 12 ? lane - 9 : 2)) : in_dy ? q - 3 * m : 0;
+    const float o0 = ((float)(hx + Fa.lo[0]) + 0.5f) * gp.hf, o1 = ((float)(hy + Fa.lo[1]) + 0.5f) * gp.hf,
+                o2 = ((float)(hz + Fa.lo[2]) + 0.5f) * gp.hf;
+    const float om = m == 0 ? o0 : (m == 1 ? o1 : o2), ol = l == 0 ? o0 : (l == 1 ? o1 : o2);
+    const float w = __shfl_sync(FULL, v[0], 0), sm = __shfl_sync(FULL, v[0], 4 + m),
+                sl = __shfl_sync(FULL, v[0], 4 + l), dm = __shfl_sync(FULL, v[0], 1 + m);
+    float x = v[0];
+    if (in_sy) x = fmaf(w, om, x);
+    else if (in_yy) x += sm * ol + om * sl + w * om * ol;
+    else if (in_dy) x = fmaf(dm, ol, x);
+    const long long f = lane == N_MOM - 1 ? (long long)cnt : lane < N_MOM ? to_fixed(x, __ldg(scl + moment_class(lane))) : 0ll;
+    if (f != 0) atomicAdd(reinterpret_cast<unsigned long long*>(acc_e + lane), (unsigned long long)f);
 }
 
 // BF16 labels: the candidate x query label products of a batch come from the
@@ -734,7 +722,7 @@ __device__ __forceinline__ void label_gram_bf16(const unsigned* __restrict__ sem
 //   4. at the unit's end each lane takes one query and forms, with y = y_q,
 //      W = k, D = X1 - k y, sum w y = k y, sum w y y^T = k y y^T,
 //      sum w d y^T = D y^T and Q = X2 - X1 y^T - y X1^T + k y y^T, which
-//      enter the same fixed-point reduction as the bit-walk kernel.
+//      enter the same reduction as those of the bit-walk kernel.
 // Scaling: w is carried as w 2^KW with 2^KW |l|max^2 <= 2^14 and the
 // features as x 2^-EX with 2^EX >= h, so every FP16 operand stays inside
 // its range; both are powers of two and undone exactly at the unit's end.
@@ -1210,10 +1198,11 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int2 unit, in
         if (qcount > 16) batches(std::integral_constant<int, 2>{});
         else batches(std::integral_constant<int, 1>{});
     }
-    // unit end: the per-query sums as they are; k_query_moments forms the moments
-    const long long at = (PARTS ? A.Q * part : 0LL) + k0;
-    float* qs8 = A.qs8 + 8 * at;
-    float* qs2 = A.qs2 + 2 * at;
+    if (!__any_sync(FULL, cnt != 0)) return;     // no pair: every sum is zero
+    // unit end: the per-query sums through shared memory (the features' place)
+    // to one lane per query, formed into the lane's moments
+    float* sq = reinterpret_cast<float*>(cf);    // [32][12] (features 0..9 used)
+    __syncwarp();
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt) {
         float (&r1)[4] = run[mt][1];
@@ -1221,139 +1210,38 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int2 unit, in
         for (int k = 0; k < 4; ++k) r1[k] += __shfl_xor_sync(FULL, r1[k], 1);    // hi and lo parts of features 8, 9
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-            const int q = 16 * mt + 8 * i + g;
-            if (q < qcount) {
-                *reinterpret_cast<float2*>(qs8 + 8 * q + 2 * t4) = make_float2(run[mt][0][2 * i], run[mt][0][2 * i + 1]);
-                if (t4 == 0) *reinterpret_cast<float2*>(qs2 + 2 * q) = make_float2(r1[2 * i], r1[2 * i + 1]);
-            }
+            float* row = sq + 12 * (16 * mt + 8 * i + g);
+            *reinterpret_cast<float2*>(row + 2 * t4) = make_float2(run[mt][0][2 * i], run[mt][0][2 * i + 1]);
+            if (t4 == 0) *reinterpret_cast<float2*>(row + 8) = make_float2(r1[2 * i], r1[2 * i + 1]);
         }
     }
-    cnt = __reduce_add_sync(FULL, cnt);
-    if (lane == 0 && cnt > 0)
-        atomicAdd(reinterpret_cast<unsigned long long*>(A.acc + (long long)e * ACC_N + N_MOM - 1),
-                  (unsigned long long)cnt);
-}
-
-// Moments of the dense path, one query per lane: from the query's k, X1 and X2
-// (sum_c w (1, x, x x^T), powers of two undone exactly) and its place y it
-// forms, with o the home cell's centre,
-//   W = k, D = X1 - k y, sum w y', sum w y'y'^T, sum w d y'^T (y' = y + o)
-//   and Q = X2 - X1 y^T - y X1^T + k y y^T.
-// Each query's moments are rounded to the edge's fixed point on their own, so
-// that the integer sums do not depend on which queries share a lane or a warp
-// (an edge's results are the same whatever other edges there are); a lane adds
-// its queries of the `per` (<= MOM_PER) groups of 32 sorted queries that its warp
-// takes, and the warp reduces once per edge it meets.  As a pass of its own every
-// lane has a query, and the reduction is paid once per 256 queries; at the end of each
-// unit of the pair kernel both cost ~1000 instructions for (LiDAR scenes) 8
-// queries in the median.
-constexpr int MOM_PER = 8;
-__global__ void __launch_bounds__(128, 4) k_query_moments(const PairArgs A, int per, const int* done) {
-    if (done && *done) return;
-    const int lane = threadIdx.x & 31;
-    const GridParams& gp = A.gp;
-    const long long w0 = ((long long)blockIdx.x * 4 + (threadIdx.x >> 5)) * per * 32;
-    long long v[32];
+    __syncwarp();
+    const float4 r0 = *reinterpret_cast<const float4*>(sq + 12 * lane), r1 = *reinterpret_cast<const float4*>(sq + 12 * lane + 4);
+    const float2 r2 = *reinterpret_cast<const float2*>(sq + 12 * lane + 8);
+    const float4 yq = lane < qcount ? A.slots[(long long)k0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float s0 = ldexpf(1.f, -sc.kw), s1 = ldexpf(1.f, sc.ex - sc.kw), s2 = ldexpf(1.f, 2 * sc.ex - sc.kw);
+    const float y[3] = {yq.x, yq.y, yq.z};
+    const float W = r0.x * s0;
+    const float X1[3] = {r0.y * s1, r0.z * s1, r0.w * s1};
+    const float X2[6] = {r1.x * s2, r1.y * s2, r1.z * s2, r1.w * s2, r2.x * s2, r2.y * s2};
+    float Sy[3], D[3], Myy[6], Mdy[9], Q[6];
 #pragma unroll
-    for (int k = 0; k < 32; ++k) v[k] = 0;
-    // edge of the sums so far: its home-cell keys, scales and frame-a grid
-    int e_cur = -1, lo0 = 0, lo1 = 0, lo2 = 0, dim0 = 1, dim1 = 1;
-    long long bin_lo = 0, bin_hi = 0;
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-    const int parts = 1 << part_shift(A, *A.n_units);
-    float c0 = 0.f, c1 = 0.f, c2 = 0.f, c3 = 0.f, c4 = 0.f, c5 = 0.f;
-    auto flush = [&]() {
-        if (e_cur < 0) return;
-        reduce_half<16>(v, lane);
-        reduce_half<8>(v, lane);
-        reduce_half<4>(v, lane);
-        reduce_half<2>(v, lane);
-        reduce_half<1>(v, lane);
-        if (lane < N_MOM - 1 && v[0] != 0)
-            atomicAdd(reinterpret_cast<unsigned long long*>(A.acc + (long long)e_cur * ACC_N + lane),
-                      (unsigned long long)v[0]);
-#pragma unroll
-        for (int k = 0; k < 32; ++k) v[k] = 0;
-    };
-    for (int r = 0; r < per; ++r) {
-        const long long k = w0 + 32LL * r + lane;
-        const uint32_t kq = k < A.Q ? A.qkey[k] : NO_KEY;
-        const bool valid = kq != NO_KEY;
-        unsigned todo = __ballot_sync(FULL, valid);
-        if (!todo) break;                    // keys of no home cell sort last
-        const long long key = (long long)(kq >> gp.key_sub);
-        float4 q = make_float4(0.f, 0.f, 0.f, 0.f), f0 = q, f1 = q;
-        float2 f2v = make_float2(0.f, 0.f);
-        if (valid) {
-            q = A.slots[k];
-            const float4* p8 = reinterpret_cast<const float4*>(A.qs8) + 2 * k;
-            f0 = p8[0];
-            f1 = p8[1];
-            f2v = reinterpret_cast<const float2*>(A.qs2)[k];
-            for (int p = 1; p < parts; ++p) {
-                const float4 g0 = p8[2 * A.Q * p], g1 = p8[2 * A.Q * p + 1];
-                const float2 g2 = reinterpret_cast<const float2*>(A.qs2)[A.Q * p + k];
-                f0 = make_float4(f0.x + g0.x, f0.y + g0.y, f0.z + g0.z, f0.w + g0.w);
-                f1 = make_float4(f1.x + g1.x, f1.y + g1.y, f1.z + g1.z, f1.w + g1.w);
-                f2v = make_float2(f2v.x + g2.x, f2v.y + g2.y);
-            }
-        }
-        while (todo) {
-            const long long kl = __shfl_sync(FULL, key, __ffs(todo) - 1);
-            if (kl < bin_lo || kl >= bin_hi) {
-                flush();
-                e_cur = find_edge_bin(A.edges, A.E, kl);
-                const EdgeDev& Ed = A.edges[e_cur];
-                const FrameDev& Fa = A.frames[Ed.a];
-                lo0 = Fa.lo[0];
-                lo1 = Fa.lo[1];
-                lo2 = Fa.lo[2];
-                dim0 = Fa.dim[0];
-                dim1 = Fa.dim[1];
-                bin_lo = Ed.bin_off;
-                bin_hi = bin_lo + (long long)dim0 * dim1 * Fa.dim[2];
-                const DenseScales sc = dense_scales(Fa.sem_norm_max, A.frames[Ed.b].sem_norm_max, gp.hf, false);
-                s0 = ldexpf(1.f, -sc.kw);
-                s1 = ldexpf(1.f, sc.ex - sc.kw);
-                s2 = ldexpf(1.f, 2 * sc.ex - sc.kw);
-                c0 = Ed.scale[MC_W];
-                c1 = Ed.scale[MC_D];
-                c2 = Ed.scale[MC_SY];
-                c3 = Ed.scale[MC_MYY];
-                c4 = Ed.scale[MC_MDY];
-                c5 = Ed.scale[MC_Q];
-            }
-            const bool mine = valid && key >= bin_lo && key < bin_hi;
-            todo &= ~__ballot_sync(FULL, mine);
-            if (mine) {
-                const int cell = (int)(key - bin_lo);
-                const int row = cell / dim0, hx = cell - row * dim0, hz = row / dim1, hy = row - hz * dim1;
-                const float o[3] = {((float)(hx + lo0) + 0.5f) * gp.hf, ((float)(hy + lo1) + 0.5f) * gp.hf,
-                                    ((float)(hz + lo2) + 0.5f) * gp.hf};
-                const float y[3] = {q.x, q.y, q.z};
-                const float w = f0.x * s0;
-                const float X1[3] = {f0.y * s1, f0.z * s1, f0.w * s1};
-                const float X2[6] = {f1.x * s2, f1.y * s2, f1.z * s2, f1.w * s2, f2v.x * s2, f2v.y * s2};
-                v[0] += to_fixed(w, c0);
-                int t6 = 0;
-#pragma unroll
-                for (int m = 0; m < 3; ++m) {
-                    const float ky = w * y[m], d = X1[m] - ky;
-                    v[1 + m] += to_fixed(d, c1);
-                    v[4 + m] += to_fixed(fmaf(w, o[m], ky), c2);
-#pragma unroll
-                    for (int l = m; l < 3; ++l, ++t6) {
-                        const float kyy = ky * y[l], kyl = w * y[l];
-                        v[7 + t6] += to_fixed(kyy + (ky * o[l] + o[m] * kyl + w * o[m] * o[l]), c3);
-                        v[22 + t6] += to_fixed(X2[t6] - X1[m] * y[l] - y[m] * X1[l] + kyy, c5);
-                    }
-#pragma unroll
-                    for (int l = 0; l < 3; ++l) v[13 + 3 * m + l] += to_fixed(fmaf(d, o[l], d * y[l]), c4);
-                }
-            }
-        }
+    for (int m = 0; m < 3; ++m) {
+        Sy[m] = W * y[m];
+        D[m] = X1[m] - Sy[m];
     }
-    flush();
+    int t6 = 0;
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+#pragma unroll
+        for (int l = m; l < 3; ++l, ++t6) {
+            Myy[t6] = Sy[m] * y[l];
+            Q[t6] = X2[t6] - X1[m] * y[l] - y[m] * X1[l] + Myy[t6];
+        }
+#pragma unroll
+        for (int l = 0; l < 3; ++l) Mdy[3 * m + l] = D[m] * y[l];
+    }
+    store_moments(W, D, Sy, Myy, Mdy, Q, cnt, Fa, hx, hy, hz, gp, A.edges[e].scale, A.acc + (long long)e * ACC_N, lane);
 }
 
 // One unit (queries of one frame-a home cell) of the pair sum: stage the queries, stream the candidates of the
@@ -2154,19 +2042,6 @@ struct MultiLaunch {
 }  // namespace
 
 int pair_unit_max(const GridParams& gp) { return (dense_path(gp) && gp.sem_bf16) ? 64 : UQ; }
-
-bool pairs_per_query(const GridParams& gp) { return dense_path(gp); }
-
-void launch_query_moments(const PairArgs& A, int num_sms, const int* done, cudaStream_t st) {
-    if (A.Q <= 0) return;
-    // groups of 32 queries per warp: as many as leave a few warps for every
-    // scheduler
-    const long long groups = (A.Q + 31) / 32;
-    int per = (int)(groups / (16LL * num_sms));
-    per = per < 1 ? 1 : (per > MOM_PER ? MOM_PER : per);
-    k_query_moments<<<blocks_for((groups + per - 1) / per, 4), 128, 0, st>>>(A, per, done);
-    count_launch();
-}
 
 void launch_pairs(const PairLaunch& L, const PairArgs& A) {
     if (A.Q <= 0) return;

@@ -103,9 +103,7 @@ size_t estimate_bytes(const Req& r) {
     for (int m = 0; m < r.K; ++m) C += cells[m];
     for (int e = 0; e < r.E; ++e) Q += (double)r.n[std::max(r.edges[2 * e], r.edges[2 * e + 1])];
     const double D = r.p.sem_dim;
-    // small problems may keep up to 8 parts of 40 bytes of sums per query
-    const double per_q = 80 + (Q <= 160000.0 && D > 0 ? 40 * 7 : 0);
-    const double bytes = N * (24 + 8 * D + 16 + 16 + 40 + 12) + Q * per_q + C * 4 +
+    const double bytes = N * (24 + 8 * D + 16 + 16 + 40 + 12) + Q * 68 + C * 4 +
                          (double)r.K * r.K * 36 * 8 * 2 + (double)r.E * 1600 + (4 << 20);
     return (size_t)(bytes * 1.25);
 }
