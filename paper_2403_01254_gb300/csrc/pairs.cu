@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(256) k_units(const uint32_t* __restrict__ key,
                 __syncthreads();
                 if (found) break;
             }
-            from = s_start;
+            from = max(s_start, 0);      // none found: the cell starts at the first query of all
         }
         const long long run = start >= 0 ? base + start : from;
         const bool st = valid && ((k - run) % uq) == 0;

@@ -1,0 +1,77 @@
+"""Binning of the queries and cutting into units, at the sizes where they change course.
+
+Cells of more queries than a block of the unit pass takes (256), whose first
+query is or is not the first of all; streams long enough to be shared by several
+warps; and query counts around the sort's tiles of 2048.  Tolerances are those of
+the parity tests (loss 1e-5, gradient and Gauss-Newton matrix 1e-4 relative); in
+the clumps every pair lies inside the cutoff, so their counts are exact.
+"""
+import numpy as np
+import pytest
+
+import oracle as O
+import scenes
+
+pytestmark = pytest.mark.gpu
+
+LOSS_TOL, GRAD_TOL, H_TOL = 1e-5, 1e-4, 1e-4
+
+
+@pytest.fixture(scope="module")
+def pk():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2403_01254_gb300 as pk
+    pk.load()
+    return pk
+
+
+def _reln(a, b):
+    return float(np.linalg.norm(np.asarray(a) - np.asarray(b)) / max(np.linalg.norm(b), 1e-300))
+
+
+def _check(pk, prob, exact_count=None):
+    ref = O.evaluate(prob, prob["poses0"])
+    g = pk.Problem.from_scene(prob)
+    try:
+        out = g.eval(prob["poses0"])
+    finally:
+        g.close()
+    if exact_count is not None:
+        assert out["edge_pairs"].tolist() == exact_count
+    assert np.abs(out["edge_pairs"] - ref["edge_pairs"]).sum() <= 3
+    assert abs(out["loss"] - ref["loss"]) <= LOSS_TOL * abs(ref["loss"])
+    assert _reln(out["grad"], ref["grad"]) <= GRAD_TOL
+    assert _reln(out["H"], ref["H"]) <= H_TOL
+
+
+def _clump(n, lead, variant):
+    """n points of each frame inside one cell; `lead` lone points of frame b in cells before it."""
+    rng = np.random.default_rng(1000 * n + lead)
+    prob = scenes.tiny_problem(seed=9, n_frames=2, n=8, extent=1.0, ell=0.15, color=variant == "color")
+    lone = np.array([[-2.0 - 0.5 * k, 0.2, 0.2] for k in range(lead)]).reshape(lead, 3)
+    box = [0.12 + 0.2 * rng.random((n, 3)) for _ in range(2)]
+    m = n + lead
+    prob["xyz"] = [np.concatenate([lone + [0.0, 9.0, 0.0], box[0]]), np.concatenate([lone, box[1]])]
+    prob["poses0"] = np.stack([np.eye(4), scenes.make_pose(
+        scenes.rot_from_axis_angle(np.array([0.0, 0.0, 1.0]), 0.05), np.array([0.01, -0.01, 0.005]))])
+    prob["edges"] = np.array([[0, 1]], np.int32)
+    prob["rgb"] = [rng.random((m, 3)) for _ in range(2)] if variant == "color" else None
+    sem = [scenes.dirichlet_labels(rng, rng.integers(0, 4, m), 4) for _ in range(2)]
+    prob["sem"] = None if variant == "plain" else sem
+    if variant == "bf16":
+        prob["sem"] = [scenes.round_to_bf16(s) for s in sem]
+        prob["params"] = dict(prob["params"], sem_bf16=1)
+    return prob
+
+
+@pytest.mark.parametrize("variant", ["plain", "fp32", "bf16", "color"])
+@pytest.mark.parametrize("n,lead", [(1, 0), (255, 0), (256, 1), (257, 0), (513, 0), (700, 5), (1025, 0)])
+def test_cells_longer_than_a_block(pk, variant, n, lead):
+    _check(pk, _clump(n, lead, variant), exact_count=[n * n])
+
+
+@pytest.mark.parametrize("n", [2047, 2048, 2049, 4097])
+def test_query_counts_around_a_sort_tile(pk, n):
+    _check(pk, scenes.tiny_problem(seed=40 + n % 7, n_frames=2, n=n, extent=2.5, ell=0.1))
