@@ -246,6 +246,7 @@ rkhsba_status build(rkhsba_ctx* c, const double* xyz, const float* sem, const fl
     layout_edges(c->edges_h.data(), E, c->frames_h.data(), c->gp, rc, &c->total_bins, &c->Q_total);
     if (c->total_bins >= (1LL << 31) - 2) return fail(c, RKHSBA_EINVAL, "total home cells exceed 2^31");
     if (c->Q_total >= (1LL << 31) - 64) return fail(c, RKHSBA_EINVAL, "more than 2^31 queries over all edges");
+    c->q_max = edge_queries_max(c->edges_h.data(), E, c->frames_h.data());
     c->qbits = 1;
     while ((1LL << c->qbits) <= c->total_bins) ++c->qbits;   // invalid key sorts last
     // three more key bits order a home cell's queries by octant, when they fit
@@ -309,6 +310,13 @@ rkhsba_status build(rkhsba_ctx* c, const double* xyz, const float* sem, const fl
 // sorted home-cell keys, sorted query records and the unit list.
 void run_binning(rkhsba_ctx* c, const double* poses, const int* done) {
     cudaStream_t st = c->stream;
+    if (c->q_max <= BIN_MAX) {
+        launch_bin_edges(BinArgs{poses, c->d_edges, c->E, c->d_frames, c->d_pt_cell, c->d_pts4, c->gp, c->tune_uq, c->d_xf,
+                                 c->d_qkey, c->d_qrec, c->d_slots, c->d_units, c->d_ucount, c->d_acc, done},
+                         c->q_max, st);
+        c->q_sorted_key = c->d_qkey;
+        return;
+    }
     const RadixWs ws = radix_ws(c->Q_total, c->qbits, c->d_qhist, c->d_scan_ws);
     launch_eval_setup(poses, c->d_edges, c->E, c->d_frames, c->gp.h, c->d_xf, c->d_scan_ws,
                       (int)scan_ws_elems(c->Q_total), c->d_ucount, c->d_acc, done, st);

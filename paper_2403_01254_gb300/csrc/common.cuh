@@ -201,6 +201,29 @@ void launch_gather(const double* xyz, const float* sem, const float* rgb, long l
 // pairs.cu
 void launch_eval_setup(const double* poses, const EdgeDev* edges, int E, const FrameDev* frames, double h, EdgeXf* xf,
                        long long* ws, int n_ws, int* ucount, long long* acc, const int* done, cudaStream_t st);
+// Binning of problems whose edges have at most BIN_MAX queries each: everything
+// that launch_eval_setup, launch_query_keys, the sort and launch_units do, with a
+// block per edge.  q_max: queries of the largest edge.
+constexpr int BIN_MAX = 4096;
+struct BinArgs {
+    const double* poses;
+    const EdgeDev* edges;
+    int E;
+    const FrameDev* frames;
+    const uint32_t* pt_cell;
+    const float4* pts4;
+    GridParams gp;
+    int uq;
+    EdgeXf* xf;
+    uint32_t* qkey;           // sorted home-cell keys, edge by edge
+    float4* qrec;             // scratch: records in query order
+    float4* slots;            // the same in sorted order
+    int2* units;
+    int* ucount;              // [4], cleared first; [0]: number of units
+    long long* acc;
+    const int* done;
+};
+void launch_bin_edges(const BinArgs& a, int q_max, cudaStream_t st);
 void launch_query_keys(const EdgeDev* edges, int E, const FrameDev* frames, const EdgeXf* xf,
                        const uint32_t* pt_cell, const float4* pts4, GridParams gp, long long Q,
                        uint32_t* qkey, float4* qrec, const RadixWs& ws, int num_sms, const int* done, cudaStream_t st);

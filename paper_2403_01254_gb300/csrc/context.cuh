@@ -64,6 +64,7 @@ struct rkhsba_ctx {
     long long* d_scan_ws = nullptr;
 
     long long total_bins = 0, Q_total = 0;
+    int q_max = 0;                     // queries of the largest edge
     int qbits = 0;                     // radix bits of the query keys
     EdgeXf* d_xf = nullptr;
     uint32_t* d_qkey = nullptr;        // home-cell key per query (then sorted)

@@ -148,6 +148,14 @@ inline void layout_edges(EdgeDev* eh, int E, const FrameDev* fh, const GridParam
     *total_q = q;
 }
 
+// Queries of the largest edge.
+inline int edge_queries_max(const EdgeDev* eh, int E, const FrameDev* fh) {
+    int m = 0;
+    for (int e = 0; e < E; ++e)
+        if (fh[eh[e].b].n_pts > m) m = fh[eh[e].b].n_pts;
+    return m;
+}
+
 // Frame -> edge incidence in edge order: frame m's entries are 2e when m is
 // edge e's first frame and 2e + 1 when it is the second.  inc_off [K + 1],
 // inc_list [2 E]; returns the number of entries.

@@ -269,13 +269,21 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
                   gp, C, d_pts4, d_sem_sorted, d_col4, d_perm_local, d_cell_start, st);
 
     // ---- evaluation ----
-    const RadixWs qws = radix_ws(Q, qbits, d_hist, d_ws);
-    launch_eval_setup(d_poses, d_edges, E, d_frames, gp.h, d_xf, d_ws, (int)scan_ws_elems(Q), d_ucount, d_acc, nullptr, st);
-    launch_query_keys(d_edges, E, d_frames, d_xf, pt_cell, d_pts4, gp, Q, d_qkey, d_qrec, qws, num_sms, nullptr, st);
-    const bool qalt = radix_sort_u32(d_qkey, d_qval, d_qkey_alt, d_qval_alt, Q, qws, d_err + 1, nullptr, st);
-    const uint32_t* qk = qalt ? d_qkey_alt : d_qkey;
-    launch_units(qk, qalt ? d_qval_alt : d_qval, d_qrec, Q, UNIT_Q, gp.key_sub, d_edges, E, d_slots, d_units,
-                 d_ucount, nullptr, st);
+    const int q_max = edge_queries_max(eh, E, fh);
+    const uint32_t* qk = d_qkey;
+    if (q_max <= BIN_MAX) {
+        launch_bin_edges(BinArgs{d_poses, d_edges, E, d_frames, pt_cell, d_pts4, gp, UNIT_Q, d_xf, d_qkey, d_qrec, d_slots,
+                                 d_units, d_ucount, d_acc, nullptr},
+                         q_max, st);
+    } else {
+        const RadixWs qws = radix_ws(Q, qbits, d_hist, d_ws);
+        launch_eval_setup(d_poses, d_edges, E, d_frames, gp.h, d_xf, d_ws, (int)scan_ws_elems(Q), d_ucount, d_acc, nullptr, st);
+        launch_query_keys(d_edges, E, d_frames, d_xf, pt_cell, d_pts4, gp, Q, d_qkey, d_qrec, qws, num_sms, nullptr, st);
+        const bool qalt = radix_sort_u32(d_qkey, d_qval, d_qkey_alt, d_qval_alt, Q, qws, d_err + 1, nullptr, st);
+        qk = qalt ? d_qkey_alt : d_qkey;
+        launch_units(qk, qalt ? d_qval_alt : d_qval, d_qrec, Q, UNIT_Q, gp.key_sub, d_edges, E, d_slots, d_units,
+                     d_ucount, nullptr, st);
+    }
     {
         PairArgs a{};
         a.qkey = qk;

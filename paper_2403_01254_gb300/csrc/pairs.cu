@@ -62,6 +62,38 @@ __device__ __forceinline__ df df_mul_f(float hi, float lo, float c) {
     return fast_two_sum(p, fmaf(lo, c, e));
 }
 
+// One edge's transform and its map of cell centres, by one warp: nine lanes an
+// entry of R_ab each, three an entry of t_ab.
+__device__ __forceinline__ void edge_transform(const double* __restrict__ poses, const EdgeDev& Ed, const FrameDev& Fb,
+                                               double h, EdgeXf& X, int lane) {
+    const double* Ta = poses + 16 * Ed.a;
+    const double* Tb = poses + 16 * Ed.b;
+    // R_ab = R_a^T R_b (lane 3 r + c: entry (r, c)),  t_ab = R_a^T (t_b - t_a) (lanes 9..11)
+    const int r = lane < 9 ? lane / 3 : lane - 9, c = lane % 3;
+    double v = 0.0, prod = 0.0;
+    if (lane < 9) {
+        for (int k = 0; k < 3; ++k) v += Ta[4 * k + r] * Tb[4 * k + c];
+        X.R[lane] = v;
+        X.Rf[lane] = (float)v;
+        // P(l) = h R l + [R (lo_b + 1/2) h + t]
+        const double A = h * v;
+        X.Ahi[lane] = (float)A;
+        X.Alo[lane] = (float)(A - (double)(float)A);
+        prod = v * ((double)Fb.lo[c] + 0.5) * h;
+    } else if (lane < 12) {
+        v = Ta[r] * (Tb[3] - Ta[3]) + Ta[4 + r] * (Tb[7] - Ta[7]) + Ta[8 + r] * (Tb[11] - Ta[11]);
+        X.t[r] = v;
+    }
+    const int src = lane >= 9 && lane < 12 ? 3 * r : 0;
+    const double p0 = __shfl_sync(FULL, prod, src), p1 = __shfl_sync(FULL, prod, src + 1),
+                 p2 = __shfl_sync(FULL, prod, src + 2);
+    if (lane >= 9 && lane < 12) {
+        const double B = v + p0 + p1 + p2;
+        X.Bhi[r] = (float)B;
+        X.Blo[r] = (float)(B - (double)(float)B);
+    }
+}
+
 // Start of an evaluation: the edges' transforms, one warp per edge (nine lanes
 // an entry of R_ab each: FP64 chains of a few operations instead of the ~100 of
 // one thread per edge, 8.4 us at 28 edges), and everything cleared that the
@@ -79,34 +111,7 @@ __global__ void __launch_bounds__(128) k_eval_setup(const double* __restrict__ p
     if (gt < 4) ucount[gt] = 0;
     const int lane = threadIdx.x & 31;
     for (int e = gt >> 5; e < E; e += nt >> 5) {
-        const double* Ta = poses + 16 * edges[e].a;
-        const double* Tb = poses + 16 * edges[e].b;
-        const FrameDev& Fb = frames[edges[e].b];
-        EdgeXf& X = xf[e];
-        // R_ab = R_a^T R_b (lane 3 r + c: entry (r, c)),  t_ab = R_a^T (t_b - t_a) (lanes 9..11)
-        const int r = lane < 9 ? lane / 3 : lane - 9, c = lane % 3;
-        double v = 0.0, prod = 0.0;
-        if (lane < 9) {
-            for (int k = 0; k < 3; ++k) v += Ta[4 * k + r] * Tb[4 * k + c];
-            X.R[lane] = v;
-            X.Rf[lane] = (float)v;
-            // P(l) = h R l + [R (lo_b + 1/2) h + t]
-            const double A = h * v;
-            X.Ahi[lane] = (float)A;
-            X.Alo[lane] = (float)(A - (double)(float)A);
-            prod = v * ((double)Fb.lo[c] + 0.5) * h;
-        } else if (lane < 12) {
-            v = Ta[r] * (Tb[3] - Ta[3]) + Ta[4 + r] * (Tb[7] - Ta[7]) + Ta[8 + r] * (Tb[11] - Ta[11]);
-            X.t[r] = v;
-        }
-        const int src = lane >= 9 && lane < 12 ? 3 * r : 0;
-        const double p0 = __shfl_sync(FULL, prod, src), p1 = __shfl_sync(FULL, prod, src + 1),
-                     p2 = __shfl_sync(FULL, prod, src + 2);
-        if (lane >= 9 && lane < 12) {
-            const double B = v + p0 + p1 + p2;
-            X.Bhi[r] = (float)B;
-            X.Blo[r] = (float)(B - (double)(float)B);
-        }
+        edge_transform(poses, edges[e], frames[edges[e].b], h, xf[e], lane);
     }
 }
 
@@ -126,6 +131,50 @@ __device__ __forceinline__ int find_edge_bin(const EdgeDev* __restrict__ edges, 
         if (edges[mid].bin_off <= bin) lo = mid; else hi = mid - 1;
     }
     return lo;
+}
+
+// Home cell of one query among frame a's cells (NO_KEY: outside the grid) and
+// its record, the FP32 offset from that cell's centre.  p: the point, relative to
+// the centre of its own cell l of frame b; s: its index.
+__device__ __forceinline__ uint32_t query_key(const FrameDev& Fa, const FrameDev& Fb, const EdgeXf& X, int l,
+                                              const float4 p, int s, const GridParams& gp, float4& rec) {
+    const float lf[3] = {(float)(l % Fb.dim[0]), (float)((l / Fb.dim[0]) % Fb.dim[1]),
+                         (float)(l / (Fb.dim[0] * Fb.dim[1]))};
+    float K[3], F[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        df P = {X.Bhi[r], X.Blo[r]};
+#pragma unroll
+        for (int c = 0; c < 3; ++c) P = df_add(P, df_mul_f(X.Ahi[3 * r + c], X.Alo[3 * r + c], lf[c]));
+        float k = floorf(P.hi * gp.hf_inv);
+        k = fminf(fmaxf(k, -4194304.f), 4194304.f);
+        df C = df_mul_f(gp.hf, gp.hf_lo, k + 0.5f);
+        df Rm = df_add(P, {-C.hi, -C.lo});
+        float f = Rm.hi + Rm.lo;
+        if (f < -0.5f * gp.hf) { k -= 1.f; C = df_mul_f(gp.hf, gp.hf_lo, k + 0.5f);
+                                 Rm = df_add(P, {-C.hi, -C.lo}); f = Rm.hi + Rm.lo; }
+        else if (f >= 0.5f * gp.hf) { k += 1.f; C = df_mul_f(gp.hf, gp.hf_lo, k + 0.5f);
+                                      Rm = df_add(P, {-C.hi, -C.lo}); f = Rm.hi + Rm.lo; }
+        K[r] = k;
+        F[r] = f;
+    }
+    const float* R = X.Rf;
+    const float vx = fmaf(R[2], p.z, fmaf(R[1], p.y, fmaf(R[0], p.x, F[0])));
+    const float vy = fmaf(R[5], p.z, fmaf(R[4], p.y, fmaf(R[3], p.x, F[1])));
+    const float vz = fmaf(R[8], p.z, fmaf(R[7], p.y, fmaf(R[6], p.x, F[2])));
+    const float mx = floorf(fmaf(vx, gp.hf_inv, 0.5f));
+    const float my = floorf(fmaf(vy, gp.hf_inv, 0.5f));
+    const float mz = floorf(fmaf(vz, gp.hf_inv, 0.5f));
+    const int hx = (int)(K[0] + mx) - Fa.lo[0];
+    const int hy = (int)(K[1] + my) - Fa.lo[1];
+    const int hz = (int)(K[2] + mz) - Fa.lo[2];
+    const float ox = fmaf(-mx, gp.hf, vx), oy = fmaf(-my, gp.hf, vy), oz = fmaf(-mz, gp.hf, vz);
+    rec = make_float4(ox, oy, oz, __int_as_float(s));
+    if (hx < 0 || hy < 0 || hz < 0 || hx >= Fa.dim[0] || hy >= Fa.dim[1] || hz >= Fa.dim[2]) return NO_KEY;
+    const uint32_t cell = (uint32_t)(((long long)hz * Fa.dim[1] + hy) * Fa.dim[0] + hx);
+    // with key_sub = 3 the low bits hold the query's octant of its home
+    // cell, so a cell's queries sort by octant and a unit's are close
+    return gp.key_sub ? (cell << 3) | (ox >= 0.f ? 1u : 0u) | (oy >= 0.f ? 2u : 0u) | (oz >= 0.f ? 4u : 0u) : cell;
 }
 
 // One thread per query: frame-a home cell key and the query's FP32 offset
@@ -151,49 +200,9 @@ __global__ void __launch_bounds__(RAD_T) k_query_keys(const EdgeDev* __restrict_
         const FrameDev& Fa = frames[Ed.a];
         const FrameDev& Fb = frames[Ed.b];
         const int s = (int)(Fb.pt_off + (q - Ed.q_off));
-        const int l = (int)((long long)pt_cell[s] - Fb.cell_off);
-        const float lf[3] = {(float)(l % Fb.dim[0]), (float)((l / Fb.dim[0]) % Fb.dim[1]),
-                             (float)(l / (Fb.dim[0] * Fb.dim[1]))};
-        const EdgeXf& X = xf[e];
-        float K[3], F[3];
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-            df P = {X.Bhi[r], X.Blo[r]};
-#pragma unroll
-            for (int c = 0; c < 3; ++c) P = df_add(P, df_mul_f(X.Ahi[3 * r + c], X.Alo[3 * r + c], lf[c]));
-            float k = floorf(P.hi * gp.hf_inv);
-            k = fminf(fmaxf(k, -4194304.f), 4194304.f);
-            df C = df_mul_f(gp.hf, gp.hf_lo, k + 0.5f);
-            df Rm = df_add(P, {-C.hi, -C.lo});
-            float f = Rm.hi + Rm.lo;
-            if (f < -0.5f * gp.hf) { k -= 1.f; C = df_mul_f(gp.hf, gp.hf_lo, k + 0.5f);
-                                     Rm = df_add(P, {-C.hi, -C.lo}); f = Rm.hi + Rm.lo; }
-            else if (f >= 0.5f * gp.hf) { k += 1.f; C = df_mul_f(gp.hf, gp.hf_lo, k + 0.5f);
-                                          Rm = df_add(P, {-C.hi, -C.lo}); f = Rm.hi + Rm.lo; }
-            K[r] = k;
-            F[r] = f;
-        }
-        const float4 p = pts4[s];
-        const float* R = X.Rf;
-        const float vx = fmaf(R[2], p.z, fmaf(R[1], p.y, fmaf(R[0], p.x, F[0])));
-        const float vy = fmaf(R[5], p.z, fmaf(R[4], p.y, fmaf(R[3], p.x, F[1])));
-        const float vz = fmaf(R[8], p.z, fmaf(R[7], p.y, fmaf(R[6], p.x, F[2])));
-        const float mx = floorf(fmaf(vx, gp.hf_inv, 0.5f));
-        const float my = floorf(fmaf(vy, gp.hf_inv, 0.5f));
-        const float mz = floorf(fmaf(vz, gp.hf_inv, 0.5f));
-        const int hx = (int)(K[0] + mx) - Fa.lo[0];
-        const int hy = (int)(K[1] + my) - Fa.lo[1];
-        const int hz = (int)(K[2] + mz) - Fa.lo[2];
-        const float ox = fmaf(-mx, gp.hf, vx), oy = fmaf(-my, gp.hf, vy), oz = fmaf(-mz, gp.hf, vz);
-        if (hx >= 0 && hy >= 0 && hz >= 0 && hx < Fa.dim[0] && hy < Fa.dim[1] && hz < Fa.dim[2]) {
-            key = (uint32_t)(Ed.bin_off + ((long long)hz * Fa.dim[1] + hy) * Fa.dim[0] + hx);
-            // with key_sub = 3 the low bits hold the query's octant of its home
-            // cell, so a cell's queries sort by octant and a unit's are close
-            if (gp.key_sub)
-                key = (key << 3) | (ox >= 0.f ? 1u : 0u) | (oy >= 0.f ? 2u : 0u) | (oz >= 0.f ? 4u : 0u);
-        }
+        const uint32_t local = query_key(Fa, Fb, xf[e], (int)((long long)pt_cell[s] - Fb.cell_off), pts4[s], s, gp, qrec[q]);
+        if (local != NO_KEY) key = (uint32_t)(Ed.bin_off << gp.key_sub) + local;
         qkey[q] = key;
-        qrec[q] = make_float4(ox, oy, oz, __int_as_float(s));
         }
         radix_count(key, q < Q, ws.npass, hist);
     }
@@ -274,6 +283,228 @@ __global__ void __launch_bounds__(256) k_units(const uint32_t* __restrict__ key,
                 make_int2((int)k, (find_edge_bin(edges, E, kk >> sub) << 7) | lo);
         }
         __syncthreads();
+    }
+}
+
+// ------------------------------------------------ binning by one block ----
+// Problems whose edges have few queries (<= BIN_MAX each) are binned by one block per
+// edge in one launch: transform, keys, the sort (in shared memory; edges' keys
+// are apart, so sorting every edge by itself sorts them all, but for the queries
+// of no home cell, which end their edge instead of the list), sorted records and
+// units.  The chain of setup, keys, a kernel per 8-bit digit and the unit pass is
+// bound by its 6 or 7 launches and the look-back between tiles: 2 x 2000 points, one
+// evaluation 138 -> 119 us and one LM iteration 89 -> 84 us (this kernel 18 us, bound by the
+// latency of its barriers and digit ranking), 60-rotation search of 2 x 4000 1283 ->
+// 1250 us.  At 5003 queries per edge it takes as long as the chain (28 us: one SM's
+// issue rate), at 8000 longer (39 us), so edges end at BIN_MAX.
+constexpr int BIN_T = 1024;
+constexpr int BIN_W = BIN_T / 32;
+
+template <int IPT>
+struct BinSmem {
+    static constexpr int CAP = BIN_T * IPT;
+    static constexpr size_t KEY = 0;                                     // [CAP] uint32
+    static constexpr size_t VAL = KEY + 4 * CAP;                         // [CAP] uint16
+    static constexpr size_t CNT = VAL + 2 * CAP;                         // [BIN_W][256] uint16
+    static constexpr size_t BYTES = CNT + 2 * BIN_W * 256;
+};
+
+template <int IPT>
+__global__ void __launch_bounds__(BIN_T) k_bin_edges(const double* __restrict__ poses, const EdgeDev* __restrict__ edges,
+                                                     const FrameDev* __restrict__ frames,
+                                                     const uint32_t* __restrict__ pt_cell,
+                                                     const float4* __restrict__ pts4, GridParams gp, int uq,
+                                                     EdgeXf* __restrict__ xf, uint32_t* qkey, float4* qrec,
+                                                     float4* slots, int2* units, int* n_units,
+                                                     long long* __restrict__ acc, const int* done) {
+    if (done && *done) return;
+    using L = BinSmem<IPT>;
+    extern __shared__ float4 smem4[];
+    unsigned char* sm = reinterpret_cast<unsigned char*>(smem4);
+    uint32_t* s_key = reinterpret_cast<uint32_t*>(sm + L::KEY);
+    uint16_t* s_val = reinterpret_cast<uint16_t*>(sm + L::VAL);
+    uint16_t(*cnt)[256] = reinterpret_cast<uint16_t(*)[256]>(sm + L::CNT);
+    __shared__ EdgeXf X;
+    __shared__ int s_part[4][256], s_off[4][256], s_sum[BIN_W], s_first[BIN_W], s_base;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    const int e = blockIdx.x;
+    const EdgeDev& Ed = edges[e];
+    const FrameDev& Fa = frames[Ed.a];
+    const FrameDev& Fb = frames[Ed.b];
+    const int n = Fb.n_pts;
+    if (warp == 0) edge_transform(poses, Ed, Fb, gp.h, X, lane);
+    else if (warp == 1) acc[(long long)e * ACC_N + lane] = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) reinterpret_cast<uint32_t*>(cnt[warp])[lane + 32 * j] = 0u;
+    __syncthreads();
+    {
+        const uint32_t* src = reinterpret_cast<const uint32_t*>(&X);
+        uint32_t* dst = reinterpret_cast<uint32_t*>(xf + e);
+        for (int i = tid; i < (int)(sizeof(EdgeXf) / 4); i += BIN_T) dst[i] = src[i];
+    }
+    // a warp's queries are one run of the edge's
+    const int at0 = warp * (32 * IPT) + lane;
+    uint32_t key[IPT];
+    int val[IPT];
+#pragma unroll
+    for (int r = 0; r < IPT; ++r) {
+        const int i = at0 + 32 * r;
+        key[r] = NO_KEY;
+        val[r] = i;
+        if (i < n) {
+            const int s = (int)Fb.pt_off + i;
+            key[r] = query_key(Fa, Fb, X, (int)((long long)pt_cell[s] - Fb.cell_off), pts4[s], s, gp,
+                               qrec[Ed.q_off + i]);
+        }
+    }
+    // stable sort by 8-bit digits; bits such that NO_KEY's lie above every cell's
+    const long long top = ((long long)Fa.dim[0] * Fa.dim[1] * Fa.dim[2]) << gp.key_sub;
+    int bits = 1;
+    while ((1LL << bits) <= top) ++bits;
+    for (int shift = 0; shift < bits; shift += 8) {
+        int rank[IPT];
+#pragma unroll
+        for (int r = 0; r < IPT; ++r) {
+            const bool valid = at0 + 32 * r < n;
+            const int d = valid ? (int)((key[r] >> shift) & 255u) : 256;
+            const unsigned peers = __match_any_sync(FULL, d);
+            const int leader = __ffs(peers) - 1;
+            int old = 0;
+            if (valid && lane == leader) {
+                old = cnt[warp][d];
+                cnt[warp][d] = (uint16_t)(old + __popc(peers));
+            }
+            rank[r] = __shfl_sync(FULL, old, leader) + __popc(peers & lt);
+            __syncwarp();
+        }
+        __syncthreads();
+        // exclusive sums over the warps, a quarter of them per group of 256 threads, then over the digits
+        {
+            const int d = tid & 255, q = tid >> 8;
+            int sum = 0;
+#pragma unroll
+            for (int w = 0; w < BIN_W / 4; ++w) {
+                const int c = cnt[q * (BIN_W / 4) + w][d];
+                cnt[q * (BIN_W / 4) + w][d] = (uint16_t)sum;
+                sum += c;
+            }
+            s_part[q][d] = sum;
+        }
+        __syncthreads();
+        int tot = 0, inc = 0;
+        if (tid < 256) {
+            tot = s_part[0][tid] + s_part[1][tid] + s_part[2][tid] + s_part[3][tid];
+            inc = tot;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(FULL, inc, o);
+                if (lane >= o) inc += u;
+            }
+            if (lane == 31) s_sum[warp] = inc;
+        }
+        __syncthreads();
+        if (tid < 256) {
+            int base = inc - tot;
+            for (int w = 0; w < warp; ++w) base += s_sum[w];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                s_off[q][tid] = base;
+                base += s_part[q][tid];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < IPT; ++r) {
+            if (at0 + 32 * r < n) {
+                const int d = (int)((key[r] >> shift) & 255u);
+                const int at = s_off[warp / (BIN_W / 4)][d] + cnt[warp][d] + rank[r];
+                s_key[at] = key[r];
+                s_val[at] = (uint16_t)val[r];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < IPT; ++r) {
+            const int i = at0 + 32 * r;
+            if (i < n) {
+                key[r] = s_key[i];
+                val[r] = s_val[i];
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) reinterpret_cast<uint32_t*>(cnt[warp])[lane + 32 * j] = 0u;
+        __syncwarp();
+    }
+    // sorted keys and records, and the last cell head at or before each query
+    const uint32_t bin0 = (uint32_t)(Ed.bin_off << gp.key_sub);
+    int start[IPT], carry = -1;
+#pragma unroll
+    for (int r = 0; r < IPT; ++r) {
+        const int i = at0 + 32 * r;
+        bool head = false;
+        if (i < n) {
+            const long long q = Ed.q_off + i;
+            slots[q] = qrec[Ed.q_off + val[r]];
+            qkey[q] = key[r] == NO_KEY ? NO_KEY : bin0 + key[r];
+            head = i == 0 || (s_key[i - 1] >> gp.key_sub) != (key[r] >> gp.key_sub);
+        }
+        const unsigned all = __ballot_sync(FULL, head);
+        const unsigned hm = all & (lt | (1u << lane));
+        start[r] = hm ? at0 - lane + 32 * r + 31 - __clz(hm) : carry;
+        if (all) carry = at0 - lane + 32 * r + 31 - __clz(all);
+    }
+    if (lane == 0) s_first[warp] = carry;
+    __syncthreads();
+    for (int w = warp - 1, open = 1; w >= 0 && open; --w) {
+        const int f = s_first[w];
+        if (f >= 0) {
+#pragma unroll
+            for (int r = 0; r < IPT; ++r)
+                if (start[r] < 0) start[r] = f;
+            open = 0;
+        }
+    }
+    // units: every uq queries of a cell
+    unsigned mine[IPT];
+    int count = 0;
+#pragma unroll
+    for (int r = 0; r < IPT; ++r) {
+        const int i = at0 + 32 * r;
+        mine[r] = __ballot_sync(FULL, i < n && key[r] != NO_KEY && ((unsigned)(i - start[r]) % (unsigned)uq) == 0u);
+        count += __popc(mine[r]);
+    }
+    if (lane == 0) s_sum[warp] = count;
+    __syncthreads();
+    if (warp == 0) {
+        const int c = s_sum[lane];
+        int inc = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(FULL, inc, o);
+            if (lane >= o) inc += u;
+        }
+        s_sum[lane] = inc - c;
+        if (lane == 31) s_base = inc ? atomicAdd(n_units, inc) : 0;
+    }
+    __syncthreads();
+    int to = s_base + s_sum[warp];
+#pragma unroll
+    for (int r = 0; r < IPT; ++r) {
+        const int i = at0 + 32 * r;
+        if ((mine[r] >> lane) & 1u) {
+            const uint32_t c = key[r] >> gp.key_sub;
+            auto same = [&](int k) { return k < n && (s_key[k] >> gp.key_sub) == c; };
+            int m = 1;                               // queries of the cell from here on, uq at most
+            while (m < uq && same(i + m)) m *= 2;
+            int lo = m / 2 + 1, hi = m < uq ? m : uq;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (same(i + mid)) lo = mid + 1; else hi = mid;
+            }
+            units[to + __popc(mine[r] & lt)] = make_int2((int)(Ed.q_off + i), (e << 7) | lo);
+        }
+        to += __popc(mine[r]);
     }
 }
 
@@ -1892,6 +2123,22 @@ int pair_blocks_per_sm(KernelT kernel, size_t smem, int* cache) {
     return *cache;
 }
 
+template <int IPT>
+void bin_edges(const BinArgs& a, cudaStream_t st) {
+    constexpr size_t smem = BinSmem<IPT>::BYTES;
+    if constexpr (smem > 36864) {                // with the static arrays more than 48 KB: opt in, once per device
+        static std::atomic<bool> opted[64];
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (dev >= 64 || !opted[dev].load(std::memory_order_acquire)) {
+            cudaFuncSetAttribute(k_bin_edges<IPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (dev < 64) opted[dev].store(true, std::memory_order_release);
+        }
+    }
+    k_bin_edges<IPT><<<(unsigned)a.E, BIN_T, smem, st>>>(a.poses, a.edges, a.frames, a.pt_cell, a.pts4, a.gp, a.uq, a.xf,
+                                                         a.qkey, a.qrec, a.slots, a.units, a.ucount, a.acc, a.done);
+}
+
 inline unsigned pair_grid(int num_sms, int resident, int ctas_per_sm) {
     const int per_sm = (ctas_per_sm > 0 && ctas_per_sm < resident) ? ctas_per_sm : resident;
     return (unsigned)(num_sms * per_sm);
@@ -2012,6 +2259,20 @@ void launch_units(const uint32_t* qkey_sorted, const int* qval_sorted, const flo
     if (uq < 1 || uq > UQ) uq = UQ;      // larger units are taken as units of 32
     k_units<<<blocks_for(Q, 256), 256, 0, st>>>(qkey_sorted, qval_sorted, qrec, Q, uq, sub, edges, E, slots, units,
                                                 n_units, done);
+    count_launch();
+}
+
+void launch_bin_edges(const BinArgs& a, int q_max, cudaStream_t st) {
+    cudaMemsetAsync(a.ucount, 0, 4 * sizeof(int), st);
+    BinArgs b = a;
+    if (b.uq < 1 || b.uq > UQ) b.uq = UQ;      // larger units are taken as units of 32
+    switch ((q_max + BIN_T - 1) / BIN_T) {     // queries per thread
+        case 0:
+        case 1: bin_edges<1>(b, st); break;
+        case 2: bin_edges<2>(b, st); break;
+        case 3: bin_edges<3>(b, st); break;
+        default: bin_edges<4>(b, st); break;
+    }
     count_launch();
 }
 

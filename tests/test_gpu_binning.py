@@ -1,10 +1,12 @@
 """Binning of the queries and cutting into units, at the sizes where they change course.
 
-Cells of more queries than a block of the unit pass takes (256), whose first
-query is or is not the first of all; streams long enough to be shared by several
-warps; and query counts around the sort's tiles of 2048.  Tolerances are those of
-the parity tests (loss 1e-5, gradient and Gauss-Newton matrix 1e-4 relative); in
-the clumps every pair lies inside the cutoff, so their counts are exact.
+Edges of at most 4096 queries are binned by one block each (1 to 4 queries a
+thread), larger ones by the tiled sort (tiles of 2048 and, from 5 M queries on,
+4096) and the unit pass (blocks of 256): sizes around each step, cells longer than a block
+whose first query is or is not the first of all, and streams long enough to be shared by
+several warps.  Tolerances are those of the parity tests (loss 1e-5, gradient and
+Gauss-Newton matrix 1e-4 relative); in the clumps every pair lies inside the cutoff, so
+their counts are exact.
 """
 import numpy as np
 import pytest
@@ -46,19 +48,18 @@ def _check(pk, prob, exact_count=None):
     assert _reln(out["H"], ref["H"]) <= H_TOL
 
 
-def _clump(n, lead, variant):
-    """n points of each frame inside one cell; `lead` lone points of frame b in cells before it."""
-    rng = np.random.default_rng(1000 * n + lead)
+def _clump(na, nb, lead, variant):
+    """na and nb points of the two frames inside one cell; `lead` lone points of frame b in cells before it."""
+    rng = np.random.default_rng(1000 * nb + lead)
     prob = scenes.tiny_problem(seed=9, n_frames=2, n=8, extent=1.0, ell=0.15, color=variant == "color")
     lone = np.array([[-2.0 - 0.5 * k, 0.2, 0.2] for k in range(lead)]).reshape(lead, 3)
-    box = [0.12 + 0.2 * rng.random((n, 3)) for _ in range(2)]
-    m = n + lead
+    box = [0.12 + 0.2 * rng.random((n, 3)) for n in (na, nb)]
     prob["xyz"] = [np.concatenate([lone + [0.0, 9.0, 0.0], box[0]]), np.concatenate([lone, box[1]])]
     prob["poses0"] = np.stack([np.eye(4), scenes.make_pose(
         scenes.rot_from_axis_angle(np.array([0.0, 0.0, 1.0]), 0.05), np.array([0.01, -0.01, 0.005]))])
-    prob["edges"] = np.array([[0, 1]], np.int32)
-    prob["rgb"] = [rng.random((m, 3)) for _ in range(2)] if variant == "color" else None
-    sem = [scenes.dirichlet_labels(rng, rng.integers(0, 4, m), 4) for _ in range(2)]
+    m = [len(x) for x in prob["xyz"]]
+    prob["rgb"] = [rng.random((k, 3)) for k in m] if variant == "color" else None
+    sem = [scenes.dirichlet_labels(rng, rng.integers(0, 4, k), 4) for k in m]
     prob["sem"] = None if variant == "plain" else sem
     if variant == "bf16":
         prob["sem"] = [scenes.round_to_bf16(s) for s in sem]
@@ -67,11 +68,13 @@ def _clump(n, lead, variant):
 
 
 @pytest.mark.parametrize("variant", ["plain", "fp32", "bf16", "color"])
-@pytest.mark.parametrize("n,lead", [(1, 0), (255, 0), (256, 1), (257, 0), (513, 0), (700, 5), (1025, 0)])
-def test_cells_longer_than_a_block(pk, variant, n, lead):
-    _check(pk, _clump(n, lead, variant), exact_count=[n * n])
+@pytest.mark.parametrize("na,nb,lead", [(1, 1, 0), (255, 255, 0), (257, 257, 0), (700, 700, 5), (1025, 1025, 0),
+                                        (40, 1024, 3), (40, 2048, 0), (40, 2049, 1), (40, 3073, 0), (40, 4096, 0),
+                                        (40, 4097, 0), (40, 4096, 1), (40, 9001, 300)])
+def test_cells_longer_than_a_block(pk, variant, na, nb, lead):
+    _check(pk, _clump(na, nb, lead, variant), exact_count=[na * nb])
 
 
-@pytest.mark.parametrize("n", [2047, 2048, 2049, 4097])
-def test_query_counts_around_a_sort_tile(pk, n):
-    _check(pk, scenes.tiny_problem(seed=40 + n % 7, n_frames=2, n=n, extent=2.5, ell=0.1))
+@pytest.mark.parametrize("n", [1023, 1025, 2048, 3073, 4096, 4097, 6145, 10240, 10241])
+def test_query_counts_around_a_tile(pk, n):
+    _check(pk, scenes.tiny_problem(seed=40 + n % 7, n_frames=2, n=n, extent=2.5 if n < 4000 else 4.0, ell=0.1))
