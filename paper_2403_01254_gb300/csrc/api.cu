@@ -17,6 +17,7 @@
 #include <cstring>
 #include <set>
 #include <string>
+#include <memory>
 #include <utility>
 #include <vector>
 
@@ -186,28 +187,36 @@ rkhsba_status build(rkhsba_ctx* c, const double* xyz, const float* sem, const fl
         RK_CUDA(c, cudaMemcpyAsync(c->d_rgb_in, rgb_used, sizeof(float) * 3 * N,
                                    on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st));
     }
-    RK_TRY(alloc(c, &c->d_pt_off, K + 1));
-    RK_CUDA(c, cudaMemcpyAsync(c->d_pt_off, c->pt_off.data(), sizeof(long long) * (K + 1),
-                               cudaMemcpyHostToDevice, st));
-    RK_TRY(alloc(c, &c->d_cmin, 3 * K));
-    RK_TRY(alloc(c, &c->d_cmax, 3 * K));
-    RK_TRY(alloc(c, &c->d_semnorm, K));
-    RK_TRY(alloc(c, &c->d_err, 4));
-    std::vector<int> big(3 * K, 0x7fffffff), small(3 * K, (int)0x80000000);
-    RK_CUDA(c, cudaMemcpyAsync(c->d_cmin, big.data(), sizeof(int) * 3 * K, cudaMemcpyHostToDevice, st));
-    RK_CUDA(c, cudaMemcpyAsync(c->d_cmax, small.data(), sizeof(int) * 3 * K, cudaMemcpyHostToDevice, st));
-    RK_CUDA(c, cudaMemsetAsync(c->d_semnorm, 0, sizeof(unsigned) * K, st));
-    RK_CUDA(c, cudaMemsetAsync(c->d_err, 0, sizeof(int) * 4, st));
+    // small arrays of the grid step and the results of an evaluation, in one
+    // block: what goes up or comes back together is one copy (each pageable copy costs
+    // several microseconds of host time)
+    const ResultLayout R(K, E);
+    RK_TRY(alloc(c, &c->d_block, (long long)R.end));
+    c->d_pt_off = reinterpret_cast<long long*>(c->d_block + R.pt_off);
+    c->d_cmin = reinterpret_cast<int*>(c->d_block + R.cmin);
+    c->d_cmax = reinterpret_cast<int*>(c->d_block + R.cmax);
+    c->d_semnorm = reinterpret_cast<unsigned*>(c->d_block + R.semn);
+    c->d_err = reinterpret_cast<int*>(c->d_block + R.err);
+    c->d_state = reinterpret_cast<LMState*>(c->d_block + R.state);
+    c->d_poses_cur = reinterpret_cast<double*>(c->d_block + R.poses);
+    c->d_F_cand = reinterpret_cast<double*>(c->d_block + R.F);
+    c->d_n_cand = reinterpret_cast<long long*>(c->d_block + R.n);
+    c->d_b_cand = reinterpret_cast<double*>(c->d_block + R.b);
+    c->d_H_cand = reinterpret_cast<double*>(c->d_block + R.H);
+    c->d_eout = reinterpret_cast<EdgeOut*>(c->d_block + R.eout);
+    std::vector<char> up(R.err + 16, 0);
+    std::memcpy(up.data() + R.pt_off, c->pt_off.data(), sizeof(long long) * (K + 1));
+    std::fill_n(reinterpret_cast<int*>(up.data() + R.cmin), 3 * K, 0x7fffffff);
+    std::fill_n(reinterpret_cast<int*>(up.data() + R.cmax), 3 * K, (int)0x80000000);
+    RK_CUDA(c, cudaMemcpyAsync(c->d_block, up.data(), up.size(), cudaMemcpyHostToDevice, st));
     launch_bbox(c->d_xyz, c->d_sem_in, c->d_rgb_in, N, K, c->d_pt_off, c->p.sem_dim, c->gp.h_inv,
                 c->d_cmin, c->d_cmax, c->d_semnorm, c->d_err, st);
-    std::vector<int> cmin(3 * K), cmax(3 * K);
-    std::vector<unsigned> semn(K);
-    int errbits = 0;
-    RK_CUDA(c, cudaMemcpyAsync(cmin.data(), c->d_cmin, sizeof(int) * 3 * K, cudaMemcpyDeviceToHost, st));
-    RK_CUDA(c, cudaMemcpyAsync(cmax.data(), c->d_cmax, sizeof(int) * 3 * K, cudaMemcpyDeviceToHost, st));
-    RK_CUDA(c, cudaMemcpyAsync(semn.data(), c->d_semnorm, sizeof(unsigned) * K, cudaMemcpyDeviceToHost, st));
-    RK_CUDA(c, cudaMemcpyAsync(&errbits, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    RK_CUDA(c, cudaMemcpyAsync(up.data(), c->d_block, up.size(), cudaMemcpyDeviceToHost, st));
     RK_CUDA(c, cudaStreamSynchronize(st));
+    const int* cmin = reinterpret_cast<const int*>(up.data() + R.cmin);
+    const int* cmax = reinterpret_cast<const int*>(up.data() + R.cmax);
+    const unsigned* semn = reinterpret_cast<const unsigned*>(up.data() + R.semn);
+    const int errbits = *reinterpret_cast<const int*>(up.data() + R.err);
     if (errbits & 1) return fail(c, RKHSBA_EINVAL, "non-finite point coordinate");
     if (errbits & 2) return fail(c, RKHSBA_EINVAL, "point coordinate beyond 2^29 grid cells");
     if (errbits & 4) return fail(c, RKHSBA_EINVAL, "non-finite label value");
@@ -215,14 +224,9 @@ rkhsba_status build(rkhsba_ctx* c, const double* xyz, const float* sem, const fl
 
     // grid layout per frame (dense, one-cell margin)
     c->frames_h.assign(K, FrameDev{});
-    if (const char* msg = layout_frames(c->frames_h.data(), K, c->pt_off.data(), cmin.data(), cmax.data(),
-                                        semn.data(), has_sem, 1LL << 20, 1LL << 30, (1LL << 31) - 2,
+    if (const char* msg = layout_frames(c->frames_h.data(), K, c->pt_off.data(), cmin, cmax, semn, has_sem, 1LL << 20, 1LL << 30, (1LL << 31) - 2,
                                         &c->C_total))
         return fail(c, RKHSBA_EINVAL, std::string(msg) + " (2^20 per axis, 2^30 per frame, 2^31 in all)");
-    RK_TRY(alloc(c, &c->d_frames, K));
-    RK_CUDA(c, cudaMemcpyAsync(c->d_frames, c->frames_h.data(), sizeof(FrameDev) * K,
-                               cudaMemcpyHostToDevice, st));
-
     // grid buffers
     const int sp = c->gp.sem_pad;
     RK_TRY(alloc(c, &c->d_keys, N));
@@ -256,21 +260,23 @@ rkhsba_status build(rkhsba_ctx* c, const double* xyz, const float* sem, const fl
                                            (long long)radix_hist_elems(c->Q_total));
     RK_TRY(alloc(c, &c->d_scan_ws, (long long)scan_ws_elems(scan_n) + 64));
     if (N == 0) RK_CUDA(c, cudaMemsetAsync(c->d_cell_start, 0, sizeof(int) * (c->C_total + 1), st));
+    // frames, edges and the incidence lists (frame -> edges, edge order kept)
+    const size_t o_edges = sizeof(FrameDev) * K, o_ioff = o_edges + sizeof(EdgeDev) * E, o_ilist = o_ioff + sizeof(int) * (K + 1);
+    up.assign(o_ilist + sizeof(int) * (2 * (size_t)E + 1), 0);
+    std::memcpy(up.data(), c->frames_h.data(), sizeof(FrameDev) * K);
+    std::memcpy(up.data() + o_edges, c->edges_h.data(), sizeof(EdgeDev) * E);
+    incidence_lists(c->edges_h.data(), E, K, reinterpret_cast<int*>(up.data() + o_ioff),
+                    reinterpret_cast<int*>(up.data() + o_ilist));
+    char* graph = nullptr;
+    RK_TRY(alloc(c, &graph, (long long)up.size()));
+    c->d_frames = reinterpret_cast<FrameDev*>(graph);
+    c->d_edges = reinterpret_cast<EdgeDev*>(graph + o_edges);
+    c->d_inc_off = reinterpret_cast<int*>(graph + o_ioff);
+    c->d_inc_list = reinterpret_cast<int*>(graph + o_ilist);
+    RK_CUDA(c, cudaMemcpyAsync(graph, up.data(), up.size(), cudaMemcpyHostToDevice, st));
     bool alt = false;
     grid_fill(c, &alt);
     RK_CUDA(c, cudaGetLastError());
-
-    RK_TRY(alloc(c, &c->d_edges, E));
-    RK_CUDA(c, cudaMemcpyAsync(c->d_edges, c->edges_h.data(), sizeof(EdgeDev) * E,
-                               cudaMemcpyHostToDevice, st));
-    // incidence lists (frame -> edges), edge order kept
-    std::vector<int> inc_off(K + 1, 0), inc_list(2 * (size_t)E + 1, 0);
-    inc_list.resize(incidence_lists(c->edges_h.data(), E, K, inc_off.data(), inc_list.data()));
-    RK_TRY(alloc(c, &c->d_inc_off, K + 1));
-    RK_TRY(alloc(c, &c->d_inc_list, (long long)inc_list.size()));
-    RK_CUDA(c, cudaMemcpyAsync(c->d_inc_off, inc_off.data(), sizeof(int) * (K + 1), cudaMemcpyHostToDevice, st));
-    RK_CUDA(c, cudaMemcpyAsync(c->d_inc_list, inc_list.data(), sizeof(int) * inc_list.size(),
-                               cudaMemcpyHostToDevice, st));
 
     // evaluation buffers
     const long long Q = c->Q_total;
@@ -285,17 +291,10 @@ rkhsba_status build(rkhsba_ctx* c, const double* xyz, const float* sem, const fl
     RK_TRY(alloc(c, &c->d_units, Q));
     RK_TRY(alloc(c, &c->d_ucount, 4));
     RK_TRY(alloc(c, &c->d_acc, (long long)E * ACC_N));
-    RK_TRY(alloc(c, &c->d_eout, E));
     const long long n6 = 6LL * K;
-    RK_TRY(alloc(c, &c->d_H_cand, n6 * n6));
     RK_TRY(alloc(c, &c->d_H_cur, n6 * n6));
-    RK_TRY(alloc(c, &c->d_b_cand, n6));
     RK_TRY(alloc(c, &c->d_b_cur, n6));
-    RK_TRY(alloc(c, &c->d_F_cand, 1));
-    RK_TRY(alloc(c, &c->d_n_cand, 1));
-    RK_TRY(alloc(c, &c->d_poses_cur, 16LL * K));
     RK_TRY(alloc(c, &c->d_poses_cand, 16LL * K));
-    RK_TRY(alloc(c, &c->d_state, 1));
     const long long nf = 6LL * (K - 1);
     RK_TRY(alloc(c, &c->d_lm_ws, nf * nf + 2 * nf + 16));
     // blocks of frame pairs without an edge stay zero: no evaluation writes them
@@ -586,25 +585,27 @@ rkhsba_status rkhsba_eval(rkhsba_ctx* c, const double* poses, double* loss, doub
     RK_CUDA(c, cudaMemcpyAsync(c->d_poses_cand, poses, sizeof(double) * 16 * c->K, cudaMemcpyHostToDevice, st));
     run_eval(c, c->d_poses_cand, nullptr);
     RK_CUDA(c, cudaGetLastError());
-    double F = 0.0;
-    int sort_err = 0;
-    RK_CUDA(c, cudaMemcpyAsync(&sort_err, c->d_err + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
-    RK_CUDA(c, cudaMemcpyAsync(&F, c->d_F_cand, sizeof(double), cudaMemcpyDeviceToHost, st));
-    std::vector<double> b;
-    if (grad) {
-        b.resize(6 * c->K);
-        RK_CUDA(c, cudaMemcpyAsync(b.data(), c->d_b_cand, sizeof(double) * 6 * c->K, cudaMemcpyDeviceToHost, st));
-    }
-    if (H_full)
-        RK_CUDA(c, cudaMemcpyAsync(H_full, c->d_H_cand, sizeof(double) * 36LL * c->K * c->K,
-                                   cudaMemcpyDeviceToHost, st));
-    std::vector<EdgeOut> eo;
-    if (H_blocks || edge_pairs) {
-        eo.resize(c->E);
-        RK_CUDA(c, cudaMemcpyAsync(eo.data(), c->d_eout, sizeof(EdgeOut) * c->E, cudaMemcpyDeviceToHost, st));
-    }
+    // everything asked for up to ONE_COPY bytes in one copy, else the matrix
+    // straight to its place
+    const ResultLayout R(c->K, c->E);
+    constexpr size_t ONE_COPY = 256 << 10;
+    const bool want_e = H_blocks || edge_pairs;
+    const size_t nH = sizeof(double) * 36 * (size_t)c->K * c->K, head = R.H - R.err, nE = R.end - R.eout;
+    const bool one = (want_e || H_full) && (want_e ? R.end : R.eout) - R.err <= ONE_COPY;
+    const size_t n1 = one ? (want_e ? R.end : R.eout) - R.err : head;
+    std::unique_ptr<char[]> res(new char[n1 + (!one && want_e ? nE : 0)]);
+    RK_CUDA(c, cudaMemcpyAsync(res.get(), c->d_block + R.err, n1, cudaMemcpyDeviceToHost, st));
+    if (!one && H_full) RK_CUDA(c, cudaMemcpyAsync(H_full, c->d_H_cand, nH, cudaMemcpyDeviceToHost, st));
+    if (!one && want_e) RK_CUDA(c, cudaMemcpyAsync(res.get() + n1, c->d_eout, nE, cudaMemcpyDeviceToHost, st));
     RK_CUDA(c, cudaStreamSynchronize(st));
-    if (sort_err) return fail(c, RKHSBA_ETIMEOUT, "a bounded wait of the radix sort gave up");
+    int err[2];
+    double F;
+    std::memcpy(err, res.get(), sizeof(err));
+    std::memcpy(&F, res.get() + (R.F - R.err), sizeof(F));
+    if (err[1]) return fail(c, RKHSBA_ETIMEOUT, "a bounded wait of the radix sort gave up");
+    const double* b = reinterpret_cast<const double*>(res.get() + (R.b - R.err));
+    const EdgeOut* eo = reinterpret_cast<const EdgeOut*>(res.get() + (one ? R.eout - R.err : n1));
+    if (one && H_full) std::memcpy(H_full, res.get() + (R.H - R.err), nH);
     if (loss) *loss = -F;
     if (grad) {
         const double scale = c->p.sigma * c->p.sigma / (c->p.ell * c->p.ell);
@@ -645,15 +646,16 @@ rkhsba_status rkhsba_iterate(rkhsba_ctx* c, int32_t n_iters) {
 
 rkhsba_status rkhsba_get_state(rkhsba_ctx* c, double* poses, rkhsba_solve_info* info) {
     if (!c) return fail(nullptr, RKHSBA_EINVAL, "ctx is NULL");
-    LMState s{};
-    int sort_err = 0;
-    RK_CUDA(c, cudaMemcpyAsync(&s, c->d_state, sizeof(LMState), cudaMemcpyDeviceToHost, c->stream));
-    RK_CUDA(c, cudaMemcpyAsync(&sort_err, c->d_err + 1, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    if (poses)
-        RK_CUDA(c, cudaMemcpyAsync(poses, c->d_poses_cur, sizeof(double) * 16 * c->K,
-                                   cudaMemcpyDeviceToHost, c->stream));
+    const ResultLayout R(c->K, c->E);
+    std::unique_ptr<char[]> res(new char[R.F - R.err]);
+    RK_CUDA(c, cudaMemcpyAsync(res.get(), c->d_block + R.err, R.F - R.err, cudaMemcpyDeviceToHost, c->stream));
     RK_CUDA(c, cudaStreamSynchronize(c->stream));
-    if (sort_err) return fail(c, RKHSBA_ETIMEOUT, "a bounded wait of the radix sort gave up");
+    LMState s{};
+    int err[2];
+    std::memcpy(err, res.get(), sizeof(err));
+    std::memcpy(&s, res.get() + (R.state - R.err), sizeof(s));
+    if (poses) std::memcpy(poses, res.get() + (R.poses - R.err), sizeof(double) * 16 * c->K);
+    if (err[1]) return fail(c, RKHSBA_ETIMEOUT, "a bounded wait of the radix sort gave up");
     if (info) {
         info->iters = s.iters;
         info->status = s.done ? s.status : RKHSBA_ENOTCONV;

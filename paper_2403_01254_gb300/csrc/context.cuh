@@ -38,6 +38,7 @@ struct rkhsba_ctx {
     std::vector<std::pair<int, int>> edge_in;   // as given by the caller (a, b)
 
     // device
+    char* d_block = nullptr;              // the arrays of ResultLayout
     long long* d_pt_off = nullptr;
     FrameDev* d_frames = nullptr;
     EdgeDev* d_edges = nullptr;

@@ -156,6 +156,29 @@ inline int edge_queries_max(const EdgeDev* eh, int E, const FrameDev* fh) {
     return m;
 }
 
+// Offsets in the block of small arrays of a problem: the point offsets, frame
+// bounds and label norms of the grid step, the error words, the LM state and
+// accepted poses, and the results of an evaluation (loss, pair count, gradient, matrix,
+// edges).
+struct ResultLayout {
+    size_t pt_off, cmin, cmax, semn, err, state, poses, F, n, b, H, eout, end;
+    ResultLayout(int K, int E) {
+        pt_off = 0;
+        cmin = sizeof(long long) * ((size_t)K + 1);
+        cmax = cmin + sizeof(int) * 3 * (size_t)K;
+        semn = cmax + sizeof(int) * 3 * (size_t)K;
+        err = (semn + sizeof(unsigned) * (size_t)K + 15) & ~size_t(15);     // four words
+        state = err + 16;
+        poses = state + sizeof(LMState);
+        F = poses + sizeof(double) * 16 * (size_t)K;
+        n = F + sizeof(double);
+        b = n + sizeof(long long);
+        H = b + sizeof(double) * 6 * (size_t)K;
+        eout = H + sizeof(double) * 36 * (size_t)K * K;
+        end = eout + sizeof(EdgeOut) * (size_t)E;
+    }
+};
+
 // Frame -> edge incidence in edge order: frame m's entries are 2e when m is
 // edge e's first frame and 2e + 1 when it is the second.  inc_off [K + 1],
 // inc_list [2 E]; returns the number of entries.

@@ -171,38 +171,45 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
     SCK(cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev));
 
     // ---- small arrays and the bounding boxes ----
+    // what goes up or comes back together lies together and is one copy
     Carve cv{base};
-    long long* d_pt_off = cv.take<long long>(K + 1);
-    int* d_cmin = cv.take<int>(3 * K);
-    int* d_cmax = cv.take<int>(3 * K);
-    unsigned* d_semn = cv.take<unsigned>(K);
-    int* d_err = cv.take<int>(4);
-    FrameDev* d_frames = cv.take<FrameDev>(K);
-    EdgeDev* d_edges = cv.take<EdgeDev>(E);
+    const ResultLayout RL(K, E);
+    unsigned char* d_block = cv.take<unsigned char>((long long)RL.end);
+    struct Graph {                        // frames, edges, incidence lists, poses
+        FrameDev frames[MAX_K];
+        EdgeDev edges[MAX_E];
+        int inc_off[MAX_K + 1], inc_list[2 * MAX_E];
+        double poses[16 * MAX_K];
+    };
+    Graph* d_graph = cv.take<Graph>(1);
     EdgeXf* d_xf = cv.take<EdgeXf>(E);
-    int* d_inc_off = cv.take<int>(K + 1);
-    int* d_inc_list = cv.take<int>(2 * E);
-    double* d_poses = cv.take<double>(16 * K);
     if (!cv.ok) return fail(RKHSBA_EINVAL, "static scratch too small");
-    int cmin[3 * MAX_K], cmax[3 * MAX_K], errbits = 0;
-    unsigned semn[MAX_K];
+    long long* d_pt_off = reinterpret_cast<long long*>(d_block + RL.pt_off);
+    int* d_cmin = reinterpret_cast<int*>(d_block + RL.cmin);
+    int* d_cmax = reinterpret_cast<int*>(d_block + RL.cmax);
+    unsigned* d_semn = reinterpret_cast<unsigned*>(d_block + RL.semn);
+    int* d_err = reinterpret_cast<int*>(d_block + RL.err);
+    constexpr size_t UP_MAX = sizeof(long long) * (MAX_K + 1) + sizeof(int) * 7 * MAX_K + 32;
+    alignas(16) unsigned char up[UP_MAX];
+    const size_t n_up = RL.err + 16;
+    std::memset(up, 0, n_up);
+    std::memcpy(up + RL.pt_off, pt_off, sizeof(long long) * (K + 1));
+    int* cmin = reinterpret_cast<int*>(up + RL.cmin);
+    int* cmax = reinterpret_cast<int*>(up + RL.cmax);
+    const unsigned* semn = reinterpret_cast<const unsigned*>(up + RL.semn);
     for (int i = 0; i < 3 * K; ++i) { cmin[i] = 0x7fffffff; cmax[i] = (int)0x80000000; }
-    SCK(cudaMemcpyAsync(d_pt_off, pt_off, sizeof(long long) * (K + 1), cudaMemcpyHostToDevice, st));
-    SCK(cudaMemcpyAsync(d_cmin, cmin, sizeof(int) * 3 * K, cudaMemcpyHostToDevice, st));
-    SCK(cudaMemcpyAsync(d_cmax, cmax, sizeof(int) * 3 * K, cudaMemcpyHostToDevice, st));
-    SCK(cudaMemsetAsync(d_semn, 0, sizeof(unsigned) * K, st));
-    SCK(cudaMemsetAsync(d_err, 0, sizeof(int) * 4, st));
+    SCK(cudaMemcpyAsync(d_block, up, n_up, cudaMemcpyHostToDevice, st));
     launch_bbox(d_xyz, d_sem, gp.color ? d_rgb : nullptr, N, K, d_pt_off, p.sem_dim, gp.h_inv, d_cmin, d_cmax,
                 d_semn, d_err, st);
-    SCK(cudaMemcpyAsync(cmin, d_cmin, sizeof(int) * 3 * K, cudaMemcpyDeviceToHost, st));
-    SCK(cudaMemcpyAsync(cmax, d_cmax, sizeof(int) * 3 * K, cudaMemcpyDeviceToHost, st));
-    SCK(cudaMemcpyAsync(semn, d_semn, sizeof(unsigned) * K, cudaMemcpyDeviceToHost, st));
-    SCK(cudaMemcpyAsync(&errbits, d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    SCK(cudaMemcpyAsync(up, d_block, n_up, cudaMemcpyDeviceToHost, st));
     SCK(cudaStreamSynchronize(st));
+    const int errbits = *reinterpret_cast<const int*>(up + RL.err);
     if (errbits) return fail(RKHSBA_EINVAL, "non-finite or out-of-range input values");
 
     // ---- grid layout, edges, fixed-point scales (host) ----
-    FrameDev fh[MAX_K];
+    Graph gh;
+    std::memset(&gh, 0, sizeof(gh));
+    FrameDev* fh = gh.frames;
     long long C = 0;
     if (const char* msg = layout_frames(fh, K, pt_off, cmin, cmax, semn, p.sem_dim > 0, MAX_CELLS, MAX_CELLS,
                                         MAX_CELLS + 1, &C))
@@ -217,8 +224,14 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
     qbits += gp.key_sub;
     int cbits = 0;
     while ((1LL << cbits) < C) ++cbits;
-    int inc_off[MAX_K + 1], inc_list[2 * MAX_E];
-    const int ninc = incidence_lists(eh, E, K, inc_off, inc_list);
+    incidence_lists(eh, E, K, gh.inc_off, gh.inc_list);
+    std::memcpy(gh.edges, eh, sizeof(EdgeDev) * E);
+    std::memcpy(gh.poses, poses, sizeof(double) * 16 * K);
+    FrameDev* d_frames = d_graph->frames;
+    EdgeDev* d_edges = d_graph->edges;
+    int* d_inc_off = d_graph->inc_off;
+    int* d_inc_list = d_graph->inc_list;
+    double* d_poses = d_graph->poses;
 
     // ---- large arrays ----
     const int sp = gp.sem_pad;
@@ -244,18 +257,14 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
     int2* d_units = cv.take<int2>(Q);
     int* d_ucount = cv.take<int>(4);
     long long* d_acc = cv.take<long long>((long long)E * ACC_N);
-    EdgeOut* d_eout = cv.take<EdgeOut>(E);
-    double* d_H = cv.take<double>(36LL * K * K);
-    double* d_b = cv.take<double>(6 * K);
-    double* d_F = cv.take<double>(1);
-    long long* d_n = cv.take<long long>(1);
+    EdgeOut* d_eout = reinterpret_cast<EdgeOut*>(d_block + RL.eout);
+    double* d_H = reinterpret_cast<double*>(d_block + RL.H);
+    double* d_b = reinterpret_cast<double*>(d_block + RL.b);
+    double* d_F = reinterpret_cast<double*>(d_block + RL.F);
+    long long* d_n = reinterpret_cast<long long*>(d_block + RL.n);
     if (!cv.ok) return fail(RKHSBA_EINVAL, "rkhsba_eval_static: problem does not fit the 32 MiB static scratch");
 
-    SCK(cudaMemcpyAsync(d_frames, fh, sizeof(FrameDev) * K, cudaMemcpyHostToDevice, st));
-    SCK(cudaMemcpyAsync(d_edges, eh, sizeof(EdgeDev) * E, cudaMemcpyHostToDevice, st));
-    SCK(cudaMemcpyAsync(d_inc_off, inc_off, sizeof(int) * (K + 1), cudaMemcpyHostToDevice, st));
-    SCK(cudaMemcpyAsync(d_inc_list, inc_list, sizeof(int) * (ninc > 0 ? ninc : 1), cudaMemcpyHostToDevice, st));
-    SCK(cudaMemcpyAsync(d_poses, poses, sizeof(double) * 16 * K, cudaMemcpyHostToDevice, st));
+    SCK(cudaMemcpyAsync(d_graph, &gh, sizeof(gh), cudaMemcpyHostToDevice, st));
 
     // ---- grid step (all temporaries that must start at zero are cleared) ----
     if (N == 0) SCK(cudaMemsetAsync(d_cell_start, 0, sizeof(int) * (C + 1), st));
@@ -309,15 +318,19 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
     launch_frame_assemble(d_edges, E, K, d_inc_off, d_inc_list, d_eout, d_H, d_b, d_F, d_n, nullptr, nullptr, st);
 
     // ---- results to the caller's host buffers ----
-    double F = 0.0;
-    double bvec[6 * MAX_K];
-    int sort_err = 0;
-    SCK(cudaMemcpyAsync(&sort_err, d_err + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
-    SCK(cudaMemcpyAsync(&F, d_F, sizeof(double), cudaMemcpyDeviceToHost, st));
-    SCK(cudaMemcpyAsync(bvec, d_b, sizeof(double) * 6 * K, cudaMemcpyDeviceToHost, st));
+    struct Head {
+        double F;
+        long long n;
+        double b[6 * MAX_K];
+    } head;
+    int err[4];
+    SCK(cudaMemcpyAsync(err, d_err, sizeof(err), cudaMemcpyDeviceToHost, st));
+    SCK(cudaMemcpyAsync(&head, d_F, RL.H - RL.F, cudaMemcpyDeviceToHost, st));
     if (H_full) SCK(cudaMemcpyAsync(H_full, d_H, sizeof(double) * 36LL * K * K, cudaMemcpyDeviceToHost, st));
     SCK(cudaStreamSynchronize(st));
     SCK(cudaGetLastError());
+    const double F = head.F, *bvec = head.b;
+    const int sort_err = err[1];
     if (sort_err) return fail(RKHSBA_ETIMEOUT, "a bounded wait of the radix sort gave up");
     if (loss) *loss = -F;
     if (grad) {
