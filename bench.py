@@ -86,7 +86,7 @@ def kernel_path(flat):
     the per-query moment sums on the tensor cores (mma.sync, BF16 or split
     FP16 operands, FP32 accumulation)."""
     if flat["color"]:
-        return "bit-walk (colour): FP32 label dot and moment sums per pair on the FP32 pipe"
+        return "lanes over queries: FP32 label dot and moment sums on the FP32 pipe"
     return ("dense tile: test, exponent and weight on the FP32 pipe (9 flops per tested element), label "
             "products and moment sums on the tensor cores (mma.sync, %s operands)"
             % ("BF16 labels / split FP16 features" if flat["P"].get("sem_bf16", 0) else "split FP16"))

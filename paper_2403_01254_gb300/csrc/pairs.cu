@@ -17,12 +17,10 @@
 //   * the dense tile unit (no colour, no pruning): every element of the
 //     32-candidate x unit tile in MMA fragment layout, label products and
 //     per-query moment sums on the tensor cores (see "dense tile path");
-//   * the bit-walk unit (colour, semantic pruning): lane = candidate, a bit
-//     mask of its pairs inside r_c, each lane walking its own set bits and
-//     folding W = sum w, D = sum w d, Q = sum w d d^T (d = x - y') per
-//     candidate.
-// Each lane's moments are rounded to 64-bit fixed point before any
-// cross-lane sum, so edge totals are exact integer sums, independent of which
+//   * the lane unit (colour, semantic pruning, no labels): lanes over the
+//     queries, all in FP32 (see "lane path").
+// A unit's moments are summed over the warp in a fixed order and rounded once to
+// 64-bit fixed point, so edge totals are exact integer sums, independent of which
 // warp ran which unit.
 //
 // No FP64 arithmetic runs per query: the frame-a position of a frame-b cell
@@ -663,32 +661,8 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
-// Per-warp shared memory, queries kept as m = -2 y and |y|^2 so that the
-// cutoff test of a candidate x is |y|^2 - 2 x.y < r_c^2 - |x|^2 (three FMA)
-// and d = x - y = x + m/2:
-//   walk  [UQ]    float4 (m_x, m_y, m_z, m_x): pairs (m_x, m_y), (m_z, m_x)
-//   test  [UQ/2]  8 floats per query pair (j, j+1):
-//                 (m_x j, m_x j+1, m_y j, m_y j+1, m_z j, m_z j+1, |y|^2 j, |y|^2 j+1)
-//   colours [UQ] float4, labels [UQ][row words], stencil rows [40] ints,
-//   per-lane unit sums [32][N_ACC] (kept in shared memory to free registers),
-//   candidate queue [CQ_N] float4 (x relative to the home centre, point index),
-//   with BF16 labels the batch's label Gram [32 queries][GRAM_LD] floats.
-// Per-lane sums over a unit, in this order: W, D (3), Q (6), sum w0 x (3),
-// sum w0 x x^T (6), sum x dc^T (9), with w0 = sum w, dc = sum w d of one
-// candidate over its queries.
-constexpr int N_ACC = 28;
 constexpr int ROWS_WORDS = 9 * 4 + 9 * 2 + 2;   // segment list of the candidate stream (Rows)
 constexpr int CQ_N = 64;            // ring of candidates that survived the unit's box test
-constexpr int GRAM_LD = 32;         // row stride (floats) of the BF16 label Gram tile, stored
-                                    // [query][candidate]: the walk's lane c reads column c,
-                                    // one bank per lane
-constexpr int A_W = 0, A_D = 1, A_Q = 4, A_SWX = 10, A_SWXX = 13, A_SXD = 19;
-
-template <int DP, bool BF16, bool COLOR>
-__host__ __device__ constexpr int warp_smem_words() {
-    return UQ * 4 + UQ * 4 + (COLOR ? UQ * 4 : 0) + UQ * SemRow<DP, BF16>::WORDS + ROWS_WORDS + 32 * N_ACC +
-           4 * CQ_N + ((BF16 && DP > 0) ? 32 * GRAM_LD : 0);
-}
 
 // The candidate stream of a unit: the points of the 3x3x3 cells around its
 // home cell are nine contiguous ranges (rows of three x-adjacent cells).  Cells
@@ -847,100 +821,17 @@ __device__ __forceinline__ void store_moments(float W, const float (&Dv)[3], con
     if (f != 0) atomicAdd(reinterpret_cast<unsigned long long*>(acc_e + lane), (unsigned long long)f);
 }
 
-// BF16 labels: the candidate x query label products of a batch come from the
-// tensor cores (mma.sync m16n8k16, BF16 in, FP32 accumulate; BF16 products
-// are exact in FP32) into a shared-memory tile; the walk reads one float per
-// pair instead of forming the dot product.
-__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-                 "{%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// Query-side (B) fragments of the Gram MMAs: lane (g, t4) holds words
-// 8 ks + t4 and 8 ks + t4 + 4 of query row 8 nt + g; the unit's queries do
-// not change from batch to batch, so they are loaded once per unit.
-template <int DP>
-struct GramB {
-    static constexpr int KS = (DP + 15) / 16;   // k16 steps; words beyond DP are zero
-    unsigned b[4][KS][2];
-    __device__ __forceinline__ void load(const float* ssq, int lane) {
-        constexpr int RW = DP / 2;
-        const int g = lane >> 2, t4 = lane & 3;
-        const unsigned* qw = reinterpret_cast<const unsigned*>(ssq);
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-            for (int ks = 0; ks < KS; ++ks) {
-                const unsigned* qrow = qw + (8 * nt + g) * RW;
-                const int w0 = 8 * ks + t4, w1 = w0 + 4;
-                b[nt][ks][0] = (w0 < RW) ? qrow[w0] : 0u;
-                b[nt][ks][1] = (w1 < RW) ? qrow[w1] : 0u;
-            }
-    }
-};
-
-// Column of candidate c in row q of the Gram tile: XOR-swizzled by q so that
-// the MMA fragment stores (four query rows of one candidate per instruction)
-// hit 32 different banks.
-__device__ __forceinline__ int gram_col(int q, int c) { return c ^ (((q >> 1) & 3) << 3); }
-
-template <int DP>
-__device__ __forceinline__ void label_gram_bf16(const unsigned* __restrict__ semw, const GramB<DP>& B, int cand_i,
-                                                unsigned has_mask, int lane, float* G) {
-    constexpr int KS = GramB<DP>::KS;
-    constexpr int RW = DP / 2;           // 32-bit words per label row
-    const int g = lane >> 2, t4 = lane & 3;
-    float acc[2][4][4];
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) acc[mt][nt][k] = 0.f;
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-        const int r0 = 16 * mt + g, r1 = r0 + 8;                 // candidate rows of this lane
-        const int i0 = __shfl_sync(FULL, cand_i, r0), i1 = __shfl_sync(FULL, cand_i, r1);
-        const bool v0 = (has_mask >> r0) & 1u, v1 = (has_mask >> r1) & 1u;
-        const unsigned* row0 = semw + (size_t)i0 * RW;
-        const unsigned* row1 = semw + (size_t)i1 * RW;
-#pragma unroll
-        for (int ks = 0; ks < KS; ++ks) {
-            const int w0 = 8 * ks + t4, w1 = w0 + 4;             // words of k = 16 ks + 2 t, + 8
-            unsigned a[4];
-            a[0] = (v0 && w0 < RW) ? __ldg(row0 + w0) : 0u;
-            a[1] = (v1 && w0 < RW) ? __ldg(row1 + w0) : 0u;
-            a[2] = (v0 && w1 < RW) ? __ldg(row0 + w1) : 0u;
-            a[3] = (v1 && w1 < RW) ? __ldg(row1 + w1) : 0u;
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) mma_bf16_16816(acc[mt][nt], a, B.b[nt][ks][0], B.b[nt][ks][1]);
-        }
-    }
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            const int c = 16 * mt + g, q = 8 * nt + 2 * t4;      // candidate row, query column
-            G[q * GRAM_LD + gram_col(q, c)] = acc[mt][nt][0];
-            G[(q + 1) * GRAM_LD + gram_col(q + 1, c)] = acc[mt][nt][1];
-            G[q * GRAM_LD + gram_col(q, c + 8)] = acc[mt][nt][2];
-            G[(q + 1) * GRAM_LD + gram_col(q + 1, c + 8)] = acc[mt][nt][3];
-        }
-}
-
 // ------------------------------------------------------ dense tile path ----
 // Labels without colour or pruning.  On the LiDAR workloads half to two
 // thirds of a batch's candidate x query tests pass the cutoff after the box
-// cull, so instead of walking each lane's set bits the warp evaluates the
+// cull, so instead of taking pairs one by one the warp evaluates the
 // whole tile in MMA fragment layout and moves the moment sums onto the tensor
 // cores:
 //   1. S = L_q L_c^T, the tile's label products (rows are the unit's queries
 //      in m tiles of 16, columns the batch's 32 candidates): BF16 labels as
 //      stored; FP32 labels scaled by a power of two and split into FP16
 //      hi + lo parts, S = hi*hi + hi*lo + lo*hi;
-//   2. per element: the exact cutoff test of the bit-walk kernel (same FP32
+//   2. per element: the exact cutoff test of the lane kernel (same FP32
 //      formula, so the same pair set), w = s 2^(kg |d|^2) (one ex2), and 0
 //      outside r_c; |d|^2 = |y|^2 - 2 x.y + |x|^2;
 //   3. the weights, now an A operand in registers (the accumulator layout of
@@ -953,7 +844,7 @@ __device__ __forceinline__ void label_gram_bf16(const unsigned* __restrict__ sem
 //   4. at the unit's end each lane takes one query and forms, with y = y_q,
 //      W = k, D = X1 - k y, sum w y = k y, sum w y y^T = k y y^T,
 //      sum w d y^T = D y^T and Q = X2 - X1 y^T - y X1^T + k y y^T, which
-//      enter the same reduction as those of the bit-walk kernel.
+//      enter the same reduction as those of the lane kernel.
 // Scaling: w is carried as w 2^KW with 2^KW |l|max^2 <= 2^14 and the
 // features as x 2^-EX with 2^EX >= h, so every FP16 operand stays inside
 // its range; both are powers of two and undone exactly at the unit's end.
@@ -1475,68 +1366,62 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int2 unit, in
     store_moments(W, D, Sy, Myy, Mdy, Q, cnt, Fa, hx, hy, hz, gp, A.edges[e].scale, A.acc + (long long)e * ACC_N, lane);
 }
 
-// One unit (queries of one frame-a home cell) of the pair sum: stage the queries, stream the candidates of the
-// 27-cell stencil, test, walk and fold, and add the unit's moments to its
-// edge.  wb is the warp's shared-memory block.
+// ------------------------------------------------------------ lane path ----
+// Everything else (colour, semantic pruning, no labels): lanes over the unit's
+// queries, all in FP32.  A unit of <= 16, 8 or 4 queries gives each of them 2, 4
+// or 8 lanes, which take every 2nd, 4th or 8th pair of candidates; a lane holds its
+// query (place, label row, colour) and its running sums W, D = sum w d and Q =
+// sum w d d^T in registers, and evaluates two candidates at a time in paired
+// FP32, those outside r_c with weight 0.  With y the lane's query, sum w y' = W y,
+// sum w y'y'^T = W y y^T and sum w d y'^T = D y^T at the unit's end.
+//
+// Bound by FP32 issue (two elements take ~22 paired instructions), on clouds of small
+// units by the latency of a unit's loads.  It replaced a walk over the set bits of a
+// per-candidate mask (lane = candidate), which folded 28 sums per candidate and
+// batch, read the queries with bank conflicts and ran as long as the lane with the
+// most pairs: four unlabelled scans of 8000 points 381 -> 298 us per evaluation, 5 x 20k
+// RGB-D with colour 210 -> 200 us.  Three CTAs per SM: 313 and 203 us.
+template <int DP, bool BF16>
+__host__ __device__ constexpr int lane_row_words() {   // row stride of the staged labels: lanes read up to 8 rows at a time
+    return SemRow<DP, BF16>::WORDS + (SemRow<DP, BF16>::WORDS % 8 == 0 && DP > 0 ? 4 : 0);
+}
+// Per-warp shared memory: the batch's candidate pairs [16][8] (x0 x0' x1 x1' x2
+// x2' thr thr'), their colours [16][8] (r r' g g' b b' - -), label rows, the
+// candidate ring, the stream's segments.
+template <int DP, bool BF16, bool COLOR>
+__host__ __device__ constexpr int warp_smem_words() {
+    return 16 * 8 + (COLOR ? 16 * 8 : 0) + 32 * lane_row_words<DP, BF16>() + 4 * CQ_N + ROWS_WORDS;
+}
+
 template <int DP, bool BF16, bool COLOR>
 __device__ __forceinline__ void pair_unit(const PairArgs& A, int2 unit, int part, int shift, float* wb, int lane) {
-    const uint32_t* __restrict__ qkey = A.qkey;
-    const float4* __restrict__ slots = A.slots;
-    const EdgeDev* __restrict__ edges = A.edges;
-    const FrameDev* __restrict__ frames = A.frames;
-    const int* __restrict__ cell_start = A.cell_start;
-    const float4* __restrict__ pts4 = A.pts4;
-    const void* __restrict__ sem_sorted = A.sem_sorted;
-    const float4* __restrict__ col4 = A.col4;
-    long long* __restrict__ acc = A.acc;
+    constexpr int SW = lane_row_words<DP, BF16>();
     const GridParams& gp = A.gp;
-    constexpr int SW = SemRow<DP, BF16>::WORDS;
-    float4* smw = reinterpret_cast<float4*>(wb);                      // [UQ] walk records
-    float* smt = wb + 4 * UQ;                                         // [UQ/2][8] test records
-    float4* scq = reinterpret_cast<float4*>(wb + 8 * UQ);             // [UQ] query colours
-    float* ssq = wb + (COLOR ? 12 : 8) * UQ;                          // [UQ][SW] query labels
-    float* ri = ssq + UQ * SW;
-    const Rows R{reinterpret_cast<int4*>(ri), reinterpret_cast<float2*>(ri + 36)};
-    float4* sacc = reinterpret_cast<float4*>(ri + ROWS_WORDS) + lane * (N_ACC / 4);   // this lane's unit sums
-    float4* cq = reinterpret_cast<float4*>(ri + ROWS_WORDS) + 32 * (N_ACC / 4);       // candidate ring
-    float* gram = reinterpret_cast<float*>(cq + CQ_N);                        // [query][candidate] (BF16)
-    const ulonglong2* walk2 = reinterpret_cast<const ulonglong2*>(smw);
-    const ulonglong2* test2 = reinterpret_cast<const ulonglong2*>(smt);
-    const u64 H2 = f2(0.5f, 0.5f);
+    float* cg = wb;
+    float* cc = wb + 16 * 8;
+    float* srow = cc + (COLOR ? 16 * 8 : 0);
+    float4* cq = reinterpret_cast<float4*>(srow + 32 * SW);
+    const Rows R{reinterpret_cast<int4*>(cq + CQ_N), reinterpret_cast<float2*>(cq + CQ_N + 9)};
+    const float INF = __int_as_float(0x7f800000);
     const int k0 = unit.x, qcount = unit.y & 127, e = unit.y >> 7;
-    const uint32_t key0 = qkey[k0] >> gp.key_sub;            // home-cell key
-    const FrameDev& Fa = frames[edges[e].a];
-    const int cell = (int)(key0 - edges[e].bin_off);
+    const uint32_t key0 = A.qkey[k0] >> gp.key_sub;            // home-cell key
+    const FrameDev& Fa = A.frames[A.edges[e].a];
+    const int cell = (int)(key0 - A.edges[e].bin_off);
     const int hx = cell % Fa.dim[0], hy = (cell / Fa.dim[0]) % Fa.dim[1], hz = cell / (Fa.dim[0] * Fa.dim[1]);
-    __syncwarp();
-    // bounding box of the unit's queries (home-centre coordinates)
-    float blo0 = __int_as_float(0x7f800000), blo1 = blo0, blo2 = blo0;
-    float bhi0 = -blo0, bhi1 = -blo0, bhi2 = -blo0;
-    {
-        const int q = lane;
-        float* tq = smt + 8 * (q >> 1) + (q & 1);
-        if (q < qcount) {
-            const float4 r = slots[(long long)k0 + q];
-            blo0 = bhi0 = r.x;
-            blo1 = bhi1 = r.y;
-            blo2 = bhi2 = r.z;
-            const int s = __float_as_int(r.w);
-            const float mx = -2.f * r.x, my = -2.f * r.y, mz = -2.f * r.z;
-            smw[q] = make_float4(mx, my, mz, mx);
-            tq[0] = mx;
-            tq[2] = my;
-            tq[4] = mz;
-            tq[6] = fmaf(r.x, r.x, fmaf(r.y, r.y, r.z * r.z));
-            if (COLOR) scq[q] = __ldg(col4 + s);
-            SemRow<DP, BF16>::stage(ssq + q * SW, sem_sorted, s);
-        } else if (q == qcount && (q & 1)) {
-            // odd count: the partner slot of the last pair never passes
-            tq[0] = 0.f;
-            tq[2] = 0.f;
-            tq[4] = 0.f;
-            tq[6] = __int_as_float(0x7f800000);
-        }
-    }
+    // 2^gs lanes per query: the lane's query, and its place among them
+    const int gs = qcount > 16 ? 0 : (qcount > 8 ? 1 : (qcount > 4 ? 2 : 3));
+    const int ql = lane & ((32 >> gs) - 1), gi = lane >> (5 - gs);
+    const bool qv = ql < qcount;
+    const float4 r = qv ? A.slots[(long long)k0 + ql] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const int sidx = __float_as_int(r.w);
+    const float mx = -2.f * r.x, my = -2.f * r.y, mz = -2.f * r.z;
+    const float mw = qv ? fmaf(r.x, r.x, fmaf(r.y, r.y, r.z * r.z)) : INF;      // an absent query fails every test
+    Sem<DP, BF16> qs;
+    if (DP > 0) qs.load(A.sem_sorted, sidx, qv);
+    float4 qc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (COLOR && qv) qc = __ldg(A.col4 + sidx);
+    float blo0 = qv ? r.x : INF, blo1 = qv ? r.y : INF, blo2 = qv ? r.z : INF;
+    float bhi0 = qv ? r.x : -INF, bhi1 = qv ? r.y : -INF, bhi2 = qv ? r.z : -INF;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         blo0 = fminf(blo0, __shfl_xor_sync(FULL, blo0, o));
@@ -1546,235 +1431,142 @@ __device__ __forceinline__ void pair_unit(const PairArgs& A, int2 unit, int part
         bhi1 = fmaxf(bhi1, __shfl_xor_sync(FULL, bhi1, o));
         bhi2 = fmaxf(bhi2, __shfl_xor_sync(FULL, bhi2, o));
     }
+    __syncwarp();
     // a candidate farther than r_c from the query box pairs with none of
     // the queries; the margin keeps every candidate the exact test passes
     const float box_thr = gp.rc2 * 1.0001f;
     int n_seg;
-    const int C = build_rows(R, cell_start, Fa, hx, hy, hz, blo0, blo1, blo2, bhi0, bhi1, bhi2, gp.hf, box_thr, lane, n_seg);
+    const int C = build_rows(R, A.cell_start, Fa, hx, hy, hz, blo0, blo1, blo2, bhi0, bhi1, bhi2, gp.hf, box_thr, lane,
+                             n_seg);
     int c_s, c_hi;                               // chunks of the stream
     part_range(C, part, shift, c_s, c_hi);
     if (c_s >= c_hi) return;
-    const int np = (qcount + 1) >> 1;
-    // BF16 labels: the Gram path leaves registers free, so the query-side MMA
-    // fragments and the per-lane unit sums live in registers instead of
-    // shared memory
-    constexpr bool REG = BF16 && DP > 0;
-    GramB<(BF16 && DP > 0) ? DP : 16> gb;
-    if constexpr (REG) gb.load(ssq, lane);
-
-    // per lane, over its candidates x with sums w0 = sum w, dc = sum w d,
-    // qc = sum w d d^T: W, D, Q and sum w0 x, sum w0 x x^T, sum x dc^T
-    float racc[REG ? N_ACC : 1];
-    if constexpr (REG) {
-#pragma unroll
-        for (int k = 0; k < N_ACC; ++k) racc[k] = 0.f;
-    } else {
-#pragma unroll
-        for (int k = 0; k < N_ACC / 4; ++k) sacc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    const u64 MX = f2(mx, mx), MY = f2(my, my), MZ = f2(mz, mz), MW = f2(mw, mw);
+    const u64 H2 = f2(0.5f, 0.5f), KG2 = f2(gp.kg, gp.kg);
+    u64 W2 = 0ull, D2[3] = {0ull, 0ull, 0ull}, Q2[6] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};   // halves: even, odd candidates
     int cnt = 0;
-    int qhead = 0, qlen = 0;                     // ring head and fill
-    Cursor cur;
-    cur.start(R, n_seg, 32 * c_s + lane);
-    while (c_s < c_hi || qlen > 0) {
-        // stream the 27-cell candidates through the box test into the
-        // ring until it holds a full batch (or the stream ends)
-        while (qlen < 32 && c_s < c_hi) {
-            bool keep = false;
-            float4 ent = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (cur.valid()) {
-                ent = cur.point(pts4, gp.hf);
-                const float e0 = fmaxf(fmaxf(blo0 - ent.x, ent.x - bhi0), 0.f);
-                const float e1 = fmaxf(fmaxf(blo1 - ent.y, ent.y - bhi1), 0.f);
-                const float e2 = fmaxf(fmaxf(blo2 - ent.z, ent.z - bhi2), 0.f);
-                keep = fmaf(e0, e0, fmaf(e1, e1, e2 * e2)) < box_thr;
+    // the batches, compiled with and without the pruning test
+    auto batches = [&](auto prune) {
+        constexpr bool PRUNE = decltype(prune)::value;
+        int qhead = 0, qlen = 0;                 // ring head and fill
+        Cursor cur;
+        cur.start(R, n_seg, 32 * c_s + lane);
+        while (c_s < c_hi || qlen > 0) {
+            // stream the 27-cell candidates through the box test into the
+            // ring until it holds a full batch (or the stream ends)
+            while (qlen < 32 && c_s < c_hi) {
+                bool keep = false;
+                float4 ent = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (cur.valid()) {
+                    ent = cur.point(A.pts4, gp.hf);
+                    const float e0 = fmaxf(fmaxf(blo0 - ent.x, ent.x - bhi0), 0.f);
+                    const float e1 = fmaxf(fmaxf(blo1 - ent.y, ent.y - bhi1), 0.f);
+                    const float e2 = fmaxf(fmaxf(blo2 - ent.z, ent.z - bhi2), 0.f);
+                    keep = fmaf(e0, e0, fmaf(e1, e1, e2 * e2)) < box_thr;
+                }
+                const unsigned bal = __ballot_sync(FULL, keep);
+                if (keep) cq[(qhead + qlen + __popc(bal & ((1u << lane) - 1u))) & (CQ_N - 1)] = ent;
+                qlen += __popc(bal);
+                ++c_s;
+                cur.next(R, n_seg);
             }
-            const unsigned bal = __ballot_sync(FULL, keep);
-            if (keep) cq[(qhead + qlen + __popc(bal & ((1u << lane) - 1u))) & (CQ_N - 1)] = ent;
-            qlen += __popc(bal);
-            ++c_s;
-            cur.next(R, n_seg);
-        }
-        __syncwarp();
-        const int nb = qlen < 32 ? qlen : 32;
-        if (nb == 0) break;                      // stream ended with the ring empty
-        const bool has = lane < nb;
-        const float4 ent = has ? cq[(qhead + lane) & (CQ_N - 1)] : make_float4(0.f, 0.f, 0.f, 0.f);
-        qhead = (qhead + nb) & (CQ_N - 1);
-        qlen -= nb;
-        __syncwarp();
-        const int i = __float_as_int(ent.w);
-        // candidate relative to the home cell centre
-        const float x0 = ent.x, x1 = ent.y, x2 = ent.z;
-        const float xx = fmaf(x0, x0, fmaf(x1, x1, x2 * x2));
-        const float thr = gp.rc2 - xx;
-        Sem<DP, BF16> cs;
-        if (DP > 0 && !BF16) cs.load(sem_sorted, i, has);
-        float4 cc = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (COLOR && has) cc = __ldg(col4 + i);
-        // cutoff test against query pairs: bit j set when |x - y_j| < r_c
-        unsigned mk = 0u;
-        {
-            const u64 X0 = f2(x0, x0), X1 = f2(x1, x1), X2 = f2(x2, x2);
-#pragma unroll 4
-            for (int pj = 0; pj < np; ++pj) {
-                const ulonglong2 a = test2[2 * pj], b = test2[2 * pj + 1];
-                const float2 t = f2_split(ffma2(X0, a.x, ffma2(X1, a.y, ffma2(X2, b.x, b.y))));
-                mk |= ((t.x < thr ? 1u : 0u) | (t.y < thr ? 2u : 0u)) << (2 * pj);
+            __syncwarp();
+            const int nb = qlen < 32 ? qlen : 32;
+            if (nb == 0) break;                  // stream ended with the ring empty
+            // lane c stages candidate c (absent ones: thr = -inf, the label row left as it is)
+            {
+                const bool has = lane < nb;
+                const float4 ent = has ? cq[(qhead + lane) & (CQ_N - 1)] : make_float4(0.f, 0.f, 0.f, 0.f);
+                const int i = __float_as_int(ent.w);
+                float* g = cg + 8 * (lane >> 1) + (lane & 1);
+                g[0] = ent.x;
+                g[2] = ent.y;
+                g[4] = ent.z;
+                g[6] = has ? gp.rc2 - fmaf(ent.x, ent.x, fmaf(ent.y, ent.y, ent.z * ent.z)) : -INF;
+                if constexpr (COLOR) {
+                    const float4 c = has ? __ldg(A.col4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    float* k = cc + 8 * (lane >> 1) + (lane & 1);
+                    k[0] = c.x;
+                    k[2] = c.y;
+                    k[4] = c.z;
+                }
+                if (has) SemRow<DP, BF16>::stage(srow + lane * SW, A.sem_sorted, i);
             }
-        }
-        if (!has) mk = 0u;
-        if constexpr (BF16 && DP > 0) {
-            label_gram_bf16<DP>(reinterpret_cast<const unsigned*>(sem_sorted), gb, i, __ballot_sync(FULL, has),
-                                lane, gram);
+            qhead = (qhead + nb) & (CQ_N - 1);
+            qlen -= nb;
+            __syncwarp();
+            const int n_it = (((nb + 1) >> 1) + (1 << gs) - 1) >> gs;
+            for (int j = 0; j < n_it; ++j) {
+                const int p = (j << gs) + gi;
+                const ulonglong2 x01 = *reinterpret_cast<const ulonglong2*>(cg + 8 * p);
+                const ulonglong2 x2t = *reinterpret_cast<const ulonglong2*>(cg + 8 * p + 4);
+                const float2 t = f2_split(ffma2(x01.x, MX, ffma2(x01.y, MY, ffma2(x2t.x, MZ, MW))));
+                const float2 thr = f2_split(x2t.y);
+                bool in0 = t.x < thr.x, in1 = t.y < thr.y;
+                const u64 E0 = ffma2(H2, MX, x01.x), E1 = ffma2(H2, MY, x01.y), E2 = ffma2(H2, MZ, x2t.x);
+                u64 arg = fmul2(ffma2(E0, E0, ffma2(E1, E1, fmul2(E2, E2))), KG2);
+                if constexpr (COLOR) {
+                    const ulonglong2 c01 = *reinterpret_cast<const ulonglong2*>(cc + 8 * p);
+                    const u64 c2 = *reinterpret_cast<const u64*>(cc + 8 * p + 4);
+                    const u64 r0 = fadd2(c01.x, f2(-qc.x, -qc.x)), r1 = fadd2(c01.y, f2(-qc.y, -qc.y)),
+                              r2 = fadd2(c2, f2(-qc.z, -qc.z));
+                    arg = ffma2(ffma2(r0, r0, ffma2(r1, r1, fmul2(r2, r2))), f2(gp.kc, gp.kc), arg);
+                }
+                const float2 a = f2_split(arg);
+                float w0 = ex2_approx(a.x), w1 = ex2_approx(a.y);
+                if constexpr (DP > 0) {
+                    const float s0 = SemRow<DP, BF16>::dot(qs, srow + (2 * p) * SW);
+                    const float s1 = SemRow<DP, BF16>::dot(qs, srow + (2 * p + 1) * SW);
+                    if constexpr (PRUNE) {
+                        in0 = in0 && s0 >= gp.sem_min;
+                        in1 = in1 && s1 >= gp.sem_min;
+                    }
+                    w0 *= s0;
+                    w1 *= s1;
+                }
+                cnt += (in0 ? 1 : 0) + (in1 ? 1 : 0);
+                const u64 w = f2(in0 ? w0 : 0.f, in1 ? w1 : 0.f);
+                const u64 WX = fmul2(w, E0), WY = fmul2(w, E1), WZ = fmul2(w, E2);
+                W2 = fadd2(W2, w);
+                D2[0] = fadd2(D2[0], WX);
+                D2[1] = fadd2(D2[1], WY);
+                D2[2] = fadd2(D2[2], WZ);
+                Q2[0] = ffma2(WX, E0, Q2[0]);
+                Q2[1] = ffma2(WX, E1, Q2[1]);
+                Q2[2] = ffma2(WX, E2, Q2[2]);
+                Q2[3] = ffma2(WY, E1, Q2[3]);
+                Q2[4] = ffma2(WY, E2, Q2[4]);
+                Q2[5] = ffma2(WZ, E2, Q2[5]);
+            }
             __syncwarp();
         }
-        const u64 XA = f2(x0, x1), XB = f2(x2, x0);
-        float w0 = 0.f, dz_s = 0.f, q12 = 0.f, q22 = 0.f;
-        u64 D01 = 0ull, Q0011 = 0ull, Q0201 = 0ull;
-        // the bit walk, compiled twice: with the semantic-pruning test
-        // only when pruning is on (a uniform branch per batch).  Each
-        // iteration takes 4 of the lane's pairs as independent dependency
-        // chains (missing ones weigh zero); at 2 CTAs per SM the registers
-        // for them are there, and the ILP hides more latency than a third
-        // CTA's warps did.
-        auto walk = [&](auto prune) {
-            constexpr bool PRUNE = decltype(prune)::value;
-            auto pair_w = [&](int j, u64& E01, u64& E20, float& ez, bool& kept) -> float {
-                const ulonglong2 m = walk2[j];
-                E01 = ffma2(H2, m.x, XA);
-                E20 = ffma2(H2, m.y, XB);
-                const float2 exy = f2_split(E01);
-                ez = f2_split(E20).x;
-                const float dd = fmaf(exy.x, exy.x, fmaf(exy.y, exy.y, ez * ez));
-                float arg = dd * gp.kg;
-                if (COLOR) {
-                    const float4 qc = scq[j];
-                    const float cr = cc.x - qc.x, cg = cc.y - qc.y, cb = cc.z - qc.z;
-                    arg = fmaf(fmaf(cr, cr, fmaf(cg, cg, cb * cb)), gp.kc, arg);
-                }
-                float s;
-                if constexpr (BF16 && DP > 0) s = gram[j * GRAM_LD + gram_col(j, lane)];
-                else s = SemRow<DP, BF16>::dot(cs, ssq + j * SW);
-                kept = true;
-                if constexpr (PRUNE) kept = s >= gp.sem_min;
-                return kept ? s * ex2_approx(arg) : 0.f;
-            };
-            auto add = [&](float w, u64 E01, u64 E20, float ez, bool kept) {
-                const u64 WXY = fmul2(f2(w, w), E01);
-                const float wz = w * ez;
-                w0 += w;
-                D01 = fadd2(D01, WXY);
-                dz_s += wz;
-                Q0011 = ffma2(WXY, E01, Q0011);
-                Q0201 = ffma2(WXY, E20, Q0201);
-                q12 = fmaf(f2_split(WXY).y, ez, q12);
-                q22 = fmaf(wz, ez, q22);
-                cnt += kept ? 1 : 0;
-            };
-            constexpr int U = 4;   // pairs per iteration
-            while (__any_sync(FULL, mk != 0u)) {
-                if (mk) {
-                    int jj[U];
-                    bool hv[U];
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        hv[u] = mk != 0u;
-                        jj[u] = hv[u] ? __ffs(mk) - 1 : 0;
-                        if (hv[u]) mk &= mk - 1u;
-                    }
-                    u64 Ea[U], Eb[U];
-                    float ez[U], w[U];
-                    bool kp[U];
-#pragma unroll
-                    for (int u = 0; u < U; ++u) w[u] = pair_w(jj[u], Ea[u], Eb[u], ez[u], kp[u]);
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        if (!hv[u]) { w[u] = 0.f; kp[u] = false; }
-                        add(w[u], Ea[u], Eb[u], ez[u], kp[u]);
-                    }
-                }
-            }
-        };
-        if (DP > 0 && gp.sem_min > -__int_as_float(0x7f800000)) walk(std::true_type{});
-        else walk(std::false_type{});
-        const float2 dxy = f2_split(D01), q0011 = f2_split(Q0011), q0201 = f2_split(Q0201);
-        const float x[3] = {x0, x1, x2};
-        const float dc[3] = {dxy.x, dxy.y, dz_s};
-        const float qc[6] = {q0011.x, q0201.y, q0201.x, q0011.y, q12, q22};
-        float a_s[REG ? 1 : N_ACC];
-        float* a = REG ? racc : a_s;
-        if constexpr (!REG) {
-#pragma unroll
-            for (int k = 0; k < N_ACC / 4; ++k) {
-                const float4 t = sacc[k];
-                a[4 * k] = t.x; a[4 * k + 1] = t.y; a[4 * k + 2] = t.z; a[4 * k + 3] = t.w;
-            }
-        }
-        a[A_W] += w0;
-#pragma unroll
-        for (int t6 = 0; t6 < 6; ++t6) a[A_Q + t6] += qc[t6];
-#pragma unroll
-        for (int mm = 0; mm < 3; ++mm) {
-            a[A_D + mm] += dc[mm];
-            const float wx = w0 * x[mm];
-            a[A_SWX + mm] += wx;
-#pragma unroll
-            for (int l = 0; l < 3; ++l) a[A_SXD + 3 * mm + l] = fmaf(x[mm], dc[l], a[A_SXD + 3 * mm + l]);
-#pragma unroll
-            for (int l = mm; l < 3; ++l) {
-                const int t6 = mm == 0 ? l : (mm == 1 ? 2 + l : 5);
-                a[A_SWXX + t6] = fmaf(wx, x[l], a[A_SWXX + t6]);
-            }
-        }
-        if constexpr (!REG) {
-#pragma unroll
-            for (int k = 0; k < N_ACC / 4; ++k)
-                sacc[k] = make_float4(a[4 * k], a[4 * k + 1], a[4 * k + 2], a[4 * k + 3]);
-        }
-    }
+    };
+    if (DP > 0 && gp.sem_min > -INF) batches(std::true_type{});
+    else batches(std::false_type{});
     if (!__any_sync(FULL, cnt != 0)) return;     // no pair: every sum is zero
-    float a_s[REG ? 1 : N_ACC];
-    float* a = REG ? racc : a_s;
-    if constexpr (!REG) {
+    auto both = [](u64 v) { const float2 h = f2_split(v); return h.x + h.y; };
+    const float W = both(W2), y[3] = {r.x, r.y, r.z};
+    float Dv[3], Sy[3], Myy[6], Mdy[9], Qm[6];
 #pragma unroll
-        for (int k = 0; k < N_ACC / 4; ++k) {
-            const float4 t = sacc[k];
-            a[4 * k] = t.x; a[4 * k + 1] = t.y; a[4 * k + 2] = t.z; a[4 * k + 3] = t.w;
+    for (int m = 0; m < 3; ++m) {
+        Dv[m] = both(D2[m]);
+        Sy[m] = W * y[m];
+    }
+    int t6 = 0;
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+#pragma unroll
+        for (int l = 0; l < 3; ++l) Mdy[3 * m + l] = Dv[m] * y[l];
+#pragma unroll
+        for (int l = m; l < 3; ++l, ++t6) {
+            Myy[t6] = Sy[m] * y[l];
+            Qm[t6] = both(Q2[t6]);
         }
     }
-    const float W = a[A_W];
-    const float Dv[3] = {a[A_D], a[A_D + 1], a[A_D + 2]};
-    const float* Qm = a + A_Q;
-    const float* Swx = a + A_SWX;
-    const float* Swxx = a + A_SWXX;
-    const float* Sxd = a + A_SXD;
-    // y' = x - d:  sum w y' = sum w0 x - D;  sum w y'y'^T = sum w0 x x^T -
-    // sum (x dc^T + dc x^T) + Q;  sum w d y'^T = sum dc x^T - Q
-    float Sy[3], Myy[6], Mdy[9];
-#pragma unroll
-    for (int mm = 0; mm < 3; ++mm) Sy[mm] = Swx[mm] - Dv[mm];
-#pragma unroll
-    for (int mm = 0; mm < 3; ++mm)
-#pragma unroll
-        for (int l = mm; l < 3; ++l) {
-            const int t6 = mm == 0 ? l : (mm == 1 ? 2 + l : 5);
-            Myy[t6] = Swxx[t6] - (Sxd[3 * mm + l] + Sxd[3 * l + mm]) + Qm[t6];
-        }
-#pragma unroll
-    for (int mm = 0; mm < 3; ++mm)
-#pragma unroll
-        for (int l = 0; l < 3; ++l) {
-            const int qi = (mm <= l) ? (mm == 0 ? l : (mm == 1 ? 2 + l : 5))
-                                     : (l == 0 ? mm : (l == 1 ? 2 + mm : 5));
-            Mdy[3 * mm + l] = Sxd[3 * l + mm] - Qm[qi];
-        }
-    store_moments(W, Dv, Sy, Myy, Mdy, Qm, cnt, Fa, hx, hy, hz, gp, edges[e].scale,
-                  acc + (long long)e * ACC_N, lane);
-
+    store_moments(W, Dv, Sy, Myy, Mdy, Qm, cnt, Fa, hx, hy, hz, gp, A.edges[e].scale, A.acc + (long long)e * ACC_N, lane);
 }
 
-// Shared-memory words per warp of the bit-walk or the dense tile unit.
+// Shared-memory words per warp of the lane or the dense tile unit.
 template <int DP, bool BF16, bool COLOR, bool DENSE>
 __host__ __device__ constexpr int unit_smem_words() {
     if constexpr (DENSE) return DenseSmem<(DP > 0 ? DP : 8), !BF16>::WORDS;
@@ -1878,13 +1670,9 @@ k_pairs_multi(const PairJob* __restrict__ jobs, int n_jobs, int* unit_counter) {
 // smallest, instead of one for every candidate that any lane takes.
 // 8 x 20k LiDAR, top_k = 8: evaluation 724 -> 645 us.  Three CTAs per SM (80
 // registers) spill: slower than the start.
-template <int DP, bool BF16>
-__host__ __device__ constexpr int topk_row_words() {   // row stride of the staged labels: lanes read up to 8 rows at a time
-    return SemRow<DP, BF16>::WORDS + (SemRow<DP, BF16>::WORDS % 8 == 0 && DP > 0 ? 4 : 0);
-}
 template <int DP, bool BF16, bool COLOR>
 __host__ __device__ constexpr int warp_smem_words_topk() {
-    return 32 * 4 + 32 * topk_row_words<DP, BF16>() + (COLOR ? 32 * 4 : 0) + 4 * CQ_N + ROWS_WORDS + 32 * 32;
+    return 32 * 4 + 32 * lane_row_words<DP, BF16>() + (COLOR ? 32 * 4 : 0) + 4 * CQ_N + ROWS_WORDS + 32 * 32;
 }
 
 // (w, i) comes before (v, j): larger weight, of equal ones the earlier point
@@ -1900,7 +1688,7 @@ k_pairs_topk(const int2* __restrict__ units, const int* __restrict__ n_units, in
              long long* __restrict__ acc, const int* done) {
     if (done && *done) return;
     extern __shared__ float4 smem4[];
-    constexpr int SW = topk_row_words<DP, BF16>();
+    constexpr int SW = lane_row_words<DP, BF16>();
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     float* wb = reinterpret_cast<float*>(smem4) + warp * warp_smem_words_topk<DP, BF16, COLOR>();
@@ -2213,7 +2001,7 @@ inline unsigned pair_grid(int num_sms, int resident, int ctas_per_sm) {
 
 // The dense tile unit serves BF16 labels without colour and without
 // semantic pruning (top_k has its own kernel); RK_NO_DENSE builds the
-// bit-walk kernel for every layout.
+// lane kernel for every layout.
 inline bool dense_path(const GridParams& gp) {
 #ifdef RK_NO_DENSE
     (void)gp;

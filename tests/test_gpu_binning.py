@@ -6,7 +6,8 @@ thread), larger ones by the tiled sort (tiles of 2048 and, from 5 M queries on,
 whose first query is or is not the first of all, and streams long enough to be shared by
 several warps.  Tolerances are those of the parity tests (loss 1e-5, gradient and
 Gauss-Newton matrix 1e-4 relative); in the clumps every pair lies inside the cutoff, so
-their counts are exact.
+their counts are exact.  Units of few queries share a query among lanes (steps at 4, 8
+and 16 queries): counts around them, with streams of a part of a batch to many.
 """
 import numpy as np
 import pytest
@@ -78,3 +79,15 @@ def test_cells_longer_than_a_block(pk, variant, na, nb, lead):
 @pytest.mark.parametrize("n", [1023, 1025, 2048, 3073, 4096, 4097, 6145, 10240, 10241])
 def test_query_counts_around_a_tile(pk, n):
     _check(pk, scenes.tiny_problem(seed=40 + n % 7, n_frames=2, n=n, extent=2.5 if n < 4000 else 4.0, ell=0.1))
+
+
+@pytest.mark.parametrize("variant,extra", [("plain", {}), ("color", {}), ("fp32", dict(sem_min=0.1)),
+                                           ("bf16", dict(sem_min=0.1)), ("plain", dict(top_k=8)),
+                                           ("color", dict(top_k=3)), ("fp32", dict(top_k=8)),
+                                           ("bf16", dict(top_k=1, sem_min=0.1))])
+@pytest.mark.parametrize("nb", [1, 4, 5, 8, 9, 16, 17, 32, 33])
+def test_units_of_few_queries(pk, variant, extra, nb):
+    for na in (1, 2, 33, 300):
+        prob = _clump(na, nb, 1, variant)
+        prob["params"] = dict(prob["params"], **extra)
+        _check(pk, prob)
