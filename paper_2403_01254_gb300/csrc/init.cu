@@ -39,23 +39,53 @@ __device__ double block_sum(double v, double* sh) {
     return r;
 }
 
+// Inputs of the rotation batch, frame a and N_ROT copies of frame b, in one launch
+// (blockIdx.y: which frame of the batch), with the partial sums of the two
+// frames' points: a copy call per array and frame was 61 to 183 of them, each
+// of some microseconds of host time.  part: [2][gridDim.x][3].
+constexpr int ROT_T = 256;
+__global__ void __launch_bounds__(ROT_T) k_rot_batch(const double* __restrict__ xyz, const float* __restrict__ sem,
+                                                     const float* __restrict__ rgb, int sem_dim, long long off_a,
+                                                     long long n_a, long long off_b, long long n_b,
+                                                     double* __restrict__ xyz_out, float* __restrict__ sem_out,
+                                                     float* __restrict__ rgb_out, double* __restrict__ part) {
+    __shared__ double sh[ROT_T / 32][3];
+    const int f = blockIdx.y;
+    const long long n = f == 0 ? n_a : n_b, so = f == 0 ? off_a : off_b, dst = f == 0 ? 0 : n_a + (f - 1) * n_b;
+    const long long t0 = blockIdx.x * (long long)ROT_T + threadIdx.x, nt = (long long)gridDim.x * ROT_T;
+    for (long long i = t0; i < 3 * n; i += nt) xyz_out[3 * dst + i] = xyz[3 * so + i];
+    if (sem)
+        for (long long i = t0; i < sem_dim * n; i += nt) sem_out[sem_dim * dst + i] = sem[sem_dim * so + i];
+    if (rgb)
+        for (long long i = t0; i < 3 * n; i += nt) rgb_out[3 * dst + i] = rgb[3 * so + i];
+    if (f >= 2) return;
+    double s[3] = {0.0, 0.0, 0.0};
+    for (long long i = t0; i < n; i += nt)
+        for (int k = 0; k < 3; ++k) s[k] += xyz[3 * (so + i) + k];
+    for (int k = 0; k < 3; ++k)
+        for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+    if ((threadIdx.x & 31) == 0)
+        for (int k = 0; k < 3; ++k) sh[threadIdx.x >> 5][k] = s[k];
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        double t = 0.0;
+        for (int w = 0; w < ROT_T / 32; ++w) t += sh[w][threadIdx.x];
+        part[3 * (f * (long long)gridDim.x + blockIdx.x) + threadIdx.x] = t;
+    }
+}
+
 // Candidate poses of the rotation search: pose 0 = T_a, pose 1 + k =
-// T_a [R_k | mu_a - R_k mu_b], mu the frame-local centroids.  One block.
-__global__ void k_rot_candidates(const double* __restrict__ xyz, long long off_a, long long n_a,
-                                 long long off_b, long long n_b, const double* __restrict__ Ta,
-                                 const double* __restrict__ R, double* __restrict__ poses) {
-    __shared__ double sh[256];
+// T_a [R_k | mu_a - R_k mu_b], mu the frame-local centroids (from the n_part
+// partial sums of each frame).  One block.
+__global__ void k_rot_candidates(const double* __restrict__ part, int n_part, long long n_a, long long n_b,
+                                 const double* __restrict__ Ta, const double* __restrict__ R,
+                                 double* __restrict__ poses) {
     __shared__ double mu[6];
-    for (int f = 0; f < 2; ++f) {
-        const long long off = f ? off_b : off_a;
-        const long long n = f ? n_b : n_a;
-        double s[3] = {0.0, 0.0, 0.0};
-        for (long long i = threadIdx.x; i < n; i += blockDim.x)
-            for (int k = 0; k < 3; ++k) s[k] += xyz[3 * (off + i) + k];
-        for (int k = 0; k < 3; ++k) {
-            const double t = block_sum(s[k], sh);
-            if (threadIdx.x == 0) mu[3 * f + k] = t / (double)n;
-        }
+    if (threadIdx.x < 6) {
+        const int f = threadIdx.x / 3, k = threadIdx.x % 3;
+        double t = 0.0;
+        for (int i = 0; i < n_part; ++i) t += part[3 * (f * n_part + i) + k];
+        mu[threadIdx.x] = t / (double)(f ? n_b : n_a);
     }
     __syncthreads();
     const int k = threadIdx.x;
@@ -319,20 +349,15 @@ rkhsba_status rkhsba_rotation_search(rkhsba_ctx* c, int32_t a, int32_t b, const 
     RK_TRY(tmp_alloc(c, bx, &d_xyz, 3 * n_child));
     if (c->d_sem_in) RK_TRY(tmp_alloc(c, bs, &d_sem, (long long)sd * n_child));
     if (c->d_rgb_in) RK_TRY(tmp_alloc(c, bc, &d_rgb, 3 * n_child));
-    for (int f = 0; f <= N_ROT; ++f) {
-        const int src = f == 0 ? a : b;
-        const long long n = f == 0 ? na : nb;
-        const long long dst = f == 0 ? 0 : na + (long long)(f - 1) * nb;
-        const long long so = c->pt_off[src];
-        RK_CUDA(c, cudaMemcpyAsync(d_xyz + 3 * dst, c->d_xyz + 3 * so, sizeof(double) * 3 * n,
-                                   cudaMemcpyDeviceToDevice, st));
-        if (d_sem)
-            RK_CUDA(c, cudaMemcpyAsync(d_sem + (long long)sd * dst, c->d_sem_in + (long long)sd * so,
-                                       sizeof(float) * sd * n, cudaMemcpyDeviceToDevice, st));
-        if (d_rgb)
-            RK_CUDA(c, cudaMemcpyAsync(d_rgb + 3 * dst, c->d_rgb_in + 3 * so, sizeof(float) * 3 * n,
-                                       cudaMemcpyDeviceToDevice, st));
-    }
+    const int n_part = (int)std::min<long long>((std::max(na, nb) + ROT_T - 1) / ROT_T, 64);
+    double* d_in = nullptr;              // rotations and T_a, results, partial sums
+    constexpr int N_IN = 9 * N_ROT + 16, N_OUT = N_ROT + 17;
+    RK_TRY(tmp_alloc(c, bp, &d_in, (long long)N_IN + N_OUT + 6 * n_part));
+    double* d_out = d_in + N_IN;
+    double* d_part = d_out + N_OUT;
+    k_rot_batch<<<dim3((unsigned)n_part, 1 + N_ROT), ROT_T, 0, st>>>(c->d_xyz, c->d_sem_in, c->d_rgb_in, sd, c->pt_off[a],
+                                                                     na, c->pt_off[b], nb, d_xyz, d_sem, d_rgb, d_part);
+    count_launch();
     std::vector<int64_t> n_pts(1 + N_ROT, nb);
     n_pts[0] = na;
     std::vector<int32_t> edges(2 * N_ROT);
@@ -349,21 +374,17 @@ rkhsba_status rkhsba_rotation_search(rkhsba_ctx* c, int32_t a, int32_t b, const 
     // rotation table and T_a
     const std::vector<Mat3>& G = icosahedral_group();
     if (G.size() != (size_t)N_ROT) return ctx_fail(c, RKHSBA_EINVAL, "icosahedral group construction failed");
-    std::vector<double> hin(9 * N_ROT + 16);
+    std::vector<double> hin(N_IN);
     for (int k = 0; k < N_ROT; ++k) std::copy(G[k].begin(), G[k].end(), hin.begin() + 9 * k);
     std::copy(poses + 16 * a, poses + 16 * a + 16, hin.begin() + 9 * N_ROT);
-    double* d_in = nullptr;
-    RK_TRY(tmp_alloc(c, bp, &d_in, (long long)hin.size() + N_ROT + 17));
-    double* d_out = d_in + hin.size();
     RK_CUDA(c, cudaMemcpyAsync(d_in, hin.data(), sizeof(double) * hin.size(), cudaMemcpyHostToDevice, st));
-    k_rot_candidates<<<1, 256, 0, st>>>(c->d_xyz, c->pt_off[a], na, c->pt_off[b], nb, d_in + 9 * N_ROT, d_in,
-                                        child->d_poses_cand);
+    k_rot_candidates<<<1, 64, 0, st>>>(d_part, n_part, na, nb, d_in + 9 * N_ROT, d_in, child->d_poses_cand);
     count_launch();
     ctx_run_eval(child, child->d_poses_cand);
     k_rot_select<<<1, 64, 0, st>>>(child->d_eout, c->self_ctx->d_eout + a, c->self_ctx->d_eout + b,
                                    child->d_poses_cand, d_out);
     count_launch();
-    std::vector<double> h(N_ROT + 17);
+    std::vector<double> h(N_OUT);
     RK_CUDA(c, cudaMemcpyAsync(h.data(), d_out, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, st));
     RK_CUDA(c, cudaStreamSynchronize(st));
     RK_CUDA(c, cudaGetLastError());
