@@ -29,6 +29,31 @@ inline void count_launch(long long n = 1) {
     t_launches += n;
 }
 
+// Kernels of a chain start while their predecessor runs out: each waits for it
+// (and for its stores) before it touches memory, and lets its own successor be
+// launched once all its blocks have started, so that only the launch
+// itself overlaps.  Without the launch attribute both are no-ops.
+// 2 x 2000 RGB-D evaluation 79 -> 72 us, 10-iteration solve 780 -> 759 us, 5 x 20k
+// evaluation 200 -> 191 us; large problems unchanged.
+__device__ __forceinline__ void chain_enter() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... P, typename... A>
+inline void launch_chained(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 constexpr int MAX_SEM = 32;     // label floats per point
 constexpr int ACC_N = 32;       // int64 accumulator slots per edge
 constexpr int N_MOM = 29;       // used slots (see MomentIndex)

@@ -37,6 +37,7 @@ __global__ void k_bbox(const double* __restrict__ xyz, const float* __restrict__
                        const float* __restrict__ rgb, long long N, int K,
                        const long long* __restrict__ pt_off, int sem_dim, double h_inv,
                        int* cmin, int* cmax, unsigned* sem_norm_bits, int* err) {
+    chain_enter();
     __shared__ float s_row[GT / 32][32 * 33];
     const double lim = 536870912.0;   // 2^29
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -135,6 +136,7 @@ __global__ void __launch_bounds__(RAD_T) k_keys(const double* __restrict__ xyz, 
                                                 const long long* __restrict__ pt_off,
                                                 const FrameDev* __restrict__ frames, double h_inv,
                                                 uint32_t* __restrict__ keys, RadixWs ws, int rounds) {
+    chain_enter();
     __shared__ int hist[RAD_PASSES][256];
 #pragma unroll
     for (int p = 0; p < RAD_PASSES; ++p) hist[p][threadIdx.x] = 0;
@@ -163,6 +165,7 @@ __global__ void k_gather(const double* __restrict__ xyz, const float* __restrict
                          float4* __restrict__ pts4, void* __restrict__ sem_sorted,
                          float4* __restrict__ col4, int* __restrict__ perm_local,
                          int* __restrict__ cell_start) {
+    chain_enter();
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < N;
          s += (long long)gridDim.x * blockDim.x) {
         const long long g = perm[s];
@@ -216,6 +219,7 @@ __global__ void k_gather(const double* __restrict__ xyz, const float* __restrict
 // of the next occupied one, the end entry N).
 __global__ void k_cell_start(const uint32_t* __restrict__ keys, long long N, long long C_total,
                              int* __restrict__ cell_start) {
+    chain_enter();
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c <= C_total;
          c += (long long)gridDim.x * blockDim.x) {
         long long lo = 0, hi = N;
@@ -229,6 +233,7 @@ __global__ void k_cell_start(const uint32_t* __restrict__ keys, long long N, lon
 }
 
 __global__ void k_iota(int* __restrict__ vals, long long n) {
+    chain_enter();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         vals[i] = (int)i;
 }
@@ -243,7 +248,7 @@ inline unsigned grid_for(long long n) {
 
 void launch_iota(int* vals, long long n, cudaStream_t st) {
     if (n <= 0) return;
-    k_iota<<<grid_for(n), GT, 0, st>>>(vals, n);
+    launch_chained(k_iota, grid_for(n), GT, 0, st, vals, n);
     count_launch();
 }
 
@@ -251,7 +256,7 @@ void launch_bbox(const double* xyz, const float* sem, const float* rgb, long lon
                  const long long* pt_off, int sem_dim, double h_inv, int* cmin, int* cmax,
                  unsigned* sem_norm_bits, int* err, cudaStream_t st) {
     if (N <= 0) return;
-    k_bbox<<<grid_for(N), GT, 0, st>>>(xyz, sem, rgb, N, K, pt_off, sem_dim, h_inv, cmin, cmax,
+    launch_chained(k_bbox, grid_for(N), GT, 0, st, xyz, sem, rgb, N, K, pt_off, sem_dim, h_inv, cmin, cmax,
                                        sem_norm_bits, err);
     count_launch();
 }
@@ -261,7 +266,7 @@ void launch_keys(const double* xyz, long long N, int K, const long long* pt_off,
                  cudaStream_t st) {
     if (N <= 0) return;
     const int rounds = radix_rounds(N, num_sms);
-    k_keys<<<(unsigned)((N + (long long)RAD_T * rounds - 1) / ((long long)RAD_T * rounds)), RAD_T, 0, st>>>(
+    launch_chained(k_keys, (unsigned)((N + (long long)RAD_T * rounds - 1) / ((long long)RAD_T * rounds)), RAD_T, 0, st, 
         xyz, N, K, pt_off, frames, h_inv, keys, ws, rounds);
     count_launch();
 }
@@ -271,9 +276,9 @@ void launch_gather(const double* xyz, const float* sem, const float* rgb, long l
                    long long C_total, float4* pts4, void* sem_sorted, float4* col4,
                    int* perm_local, int* cell_start, cudaStream_t st) {
     if (N <= 0) return;
-    k_gather<<<grid_for(N), GT, 0, st>>>(xyz, sem, rgb, N, K, pt_off, keys, perm, gp, C_total,
+    launch_chained(k_gather, grid_for(N), GT, 0, st, xyz, sem, rgb, N, K, pt_off, keys, perm, gp, C_total,
                                          pts4, sem_sorted, col4, perm_local, cell_start);
-    k_cell_start<<<grid_for(C_total + 1), GT, 0, st>>>(keys, N, C_total, cell_start);
+    launch_chained(k_cell_start, grid_for(C_total + 1), GT, 0, st, keys, N, C_total, cell_start);
     count_launch(2);
 }
 

@@ -102,6 +102,7 @@ __global__ void __launch_bounds__(128) k_eval_setup(const double* __restrict__ p
                                                     EdgeXf* __restrict__ xf, long long* __restrict__ ws, int n_ws,
                                                     int* __restrict__ ucount, long long* __restrict__ acc,
                                                     const int* done) {
+    chain_enter();
     if (done && *done) return;
     const int gt = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
     for (int i = gt; i < n_ws; i += nt) ws[i] = 0;
@@ -184,6 +185,7 @@ __global__ void __launch_bounds__(RAD_T) k_query_keys(const EdgeDev* __restrict_
                                                       const float4* __restrict__ pts4, GridParams gp, long long Q,
                                                       uint32_t* __restrict__ qkey, float4* __restrict__ qrec,
                                                       RadixWs ws, int rounds, const int* done) {
+    chain_enter();
     if (done && *done) return;
     __shared__ int hist[RAD_PASSES][256];
 #pragma unroll
@@ -220,6 +222,7 @@ __global__ void __launch_bounds__(256) k_units(const uint32_t* __restrict__ key,
                                                const EdgeDev* __restrict__ edges, int E,
                                                float4* __restrict__ slots, int2* __restrict__ units,
                                                int* __restrict__ n_units, const int* done) {
+    chain_enter();
     if (done && *done) return;
     __shared__ int s_cnt[8], s_first[8];
     __shared__ int s_base, s_start;
@@ -315,6 +318,7 @@ __global__ void __launch_bounds__(BIN_T) k_bin_edges(const double* __restrict__ 
                                                      EdgeXf* __restrict__ xf, uint32_t* qkey, float4* qrec,
                                                      float4* slots, int2* units, int* n_units,
                                                      long long* __restrict__ acc, const int* done) {
+    chain_enter();
     if (done && *done) return;
     using L = BinSmem<IPT>;
     extern __shared__ float4 smem4[];
@@ -1586,6 +1590,7 @@ __device__ __forceinline__ void run_unit(const PairArgs& A, int item, int shift,
 template <int DP, bool BF16, bool COLOR, bool DENSE, bool PARTS>
 __global__ void __launch_bounds__(PAIR_T, 2)
 k_pairs(int* unit_counter, const PairArgs A, const int* done) {
+    chain_enter();
     if (done && *done) return;
     extern __shared__ float4 smem4[];
     const int lane = threadIdx.x & 31;
@@ -1686,6 +1691,7 @@ k_pairs_topk(const int2* __restrict__ units, const int* __restrict__ n_units, in
              const int* __restrict__ cell_start, const float4* __restrict__ pts4,
              const void* __restrict__ sem_sorted, const float4* __restrict__ col4, GridParams gp,
              long long* __restrict__ acc, const int* done) {
+    chain_enter();
     if (done && *done) return;
     extern __shared__ float4 smem4[];
     constexpr int SW = lane_row_words<DP, BF16>();
@@ -1990,7 +1996,7 @@ void bin_edges(const BinArgs& a, cudaStream_t st) {
             if (dev < 64) opted[dev].store(true, std::memory_order_release);
         }
     }
-    k_bin_edges<IPT><<<(unsigned)a.E, BIN_T, smem, st>>>(a.poses, a.edges, a.frames, a.pt_cell, a.pts4, a.gp, a.uq, a.xf,
+    launch_chained(k_bin_edges<IPT>, (unsigned)a.E, BIN_T, smem, st, a.poses, a.edges, a.frames, a.pt_cell, a.pts4, a.gp, a.uq, a.xf,
                                                          a.qkey, a.qrec, a.slots, a.units, a.ucount, a.acc, a.done);
 }
 
@@ -2016,7 +2022,7 @@ void launch_k_pairs(const PairLaunch& L, const PairArgs& A) {
     const size_t smem = sizeof(float) * (PAIR_T / 32) * unit_smem_words<DP, BF16, COLOR, DENSE>();
     static int resident = 0;   // opt in to > 48 KB and size the persistent grid, once per instantiation
     const int r = pair_blocks_per_sm(k_pairs<DP, BF16, COLOR, DENSE, PARTS>, smem, &resident);
-    k_pairs<DP, BF16, COLOR, DENSE, PARTS><<<pair_grid(L.num_sms, r, L.ctas_per_sm), PAIR_T, smem, L.stream>>>(
+    launch_chained(k_pairs<DP, BF16, COLOR, DENSE, PARTS>, pair_grid(L.num_sms, r, L.ctas_per_sm), PAIR_T, smem, L.stream, 
         L.unit_counter, A, L.done);
 }
 
@@ -2026,7 +2032,7 @@ void run_pairs(const PairLaunch& L, const PairArgs& A) {
         const size_t smem = sizeof(float) * (PAIR_T / 32) * warp_smem_words_topk<DP, BF16, COLOR>();
         static int resident = 0;
         const int r = pair_blocks_per_sm(k_pairs_topk<DP, BF16, COLOR>, smem, &resident);
-        k_pairs_topk<DP, BF16, COLOR><<<pair_grid(L.num_sms, r, L.ctas_per_sm), PAIR_T, smem, L.stream>>>(
+        launch_chained(k_pairs_topk<DP, BF16, COLOR>, pair_grid(L.num_sms, r, L.ctas_per_sm), PAIR_T, smem, L.stream, 
             A.units, A.n_units, L.unit_counter, A.qkey, A.slots, A.edges, A.frames, A.cell_start, A.pts4,
             A.sem_sorted, A.col4, A.gp, A.acc, L.done);
         return;
@@ -2092,7 +2098,7 @@ bool with_label_layout(const GridParams& gp, const F& f) {
 
 void launch_eval_setup(const double* poses, const EdgeDev* edges, int E, const FrameDev* frames, double h, EdgeXf* xf,
                        long long* ws, int n_ws, int* ucount, long long* acc, const int* done, cudaStream_t st) {
-    k_eval_setup<<<(unsigned)(E < 4 * 592 ? (E + 3) / 4 : 592), 128, 0, st>>>(poses, edges, E, frames, h, xf, ws, n_ws,
+    launch_chained(k_eval_setup, (unsigned)(E < 4 * 592 ? (E + 3) / 4 : 592), 128, 0, st, poses, edges, E, frames, h, xf, ws, n_ws,
                                                                               ucount, acc, done);
     count_launch();
 }
@@ -2102,7 +2108,7 @@ void launch_query_keys(const EdgeDev* edges, int E, const FrameDev* frames, cons
                        uint32_t* qkey, float4* qrec, const RadixWs& ws, int num_sms, const int* done, cudaStream_t st) {
     if (Q <= 0) return;
     const int rounds = radix_rounds(Q, num_sms);
-    k_query_keys<<<(unsigned)((Q + (long long)RAD_T * rounds - 1) / ((long long)RAD_T * rounds)), RAD_T, 0, st>>>(
+    launch_chained(k_query_keys, (unsigned)((Q + (long long)RAD_T * rounds - 1) / ((long long)RAD_T * rounds)), RAD_T, 0, st, 
         edges, E, frames, xf, pt_cell, pts4, gp, Q, qkey, qrec, ws, rounds, done);
     count_launch();
 }
@@ -2112,7 +2118,7 @@ void launch_units(const uint32_t* qkey_sorted, const int* qval_sorted, const flo
                   cudaStream_t st) {
     if (Q <= 0) return;
     if (uq < 1 || uq > UQ) uq = UQ;      // larger units are taken as units of 32
-    k_units<<<blocks_for(Q, 256), 256, 0, st>>>(qkey_sorted, qval_sorted, qrec, Q, uq, sub, edges, E, slots, units,
+    launch_chained(k_units, blocks_for(Q, 256), 256, 0, st, qkey_sorted, qval_sorted, qrec, Q, uq, sub, edges, E, slots, units,
                                                 n_units, done);
     count_launch();
 }

@@ -61,6 +61,7 @@ __global__ void __launch_bounds__(RAD_T) k_onesweep(const uint32_t* __restrict__
                                                     const unsigned long long* __restrict__ counts,
                                                     unsigned long long* status, int* tile_ctr, int* err,
                                                     int spin_limit, const int* done) {
+    chain_enter();
     if (done && *done) return;
     constexpr int TILE = RAD_T * IPT;
     __shared__ int s_tile;
@@ -183,7 +184,7 @@ void sort_passes(uint32_t* keys, int* vals, uint32_t* keys_alt, int* vals_alt, l
     int* vo = vals_alt;
     for (int p = 0; p < ws.npass; ++p) {
         auto kernel = p == 0 ? k_onesweep<IPT, true> : k_onesweep<IPT, false>;
-        kernel<<<(unsigned)nb, RAD_T, 0, st>>>(ki, vi, ko, vo, n, 8 * p, ws.counts + 256 * p,
+        launch_chained(kernel, (unsigned)nb, RAD_T, 0, st, ki, vi, ko, vo, n, 8 * p, ws.counts + 256 * p,
                                                ws.status + (size_t)256 * nb * p, ws.ctr + p, err, SPIN_LIMIT, done);
         count_launch();
         std::swap(ki, ko);

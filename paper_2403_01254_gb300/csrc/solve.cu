@@ -37,6 +37,7 @@ __device__ __forceinline__ double skew_at(const double* v, int i, int j) {
 __global__ void __launch_bounds__(64) k_edge_assemble(const EdgeDev* __restrict__ edges, const EdgeXf* __restrict__ xf,
                                                       const long long* __restrict__ acc, double sigma2,
                                                       EdgeOut* __restrict__ out, const int* done) {
+    chain_enter();
     if (done && *done) return;
     __shared__ double m[28], R[9], t[3];
     __shared__ double Mxx[9], Mxt[9], Mtt[9], Sx[3], St[3], T1[9], Mb[9], Sb[3], KtR[9], KxR[9], NR[9];
@@ -177,6 +178,7 @@ __global__ void __launch_bounds__(FA_T) k_frame_assemble(const EdgeDev* __restri
                                                          const EdgeOut* __restrict__ eo, double* __restrict__ H,
                                                          double* __restrict__ b, double* __restrict__ F,
                                                          long long* __restrict__ npairs, const int* done, LMStep lm) {
+    chain_enter();
     if (done && *done) return;
     __shared__ double s_F[FA_T];
     __shared__ long long s_n[FA_T];
@@ -378,6 +380,7 @@ __global__ void __launch_bounds__(LM_T) k_lm_solve(int K, const double* __restri
                                                    const double* __restrict__ Tcur,
                                                    double* __restrict__ Tcand, LMState* S,
                                                    double* __restrict__ ws) {
+    chain_enter();
     extern __shared__ double sm[];
     __shared__ double red[33];
     __shared__ int fail;
@@ -607,14 +610,14 @@ __global__ void k_copy_if(const LMState* S, double* __restrict__ dst, const doub
 
 void launch_edge_assemble(const EdgeDev* edges, int E, const EdgeXf* xf, const long long* acc,
                           double sigma2, EdgeOut* out, const int* done, cudaStream_t st) {
-    k_edge_assemble<<<E, 64, 0, st>>>(edges, xf, acc, sigma2, out, done);
+    launch_chained(k_edge_assemble, E, 64, 0, st, edges, xf, acc, sigma2, out, done);
     count_launch();
 }
 
 void launch_frame_assemble(const EdgeDev* edges, int E, int K, const int* inc_off,
                            const int* inc_list, const EdgeOut* eout, double* H, double* b,
                            double* F, long long* npairs, const int* done, const LMStep* lm, cudaStream_t st) {
-    k_frame_assemble<<<K + E + 1, FA_T, 0, st>>>(edges, E, K, inc_off, inc_list, eout, H, b, F, npairs, done,
+    launch_chained(k_frame_assemble, K + E + 1, FA_T, 0, st, edges, E, K, inc_off, inc_list, eout, H, b, F, npairs, done,
                                                  lm ? *lm : LMStep{});
     count_launch();
     const long long nH = 36LL * K * K;
@@ -662,7 +665,7 @@ void launch_lm_solve(int K, const double* H_cur, const double* b_cur, const doub
     // hold, so warps that the system has no rows for are left out (two frames: 18.9 us
     // with 512 threads; a 10-iteration solve 838 -> 811 us)
     const int threads = n <= 12 ? 64 : (n <= 30 ? 128 : LM_T);
-    k_lm_solve<<<1, threads, smem, st>>>(K, H_cur, b_cur, poses_cur, poses_cand, st_dev, ws);
+    launch_chained(k_lm_solve, 1, threads, smem, st, K, H_cur, b_cur, poses_cur, poses_cand, st_dev, ws);
     count_launch();
 }
 
