@@ -161,7 +161,8 @@ constexpr int MAX_PAIR_JOBS = 64;   // problems in one batched pair launch
 // warps per SM) are wanted, in 2^3 parts per unit at most.  A problem of more
 // queries than 32 per wanted item has the items as units; the top_k variant's
 // selection needs a unit's whole stream.  Measured with 1, 2 and 4 items per
-// warp: four scans of 8000 points of one object, without labels, 492 us per
+// warp and the walk that the lane unit replaced: four scans of 8000 points of one
+// object, without labels, 492 us per
 // pair launch uncut, 289 / 272 / 266 us; an RGB-D pair of 2000 points 16 us uncut,
 // 18 / 24 / 24 us (short streams gain nothing).
 constexpr int PART_MAX = 3;
