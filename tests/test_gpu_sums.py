@@ -1,0 +1,70 @@
+"""What the sums of the pair kernels hold: values that must not enter them, and bits that must.
+
+Scenes are built so that the right sums are known without a reference of the same
+precision: weights that are FP32 numbers (pairs at distance zero), counts that are exact.
+"""
+import numpy as np
+import pytest
+
+import oracle as O
+import scenes
+
+pytestmark = pytest.mark.gpu
+
+LOSS_TOL, GRAD_TOL, H_TOL = 1e-5, 1e-4, 1e-4
+ELL = 0.25
+H_CELL = 3.0 * ELL * (1.0 + 1.0 / 1024.0)      # the grid's cell edge
+
+
+@pytest.fixture(scope="module")
+def pk():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2403_01254_gb300 as pk
+    pk.load()
+    return pk
+
+
+def _reln(a, b):
+    return float(np.linalg.norm(np.asarray(a) - np.asarray(b)) / max(np.linalg.norm(b), 1e-300))
+
+
+def _pair(xa, xb, sem=None, rgb=None, **params):
+    return dict(xyz=[np.asarray(xa, np.float64), np.asarray(xb, np.float64)], sem=sem, rgb=rgb,
+                edges=np.array([[0, 1]], np.int32), poses0=np.stack([np.eye(4), np.eye(4)]),
+                params=dict(dict(ell=ELL, cutoff_mult=3.0, sigma=1.0, sem_bf16=0), **params))
+
+
+def _eval(pk, prob, **kw):
+    g = pk.Problem.from_scene(prob)
+    try:
+        return g.eval(prob["poses0"], **kw)
+    finally:
+        g.close()
+
+
+# Labels of 1e25: their products with each other (BF16) or their FP16 parts (FP32 labels) are
+# infinite.  The two points that carry them are farther than r_c from every point of
+# the other frame, but lie in the box of the other points, so they share tiles with them.
+@pytest.mark.parametrize("bf16", [0, 1])
+def test_infinite_label_products_outside_the_cutoff(pk, bf16):
+    at = lambda *f: (0.5 + np.array(f)) * H_CELL
+    near = [at(-0.48, -0.48, -0.48), at(0.48, 0.48, 0.48)]
+    rng = np.random.default_rng(3)
+    jit = lambda n: 0.003 * rng.standard_normal((n, 3))
+    xa = np.concatenate([near[0] + jit(20), near[1] + jit(20), at(0.48, -0.48, 0.0)[None]])
+    xb = np.concatenate([near[0] + jit(9), near[1] + jit(8), at(-0.48, 0.48, 0.0)[None]])
+    sem = []
+    for x in (xa, xb):
+        s = scenes.round_to_bf16(scenes.dirichlet_labels(rng, rng.integers(0, 4, len(x)), 4))
+        s[-1] = 2.0 ** 83
+        sem.append(s)
+    prob = _pair(xa, xb, sem, sem_bf16=bf16)
+    ref = O.evaluate(prob, prob["poses0"])
+    assert ref["edge_pairs"].tolist() == [20 * 9 + 20 * 8]
+    out = _eval(pk, prob)
+    assert out["edge_pairs"].tolist() == ref["edge_pairs"].tolist()
+    assert abs(out["loss"] - ref["loss"]) <= LOSS_TOL * abs(ref["loss"])
+    assert _reln(out["grad"], ref["grad"]) <= GRAD_TOL
+    assert _reln(out["H"], ref["H"]) <= H_TOL
