@@ -68,3 +68,23 @@ def test_infinite_label_products_outside_the_cutoff(pk, bf16):
     assert abs(out["loss"] - ref["loss"]) <= LOSS_TOL * abs(ref["loss"])
     assert _reln(out["grad"], ref["grad"]) <= GRAD_TOL
     assert _reln(out["H"], ref["H"]) <= H_TOL
+
+
+# Eight queries at the corners of their home cell, each with one candidate at its own
+# place: a weight per lane that FP32 holds, whose sum (25 bits and more) it does not.  Only the
+# rounding to 2^-51 (the fixed point's step for 8 x 8 points and labels of 4) is left.
+@pytest.mark.parametrize("bf16,extra", [(0, dict(sem_min=1e-12)), (1, dict(sem_min=1e-12)), (0, dict(ell_color=0.2)),
+                                        (1, dict(ell_color=0.2)), (0, dict(top_k=1)), (1, dict(top_k=3))])
+def test_lanes_of_a_unit_are_summed_without_rounding(pk, bf16, extra):
+    corners = np.array([[x, y, z] for z in (-1, 1) for y in (-1, 1) for x in (-1, 1)], np.float64)
+    xyz = (0.5 + 0.4998 * corners) * H_CELL
+    for big in range(8):
+        s = np.zeros((8, 4))
+        s[:, 1] = 3.0 * 2.0 ** -11
+        s[big, 1] = 4.0
+        rgb = [np.full((8, 3), 0.25)] * 2 if "ell_color" in extra else None
+        out = _eval(pk, _pair(xyz, xyz, [s, s], rgb, sem_bf16=bf16, **extra))
+        want = 16.0 + 7 * 9 * 2.0 ** -22
+        assert out["edge_pairs"].tolist() == [8]
+        assert abs(-out["loss"] - want) <= 1e-12 * want
+        assert abs(out["H"][0, 0] - want) <= 1e-12 * want
