@@ -1001,7 +1001,8 @@ struct DenseSmem {
                                                                   //   ldmatrix)
     static constexpr int RING = CF + 32 * 12;                     // [CQ_N] float4 candidate ring
     static constexpr int ROWS = RING + 4 * CQ_N;                  // the stream's segments
-    static constexpr int WORDS = ROWS + ROWS_WORDS;
+    static constexpr int OLD = ROWS + ROWS_WORDS;                 // [4][32] float4: the lanes' sums over earlier pieces
+    static constexpr int WORDS = OLD + 4 * 32 * 4;
 };
 
 // Power-of-two scales of the dense path's FP16 operands, from the frames'
@@ -1239,11 +1240,11 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int2 unit, in
             for (int k = 0; k < 4; ++k) run[mt][n2][k] = 0.f;
     int cnt = 0;
     // the batches, compiled for one and for two m tiles
-    auto batches = [&](auto mtc) {
+    auto batches = [&](auto mtc, int c_s, int c_hi) {
         constexpr int MT = decltype(mtc)::value;
-        int c_s = c_lo, qhead = 0, qlen = 0;
+        int qhead = 0, qlen = 0;
         Cursor cur;
-        cur.start(R, n_seg, 32 * c_lo + lane);
+        cur.start(R, n_seg, 32 * c_s + lane);
         while (c_s < c_hi || qlen > 0) {
             while (qlen < 32 && c_s < c_hi) {
                 bool keep = false;
@@ -1366,10 +1367,40 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int2 unit, in
             }
         }
     };
-    if (c_lo < c_hi) {
-        if (qcount > 16) batches(std::integral_constant<int, 2>{});
-        else batches(std::integral_constant<int, 1>{});
-    }
+    // Streams of more than PIECE chunks are taken in pieces of that length, whose sums are added up
+    // in shared memory: no chain of FP32 additions is longer than 2 PIECE (and one per
+    // piece).  Every piece ends with a batch that is not full (a batch in sixty), and the inner loop
+    // stays as it was: sums folded inside it, every 8 or 32 batches, cost 3% of every case.
+    constexpr int PIECE = 64;
+    float4* older = reinterpret_cast<float4*>(wb + L::OLD) + lane;
+    auto pieces = [&](auto mtc) {
+        constexpr int MT = decltype(mtc)::value;
+#pragma unroll 1
+        for (int c0 = c_lo; c0 < c_hi; c0 += PIECE) {
+            batches(mtc, c0, min(c0 + PIECE, c_hi));
+            if (c_hi - c_lo <= PIECE) break;
+            const bool first = c0 == c_lo, last = c0 + PIECE >= c_hi;
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                for (int n2 = 0; n2 < 2; ++n2) {
+                    float(&r)[4] = run[mt][n2];
+                    float4& o = older[32 * (2 * mt + n2)];
+                    float4 v = make_float4(r[0], r[1], r[2], r[3]);
+                    if (!first) v = make_float4(o.x + v.x, o.y + v.y, o.z + v.z, o.w + v.w);
+                    if (!last) {
+                        o = v;
+                        v = make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+                    r[0] = v.x;
+                    r[1] = v.y;
+                    r[2] = v.z;
+                    r[3] = v.w;
+                }
+        }
+    };
+    if (qcount > 16) pieces(std::integral_constant<int, 2>{});
+    else pieces(std::integral_constant<int, 1>{});
     if (!__any_sync(FULL, cnt != 0)) return;     // no pair: every sum is zero
     // unit end: the per-query sums through shared memory (the features' place)
     // to one lane per query, formed into the lane's moments
@@ -1493,7 +1524,17 @@ __device__ __forceinline__ void pair_unit(const PairArgs& A, int2 unit, int part
     if (c_s >= c_hi) return;
     const u64 MX = f2(mx, mx), MY = f2(my, my), MZ = f2(mz, mz), MW = f2(mw, mw);
     const u64 H2 = f2(0.5f, 0.5f), KG2 = f2(gp.kg, gp.kg);
-    u64 W2 = 0ull, D2[3] = {0ull, 0ull, 0ull}, Q2[6] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};   // halves: even, odd candidates
+    // W, D and Q of the last <= 32 candidate pairs (halves: even, odd candidates), and of all before
+    // them.  One chain of additions over the whole stream was off by up to 1.2e-4 at 25 600
+    // candidates of equal weight (the loss promises 1e-5), these by 4e-6; four unlabelled scans of
+    // 8000 points take 288 us with either.
+    u64 S2[10];
+    float T[10];
+#pragma unroll
+    for (int k = 0; k < 10; ++k) {
+        S2[k] = 0ull;
+        T[k] = 0.f;
+    }
     int cnt = 0;
     // the batches, compiled with and without the pruning test
     auto batches = [&](auto prune) {
@@ -1501,105 +1542,124 @@ __device__ __forceinline__ void pair_unit(const PairArgs& A, int2 unit, int part
         int qhead = 0, qlen = 0;                 // ring head and fill
         Cursor cur;
         cur.start(R, n_seg, 32 * c_s + lane);
-        while (c_s < c_hi || qlen > 0) {
-            // stream the 27-cell candidates through the box test into the
-            // ring until it holds a full batch (or the stream ends)
-            while (qlen < 32 && c_s < c_hi) {
-                bool keep = false;
-                float4 ent = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (cur.valid()) {
-                    ent = cur.point(A.pts4, gp.hf);
-                    const float e0 = fmaxf(fmaxf(blo0 - ent.x, ent.x - bhi0), 0.f);
-                    const float e1 = fmaxf(fmaxf(blo1 - ent.y, ent.y - bhi1), 0.f);
-                    const float e2 = fmaxf(fmaxf(blo2 - ent.z, ent.z - bhi2), 0.f);
-                    keep = fmaf(e0, e0, fmaf(e1, e1, e2 * e2)) < box_thr;
-                }
-                const unsigned bal = __ballot_sync(FULL, keep);
-                if (keep) cq[(qhead + qlen + __popc(bal & ((1u << lane) - 1u))) & (CQ_N - 1)] = ent;
-                qlen += __popc(bal);
-                ++c_s;
-                cur.next(R, n_seg);
-            }
-            __syncwarp();
-            const int nb = qlen < 32 ? qlen : 32;
-            if (nb == 0) break;                  // stream ended with the ring empty
-            // lane c stages candidate c (absent ones: thr = -inf, the label row left as it is)
-            {
-                const bool has = lane < nb;
-                const float4 ent = has ? cq[(qhead + lane) & (CQ_N - 1)] : make_float4(0.f, 0.f, 0.f, 0.f);
-                const int i = __float_as_int(ent.w);
-                float* g = cg + 8 * (lane >> 1) + (lane & 1);
-                g[0] = ent.x;
-                g[2] = ent.y;
-                g[4] = ent.z;
-                g[6] = has ? gp.rc2 - fmaf(ent.x, ent.x, fmaf(ent.y, ent.y, ent.z * ent.z)) : -INF;
-                if constexpr (COLOR) {
-                    const float4 c = has ? __ldg(A.col4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    float* k = cc + 8 * (lane >> 1) + (lane & 1);
-                    k[0] = c.x;
-                    k[2] = c.y;
-                    k[4] = c.z;
-                }
-                if (has) SemRow<DP, BF16>::stage(srow + lane * SW, A.sem_sorted, i);
-            }
-            qhead = (qhead + nb) & (CQ_N - 1);
-            qlen -= nb;
-            __syncwarp();
-            const int n_it = (((nb + 1) >> 1) + (1 << gs) - 1) >> gs;
-            for (int j = 0; j < n_it; ++j) {
-                const int p = (j << gs) + gi;
-                const ulonglong2 x01 = *reinterpret_cast<const ulonglong2*>(cg + 8 * p);
-                const ulonglong2 x2t = *reinterpret_cast<const ulonglong2*>(cg + 8 * p + 4);
-                const float2 t = f2_split(ffma2(x01.x, MX, ffma2(x01.y, MY, ffma2(x2t.x, MZ, MW))));
-                const float2 thr = f2_split(x2t.y);
-                bool in0 = t.x < thr.x, in1 = t.y < thr.y;
-                const u64 E0 = ffma2(H2, MX, x01.x), E1 = ffma2(H2, MY, x01.y), E2 = ffma2(H2, MZ, x2t.x);
-                u64 arg = fmul2(ffma2(E0, E0, ffma2(E1, E1, fmul2(E2, E2))), KG2);
-                if constexpr (COLOR) {
-                    const ulonglong2 c01 = *reinterpret_cast<const ulonglong2*>(cc + 8 * p);
-                    const u64 c2 = *reinterpret_cast<const u64*>(cc + 8 * p + 4);
-                    const u64 r0 = fadd2(c01.x, f2(-qc.x, -qc.x)), r1 = fadd2(c01.y, f2(-qc.y, -qc.y)),
-                              r2 = fadd2(c2, f2(-qc.z, -qc.z));
-                    arg = ffma2(ffma2(r0, r0, ffma2(r1, r1, fmul2(r2, r2))), f2(gp.kc, gp.kc), arg);
-                }
-                const float2 a = f2_split(arg);
-                float w0 = ex2_approx(a.x), w1 = ex2_approx(a.y);
-                if constexpr (DP > 0) {
-                    const float s0 = SemRow<DP, BF16>::dot(qs, srow + (2 * p) * SW);
-                    const float s1 = SemRow<DP, BF16>::dot(qs, srow + (2 * p + 1) * SW);
-                    if constexpr (PRUNE) {
-                        in0 = in0 && s0 >= gp.sem_min;
-                        in1 = in1 && s1 >= gp.sem_min;
+        bool more = true;
+        for (;;) {
+            // batches of up to 16 additions, until another one could make more than 32
+#pragma unroll 1
+            for (int chain = 0; chain <= 16;) {
+                more = c_s < c_hi || qlen > 0;
+                if (!more) break;
+                // stream the 27-cell candidates through the box test into the
+                // ring until it holds a full batch (or the stream ends)
+                while (qlen < 32 && c_s < c_hi) {
+                    bool keep = false;
+                    float4 ent = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (cur.valid()) {
+                        ent = cur.point(A.pts4, gp.hf);
+                        const float e0 = fmaxf(fmaxf(blo0 - ent.x, ent.x - bhi0), 0.f);
+                        const float e1 = fmaxf(fmaxf(blo1 - ent.y, ent.y - bhi1), 0.f);
+                        const float e2 = fmaxf(fmaxf(blo2 - ent.z, ent.z - bhi2), 0.f);
+                        keep = fmaf(e0, e0, fmaf(e1, e1, e2 * e2)) < box_thr;
                     }
-                    w0 *= s0;
-                    w1 *= s1;
+                    const unsigned bal = __ballot_sync(FULL, keep);
+                    if (keep) cq[(qhead + qlen + __popc(bal & ((1u << lane) - 1u))) & (CQ_N - 1)] = ent;
+                    qlen += __popc(bal);
+                    ++c_s;
+                    cur.next(R, n_seg);
                 }
-                cnt += (in0 ? 1 : 0) + (in1 ? 1 : 0);
-                const u64 w = f2(in0 ? w0 : 0.f, in1 ? w1 : 0.f);
-                const u64 WX = fmul2(w, E0), WY = fmul2(w, E1), WZ = fmul2(w, E2);
-                W2 = fadd2(W2, w);
-                D2[0] = fadd2(D2[0], WX);
-                D2[1] = fadd2(D2[1], WY);
-                D2[2] = fadd2(D2[2], WZ);
-                Q2[0] = ffma2(WX, E0, Q2[0]);
-                Q2[1] = ffma2(WX, E1, Q2[1]);
-                Q2[2] = ffma2(WX, E2, Q2[2]);
-                Q2[3] = ffma2(WY, E1, Q2[3]);
-                Q2[4] = ffma2(WY, E2, Q2[4]);
-                Q2[5] = ffma2(WZ, E2, Q2[5]);
+                __syncwarp();
+                const int nb = qlen < 32 ? qlen : 32;
+                more = nb != 0;                      // stream ended with the ring empty
+                if (!more) break;
+                // lane c stages candidate c (absent ones: thr = -inf, the label row left as it is)
+                {
+                    const bool has = lane < nb;
+                    const float4 ent = has ? cq[(qhead + lane) & (CQ_N - 1)] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    const int i = __float_as_int(ent.w);
+                    float* g = cg + 8 * (lane >> 1) + (lane & 1);
+                    g[0] = ent.x;
+                    g[2] = ent.y;
+                    g[4] = ent.z;
+                    g[6] = has ? gp.rc2 - fmaf(ent.x, ent.x, fmaf(ent.y, ent.y, ent.z * ent.z)) : -INF;
+                    if constexpr (COLOR) {
+                        const float4 c = has ? __ldg(A.col4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        float* k = cc + 8 * (lane >> 1) + (lane & 1);
+                        k[0] = c.x;
+                        k[2] = c.y;
+                        k[4] = c.z;
+                    }
+                    if (has) SemRow<DP, BF16>::stage(srow + lane * SW, A.sem_sorted, i);
+                }
+                qhead = (qhead + nb) & (CQ_N - 1);
+                qlen -= nb;
+                __syncwarp();
+                const int n_it = (((nb + 1) >> 1) + (1 << gs) - 1) >> gs;
+                for (int j = 0; j < n_it; ++j) {
+                    const int p = (j << gs) + gi;
+                    const ulonglong2 x01 = *reinterpret_cast<const ulonglong2*>(cg + 8 * p);
+                    const ulonglong2 x2t = *reinterpret_cast<const ulonglong2*>(cg + 8 * p + 4);
+                    const float2 t = f2_split(ffma2(x01.x, MX, ffma2(x01.y, MY, ffma2(x2t.x, MZ, MW))));
+                    const float2 thr = f2_split(x2t.y);
+                    bool in0 = t.x < thr.x, in1 = t.y < thr.y;
+                    const u64 E0 = ffma2(H2, MX, x01.x), E1 = ffma2(H2, MY, x01.y), E2 = ffma2(H2, MZ, x2t.x);
+                    u64 arg = fmul2(ffma2(E0, E0, ffma2(E1, E1, fmul2(E2, E2))), KG2);
+                    if constexpr (COLOR) {
+                        const ulonglong2 c01 = *reinterpret_cast<const ulonglong2*>(cc + 8 * p);
+                        const u64 c2 = *reinterpret_cast<const u64*>(cc + 8 * p + 4);
+                        const u64 r0 = fadd2(c01.x, f2(-qc.x, -qc.x)), r1 = fadd2(c01.y, f2(-qc.y, -qc.y)),
+                                  r2 = fadd2(c2, f2(-qc.z, -qc.z));
+                        arg = ffma2(ffma2(r0, r0, ffma2(r1, r1, fmul2(r2, r2))), f2(gp.kc, gp.kc), arg);
+                    }
+                    const float2 a = f2_split(arg);
+                    float w0 = ex2_approx(a.x), w1 = ex2_approx(a.y);
+                    if constexpr (DP > 0) {
+                        const float s0 = SemRow<DP, BF16>::dot(qs, srow + (2 * p) * SW);
+                        const float s1 = SemRow<DP, BF16>::dot(qs, srow + (2 * p + 1) * SW);
+                        if constexpr (PRUNE) {
+                            in0 = in0 && s0 >= gp.sem_min;
+                            in1 = in1 && s1 >= gp.sem_min;
+                        }
+                        w0 *= s0;
+                        w1 *= s1;
+                    }
+                    cnt += (in0 ? 1 : 0) + (in1 ? 1 : 0);
+                    const u64 w = f2(in0 ? w0 : 0.f, in1 ? w1 : 0.f);
+                    const u64 WX = fmul2(w, E0), WY = fmul2(w, E1), WZ = fmul2(w, E2);
+                    S2[0] = fadd2(S2[0], w);
+                    S2[1] = fadd2(S2[1], WX);
+                    S2[2] = fadd2(S2[2], WY);
+                    S2[3] = fadd2(S2[3], WZ);
+                    S2[4] = ffma2(WX, E0, S2[4]);
+                    S2[5] = ffma2(WX, E1, S2[5]);
+                    S2[6] = ffma2(WX, E2, S2[6]);
+                    S2[7] = ffma2(WY, E1, S2[7]);
+                    S2[8] = ffma2(WY, E2, S2[8]);
+                    S2[9] = ffma2(WZ, E2, S2[9]);
+                }
+                chain += n_it;
+                __syncwarp();
             }
-            __syncwarp();
+            if (!more) break;
+#pragma unroll
+            for (int k = 0; k < 10; ++k) {
+                const float2 h = f2_split(S2[k]);
+                T[k] += h.x + h.y;
+                S2[k] = 0ull;
+            }
         }
     };
     if (DP > 0 && gp.sem_min > -INF) batches(std::true_type{});
     else batches(std::false_type{});
     if (!__any_sync(FULL, cnt != 0)) return;     // no pair: every sum is zero
-    auto both = [](u64 v) { const float2 h = f2_split(v); return h.x + h.y; };
-    const float W = both(W2), y[3] = {r.x, r.y, r.z};
+    auto both = [&](int k) {
+        const float2 h = f2_split(S2[k]);
+        return T[k] + (h.x + h.y);
+    };
+    const float W = both(0), y[3] = {r.x, r.y, r.z};
     float Dv[3], Sy[3], Myy[6], Mdy[9], Qm[6];
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
-        Dv[m] = both(D2[m]);
+        Dv[m] = both(1 + m);
         Sy[m] = W * y[m];
     }
     int t6 = 0;
@@ -1610,7 +1670,7 @@ __device__ __forceinline__ void pair_unit(const PairArgs& A, int2 unit, int part
 #pragma unroll
         for (int l = m; l < 3; ++l, ++t6) {
             Myy[t6] = Sy[m] * y[l];
-            Qm[t6] = both(Q2[t6]);
+            Qm[t6] = both(4 + t6);
         }
     }
     store_moments(W, Dv, Sy, Myy, Mdy, Qm, cnt, Fa, hx, hy, hz, gp, A.edges[e].scale, A.acc + (long long)e * ACC_N, lane);

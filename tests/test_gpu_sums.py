@@ -88,3 +88,32 @@ def test_lanes_of_a_unit_are_summed_without_rounding(pk, bf16, extra):
         assert out["edge_pairs"].tolist() == [8]
         assert abs(-out["loss"] - want) <= 1e-12 * want
         assert abs(out["H"][0, 0] - want) <= 1e-12 * want
+
+
+# Every candidate and every query at the centre of one cell: each weight is the label product
+# c, so a chain of n FP32 additions of it is off by up to n 2^-24, in one direction.  Chains
+# end after 32 additions (lane unit) or 128 (dense unit), which are then added up: a few hundred in
+# all for 51 200 candidates, where one chain would have 25 600 or 3 200.  The loss's tolerance
+# is what every problem is promised.
+def _one_cell(n, nb, c, **extra):
+    xyz = [np.full((k, 3), 0.5 * H_CELL) for k in (n, nb)]
+    return _pair(*xyz, [np.full((n, 1), c), np.ones((nb, 1))], **extra)
+
+
+@pytest.mark.parametrize("c", [0.55, 0.6, 0.8371, 0.9, 1.0 / 3.0])
+@pytest.mark.parametrize("nb", [3, 7, 13, 40])
+def test_long_streams_of_equal_weights(pk, nb, c):
+    n, c = 51200, float(np.float32(c))
+    out = _eval(pk, _one_cell(n, nb, c, sem_min=1e-12))
+    assert out["edge_pairs"].tolist() == [n * nb]
+    assert abs(-out["loss"] / (n * nb * c) - 1.0) <= LOSS_TOL
+
+
+@pytest.mark.parametrize("c", [0.6, 0.8371])
+def test_long_streams_of_equal_weights_dense(pk, c):
+    # 20 bits of c: exact in the labels' and the weights' two FP16 parts; queries enough that no
+    # stream is shared by several warps
+    n, nb, c = 51200, 160000, round(c * 2 ** 20) / 2.0 ** 20
+    out = _eval(pk, _one_cell(n, nb, c))
+    assert out["edge_pairs"].tolist() == [n * nb]
+    assert abs(-out["loss"] / (n * nb * c) - 1.0) <= LOSS_TOL
