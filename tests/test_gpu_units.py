@@ -1,0 +1,55 @@
+"""How the queries of an evaluation are cut into units of work, where cells or problems are out of the ordinary."""
+import numpy as np
+import pytest
+
+import scenes
+
+pytestmark = pytest.mark.gpu
+
+ELL = 0.25
+H_CELL = 3.0 * ELL * (1.0 + 1.0 / 1024.0)      # the grid's cell edge
+
+
+@pytest.fixture(scope="module")
+def pk():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2403_01254_gb300 as pk
+    pk.load()
+    return pk
+
+
+def _plain(xa, xb):
+    return dict(xyz=[np.asarray(xa), np.asarray(xb)], sem=None, rgb=None, edges=np.array([[0, 1]], np.int32),
+                poses0=np.stack([np.eye(4), np.eye(4)]), params=dict(ell=ELL, cutoff_mult=3.0, sigma=1.0))
+
+
+def _milliseconds(pk, prob):
+    """Device time of an evaluation: the profiler's phases, the fastest of 20."""
+    from paper_2403_01254_gb300 import rkhsba as rb
+    g = pk.Problem.from_scene(prob)
+    try:
+        best = np.inf
+        for _ in range(20):
+            rb.rkhsba_profile(g.ctx, 1)
+            g.eval(prob["poses0"])
+            best = min(best, sum(ms for ms, _ in rb.rkhsba_profile(g.ctx, 0, read=True).values()))
+    finally:
+        g.close()
+    return best
+
+
+def test_a_cell_of_many_queries_costs_what_many_cells_do(pk):
+    # 400 000 queries of one home cell, 300 lone ones before it, against the same number over 4096
+    # cells: binning is a few passes over them either way, the pairs a fraction of it
+    rng = np.random.default_rng(5)
+    n = 400_000
+    few = (0.5 + 0.1 * rng.standard_normal((8, 3))) * H_CELL
+    lone = np.stack([np.array([0.5, 0.5, -1.5 - k]) * H_CELL for k in range(300)])
+    one = np.concatenate([lone, (0.5 + 0.2 * (rng.random((n, 3)) - 0.5)) * H_CELL])
+    many = 16.0 * rng.random((n + 300, 3)) * H_CELL
+    corner = np.array([[0.5, 0.5, -302.5], [0.5, 0.5, 0.5], [15.5, 15.5, 15.5]]) * H_CELL      # the grid holds all cells
+    t_one = _milliseconds(pk, _plain(np.concatenate([few, corner[:1]]), one))
+    t_many = _milliseconds(pk, _plain(np.concatenate([few, corner[1:]]), many))
+    assert t_one <= 3.0 * t_many, (t_one, t_many)
