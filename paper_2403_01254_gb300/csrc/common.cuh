@@ -134,10 +134,9 @@ struct PairArgs {
     const uint32_t* qkey;     // sorted home-cell keys of the queries
     const float4* slots;      // sorted query records (offset from the home centre, point index)
     long long Q;              // queries over all edges
-    const int2* units;        // (first sorted query, edge << 7 | queries)
+    const int2* units;        // units and parts of units: see unit_record
     const int* n_units;
-    int part_max, part_target;   // a unit's stream is cut into up to 2^part_max parts until there are
-                                 //   part_target items (part_max = 0: never)
+    int cut;                  // whether any unit of the problem may come in parts
     const EdgeDev* edges;
     const FrameDev* frames;
     const int* cell_start;
@@ -157,19 +156,43 @@ struct PairJob {
 };
 constexpr int MAX_PAIR_JOBS = 64;   // problems in one batched pair launch
 
-// Cutting of units into parts: items for two per resident warp (16
-// warps per SM) are wanted, in 2^3 parts per unit at most.  A problem of more
-// queries than 32 per wanted item has the items as units; the top_k variant's
-// selection needs a unit's whole stream.  Measured with 1, 2 and 4 items per
-// warp and the walk that the lane unit replaced: four scans of 8000 points of one
-// object, without labels, 492 us per
-// pair launch uncut, 289 / 272 / 266 us; an RGB-D pair of 2000 points 16 us uncut,
-// 18 / 24 / 24 us (short streams gain nothing).
-constexpr int PART_MAX = 3;
-inline int part_target_for(int num_sms) { return 32 * num_sms; }
-inline int part_max_for(const GridParams& gp, long long Q, int num_sms) {
-    return (gp.top_k > 0 || Q > 32LL * part_target_for(num_sms)) ? 0 : PART_MAX;
+// Cutting of units into parts.  A few dense clouds make few units with long candidate
+// streams, fewer than the chip has warps, and the launch took as long as the longest of them.  So
+// a unit comes in 2^s <= 8 parts, each an even share of its stream, as long as a part has
+// CUT_POINTS points of the 27 cells to go through.  Small edges have few units, so an eighth of
+// their queries will do (CUT_SMALL at least); large ones have many, so a part takes a 64th of their
+// queries, and those of more than CUT_EDGE are not cut.  Each part is rounded to fixed point by itself,
+// so the rule looks at the unit and at its edge alone, and an edge's results do not depend on what else
+// is evaluated, nor on the chip.  The top_k variant's selection needs a unit's whole stream.  A unit of q
+// queries has 2 q parts at most, so a list of 2 Q records holds all.
+//
+// Evaluations, us, against parts counted from the problem's units and the chip's warps (two items per warp; an
+// edge then had other bits among other edges): unlabelled scans 4 x 8000 284 -> 276, 5 x 8000 428 -> 387, LiDAR
+// 8 x 20k 352 -> 348, 4 x 20k pruned 235 -> 204, 5 x 60k 547 -> 489, fresh 4 x 30k 427 -> 404.  It costs where one
+// edge had the chip for itself: scans 2 x 2000 75 -> 82, 2 x 8000 126 -> 127, LiDAR 2 x 20k 103 -> 111, 2 x 36k pruned
+// 165 -> 195, 2 x 100k 325 -> 389; and the count of the points: ten-iteration solve of 2 x 2000 RGB-D points 748 -> 775.
+// Parts of 512 points: scans 2 x 8000 138, LiDAR 2 x 20k 117; edges of 65 536 queries in parts of 512, too: 10 x 50k
+// window step 3.54 -> 3.65 ms; of 100k: 64 x 100k mapping 62.5 -> 70.1 ms.
+constexpr int CUT_EDGE = 65536, CUT_POINTS = 256, CUT_SMALL = 128;
+inline bool cut_possible(const GridParams& gp, const EdgeDev* edges, int E, const FrameDev* frames) {
+    if (gp.top_k > 0) return false;
+    for (int e = 0; e < E; ++e)
+        if (frames[edges[e].b].n_pts <= CUT_EDGE) return true;
+    return false;
 }
+
+// Record of a unit (of the part `part` of its 2^s): first sorted query, and edge (23 bits), queries - 1
+// (5 bits), 2^s + part (4 bits).
+__host__ __device__ inline int2 unit_record(int first, int edge, int queries, int s, int part) {
+    int2 r;
+    r.x = first;
+    r.y = (int)((unsigned)edge << 9 | (unsigned)(queries - 1) << 4 | (unsigned)((1 << s) + part));
+    return r;
+}
+__device__ __forceinline__ int unit_edge(int2 u) { return (int)((unsigned)u.y >> 9); }
+__device__ __forceinline__ int unit_queries(int2 u) { return ((u.y >> 4) & 31) + 1; }
+__device__ __forceinline__ int unit_shift(int2 u) { return 31 - __clz(u.y & 15); }
+__device__ __forceinline__ int unit_part(int2 u) { return (u.y & 15) - (1 << unit_shift(u)); }
 
 // Launch state of a single-problem pair launch.
 struct PairLaunch {
@@ -238,13 +261,14 @@ struct BinArgs {
     const FrameDev* frames;
     const uint32_t* pt_cell;
     const float4* pts4;
+    const int* cell_start;
     GridParams gp;
     int uq;
     EdgeXf* xf;
     uint32_t* qkey;           // sorted home-cell keys, edge by edge
     float4* qrec;             // scratch: records in query order
     float4* slots;            // the same in sorted order
-    int2* units;
+    int2* units;              // [2 Q]
     int* ucount;              // [4], cleared first; [0]: number of units
     long long* acc;
     const int* done;
@@ -254,8 +278,8 @@ void launch_query_keys(const EdgeDev* edges, int E, const FrameDev* frames, cons
                        const uint32_t* pt_cell, const float4* pts4, GridParams gp, long long Q,
                        uint32_t* qkey, float4* qrec, const RadixWs& ws, int num_sms, const int* done, cudaStream_t st);
 void launch_units(const uint32_t* qkey_sorted, const int* qval_sorted, const float4* qrec, long long Q, int uq,
-                  int sub, const EdgeDev* edges, int E, float4* slots, int2* units, int* n_units, const int* done,
-                  cudaStream_t st);
+                  const GridParams& gp, const EdgeDev* edges, int E, const FrameDev* frames, const int* cell_start,
+                  float4* slots, int2* units, int* n_units, const int* done, cudaStream_t st);
 void launch_pairs(const PairLaunch& L, const PairArgs& A);
 // Largest unit_queries setting of this layout: 64 for the dense tile kernel
 // with BF16 labels, else 32 (64 is taken as two units of 32).

@@ -66,6 +66,7 @@ struct rkhsba_ctx {
 
     long long total_bins = 0, Q_total = 0;
     int q_max = 0;                     // queries of the largest edge
+    bool cut = false;                  // units may come in parts
     int qbits = 0;                     // radix bits of the query keys
     EdgeXf* d_xf = nullptr;
     uint32_t* d_qkey = nullptr;        // home-cell key per query (then sorted)
@@ -127,8 +128,7 @@ struct rkhsba_ctx {
         a.acc = d_acc;
         a.units = d_units;
         a.n_units = d_ucount;
-        a.part_max = rk::part_max_for(gp, Q_total, num_sms);
-        a.part_target = rk::part_target_for(num_sms);
+        a.cut = cut;
         a.E = E;
         a.gp = gp;
         return a;

@@ -210,17 +210,70 @@ __global__ void __launch_bounds__(RAD_T) k_query_keys(const EdgeDev* __restrict_
     radix_finish(ws, hist);
 }
 
+// log2 of the parts that a unit of n queries of home cell `cell` comes in (see common.cuh): edge
+// and unit decide, nothing else.  n_b: queries of the edge.
+__device__ __forceinline__ int cut_shift(const GridParams& gp, const FrameDev& Fa, int n_b,
+                                         const int* __restrict__ cell_start, int cell, int n) {
+    if (gp.top_k > 0 || n_b > CUT_EDGE) return 0;
+    const int least = max(min(max(n_b >> 3, CUT_SMALL), CUT_POINTS), n_b >> 6);
+    // Runs of cells by their places in the flat grid (at its very edge, where a row would leave
+    // it, other cells are counted, which make as good a rule).  First, for each of the three planes, all
+    // cells from the first to the last of its nine: a bound that takes six reads; the eighteen of the
+    // nine rows for every unit of a sparse cloud took a ten-iteration solve of 2 x 2000 points from
+    // 746 to 785 us.
+    const int dx = Fa.dim[0], plane = dx * Fa.dim[1], cells = plane * Fa.dim[2];
+    const int* c = cell_start + Fa.cell_off;
+    auto points = [&](int from, int to) { return __ldg(c + min(max(to + 1, 0), cells)) - __ldg(c + min(max(from, 0), cells)); };
+    long long most = 0;
+#pragma unroll
+    for (int z = -1; z <= 1; ++z) most += points(cell + z * plane - dx - 1, cell + z * plane + dx + 1);
+    if (most < 2 * least) return 0;
+    int in_row[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const int at = cell + (k % 3 - 1) * dx + (k / 3 - 1) * plane;
+        in_row[k] = points(at - 1, at + 1);
+    }
+    long long all = 0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) all += in_row[k];
+    int s = 0;
+    while (s < 3 && (1 << s) <= n && (all >> (s + 1)) >= least) ++s;
+    return s;
+}
+
+// Place of a lane's records among the warp's (2^s each where `start` holds), and their number.
+__device__ __forceinline__ int unit_places(bool start, int s, int lane, int& total) {
+    const unsigned m = __ballot_sync(FULL, start);
+    int at = __popc(m & ((1u << lane) - 1u));
+    total = __popc(m);
+    if (__any_sync(FULL, s > 0)) {
+        int more = (1 << s) - 1, inc = more;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(FULL, inc, o);
+            if (lane >= o) inc += u;
+        }
+        at += inc - more;
+        total += __shfl_sync(FULL, inc, 31);
+    }
+    return at;
+}
+
 // Sorted query records and the unit list, in one pass over the sorted keys: a
 // unit starts at the first query of a home cell and every uq queries after.
 // A block takes 256 sorted queries; where its first one continues a cell of
 // an earlier block, the block looks for that cell's first query.  One atomic per block reserves its slots in the
-// unit list; a record is (first sorted query, edge << 7 | queries), so that
-// no warp of the pair kernels searches for either.
+// unit list; a record holds edge and queries, so that no warp of the pair
+// kernels searches for either.
 __global__ void __launch_bounds__(256) k_units(const uint32_t* __restrict__ key, const int* __restrict__ val,
-                                               const float4* __restrict__ qrec, long long Q, int uq, int sub,
+                                               const float4* __restrict__ qrec, long long Q, int uq, GridParams gp,
                                                const EdgeDev* __restrict__ edges, int E,
+                                               const FrameDev* __restrict__ frames,
+                                               const int* __restrict__ cell_start,
                                                float4* __restrict__ slots, int2* __restrict__ units,
                                                int* __restrict__ n_units, const int* done) {
+    const int sub = gp.key_sub;
     chain_enter();
     if (done && *done) return;
     __shared__ int s_cnt[8], s_first[8];
@@ -266,8 +319,24 @@ __global__ void __launch_bounds__(256) k_units(const uint32_t* __restrict__ key,
         }
         const long long run = start >= 0 ? base + start : from;
         const bool st = valid && ((k - run) % uq) == 0;
-        const unsigned m = __ballot_sync(FULL, st);
-        if (lane == 0) s_cnt[warp] = __popc(m);
+        int e = 0, n = 0, s = 0;
+        if (st) {
+            // queries of the cell from here on, uq at most (gallop, then bisect)
+            int m = 1;
+            while (m < uq && k + m < Q && (key[k + m] >> sub) == (kk >> sub)) m *= 2;
+            int lo = m / 2 + 1, hi = m < uq ? m : uq;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (k + mid < Q && (key[k + mid] >> sub) == (kk >> sub)) lo = mid + 1; else hi = mid;
+            }
+            n = lo;
+            e = find_edge_bin(edges, E, kk >> sub);
+            s = cut_shift(gp, frames[edges[e].a], frames[edges[e].b].n_pts, cell_start,
+                          (int)((kk >> sub) - edges[e].bin_off), n);
+        }
+        int total;
+        const int at = unit_places(st, s, lane, total);
+        if (lane == 0) s_cnt[warp] = total;
         __syncthreads();
         if (threadIdx.x == 0) {
             int tot = 0;
@@ -275,18 +344,9 @@ __global__ void __launch_bounds__(256) k_units(const uint32_t* __restrict__ key,
             s_base = tot ? atomicAdd(n_units, tot) : 0;
         }
         __syncthreads();
-        if (st) {
-            // queries of the cell from here on, uq at most (gallop, then bisect)
-            int n = 1;
-            while (n < uq && k + n < Q && (key[k + n] >> sub) == (kk >> sub)) n *= 2;
-            int lo = n / 2 + 1, hi = n < uq ? n : uq;
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (k + mid < Q && (key[k + mid] >> sub) == (kk >> sub)) lo = mid + 1; else hi = mid;
-            }
-            units[s_base + s_cnt[warp] + __popc(m & ((1u << lane) - 1u))] =
-                make_int2((int)k, (find_edge_bin(edges, E, kk >> sub) << 7) | lo);
-        }
+        if (st)
+            for (int part = 0; part < 1 << s; ++part)
+                units[s_base + s_cnt[warp] + at + part] = unit_record((int)k, e, n, s, part);
         __syncthreads();
     }
 }
@@ -318,7 +378,8 @@ template <int IPT>
 __global__ void __launch_bounds__(BIN_T) k_bin_edges(const double* __restrict__ poses, const EdgeDev* __restrict__ edges,
                                                      const FrameDev* __restrict__ frames,
                                                      const uint32_t* __restrict__ pt_cell,
-                                                     const float4* __restrict__ pts4, GridParams gp, int uq,
+                                                     const float4* __restrict__ pts4,
+                                                     const int* __restrict__ cell_start, GridParams gp, int uq,
                                                      EdgeXf* __restrict__ xf, uint32_t* qkey, float4* qrec,
                                                      float4* slots, int2* units, int* n_units,
                                                      long long* __restrict__ acc, const int* done) {
@@ -472,13 +533,29 @@ __global__ void __launch_bounds__(BIN_T) k_bin_edges(const double* __restrict__ 
         }
     }
     // units: every uq queries of a cell
-    unsigned mine[IPT];
-    int count = 0;
+    int at[IPT], n_s[IPT], count = 0;            // place in the warp's records; queries << 2 | log2 of the parts
 #pragma unroll
     for (int r = 0; r < IPT; ++r) {
         const int i = at0 + 32 * r;
-        mine[r] = __ballot_sync(FULL, i < n && key[r] != NO_KEY && ((unsigned)(i - start[r]) % (unsigned)uq) == 0u);
-        count += __popc(mine[r]);
+        const bool st = i < n && key[r] != NO_KEY && ((unsigned)(i - start[r]) % (unsigned)uq) == 0u;
+        int s = 0;
+        n_s[r] = 0;
+        if (st) {
+            const uint32_t c = key[r] >> gp.key_sub;
+            auto same = [&](int k) { return k < n && (s_key[k] >> gp.key_sub) == c; };
+            int m = 1;                               // queries of the cell from here on, uq at most
+            while (m < uq && same(i + m)) m *= 2;
+            int lo = m / 2 + 1, hi = m < uq ? m : uq;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (same(i + mid)) lo = mid + 1; else hi = mid;
+            }
+            s = cut_shift(gp, Fa, n, cell_start, (int)c, lo);
+            n_s[r] = lo << 2 | s;
+        }
+        int total;
+        at[r] = count + unit_places(st, s, lane, total);
+        count += total;
     }
     if (lane == 0) s_sum[warp] = count;
     __syncthreads();
@@ -494,24 +571,12 @@ __global__ void __launch_bounds__(BIN_T) k_bin_edges(const double* __restrict__ 
         if (lane == 31) s_base = inc ? atomicAdd(n_units, inc) : 0;
     }
     __syncthreads();
-    int to = s_base + s_sum[warp];
+    const int to = s_base + s_sum[warp];
 #pragma unroll
-    for (int r = 0; r < IPT; ++r) {
-        const int i = at0 + 32 * r;
-        if ((mine[r] >> lane) & 1u) {
-            const uint32_t c = key[r] >> gp.key_sub;
-            auto same = [&](int k) { return k < n && (s_key[k] >> gp.key_sub) == c; };
-            int m = 1;                               // queries of the cell from here on, uq at most
-            while (m < uq && same(i + m)) m *= 2;
-            int lo = m / 2 + 1, hi = m < uq ? m : uq;
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (same(i + mid)) lo = mid + 1; else hi = mid;
-            }
-            units[to + __popc(mine[r] & lt)] = make_int2((int)(Ed.q_off + i), (e << 7) | lo);
-        }
-        to += __popc(mine[r]);
-    }
+    for (int r = 0; r < IPT; ++r)
+        if (n_s[r])
+            for (int part = 0; part < 1 << (n_s[r] & 3); ++part)
+                units[to + at[r] + part] = unit_record((int)(Ed.q_off + at0 + 32 * r), e, n_s[r] >> 2, n_s[r] & 3, part);
 }
 
 // round(v * scale) to the nearest integer (ties to even) as int64, for
@@ -754,16 +819,6 @@ struct Cursor {
     }
 };
 
-// Parts that the candidate stream of a unit is cut into, as a power of two
-// (log2): problems with few units (dense small clouds) would leave most warps
-// idle behind a few long streams, so their units are shared by up to
-// 2^part_max warps until part_target items are there.  Set by the problem's own
-// units alone, so that its results do not depend on what shares a launch.
-__device__ __forceinline__ int part_shift(const PairArgs& A, int n_units) {
-    int s = 0;
-    while (s < A.part_max && ((long long)n_units << s) < A.part_target) ++s;
-    return s;
-}
 // Chunks [c0, c1) of 32 stream points that part `part` of 2^shift takes: an
 // even share, but four at least (short streams stay whole, and their other
 // parts are empty).
@@ -1149,7 +1204,7 @@ __device__ __forceinline__ void gram_chunks(float (&s)[4], const unsigned (&qa)[
 // shared-memory pipe was the kernel's bound (82% busy on the mapping workload,
 // 98 wavefronts per 16 x 32 tile; 32 here).
 template <int DP, bool SPLIT, bool PARTS>
-__device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int2 unit, int part, int shift, float* wb, int lane) {
+__device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int2 unit, float* wb, int lane) {
     using L = DenseSmem<DP, SPLIT>;
     constexpr int LW = L::LW, PW = L::PW;
     constexpr int NKC = L::DPH / 8;             // 8-wide chunks of a label row part (1..4)
@@ -1162,7 +1217,7 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int2 unit, in
     const int g = lane >> 2, t4 = lane & 3;
     const float INF = __int_as_float(0x7f800000);
 
-    const int k0 = unit.x, qcount = unit.y & 127, e = unit.y >> 7;
+    const int k0 = unit.x, qcount = unit_queries(unit), e = unit_edge(unit);
     const uint32_t key0 = A.qkey[k0] >> gp.key_sub;
     const FrameDev& Fa = A.frames[A.edges[e].a];
     const FrameDev& Fb = A.frames[A.edges[e].b];
@@ -1214,7 +1269,7 @@ __device__ __forceinline__ void pair_unit_dense(const PairArgs& A, int2 unit, in
     const int C = build_rows(R, A.cell_start, Fa, hx, hy, hz, blo0, blo1, blo2, bhi0, bhi1, bhi2, gp.hf, box_thr, lane,
                              n_seg);
     int c_lo = 0, c_hi = (int)(((long long)C + 31) >> 5);    // chunks of the stream
-    if constexpr (PARTS) part_range(C, part, shift, c_lo, c_hi);
+    if constexpr (PARTS) part_range(C, unit_part(unit), unit_shift(unit), c_lo, c_hi);
     // query label rows (zero rows for absent queries) as A fragments, through
     // the candidates' rows
     {
@@ -1479,7 +1534,7 @@ __host__ __device__ constexpr int warp_smem_words() {
 }
 
 template <int DP, bool BF16, bool COLOR>
-__device__ __forceinline__ void pair_unit(const PairArgs& A, int2 unit, int part, int shift, float* wb, int lane) {
+__device__ __forceinline__ void pair_unit(const PairArgs& A, int2 unit, float* wb, int lane) {
     constexpr int SW = lane_row_words<DP, BF16>();
     const GridParams& gp = A.gp;
     float* cg = wb;
@@ -1488,7 +1543,7 @@ __device__ __forceinline__ void pair_unit(const PairArgs& A, int2 unit, int part
     float4* cq = reinterpret_cast<float4*>(srow + 32 * SW);
     const Rows R{reinterpret_cast<int4*>(cq + CQ_N), reinterpret_cast<float2*>(cq + CQ_N + 9)};
     const float INF = __int_as_float(0x7f800000);
-    const int k0 = unit.x, qcount = unit.y & 127, e = unit.y >> 7;
+    const int k0 = unit.x, qcount = unit_queries(unit), e = unit_edge(unit);
     const uint32_t key0 = A.qkey[k0] >> gp.key_sub;            // home-cell key
     const FrameDev& Fa = A.frames[A.edges[e].a];
     const int cell = (int)(key0 - A.edges[e].bin_off);
@@ -1524,7 +1579,7 @@ __device__ __forceinline__ void pair_unit(const PairArgs& A, int2 unit, int part
     const int C = build_rows(R, A.cell_start, Fa, hx, hy, hz, blo0, blo1, blo2, bhi0, bhi1, bhi2, gp.hf, box_thr, lane,
                              n_seg);
     int c_s, c_hi;                               // chunks of the stream
-    part_range(C, part, shift, c_s, c_hi);
+    part_range(C, unit_part(unit), unit_shift(unit), c_s, c_hi);
     if (c_s >= c_hi) return;
     const u64 MX = f2(mx, mx), MY = f2(my, my), MZ = f2(mz, mz), MW = f2(mw, mw);
     const u64 H2 = f2(0.5f, 0.5f), KG2 = f2(gp.kg, gp.kg);
@@ -1690,11 +1745,10 @@ __host__ __device__ constexpr int unit_smem_words() {
 // PARTS false (the dense path of problems that never cut units): the kernel
 // without part numbers, 2% faster on the mapping and window workloads.
 template <int DP, bool BF16, bool COLOR, bool DENSE, bool PARTS>
-__device__ __forceinline__ void run_unit(const PairArgs& A, int item, int shift, float* wb, int lane) {
-    const int2 unit = A.units[PARTS ? item >> shift : item];
-    const int part = PARTS ? item & ((1 << shift) - 1) : 0;
-    if constexpr (DENSE && DP > 0 && !COLOR) pair_unit_dense<DP, !BF16, PARTS>(A, unit, part, shift, wb, lane);
-    else pair_unit<DP, BF16, COLOR>(A, unit, part, shift, wb, lane);
+__device__ __forceinline__ void run_unit(const PairArgs& A, int item, float* wb, int lane) {
+    const int2 unit = A.units[item];
+    if constexpr (DENSE && DP > 0 && !COLOR) pair_unit_dense<DP, !BF16, PARTS>(A, unit, wb, lane);
+    else pair_unit<DP, BF16, COLOR>(A, unit, wb, lane);
 }
 
 template <int DP, bool BF16, bool COLOR, bool DENSE, bool PARTS>
@@ -1706,14 +1760,13 @@ k_pairs(int* unit_counter, const PairArgs A, const int* done) {
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     float* wb = reinterpret_cast<float*>(smem4) + warp * unit_smem_words<DP, BF16, COLOR, DENSE>();
-    const int shift = PARTS ? part_shift(A, *A.n_units) : 0;
-    const int items = *A.n_units << shift;
+    const int items = *A.n_units;
     for (;;) {
         int u = 0;
         if (lane == 0) u = atomicAdd(unit_counter, 1);
         u = __shfl_sync(FULL, u, 0);
         if (u >= items) break;
-        run_unit<DP, BF16, COLOR, DENSE, PARTS>(A, u, shift, wb, lane);
+        run_unit<DP, BF16, COLOR, DENSE, PARTS>(A, u, wb, lane);
     }
 }
 
@@ -1726,7 +1779,7 @@ k_pairs(int* unit_counter, const PairArgs A, const int* done) {
 template <int DP, bool BF16, bool COLOR, bool DENSE>
 __global__ void __launch_bounds__(PAIR_T, 2)
 k_pairs_multi(const PairJob* __restrict__ jobs, int n_jobs, int* unit_counter) {
-    __shared__ int s_pref[MAX_PAIR_JOBS + 1], s_shift[MAX_PAIR_JOBS];
+    __shared__ int s_pref[MAX_PAIR_JOBS + 1];
     extern __shared__ float4 smem4[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -1738,8 +1791,6 @@ k_pairs_multi(const PairJob* __restrict__ jobs, int n_jobs, int* unit_counter) {
             if (j < n_jobs) {
                 const int* dn = jobs[j].done;
                 n = (dn && *dn) ? 0 : *jobs[j].a.n_units;
-                s_shift[j] = part_shift(jobs[j].a, n);
-                n <<= s_shift[j];
             }
             int inc = n;
 #pragma unroll
@@ -1765,7 +1816,7 @@ k_pairs_multi(const PairJob* __restrict__ jobs, int n_jobs, int* unit_counter) {
             const int mid = (lo + hi + 1) >> 1;
             if (s_pref[mid] <= u) lo = mid; else hi = mid - 1;
         }
-        run_unit<DP, BF16, COLOR, DENSE, true>(jobs[lo].a, u - s_pref[lo], s_shift[lo], wb, lane);
+        run_unit<DP, BF16, COLOR, DENSE, true>(jobs[lo].a, u - s_pref[lo], wb, lane);
     }
 }
 
@@ -1822,7 +1873,7 @@ k_pairs_topk(const int2* __restrict__ units, const int* __restrict__ n_units, in
         u = __shfl_sync(FULL, u, 0);
         if (u >= nu) break;
         const int2 unit = units[u];
-        const int k0 = unit.x, qcount = unit.y & 127, e = unit.y >> 7;
+        const int k0 = unit.x, qcount = unit_queries(unit), e = unit_edge(unit);
         const uint32_t key0 = qkey[k0] >> gp.key_sub;
         const FrameDev& Fa = frames[edges[e].a];
         const int cell = (int)(key0 - edges[e].bin_off);
@@ -2034,8 +2085,8 @@ k_emit_pairs(const int2* __restrict__ units, const int* __restrict__ n_units, in
         u = __shfl_sync(FULL, u, 0);
         if (u >= nu) break;
         const int2 unit = units[u];
-        const int k0 = unit.x, qcount = unit.y & 127, e = unit.y >> 7;
-        if (e != edge_sel) continue;
+        const int k0 = unit.x, qcount = unit_queries(unit), e = unit_edge(unit);
+        if (e != edge_sel || unit_part(unit) > 0) continue;      // the first part lists the whole unit
         const uint32_t key0 = qkey[k0] >> gp.key_sub;
         const FrameDev& Fa = frames[edges[e].a];
         const int cell = (int)(key0 - edges[e].bin_off);
@@ -2106,7 +2157,8 @@ void bin_edges(const BinArgs& a, cudaStream_t st) {
             if (dev < 64) opted[dev].store(true, std::memory_order_release);
         }
     }
-    launch_chained(k_bin_edges<IPT>, (unsigned)a.E, BIN_T, smem, st, a.poses, a.edges, a.frames, a.pt_cell, a.pts4, a.gp, a.uq, a.xf,
+    launch_chained(k_bin_edges<IPT>, (unsigned)a.E, BIN_T, smem, st, a.poses, a.edges, a.frames, a.pt_cell, a.pts4,
+                   a.cell_start, a.gp, a.uq, a.xf,
                                                          a.qkey, a.qrec, a.slots, a.units, a.ucount, a.acc, a.done);
 }
 
@@ -2149,7 +2201,7 @@ void run_pairs(const PairLaunch& L, const PairArgs& A) {
     }
     if constexpr (DP > 0 && !COLOR) {
         if (dense_path(A.gp)) {
-            if (A.part_max > 0) launch_k_pairs<DP, BF16, COLOR, true, true>(L, A);
+            if (A.cut) launch_k_pairs<DP, BF16, COLOR, true, true>(L, A);
             else launch_k_pairs<DP, BF16, COLOR, true, false>(L, A);
             return;
         }
@@ -2224,12 +2276,12 @@ void launch_query_keys(const EdgeDev* edges, int E, const FrameDev* frames, cons
 }
 
 void launch_units(const uint32_t* qkey_sorted, const int* qval_sorted, const float4* qrec, long long Q, int uq,
-                  int sub, const EdgeDev* edges, int E, float4* slots, int2* units, int* n_units, const int* done,
-                  cudaStream_t st) {
+                  const GridParams& gp, const EdgeDev* edges, int E, const FrameDev* frames, const int* cell_start,
+                  float4* slots, int2* units, int* n_units, const int* done, cudaStream_t st) {
     if (Q <= 0) return;
     if (uq < 1 || uq > UQ) uq = UQ;      // larger units are taken as units of 32
-    launch_chained(k_units, blocks_for(Q, 256), 256, 0, st, qkey_sorted, qval_sorted, qrec, Q, uq, sub, edges, E, slots, units,
-                                                n_units, done);
+    launch_chained(k_units, blocks_for(Q, 256), 256, 0, st, qkey_sorted, qval_sorted, qrec, Q, uq, gp, edges, E,
+                   frames, cell_start, slots, units, n_units, done);
     count_launch();
 }
 

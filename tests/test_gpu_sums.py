@@ -117,3 +117,21 @@ def test_long_streams_of_equal_weights_dense(pk, c):
     out = _eval(pk, _one_cell(n, nb, c))
     assert out["edge_pairs"].tolist() == [n * nb]
     assert abs(-out["loss"] / (n * nb * c) - 1.0) <= LOSS_TOL
+
+
+# An edge's sums do not depend on what else is evaluated with it, also where long streams are
+# shared by several warps.
+@pytest.mark.parametrize("variant", ["plain", "fp32", "bf16", "color"])
+def test_an_edge_alone_equals_the_same_edge_among_others(pk, variant):
+    for n, extent in ((900, 1.2), (2500, 1.5)):
+        prob = scenes.tiny_problem(seed=61, n_frames=5, n=n, extent=extent, ell=0.15, color=variant == "color")
+        if variant == "plain":
+            prob["sem"] = None
+        if variant == "bf16":
+            prob["sem"] = [scenes.round_to_bf16(s) for s in prob["sem"]]
+            prob["params"] = dict(prob["params"], sem_bf16=1)
+        full = _eval(pk, prob, want_blocks=True)
+        for e in (0, 4, 9):
+            alone = _eval(pk, dict(prob, edges=np.asarray(prob["edges"])[e:e + 1]), want_blocks=True)
+            assert alone["edge_pairs"][0] == full["edge_pairs"][e]
+            assert np.array_equal(alone["H_blocks"][0], full["H_blocks"][e])
