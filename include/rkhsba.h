@@ -340,12 +340,13 @@ rkhsba_status rkhsba_solve_ell_decay(rkhsba_ctx* ctx, const rkhsba_ell_schedule*
  * pick launch shapes of the sparse double sum of Sec. III-B per workload).
  *
  * Three knobs change the speed of the pair stage but not its results beyond
- * FP32 rounding (pair sets and the exact fixed-point sums do not change):
+ * FP32 rounding (pair sets do not change; the sums of a unit of work are
+ * rounded once, so other units round elsewhere):
  *   cell_scale    grid cell edge in units of r_c (params.cell_scale, fixed
  *                 at rkhsba_create: the grids are built for it)
  *   unit_queries  queries of one home cell handed to a warp at a time (1..32;
- *                 1..64 for BF16 labels without colour, pruning or top_k,
- *                 whose dense pair kernel takes units of up to 64 queries)
+ *                 for BF16 labels without colour, pruning or top_k 33..64 are
+ *                 accepted as well, and mean 32)
  *   ctas_per_sm   resident CTAs per SM of the persistent pair launch
  *                 (0: as many as fit)
  * ------------------------------------------------------------------------ */
@@ -362,9 +363,10 @@ rkhsba_status rkhsba_get_tuning(const rkhsba_ctx* ctx, rkhsba_tuning* out);
 
 /*
  * rkhsba_autotune -- time the evaluation of one problem under every
- * candidate setting (cell_scale 1, 1.25, 1.5 x unit_queries 32, 16 and,
- * where the pair kernel takes it, 64 x ctas_per_sm all, 1; the default
- * setting first) and report the fastest.
+ * candidate setting (cell_scale 1, 1.25, 1.5 x unit_queries 32, 16 x
+ * ctas_per_sm all, 1; the default setting first) and report the fastest.
+ * Where unit_queries 64 is accepted it is listed too, with the times of 32,
+ * which it means, and is never the one reported.
  * For each cell size a temporary context is built from the inputs
  * (arguments as for rkhsba_create, or as for rkhsba_create_device when
  * inputs_on_device is 1); each setting is run once untimed, then at least
@@ -373,8 +375,8 @@ rkhsba_status rkhsba_get_tuning(const rkhsba_ctx* ctx, rkhsba_tuning* out);
  * kept unless another is faster by more than 3%.
  *   best      HOST out: the chosen setting and its mean time (ms)
  *   table     HOST out [table_cap] (may be NULL when table_cap is 0): every
- *             setting tried, in order; *n_table receives the count (12, or
- *             18 with 64-query units)
+ *             setting, in order; *n_table receives the count (12, or 18 where
+ *             unit_queries 64 is accepted)
  * Creating a context with params.cell_scale = best.cell_scale and calling
  * rkhsba_set_tuning(ctx, best.unit_queries, best.ctas_per_sm) applies it.
  * Synchronous; holds one temporary context at a time.

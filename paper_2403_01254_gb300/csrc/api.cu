@@ -808,7 +808,9 @@ rkhsba_status rkhsba_get_tuning(const rkhsba_ctx* c, rkhsba_tuning* out) {
 // assembly) is timed with CUDA events on the stream after one untimed run,
 // over at least `reps` evaluations and at least 20 ms.  The default setting
 // (the first candidate) is kept unless another is faster by more than 3%,
-// so timing noise on small problems does not move it.
+// so timing noise on small problems does not move it.  Units of 64 queries, where
+// they are accepted, are units of 32: such a setting is listed with the time of its
+// 32-query one, is not timed again and never chosen.
 rkhsba_status rkhsba_autotune(int32_t n_frames, const int64_t* n_points, const double* xyz, const float* sem,
                               const float* rgb, int32_t n_edges, const int32_t* edges,
                               const rkhsba_params* params, int32_t inputs_on_device, const double* poses,
@@ -820,8 +822,9 @@ rkhsba_status rkhsba_autotune(int32_t n_frames, const int64_t* n_points, const d
     // the default setting (cell_scale 1, 32 queries per unit, all CTAs that
     // fit) is timed first
     static const double scales[] = {1.0, 1.25, 1.5};
-    static const int uqs_all[] = {32, 16, 64};   // 64 only where the pair kernel takes it
+    static const int uqs_all[] = {32, 16, 64};   // 64 only where it is accepted, as a name of 32
     static const int ctas[] = {0, 1};
+    double ms_32[2] = {0.0, 0.0};                // of the cell size in hand, by CTA count
     int n = 0;
     best->ms = -1.0;
     rkhsba_tuning dflt{};
@@ -845,6 +848,11 @@ rkhsba_status rkhsba_autotune(int32_t n_frames, const int64_t* n_points, const d
             for (int uq : uqs_all)
                 for (int ct : ctas) {
                     if (uq > pair_unit_max(c->gp)) continue;
+                    if (uq > UNIT_Q) {
+                        if (n < table_cap) table[n] = rkhsba_tuning{sc, uq, ct, ms_32[ct]};
+                        ++n;
+                        continue;
+                    }
                     c->tune_uq = uq;
                     c->tune_ctas = ct;
                     float ms = 0.f, ms0 = 0.f;
@@ -863,6 +871,7 @@ rkhsba_status rkhsba_autotune(int32_t n_frames, const int64_t* n_points, const d
                         break;
                     }
                     rkhsba_tuning t{sc, uq, ct, (double)ms / nrep};
+                    if (uq == UNIT_Q) ms_32[ct] = t.ms;
                     if (n < table_cap) table[n] = t;
                     if (n == 0) dflt = t;
                     ++n;

@@ -53,3 +53,27 @@ def test_a_cell_of_many_queries_costs_what_many_cells_do(pk):
     t_one = _milliseconds(pk, _plain(np.concatenate([few, corner[:1]]), one))
     t_many = _milliseconds(pk, _plain(np.concatenate([few, corner[1:]]), many))
     assert t_one <= 3.0 * t_many, (t_one, t_many)
+
+
+def test_33_to_64_queries_mean_32_and_are_not_timed_again(pk):
+    from paper_2403_01254_gb300 import rkhsba as rb
+    prob = scenes.window_problem(seed=78, window=3, n_points=6000)
+    outs = []
+    for uq in (32, 33, 48, 64):
+        g = pk.Problem.from_scene(prob)
+        try:
+            g.set_tuning(uq, 0)
+            outs.append(g.eval(prob["poses0"]))
+        finally:
+            g.close()
+    for o in outs[1:]:
+        assert o["loss"] == outs[0]["loss"] and np.array_equal(o["grad"], outs[0]["grad"])
+        assert np.array_equal(o["H"], outs[0]["H"])
+    n = np.array([len(x) for x in prob["xyz"]], np.int64)
+    xyz = np.ascontiguousarray(np.concatenate(prob["xyz"]))
+    sem = np.ascontiguousarray(np.concatenate(prob["sem"]).astype(np.float32))
+    params = pk.make_params(0.3, sem_dim=sem.shape[1], sem_bf16=1)
+    best, table = rb.rkhsba_autotune(n, xyz, sem, None, prob["edges"], params, prob["poses0"], reps=1)
+    by = {(t["cell_scale"], t["unit_queries"], t["ctas_per_sm"]): t["ms"] for t in table}
+    same = [by[s, 64, c] == by[s, 32, c] for s in (1.0, 1.25, 1.5) for c in (0, 1)]
+    assert all(same) and best["unit_queries"] <= 32
