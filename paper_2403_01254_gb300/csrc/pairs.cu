@@ -26,6 +26,7 @@
 // No FP64 arithmetic runs per query: the frame-a position of a frame-b cell
 // centre comes from a per-edge affine map held as double-float pairs, evaluated
 // with error-free transformations (Dekker product, Knuth sum) on the FP32 pipe.
+#include "per_device.h"
 #include "radix.cuh"
 
 #include <type_traits>
@@ -2132,30 +2133,40 @@ inline unsigned blocks_for(long long n, int t) {
     return (unsigned)b;
 }
 
-// Resident CTAs per SM of a pair kernel at its shared-memory size (queried
-// once per instantiation; the dynamic shared memory opt-in is set then).
+int current_device() {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return dev;
+}
+
+// Opts a kernel in to its dynamic shared memory, which counts for the current device
+// alone.
 template <typename KernelT>
-int pair_blocks_per_sm(KernelT kernel, size_t smem, int* cache) {
-    if (!*cache) {
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        int b = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, PAIR_T, smem);
-        *cache = b < 1 ? 1 : b;
-    }
-    return *cache;
+bool opt_in(KernelT kernel, size_t smem) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
+}
+
+// Resident CTAs per SM of a pair kernel at its shared-memory size (queried
+// once per instantiation and device; the opt-in is set then).  A failure is not kept, and the launch
+// that follows reports it.
+template <typename KernelT>
+int pair_blocks_per_sm(KernelT kernel, size_t smem, PerDevice& cache) {
+    const int b = cache.get(current_device(), [&] {
+        int n = 0;
+        if (!opt_in(kernel, smem) ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, PAIR_T, smem) != cudaSuccess)
+            return 0;
+        return n < 1 ? 1 : n;
+    });
+    return b < 1 ? 1 : b;
 }
 
 template <int IPT>
 void bin_edges(const BinArgs& a, cudaStream_t st) {
     constexpr size_t smem = BinSmem<IPT>::BYTES;
-    if constexpr (smem > 36864) {                // with the static arrays more than 48 KB: opt in, once per device
-        static std::atomic<bool> opted[64];
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (dev >= 64 || !opted[dev].load(std::memory_order_acquire)) {
-            cudaFuncSetAttribute(k_bin_edges<IPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (dev < 64) opted[dev].store(true, std::memory_order_release);
-        }
+    if constexpr (smem > 36864) {                // with the static arrays more than 48 KB
+        static PerDevice opted;
+        opted.get(current_device(), [] { return opt_in(k_bin_edges<IPT>, smem) ? 1 : 0; });
     }
     launch_chained(k_bin_edges<IPT>, (unsigned)a.E, BIN_T, smem, st, a.poses, a.edges, a.frames, a.pt_cell, a.pts4,
                    a.cell_start, a.gp, a.uq, a.xf,
@@ -2182,8 +2193,8 @@ inline bool dense_path(const GridParams& gp) {
 template <int DP, bool BF16, bool COLOR, bool DENSE, bool PARTS>
 void launch_k_pairs(const PairLaunch& L, const PairArgs& A) {
     const size_t smem = sizeof(float) * (PAIR_T / 32) * unit_smem_words<DP, BF16, COLOR, DENSE>();
-    static int resident = 0;   // opt in to > 48 KB and size the persistent grid, once per instantiation
-    const int r = pair_blocks_per_sm(k_pairs<DP, BF16, COLOR, DENSE, PARTS>, smem, &resident);
+    static PerDevice resident;
+    const int r = pair_blocks_per_sm(k_pairs<DP, BF16, COLOR, DENSE, PARTS>, smem, resident);
     launch_chained(k_pairs<DP, BF16, COLOR, DENSE, PARTS>, pair_grid(L.num_sms, r, L.ctas_per_sm), PAIR_T, smem, L.stream, 
         L.unit_counter, A, L.done);
 }
@@ -2192,8 +2203,8 @@ template <int DP, bool BF16, bool COLOR>
 void run_pairs(const PairLaunch& L, const PairArgs& A) {
     if (A.gp.top_k > 0) {
         const size_t smem = sizeof(float) * (PAIR_T / 32) * warp_smem_words_topk<DP, BF16, COLOR>();
-        static int resident = 0;
-        const int r = pair_blocks_per_sm(k_pairs_topk<DP, BF16, COLOR>, smem, &resident);
+        static PerDevice resident;
+        const int r = pair_blocks_per_sm(k_pairs_topk<DP, BF16, COLOR>, smem, resident);
         launch_chained(k_pairs_topk<DP, BF16, COLOR>, pair_grid(L.num_sms, r, L.ctas_per_sm), PAIR_T, smem, L.stream, 
             A.units, A.n_units, L.unit_counter, A.qkey, A.slots, A.edges, A.frames, A.cell_start, A.pts4,
             A.sem_sorted, A.col4, A.gp, A.acc, L.done);
@@ -2213,8 +2224,8 @@ template <int DP, bool BF16, bool COLOR, bool DENSE>
 void launch_k_pairs_multi(const PairJob* jobs, int n_jobs, int* counter, int num_sms, int ctas_per_sm,
                           cudaStream_t st) {
     const size_t smem = sizeof(float) * (PAIR_T / 32) * unit_smem_words<DP, BF16, COLOR, DENSE>();
-    static int resident = 0;   // opt in to > 48 KB and size the persistent grid, once per instantiation
-    const int r = pair_blocks_per_sm(k_pairs_multi<DP, BF16, COLOR, DENSE>, smem, &resident);
+    static PerDevice resident;
+    const int r = pair_blocks_per_sm(k_pairs_multi<DP, BF16, COLOR, DENSE>, smem, resident);
     k_pairs_multi<DP, BF16, COLOR, DENSE><<<pair_grid(num_sms, r, ctas_per_sm), PAIR_T, smem, st>>>(
         jobs, n_jobs, counter);
 }

@@ -12,6 +12,7 @@
 // original cost F increases (Sec. V-C); the weights are recomputed at the new
 // poses by the next evaluation (Sec. V-A, last paragraph).
 #include "common.cuh"
+#include "per_device.h"
 
 #include <algorithm>
 
@@ -632,15 +633,17 @@ void launch_lm_solve(int K, const double* H_cur, const double* b_cur, const doub
     const int n = 6 * (K - 1);
     // factor A (n x n), right-hand side y (n) and pivot reciprocals rinv (n)
     size_t smem = (n <= LM_SMEM_N) ? (size_t)(n * n + 2 * n) * sizeof(double) : 0;
-    // opt in once to the largest factor kept in shared memory (not a stream
+    // opt in once per device to the largest factor kept in shared memory (not a stream
     // operation, so it must not happen while an iteration is being captured;
     // the first call of any context runs before capture)
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaFuncSetAttribute(k_lm_solve, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)((size_t)(LM_SMEM_N * LM_SMEM_N + 2 * LM_SMEM_N) * sizeof(double)));
-        attr_set = true;
-    }
+    static PerDevice opted;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    opted.get(dev, [] {
+        return cudaFuncSetAttribute(k_lm_solve, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)((size_t)(LM_SMEM_N * LM_SMEM_N + 2 * LM_SMEM_N) * sizeof(double))) ==
+                       cudaSuccess ? 1 : 0;
+    });
     if (n >= LM_BLOCKED_N) {
         const int nt = (n + CT - 1) / CT;
         const long long nn = (long long)n * n;
