@@ -194,7 +194,7 @@ rkhsba_status rkhsba_edge_pairs(rkhsba_ctx* ctx, const double* poses, int32_t ed
 /*
  * rkhsba_profile -- CUDA-event timing of the phases of the hot path on the
  * context stream: [0] grid build, [1] transforms + query binning, [2] pair
- * kernel, [3] FP64 assembly, [4] LM solve + accept.
+ * kernel, [3] FP64 assembly (with the LM loop's accept step), [4] LM solve.
  *   enable    1: clear and start recording; 0: stop recording
  *   ms        [5] summed milliseconds of the recorded launches, or NULL
  *   launches  [5] number of recorded launches per phase, or NULL

@@ -125,8 +125,6 @@ void grid_fill(rkhsba_ctx* c, bool* keys_in_alt) {
     const RadixWs ws = radix_ws(c->N, nbits, c->d_hist, c->d_scan_ws);
     cudaMemsetAsync(c->d_scan_ws, 0, sizeof(long long) * scan_ws_elems(c->N), st);
     launch_keys(c->d_xyz, c->N, c->K, c->d_pt_off, c->d_frames, c->gp.h_inv, c->d_keys, ws, c->num_sms, st);
-    if (ws.npass == 0)      // one cell: the input order is the order
-        launch_iota(c->d_vals, c->N, st);
     const bool alt = radix_sort_u32(c->d_keys, c->d_vals, c->d_keys_alt, c->d_vals_alt, c->N, ws, c->d_err + 1, nullptr,
                                     st);
     const uint32_t* keys = alt ? c->d_keys_alt : c->d_keys;
@@ -452,7 +450,7 @@ bool capture_graph(rkhsba_ctx* c, cudaGraphExec_t* exec, long long* kernels, Fn 
 
 // n LM iterations.  After the first evaluation has run (kernel attributes and
 // occupancy are then settled), one iteration is captured into a CUDA graph
-// and replayed, which removes the per-kernel launch cost of the ~30 small
+// and replayed, which removes the per-kernel launch cost of the 5 to 12
 // launches of an iteration.  With the phase profiler on, or when capture is
 // not possible, the iterations are launched one kernel at a time.
 void lm_iterate(rkhsba_ctx* c, int n) {
@@ -552,7 +550,6 @@ PairJob ctx_pair_job(const rkhsba_ctx* c) {
 GridParams ctx_layout(const rkhsba_ctx* c) { return c->gp; }
 int ctx_num_sms(const rkhsba_ctx* c) { return c->num_sms; }
 int ctx_tune_ctas(const rkhsba_ctx* c) { return c->tune_ctas; }
-int ctx_tune_uq(const rkhsba_ctx* c) { return c->tune_uq; }
 cudaStream_t ctx_stream(const rkhsba_ctx* c) { return c->stream; }
 const void* ctx_state_dev(const rkhsba_ctx* c) { return c->d_state; }
 const double* ctx_poses_dev(const rkhsba_ctx* c) { return c->d_poses_cur; }
@@ -587,8 +584,9 @@ rkhsba_status rkhsba_eval(rkhsba_ctx* c, const double* poses, double* loss, doub
     RK_CUDA(c, cudaMemcpyAsync(c->d_poses_cand, poses, sizeof(double) * 16 * c->K, cudaMemcpyHostToDevice, st));
     run_eval(c, c->d_poses_cand, nullptr);
     RK_CUDA(c, cudaGetLastError());
-    // everything asked for up to ONE_COPY bytes in one copy, else the matrix
-    // straight to its place
+    // everything asked for in one copy up to ONE_COPY bytes, else the matrix straight to its
+    // place (a copy costs several microseconds of host time; where the line lies between that and
+    // the second copy of a large matrix in host memory was not measured)
     const ResultLayout R(c->K, c->E);
     constexpr size_t ONE_COPY = 256 << 10;
     const bool want_e = H_blocks || edge_pairs;

@@ -57,10 +57,7 @@ inline void launch_chained(void (*kernel)(P...), dim3 grid, unsigned block, size
 constexpr int MAX_SEM = 32;     // label floats per point
 constexpr int ACC_N = 32;       // int64 accumulator slots per edge
 constexpr int N_MOM = 29;       // used slots (see MomentIndex)
-#ifndef RK_UNIT_Q
-#define RK_UNIT_Q 32
-#endif
-constexpr int UNIT_Q = RK_UNIT_Q;   // queries of one home cell per warp unit (32 or 64)
+constexpr int UNIT_Q = 32;      // queries of one home cell per unit, at most
 
 // Fixed-point accumulator layout per edge.  All sums are over the pairs of the
 // edge, in frame-a coordinates: d = x - y', y' = T_ab y.
@@ -144,7 +141,6 @@ struct PairArgs {
     const void* sem_sorted;   // label rows in the same order (FP32 or BF16), or NULL
     const float4* col4;       // colours in the same order, or NULL
     long long* acc;           // [E][ACC_N] fixed-point moments
-    int E;
     GridParams gp;
 };
 
@@ -235,7 +231,6 @@ bool radix_sort_u32(uint32_t* keys, int* vals, uint32_t* keys_alt, int* vals_alt
                     int* err, const int* done, cudaStream_t st);
 
 // grid.cu
-void launch_iota(int* vals, long long n, cudaStream_t st);
 void launch_bbox(const double* xyz, const float* sem, const float* rgb, long long N, int K,
                  const long long* pt_off, int sem_dim, double h_inv, int* cmin, int* cmax,
                  unsigned* sem_norm_bits, int* err, cudaStream_t st);
@@ -339,5 +334,4 @@ PairJob ctx_pair_job(const rkhsba_ctx* c);
 GridParams ctx_layout(const rkhsba_ctx* c);
 int ctx_num_sms(const rkhsba_ctx* c);
 int ctx_tune_ctas(const rkhsba_ctx* c);
-int ctx_tune_uq(const rkhsba_ctx* c);
 }  // namespace rk

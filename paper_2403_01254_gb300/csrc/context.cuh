@@ -129,7 +129,6 @@ struct rkhsba_ctx {
         a.units = d_units;
         a.n_units = d_ucount;
         a.cut = cut;
-        a.E = E;
         a.gp = gp;
         return a;
     }

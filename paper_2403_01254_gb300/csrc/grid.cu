@@ -232,12 +232,6 @@ __global__ void k_cell_start(const uint32_t* __restrict__ keys, long long N, lon
     }
 }
 
-__global__ void k_iota(int* __restrict__ vals, long long n) {
-    chain_enter();
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        vals[i] = (int)i;
-}
-
 inline unsigned grid_for(long long n) {
     long long b = (n + GT - 1) / GT;
     if (b < 1) b = 1;
@@ -245,12 +239,6 @@ inline unsigned grid_for(long long n) {
     return (unsigned)b;
 }
 }  // namespace
-
-void launch_iota(int* vals, long long n, cudaStream_t st) {
-    if (n <= 0) return;
-    launch_chained(k_iota, grid_for(n), GT, 0, st, vals, n);
-    count_launch();
-}
 
 void launch_bbox(const double* xyz, const float* sem, const float* rgb, long long N, int K,
                  const long long* pt_off, int sem_dim, double h_inv, int* cmin, int* cmax,

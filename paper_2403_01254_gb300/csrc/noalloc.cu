@@ -272,7 +272,6 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
     const RadixWs gws = radix_ws(N, cbits, d_hist, d_ws);
     SCK(cudaMemsetAsync(d_ws, 0, sizeof(long long) * scan_ws_elems(N), st));
     launch_keys(d_xyz, N, K, d_pt_off, d_frames, gp.h_inv, d_keys, gws, num_sms, st);
-    if (gws.npass == 0) launch_iota(d_vals, N, st);
     const bool alt = radix_sort_u32(d_keys, d_vals, d_keys_alt, d_vals_alt, N, gws, d_err + 1, nullptr, st);
     const uint32_t* pt_cell = alt ? d_keys_alt : d_keys;
     launch_gather(d_xyz, d_sem, gp.color ? d_rgb : nullptr, N, K, d_pt_off, pt_cell, alt ? d_vals_alt : d_vals,
@@ -309,7 +308,6 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
         a.units = d_units;
         a.n_units = d_ucount;
         a.cut = cut;
-        a.E = E;
         a.gp = gp;
         launch_pairs(PairLaunch{d_ucount + 1, nullptr, num_sms, 0, st}, a);
     }

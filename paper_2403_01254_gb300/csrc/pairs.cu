@@ -6,9 +6,9 @@
 // |T_a x - T_b y| = |x - T_ab y|) and keyed by the frame-a grid cell holding
 // it.  A stable radix sort groups the queries by home cell (order inside a
 // cell = frame-b order, so results do not depend on thread timing), and the
-// groups are cut into units of <= 32 (or 64) queries.  A warp takes one unit,
-// stages its queries in shared memory and streams the candidates of the 27
-// surrounding cells, 32 at a time, through a box test against the unit's
+// groups are cut into units of <= 32 queries.  A warp takes one unit, or one part
+// of a unit with a long stream, holds its queries in registers and streams the candidates
+// of the 27 surrounding cells, 32 at a time, through a box test against the unit's
 // queries.  For every candidate x query pair inside r_c the weight
 //     w = <l_i, l_j> * k_c(c_i, c_j) * exp(-|d|^2 / (2 ell^2))      Eq. (irls_weight)
 // enters the sums that fix the 28 edge moments (layout in common.cuh), and
@@ -19,9 +19,9 @@
 //     per-query moment sums on the tensor cores (see "dense tile path");
 //   * the lane unit (colour, semantic pruning, no labels): lanes over the
 //     queries, all in FP32 (see "lane path").
-// A unit's moments are summed over the warp in a fixed order and rounded once to
-// 64-bit fixed point, so edge totals are exact integer sums, independent of which
-// warp ran which unit.
+// The moments of a unit (of each of its parts) are summed over the warp in a fixed order and
+// rounded to 64-bit fixed point, so edge totals are exact integer sums, independent of which
+// warp ran which unit and of the other edges.
 //
 // No FP64 arithmetic runs per query: the frame-a position of a frame-b cell
 // centre comes from a per-edge affine map held as double-float pairs, evaluated
@@ -726,8 +726,8 @@ struct SemRow<0, false> {
 
 
 constexpr int PAIR_T = 256;
-constexpr int UQ = UNIT_Q;          // queries per unit: one 32-bit mask word
-static_assert(UQ == 32, "units hold 32 queries");
+constexpr int UQ = UNIT_Q;
+static_assert(UQ == 32, "a lane for every query of a unit");
 
 __device__ __forceinline__ float ex2_approx(float x) {
     float y;
@@ -1598,7 +1598,7 @@ __device__ __forceinline__ void pair_unit(const PairArgs& A, int2 unit, float* w
     int cnt = 0;
     // the batches, compiled with and without the pruning test
     auto batches = [&](auto prune) {
-        constexpr bool PRUNE = decltype(prune)::value;
+        [[maybe_unused]] constexpr bool PRUNE = decltype(prune)::value;
         int qhead = 0, qlen = 0;                 // ring head and fill
         Cursor cur;
         cur.start(R, n_seg, 32 * c_s + lane);

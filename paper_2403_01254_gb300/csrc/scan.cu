@@ -192,7 +192,7 @@ void sort_passes(uint32_t* keys, int* vals, uint32_t* keys_alt, int* vals_alt, l
     }
 }
 // Tiles of 4096 keys once there are enough of them for every SM several times
-// over (half the records per key: 51.6 M keys, see the launch), else of 2048.
+// over (half the records per key), else of 2048.
 constexpr long long BIG_SORT = 4096LL * 152 * 8;
 }  // namespace
 

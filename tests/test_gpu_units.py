@@ -77,3 +77,19 @@ def test_33_to_64_queries_mean_32_and_are_not_timed_again(pk):
     by = {(t["cell_scale"], t["unit_queries"], t["ctas_per_sm"]): t["ms"] for t in table}
     same = [by[s, 64, c] == by[s, 32, c] for s in (1.0, 1.25, 1.5) for c in (0, 1)]
     assert all(same) and best["unit_queries"] <= 32
+
+
+@pytest.mark.parametrize("top_k", [0, 1, 3, 8])
+@pytest.mark.parametrize("na,nb", [(1, 1), (1, 3), (2, 1), (3, 1), (2, 5), (33, 9), (300, 17)])
+def test_few_pairs_are_counted_exactly(pk, na, nb, top_k):
+    # all of them far inside the cutoff
+    rng = np.random.default_rng(10 * na + nb)
+    box = [(0.5 + 0.1 * rng.random((n, 3))) * H_CELL for n in (na, nb)]
+    prob = _plain(*box)
+    prob["params"] = dict(prob["params"], top_k=top_k)
+    g = pk.Problem.from_scene(prob)
+    try:
+        out = g.eval(prob["poses0"])
+    finally:
+        g.close()
+    assert out["edge_pairs"].tolist() == [nb * (min(top_k, na) if top_k else na)]
