@@ -249,7 +249,7 @@ rkhsba_status build(rkhsba_ctx* c, const double* xyz, const float* sem, const fl
     if (c->total_bins >= (1LL << 31) - 2) return fail(c, RKHSBA_EINVAL, "total home cells exceed 2^31");
     if (c->Q_total >= (1LL << 31) - 64) return fail(c, RKHSBA_EINVAL, "more than 2^31 queries over all edges");
     c->q_max = edge_queries_max(c->edges_h.data(), E, c->frames_h.data());
-    c->cut = cut_possible(c->gp, c->edges_h.data(), E, c->frames_h.data());
+    c->cut_edge = cut_edge_for(c->gp, c->edges_h.data(), E, c->frames_h.data(), c->Q_total);
     c->qbits = 1;
     while ((1LL << c->qbits) <= c->total_bins) ++c->qbits;   // invalid key sorts last
     // three more key bits order a home cell's queries by octant, when they fit
@@ -287,7 +287,7 @@ rkhsba_status build(rkhsba_ctx* c, const double* xyz, const float* sem, const fl
     RK_TRY(alloc(c, &c->d_qhist, (long long)radix_hist_elems(Q)));
     RK_TRY(alloc(c, &c->d_qrec, Q));
     RK_TRY(alloc(c, &c->d_slots, Q));
-    RK_TRY(alloc(c, &c->d_units, c->cut ? 2 * Q : Q));
+    RK_TRY(alloc(c, &c->d_units, c->cut_edge ? 2 * Q : Q));
     RK_TRY(alloc(c, &c->d_ucount, 4));
     RK_TRY(alloc(c, &c->d_acc, (long long)E * ACC_N));
     const long long n6 = 6LL * K;
@@ -310,7 +310,7 @@ void run_binning(rkhsba_ctx* c, const double* poses, const int* done) {
     cudaStream_t st = c->stream;
     if (c->q_max <= BIN_MAX) {
         launch_bin_edges(BinArgs{poses, c->d_edges, c->E, c->d_frames, c->d_pt_cell, c->d_pts4, c->d_cell_start, c->gp,
-                                 c->tune_uq, c->d_xf,
+                                 c->tune_uq, c->cut_edge, c->d_xf,
                                  c->d_qkey, c->d_qrec, c->d_slots, c->d_units, c->d_ucount, c->d_acc, done},
                          c->q_max, st);
         c->q_sorted_key = c->d_qkey;
@@ -325,8 +325,8 @@ void run_binning(rkhsba_ctx* c, const double* poses, const int* done) {
                                     done, st);
     c->q_sorted_key = alt ? c->d_qkey_alt : c->d_qkey;
     const int* qv = alt ? c->d_qval_alt : c->d_qval;
-    launch_units(c->q_sorted_key, qv, c->d_qrec, c->Q_total, c->tune_uq, c->gp, c->d_edges, c->E, c->d_frames,
-                 c->d_cell_start, c->d_slots, c->d_units, c->d_ucount, done, st);
+    launch_units(c->q_sorted_key, qv, c->d_qrec, c->Q_total, c->tune_uq, c->gp.key_sub, c->cut_edge, c->d_edges, c->E,
+                 c->d_frames, c->d_cell_start, c->d_slots, c->d_units, c->d_ucount, done, st);
 }
 
 // One evaluation at the device poses `poses`, results into the cand

@@ -160,7 +160,8 @@ constexpr int MAX_PAIR_JOBS = 64;   // problems in one batched pair launch
 // queries, and those of more than CUT_EDGE are not cut.  Each part is rounded to fixed point by itself,
 // so the rule looks at the unit and at its edge alone, and an edge's results do not depend on what else
 // is evaluated, nor on the chip.  The top_k variant's selection needs a unit's whole stream.  A unit of q
-// queries has 2 q parts at most, so a list of 2 Q records holds all.
+// queries has 2 q parts at most, so a list of 2 Q records holds all; records are counted in 31 bits, so
+// problems of 2^30 queries and more are not cut at all.
 //
 // Evaluations, us, against parts counted from the problem's units and the chip's warps (two items per warp; an
 // edge then had other bits among other edges): unlabelled scans 4 x 8000 284 -> 276, 5 x 8000 428 -> 387, LiDAR
@@ -170,11 +171,12 @@ constexpr int MAX_PAIR_JOBS = 64;   // problems in one batched pair launch
 // Parts of 512 points: scans 2 x 8000 138, LiDAR 2 x 20k 117; edges of 65 536 queries in parts of 512, too: 10 x 50k
 // window step 3.54 -> 3.65 ms; of 100k: 64 x 100k mapping 62.5 -> 70.1 ms.
 constexpr int CUT_EDGE = 65536, CUT_POINTS = 256, CUT_SMALL = 128;
-inline bool cut_possible(const GridParams& gp, const EdgeDev* edges, int E, const FrameDev* frames) {
-    if (gp.top_k > 0) return false;
+// Queries up to which a problem's edges are cut; 0 where none of them is.
+inline int cut_edge_for(const GridParams& gp, const EdgeDev* edges, int E, const FrameDev* frames, long long Q) {
+    if (gp.top_k > 0 || Q >= 1LL << 30) return 0;
     for (int e = 0; e < E; ++e)
-        if (frames[edges[e].b].n_pts <= CUT_EDGE) return true;
-    return false;
+        if (frames[edges[e].b].n_pts <= CUT_EDGE) return CUT_EDGE;
+    return 0;
 }
 
 // Record of a unit (of the part `part` of its 2^s): first sorted query, and edge (23 bits), queries - 1
@@ -258,7 +260,7 @@ struct BinArgs {
     const float4* pts4;
     const int* cell_start;
     GridParams gp;
-    int uq;
+    int uq, cut_edge;
     EdgeXf* xf;
     uint32_t* qkey;           // sorted home-cell keys, edge by edge
     float4* qrec;             // scratch: records in query order
@@ -273,7 +275,7 @@ void launch_query_keys(const EdgeDev* edges, int E, const FrameDev* frames, cons
                        const uint32_t* pt_cell, const float4* pts4, GridParams gp, long long Q,
                        uint32_t* qkey, float4* qrec, const RadixWs& ws, int num_sms, const int* done, cudaStream_t st);
 void launch_units(const uint32_t* qkey_sorted, const int* qval_sorted, const float4* qrec, long long Q, int uq,
-                  const GridParams& gp, const EdgeDev* edges, int E, const FrameDev* frames, const int* cell_start,
+                  int sub, int cut_edge, const EdgeDev* edges, int E, const FrameDev* frames, const int* cell_start,
                   float4* slots, int2* units, int* n_units, const int* done, cudaStream_t st);
 void launch_pairs(const PairLaunch& L, const PairArgs& A);
 // Largest unit_queries setting of this layout: 64 for the dense tile kernel

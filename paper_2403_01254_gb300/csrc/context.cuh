@@ -66,7 +66,7 @@ struct rkhsba_ctx {
 
     long long total_bins = 0, Q_total = 0;
     int q_max = 0;                     // queries of the largest edge
-    bool cut = false;                  // units may come in parts
+    int cut_edge = 0;                  // queries up to which edges have units in parts
     int qbits = 0;                     // radix bits of the query keys
     EdgeXf* d_xf = nullptr;
     uint32_t* d_qkey = nullptr;        // home-cell key per query (then sorted)
@@ -119,6 +119,7 @@ struct rkhsba_ctx {
         a.qkey = q_sorted_key;
         a.slots = d_slots;
         a.Q = Q_total;
+        a.cut = cut_edge > 0;
         a.edges = d_edges;
         a.frames = d_frames;
         a.cell_start = d_cell_start;
@@ -128,7 +129,6 @@ struct rkhsba_ctx {
         a.acc = d_acc;
         a.units = d_units;
         a.n_units = d_ucount;
-        a.cut = cut;
         a.gp = gp;
         return a;
     }

@@ -254,8 +254,8 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
     int* d_qval_alt = cv.take<int>(Q);
     float4* d_qrec = cv.take<float4>(Q);
     float4* d_slots = cv.take<float4>(Q);
-    const bool cut = cut_possible(gp, eh, E, fh);
-    int2* d_units = cv.take<int2>(cut ? 2 * Q : Q);
+    const int cut_edge = cut_edge_for(gp, eh, E, fh, Q);
+    int2* d_units = cv.take<int2>(cut_edge ? 2 * Q : Q);
     int* d_ucount = cv.take<int>(4);
     long long* d_acc = cv.take<long long>((long long)E * ACC_N);
     EdgeOut* d_eout = reinterpret_cast<EdgeOut*>(d_block + RL.eout);
@@ -281,7 +281,7 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
     const int q_max = edge_queries_max(eh, E, fh);
     const uint32_t* qk = d_qkey;
     if (q_max <= BIN_MAX) {
-        launch_bin_edges(BinArgs{d_poses, d_edges, E, d_frames, pt_cell, d_pts4, d_cell_start, gp, UNIT_Q, d_xf, d_qkey, d_qrec, d_slots,
+        launch_bin_edges(BinArgs{d_poses, d_edges, E, d_frames, pt_cell, d_pts4, d_cell_start, gp, UNIT_Q, cut_edge, d_xf, d_qkey, d_qrec, d_slots,
                                  d_units, d_ucount, d_acc, nullptr},
                          q_max, st);
     } else {
@@ -290,7 +290,7 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
         launch_query_keys(d_edges, E, d_frames, d_xf, pt_cell, d_pts4, gp, Q, d_qkey, d_qrec, qws, num_sms, nullptr, st);
         const bool qalt = radix_sort_u32(d_qkey, d_qval, d_qkey_alt, d_qval_alt, Q, qws, d_err + 1, nullptr, st);
         qk = qalt ? d_qkey_alt : d_qkey;
-        launch_units(qk, qalt ? d_qval_alt : d_qval, d_qrec, Q, UNIT_Q, gp, d_edges, E, d_frames, d_cell_start,
+        launch_units(qk, qalt ? d_qval_alt : d_qval, d_qrec, Q, UNIT_Q, gp.key_sub, cut_edge, d_edges, E, d_frames, d_cell_start,
                      d_slots, d_units, d_ucount, nullptr, st);
     }
     {
@@ -307,7 +307,7 @@ extern "C" rkhsba_status rkhsba_eval_static(int32_t n_frames, const int64_t* n_p
         a.acc = d_acc;
         a.units = d_units;
         a.n_units = d_ucount;
-        a.cut = cut;
+        a.cut = cut_edge > 0;
         a.gp = gp;
         launch_pairs(PairLaunch{d_ucount + 1, nullptr, num_sms, 0, st}, a);
     }

@@ -213,9 +213,9 @@ __global__ void __launch_bounds__(RAD_T) k_query_keys(const EdgeDev* __restrict_
 
 // log2 of the parts that a unit of n queries of home cell `cell` comes in (see common.cuh): edge
 // and unit decide, nothing else.  n_b: queries of the edge.
-__device__ __forceinline__ int cut_shift(const GridParams& gp, const FrameDev& Fa, int n_b,
+__device__ __forceinline__ int cut_shift(int cut_edge, const FrameDev& Fa, int n_b,
                                          const int* __restrict__ cell_start, int cell, int n) {
-    if (gp.top_k > 0 || n_b > CUT_EDGE) return 0;
+    if (n_b > cut_edge) return 0;
     const int least = max(min(max(n_b >> 3, CUT_SMALL), CUT_POINTS), n_b >> 6);
     // Runs of cells by their places in the flat grid (at its very edge, where a row would leave
     // it, other cells are counted, which make as good a rule).  First, for each of the three planes, all
@@ -268,13 +268,13 @@ __device__ __forceinline__ int unit_places(bool start, int s, int lane, int& tot
 // unit list; a record holds edge and queries, so that no warp of the pair
 // kernels searches for either.
 __global__ void __launch_bounds__(256) k_units(const uint32_t* __restrict__ key, const int* __restrict__ val,
-                                               const float4* __restrict__ qrec, long long Q, int uq, GridParams gp,
+                                               const float4* __restrict__ qrec, long long Q, int uq, int sub,
+                                               int cut_edge,
                                                const EdgeDev* __restrict__ edges, int E,
                                                const FrameDev* __restrict__ frames,
                                                const int* __restrict__ cell_start,
                                                float4* __restrict__ slots, int2* __restrict__ units,
                                                int* __restrict__ n_units, const int* done) {
-    const int sub = gp.key_sub;
     chain_enter();
     if (done && *done) return;
     __shared__ int s_cnt[8], s_first[8];
@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(256) k_units(const uint32_t* __restrict__ key,
             }
             n = lo;
             e = find_edge_bin(edges, E, kk >> sub);
-            s = cut_shift(gp, frames[edges[e].a], frames[edges[e].b].n_pts, cell_start,
+            s = cut_shift(cut_edge, frames[edges[e].a], frames[edges[e].b].n_pts, cell_start,
                           (int)((kk >> sub) - edges[e].bin_off), n);
         }
         int total;
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(BIN_T) k_bin_edges(const double* __restrict__ 
                                                      const FrameDev* __restrict__ frames,
                                                      const uint32_t* __restrict__ pt_cell,
                                                      const float4* __restrict__ pts4,
-                                                     const int* __restrict__ cell_start, GridParams gp, int uq,
+                                                     const int* __restrict__ cell_start, GridParams gp, int uq, int cut_edge,
                                                      EdgeXf* __restrict__ xf, uint32_t* qkey, float4* qrec,
                                                      float4* slots, int2* units, int* n_units,
                                                      long long* __restrict__ acc, const int* done) {
@@ -551,7 +551,7 @@ __global__ void __launch_bounds__(BIN_T) k_bin_edges(const double* __restrict__ 
                 const int mid = (lo + hi) >> 1;
                 if (same(i + mid)) lo = mid + 1; else hi = mid;
             }
-            s = cut_shift(gp, Fa, n, cell_start, (int)c, lo);
+            s = cut_shift(cut_edge, Fa, n, cell_start, (int)c, lo);
             n_s[r] = lo << 2 | s;
         }
         int total;
@@ -2169,7 +2169,7 @@ void bin_edges(const BinArgs& a, cudaStream_t st) {
         opted.get(current_device(), [] { return opt_in(k_bin_edges<IPT>, smem) ? 1 : 0; });
     }
     launch_chained(k_bin_edges<IPT>, (unsigned)a.E, BIN_T, smem, st, a.poses, a.edges, a.frames, a.pt_cell, a.pts4,
-                   a.cell_start, a.gp, a.uq, a.xf,
+                   a.cell_start, a.gp, a.uq, a.cut_edge, a.xf,
                                                          a.qkey, a.qrec, a.slots, a.units, a.ucount, a.acc, a.done);
 }
 
@@ -2287,11 +2287,11 @@ void launch_query_keys(const EdgeDev* edges, int E, const FrameDev* frames, cons
 }
 
 void launch_units(const uint32_t* qkey_sorted, const int* qval_sorted, const float4* qrec, long long Q, int uq,
-                  const GridParams& gp, const EdgeDev* edges, int E, const FrameDev* frames, const int* cell_start,
+                  int sub, int cut_edge, const EdgeDev* edges, int E, const FrameDev* frames, const int* cell_start,
                   float4* slots, int2* units, int* n_units, const int* done, cudaStream_t st) {
     if (Q <= 0) return;
     if (uq < 1 || uq > UQ) uq = UQ;      // larger units are taken as units of 32
-    launch_chained(k_units, blocks_for(Q, 256), 256, 0, st, qkey_sorted, qval_sorted, qrec, Q, uq, gp, edges, E,
+    launch_chained(k_units, blocks_for(Q, 256), 256, 0, st, qkey_sorted, qval_sorted, qrec, Q, uq, sub, cut_edge, edges, E,
                    frames, cell_start, slots, units, n_units, done);
     count_launch();
 }
